@@ -1813,6 +1813,28 @@ static bmlp_status packed_operand(bmlp_ctx* ctx, const void* R, int64_t n, int32
     return to_packed(ctx, in, fmt, n, *P, words_of(n), s);
 }
 
+// Whether [a, a + na) and [b, b + nb) share a byte.
+static bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + nb && y < x + na;
+}
+
+// An operator's input on the device (host memory is staged), copied into a workspace slot when it overlaps the output
+// otherwise than as the same matrix (`same_ok`: an element-wise operator may then run in place).
+static bmlp_status operator_in(bmlp_ctx* ctx, const void* p, size_t bytes, const OutView& ov, bool same_ok, int stage_slot,
+                               int copy_slot, cudaStream_t s, const void** dev) {
+    Operand o;
+    ST(stage_in(ctx, p, bytes, stage_slot, s, &o));
+    *dev = o.dev;
+    if (!o.host && overlap(o.dev, bytes, ov.dev, ov.bytes) && !(same_ok && o.dev == ov.dev)) {
+        void* d = nullptr;
+        ST(ws_get(ctx, copy_slot, bytes, &d));
+        CK(cudaMemcpyAsync(d, o.dev, bytes, cudaMemcpyDeviceToDevice, s), "copy input");
+        *dev = d;
+    }
+    return BMLP_OK;
+}
+
 static bmlp_status core_transpose(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt, void* out, cudaStream_t s) {
     if (!ctx) return BMLP_ERR_INVALID_ARG;
     ST(op_args(ctx, n, fmt));
@@ -1821,16 +1843,23 @@ static bmlp_status core_transpose(bmlp_ctx* ctx, const void* R, int64_t n, int32
     DeviceGuard g(ctx->device);
     reset_stats(ctx, 0, n);
     const int64_t ldw = words_of(n);
-    uint64_t *P = nullptr, *PT = nullptr;
+    OutView ov;
+    ST(stage_out(ctx, out, fmt_bytes(fmt, n, n), WS_OUT, &ov));
+    if (fmt == BMLP_FMT_PACKED64) {
+        const void* in = nullptr;
+        ST(operator_in(ctx, R, ov.bytes, ov, false, WS_IN0, WS_PIPE0, s, &in));
+        CK(launch_bit_transpose(static_cast<const uint64_t*>(in), static_cast<uint64_t*>(ov.dev), n, ldw, s),
+           "transpose launch");
+        ctx->stats.launches++;
+        return finish_out(ctx, ov, s);
+    }
+    uint64_t* P = nullptr;
     ST(packed_operand(ctx, R, n, fmt, WS_IN0, WS_PIPE0, s, &P));
     void* pt = nullptr;
     ST(ws_get(ctx, WS_PIPE1, static_cast<size_t>(n * ldw * 8), &pt));
-    PT = static_cast<uint64_t*>(pt);
-    CK(launch_bit_transpose(P, PT, n, ldw, s), "transpose launch");
+    CK(launch_bit_transpose(P, static_cast<uint64_t*>(pt), n, ldw, s), "transpose launch");
     ctx->stats.launches++;
-    OutView ov;
-    ST(stage_out(ctx, out, fmt_bytes(fmt, n, n), WS_OUT, &ov));
-    ST(packed_out(ctx, PT, ldw, n, fmt, ov.dev, 0, s));
+    ST(packed_out(ctx, static_cast<uint64_t*>(pt), ldw, n, fmt, ov.dev, 0, s));
     return finish_out(ctx, ov, s);
 }
 
@@ -1841,26 +1870,35 @@ static bmlp_status core_union(bmlp_ctx* ctx, const void* A, const void* B, int64
     if (!A || !B || !out) return set_err(ctx, BMLP_ERR_INVALID_ARG, "null matrix pointer");
     DeviceGuard g(ctx->device);
     reset_stats(ctx, 0, n);
-    const int64_t ldw = words_of(n);
-    uint64_t *PA = nullptr, *PB = nullptr;
-    ST(packed_operand(ctx, A, n, fmt, WS_IN0, WS_PIPE0, s, &PA));
-    ST(packed_operand(ctx, B, n, fmt, WS_IN1, WS_PIPE1, s, &PB));
-    launch_packed_or(PA, ldw, PB, ldw, n, n, s);
-    ctx->stats.launches++;
-    CK(cudaGetLastError(), "union launch");
     OutView ov;
     ST(stage_out(ctx, out, fmt_bytes(fmt, n, n), WS_OUT, &ov));
-    ST(packed_out(ctx, PA, ldw, n, fmt, ov.dev, 0, s));
+    const void *a = nullptr, *b = nullptr;
+    ST(operator_in(ctx, A, ov.bytes, ov, true, WS_IN0, WS_PIPE0, s, &a));
+    ST(operator_in(ctx, B, ov.bytes, ov, true, WS_IN1, WS_PIPE1, s, &b));
+    if (fmt == BMLP_FMT_U8)
+        launch_u8_union(static_cast<const uint8_t*>(a), static_cast<const uint8_t*>(b), n, static_cast<uint8_t*>(ov.dev), s);
+    else
+        launch_packed_union(static_cast<const uint64_t*>(a), static_cast<const uint64_t*>(b), n,
+                            static_cast<uint64_t*>(ov.dev), s);
+    ctx->stats.launches++;
+    CK(cudaGetLastError(), "union launch");
     return finish_out(ctx, ov, s);
 }
 
-// Device view of an optional packed type vector (null = every constant).
+// Device view of an optional packed type vector (null = every constant); copied when it overlaps the output `ov`.
 static bmlp_status type_vector(bmlp_ctx* ctx, const uint64_t* v, int64_t n, int slot, cudaStream_t s,
-                               const uint64_t** dv) {
+                               const uint64_t** dv, const OutView* ov = nullptr) {
     *dv = nullptr;
     if (!v) return BMLP_OK;
+    const size_t bytes = static_cast<size_t>(words_of(n) * 8);
     Operand o;
-    ST(stage_in(ctx, v, static_cast<size_t>(words_of(n) * 8), slot, s, &o));
+    ST(stage_in(ctx, v, bytes, slot, s, &o));
+    if (ov != nullptr && !o.host && overlap(o.dev, bytes, ov->dev, ov->bytes)) {
+        void* d = nullptr;
+        ST(ws_get(ctx, slot, bytes, &d));
+        CK(cudaMemcpyAsync(d, o.dev, bytes, cudaMemcpyDeviceToDevice, s), "copy type vector");
+        o.dev = d;
+    }
     *dv = static_cast<const uint64_t*>(o.dev);
     return BMLP_OK;
 }
@@ -1874,17 +1912,19 @@ static bmlp_status core_negate(bmlp_ctx* ctx, const void* R, int64_t n, int32_t 
     DeviceGuard g(ctx->device);
     reset_stats(ctx, 0, n);
     const int64_t ldw = words_of(n);
-    uint64_t* P = nullptr;
-    ST(packed_operand(ctx, R, n, fmt, WS_IN0, WS_PIPE0, s, &P));
-    const uint64_t *dr = nullptr, *dc = nullptr;
-    ST(type_vector(ctx, rows, n, WS_SRC, s, &dr));
-    ST(type_vector(ctx, cols, n, WS_VEC0, s, &dc));
-    launch_packed_negate(P, ldw, n, dr, dc, P, ldw, s);
-    ctx->stats.launches++;
-    CK(cudaGetLastError(), "negate launch");
     OutView ov;
     ST(stage_out(ctx, out, fmt_bytes(fmt, n, n), WS_OUT, &ov));
-    ST(packed_out(ctx, P, ldw, n, fmt, ov.dev, 0, s));
+    const void* in = nullptr;
+    ST(operator_in(ctx, R, ov.bytes, ov, true, WS_IN0, WS_PIPE0, s, &in));
+    const uint64_t *dr = nullptr, *dc = nullptr;
+    ST(type_vector(ctx, rows, n, WS_SRC, s, &dr, &ov));
+    ST(type_vector(ctx, cols, n, WS_VEC0, s, &dc, &ov));
+    if (fmt == BMLP_FMT_U8)
+        launch_u8_negate(static_cast<const uint8_t*>(in), n, dr, dc, static_cast<uint8_t*>(ov.dev), s);
+    else
+        launch_packed_negate(static_cast<const uint64_t*>(in), ldw, n, dr, dc, static_cast<uint64_t*>(ov.dev), ldw, s);
+    ctx->stats.launches++;
+    CK(cudaGetLastError(), "negate launch");
     return finish_out(ctx, ov, s);
 }
 

@@ -244,6 +244,12 @@ void launch_input_block_flags(const void* in, int32_t fmt, int64_t ldw_in, int64
 // out = rows x cols AND NOT in over n x n packed rows (null vector = all constants)
 void launch_packed_negate(const uint64_t* in, int64_t ldw_in, int64_t n, const uint64_t* rows, const uint64_t* cols,
                           uint64_t* out, int64_t ldw_out, cudaStream_t s);
+// the union of two n x n matrices (packed rows of ceil(n / 64) words, or bytes) into out, and NEG on bytes (as
+// launch_packed_negate); out may be an input
+void launch_packed_union(const uint64_t* A, const uint64_t* B, int64_t n, uint64_t* out, cudaStream_t s);
+void launch_u8_union(const uint8_t* A, const uint8_t* B, int64_t n, uint8_t* out, cudaStream_t s);
+void launch_u8_negate(const uint8_t* in, int64_t n, const uint64_t* rows, const uint64_t* cols, uint8_t* out,
+                      cudaStream_t s);
 // E4M3 bytes -> 0 / 1 in place (0x00 and 0x80 are zero, any other byte one), and 0 / 1 -> E4M3 0x00 / 0x38
 void launch_e4m3_bytes_to_01(uint8_t* p, int64_t bytes, cudaStream_t s);
 void launch_01_to_e4m3_bytes(uint8_t* p, int64_t bytes, cudaStream_t s);

@@ -537,9 +537,11 @@ __device__ __forceinline__ void bit_transpose_tile(const uint64_t* __restrict__ 
 }
 
 // The whole-matrix transpose, a tile of 256 rows (4 groups of 64) x 8 words (512 columns) per block: the tile is
-// read with sector-wide loads into shared memory, transposed 64 x 64 at a time by warp ballots (all-zero blocks
-// skipped), and written as 512 output rows x 4 words (one 32-byte sector each). Every word of out, padding words
-// included, is written.
+// read with sector-wide loads into shared memory, transposed 64 x 64 at a time as four 32 x 32 blocks in registers
+// (five shuffles each; two ballots and two selects per column, as before, bound the kernel by its instructions: 57 us
+// at n = 14,541, 26 MB each way, against 16.5 us now), and written as 512 output rows x 4 words (one 32-byte sector
+// each). Every word of out, padding words included, is written; bits
+// at columns >= n are ignored (their output rows do not exist).
 constexpr int kTrRows = 256, kTrWords = 8;
 __global__ void __launch_bounds__(256) bit_transpose_kernel(const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
                                                             int64_t n, int64_t ldw) {
@@ -561,13 +563,17 @@ __global__ void __launch_bounds__(256) bit_transpose_kernel(const uint64_t* __re
         ti[k >> 3][k & 7] = v[j];
     }
     __syncthreads();
-    for (int b = warp; b < 4 * kTrWords; b += 8) {
-        const int g = b / kTrWords, w = b % kTrWords;
+#pragma unroll
+    for (int j = 0; j < kTrWords / 2; ++j) {
+        const int b = warp + 8 * j, g = b / kTrWords, w = b % kTrWords;
         const uint64_t a0 = ti[64 * g + lane][w], a1 = ti[64 * g + lane + 32][w];
-        uint64_t c0 = 0ull, c1 = 0ull;
-        if (__any_sync(FULL, (a0 | a1) != 0ull)) warp_transpose64(a0, a1, lane, c0, c1);
-        to[64 * w + lane][g] = c0;  // output row 64 (w0 + w) + lane, word 4 blockIdx.y + g
-        to[64 * w + lane + 32][g] = c1;
+        // output row lane (of the word's 64) holds rows 0 .. 31 of the group in its low half, 32 .. 63 in its high one
+        const uint32_t l0 = warp_transpose32(static_cast<uint32_t>(a0), lane);
+        const uint32_t l1 = warp_transpose32(static_cast<uint32_t>(a1), lane);
+        const uint32_t h0 = warp_transpose32(static_cast<uint32_t>(a0 >> 32), lane);
+        const uint32_t h1 = warp_transpose32(static_cast<uint32_t>(a1 >> 32), lane);
+        to[64 * w + lane][g] = static_cast<uint64_t>(l0) | (static_cast<uint64_t>(l1) << 32);
+        to[64 * w + lane + 32][g] = static_cast<uint64_t>(h0) | (static_cast<uint64_t>(h1) << 32);
     }
     __syncthreads();
     for (int k = tid; k < kTrWords * 64 * 4; k += 256) {

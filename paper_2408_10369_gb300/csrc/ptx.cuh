@@ -291,4 +291,20 @@ __host__ __device__ constexpr uint32_t idesc_mxf4_ue8m0(int M, int N) {
            (static_cast<uint32_t>(M >> 4) << 24);
 }
 
+// The 32 x 32 bit block held by a warp, one 32-bit row per lane (bit j =
+// column j), transposed: lane j receives column j (bit i = row i). Five
+// exchange stages, each swapping the off-diagonal s x s sub-blocks of every
+// 2s x 2s block between lanes L and L ^ s.
+__device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane) {
+    const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+    for (int st = 0; st < 5; ++st) {
+        const int sh = 16 >> st;
+        const uint32_t m = masks[st];  // the columns j with (j & sh) == 0
+        const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, sh);
+        x = (lane & sh) ? ((x & ~m) | ((y >> sh) & m)) : ((x & m) | ((y & m) << sh));
+    }
+    return x;
+}
+
 }  // namespace bmlp
