@@ -136,7 +136,7 @@ struct bmlp_ctx {
     int sm_count = 0;
     int clock_khz = 0;           // SM clock rate, read once (the query takes hundreds of microseconds)
     char err[512] = {0};
-    bmlp::DevBuf ws[40];
+    bmlp::DevBuf ws[48];
     void* batch = nullptr;       // cached grouped-batch graph (batch.cu)
     int tune[32];                // autotuned engine per size bucket (-1 = unknown)
     int* d_ctl = nullptr;        // device control words (see CTL_* below)
@@ -380,6 +380,12 @@ cudaError_t launch_square_cost(const int64_t* wptr, const int32_t* widx, const u
                                unsigned long long* cost, int sms, cudaStream_t s);
 // (R+ + {(u, v)})+ in place on a transitive R+ (n packed rows of ldw words)
 cudaError_t launch_insert_fact(uint64_t* P, int64_t n, int64_t ldw, int64_t u, int64_t v, int sms, cudaStream_t s);
+// The same for m <= kInsertChunk facts at once (pairs: m x 2 constants in device memory, checked by the caller) through
+// insert_chunk_words(ldw) words of scratch.
+constexpr int kInsertChunk = 1024;
+int64_t insert_chunk_words(int64_t ldw);
+cudaError_t launch_insert_chunk(uint64_t* P, int64_t n, int64_t ldw, const int32_t* pairs, int m, uint64_t* scratch,
+                                int sms, cudaStream_t s);
 // out = in^T on n x n packed rows of ldw words (every word of out written, padding words with zeros)
 cudaError_t launch_bit_transpose(const uint64_t* in, uint64_t* out, int64_t n, int64_t ldw, cudaStream_t s);
 int smp_packed_max_words();

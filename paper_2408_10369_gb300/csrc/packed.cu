@@ -1038,6 +1038,106 @@ __global__ void insert_fact_kernel(uint64_t* __restrict__ P, int64_t n, int64_t 
     }
 }
 
+// ---- incremental closure: a chunk of up to kInsertChunk facts at once on a transitive R+ (three launches)
+// With Y_k = R+_{v_k} + e_{v_k} and the links k -> l iff v_k = u_l or R+ holds (v_k, u_l), everything the grown
+// relation derives from v_k is W_k = Y_k OR (OR of Y_l over the facts l that k reaches along links), and row i gains W_k
+// for every k with i = u_k or R+ holds (i, u_k). One launch per fact, as before, costs a launch's latency each (4 to
+// 6 us) and reads one word of all n rows; a chunk reads every row once. Bound by HBM/L2 reads of the n rows when few
+// rows change, else by the words that the rows gain: n = 14,541 and 1,000 facts, 6,180 us before, 140 us now.
+// R+ is transitive, so a fact whose v_k is already in a row adds nothing that the row's other facts do not bring: if
+// i reaches v_k, it also reaches every u_l that v_k links to. The same holds for Y_l inside W_k.
+constexpr int kInsertWarps = 8;
+
+// Links of the chunk: bit l of row k of G (mw words per row). A block per fact k.
+__global__ void __launch_bounds__(kInsertWarps * 32) insert_links_kernel(const uint64_t* __restrict__ P, int64_t ldw,
+                                                                         const int32_t* __restrict__ pairs, int m, int mw,
+                                                                         uint32_t* __restrict__ G) {
+    const int k = blockIdx.x;
+    const int64_t v = pairs[2 * k + 1];
+    const uint64_t* row = P + v * ldw;
+    for (int l = threadIdx.x; l < mw * 64; l += blockDim.x) {  // whole warps run: mw * 64 is a multiple of 32
+        const int64_t u = l < m ? pairs[2 * l] : 0;
+        const unsigned b = __ballot_sync(FULL, l < m && (u == v || ((row[u >> 6] >> (u & 63)) & 1ull) != 0ull));
+        if ((l & 31) == 0) G[static_cast<int64_t>(k) * 2 * mw + (l >> 5)] = b;
+    }
+}
+
+// W_k, a warp per fact: the facts that k reaches along links by a search on G (all of it in shared memory, a lane per
+// word of the reached set), then the OR of their Y rows.
+__global__ void __launch_bounds__(kInsertWarps * 32) insert_reach_kernel(const uint64_t* __restrict__ P, int64_t n,
+                                                                         int64_t ldw, const int32_t* __restrict__ pairs,
+                                                                         int m, int mw, const uint64_t* __restrict__ G,
+                                                                         uint64_t* W) {
+    extern __shared__ uint64_t ins_g[];
+    for (int x = threadIdx.x; x < m * mw; x += blockDim.x) ins_g[x] = G[x];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int k = blockIdx.x * kInsertWarps + (threadIdx.x >> 5);
+    if (k >= m) return;
+    uint64_t reach = lane < mw ? ins_g[k * mw + lane] : 0ull;  // mw <= 32
+    uint64_t todo = reach;
+    while (true) {
+        const unsigned any = __ballot_sync(FULL, todo != 0ull);
+        if (any == 0u) break;
+        const int src = __ffs(any) - 1;
+        const int bit = __ffsll(static_cast<long long>(__shfl_sync(FULL, todo, src))) - 1;
+        if (lane == src) todo &= todo - 1ull;
+        const uint64_t more = lane < mw ? ins_g[(src * 64 + bit) * mw + lane] & ~reach : 0ull;
+        reach |= more;
+        todo |= more;
+    }
+    const int64_t wpr = (n + 63) >> 6;
+    uint64_t* w = W + static_cast<int64_t>(k) * ldw;
+    const auto add = [&](int l, bool first) {
+        const int64_t v = pairs[2 * l + 1];
+        if (!first && ((w[v >> 6] >> (v & 63)) & 1ull)) return;  // uniform: every lane reads the same word
+        const uint64_t* y = P + v * ldw;
+        __syncwarp();
+        for (int64_t x = lane; x < wpr; x += 32)
+            w[x] = (first ? 0ull : w[x]) | y[x] | (x == (v >> 6) ? 1ull << (v & 63) : 0ull);
+        __syncwarp();
+    };
+    add(k, true);
+    for (int src = 0; src < mw; ++src) {
+        uint64_t bits = __shfl_sync(FULL, reach, src);
+        while (bits) {
+            add(src * 64 + __ffsll(static_cast<long long>(bits)) - 1, false);
+            bits &= bits - 1ull;
+        }
+    }
+}
+
+// Row i gains W_k for every fact k with i = u_k or (i, u_k) in the row; a warp per row, the facts tested 32 at a time.
+__global__ void __launch_bounds__(kInsertWarps * 32) insert_rows_kernel(uint64_t* P, int64_t n, int64_t ldw,
+                                                                        const int32_t* __restrict__ pairs, int m,
+                                                                        const uint64_t* __restrict__ W) {
+    const int lane = threadIdx.x & 31;
+    const int64_t wpr = (n + 63) >> 6;
+    const int64_t warps = static_cast<int64_t>(gridDim.x) * kInsertWarps;
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * kInsertWarps + (threadIdx.x >> 5); i < n; i += warps) {
+        uint64_t* row = P + i * ldw;
+        for (int k0 = 0; k0 < m; k0 += 32) {
+            const int k = k0 + lane;
+            const int64_t u = k < m ? pairs[2 * k] : 0;
+            unsigned hit = __ballot_sync(FULL, k < m && (u == i || ((row[u >> 6] >> (u & 63)) & 1ull) != 0ull));
+            while (hit) {
+                const int kk = k0 + __ffs(hit) - 1;
+                hit &= hit - 1u;
+                const int64_t v = pairs[2 * kk + 1];
+                const bool has = ((row[v >> 6] >> (v & 63)) & 1ull) != 0ull;  // uniform
+                __syncwarp();
+                if (has) continue;
+                const uint64_t* w = W + static_cast<int64_t>(kk) * ldw;
+                for (int64_t x = lane; x < wpr; x += 32) {
+                    const uint64_t r = row[x], g = r | w[x];
+                    if (g != r) row[x] = g;
+                }
+                __syncwarp();
+            }
+        }
+    }
+}
+
 // ---- one squaring step on packed rows through the word index of R:
 // C_i = R_i | OR_{k in R_i} R_k, where row k contributes only its nonzero
 // words (push_balanced), so the cost follows the index, not n / 64 words per k.
@@ -1578,6 +1678,26 @@ cudaError_t launch_product_packed(const uint64_t* A, const uint64_t* B, uint64_t
 
 cudaError_t launch_insert_fact(uint64_t* P, int64_t n, int64_t ldw, int64_t u, int64_t v, int sms, cudaStream_t s) {
     insert_fact_kernel<<<warps_grid(n, sms), 256, 0, s>>>(P, n, ldw, u, v);
+    return cudaGetLastError();
+}
+
+int64_t insert_chunk_words(int64_t ldw) { return kInsertChunk * (kInsertChunk / 64 + ldw); }
+
+cudaError_t launch_insert_chunk(uint64_t* P, int64_t n, int64_t ldw, const int32_t* pairs, int m, uint64_t* scratch,
+                                int sms, cudaStream_t s) {
+    if (m <= 0) return cudaSuccess;
+    if (m > kInsertChunk) return cudaErrorInvalidValue;
+    const int mw = (m + 63) / 64;
+    uint64_t* G = scratch;
+    uint64_t* W = scratch + kInsertChunk * (kInsertChunk / 64);
+    const int smem = m * mw * 8;  // at most 128 KiB
+    cudaError_t e = cudaFuncSetAttribute(insert_reach_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kInsertChunk * (kInsertChunk / 64) * 8);
+    if (e != cudaSuccess) return e;
+    insert_links_kernel<<<m, kInsertWarps * 32, 0, s>>>(P, ldw, pairs, m, mw, reinterpret_cast<uint32_t*>(G));
+    insert_reach_kernel<<<(m + kInsertWarps - 1) / kInsertWarps, kInsertWarps * 32, smem, s>>>(P, n, ldw, pairs, m, mw, G,
+                                                                                              W);
+    insert_rows_kernel<<<warps_grid(n, sms), kInsertWarps * 32, 0, s>>>(P, n, ldw, pairs, m, W);
     return cudaGetLastError();
 }
 
