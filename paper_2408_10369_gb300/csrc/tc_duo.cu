@@ -21,10 +21,10 @@
 //               tcgen05.mma.cta_group::2 kind::mxf4 of M=256, N=256 into TMEM
 //               columns 0..255 and one of M=256, N=224 into columns 256..479
 //               (in each CTA); the unit scale factors fill columns 480..511;
-//   warps 2..5  epilogue (both CTAs): drains the accumulator into registers as
-//               bits and frees it at once, then computes R' = R | [C > 0],
-//               writes R' and R'^T (transposed through warp ballots) and
-//               raises `changed` if R' != R.
+//   warps 2..5  epilogue (both CTAs): loads the tile's old R while the MMAs
+//               run, drains the accumulator into registers as bits and frees
+//               it at once, then computes R' = R | [C > 0], writes R' and R'^T
+//               (transposed in registers) and raises `changed` if R' != R.
 // Every mbarrier wait is bounded; on expiry the CTA records an error code,
 // waits (bounded) for its own copies and MMAs in flight, frees TMEM and exits.
 #include <cudaTypedefs.h>
@@ -180,19 +180,6 @@ __device__ __forceinline__ void f4_drain(uint32_t taddr, uint32_t (&cb)[CHUNKS])
     }
 }
 
-// cb[c] for a run-time c through selects, so that cb stays in registers.
-template <int CHUNKS>
-__device__ __forceinline__ uint32_t f4_pick(const uint32_t (&cb)[CHUNKS], int c) {
-    uint32_t v = 0;
-#pragma unroll
-    for (int j = 0; j < CHUNKS; ++j) v = (j == c) ? cb[j] : v;
-    return v;
-}
-
-// Epilogue, part 2: R' = R | C for row (mb, quarter, lane) of the pair tile
-// whose first column is col_base: writes R' and, through warp ballots, R'^T
-// for every 32-column chunk below n_pad; returns the bits that changed
-// (nonzero in some lane iff R' != R in this warp's rows).
 // E4M3 bytes: 4 bytes -> 4 bits (bit k = byte k nonzero), and back (0 / one).
 __device__ __forceinline__ uint32_t e4_bits4(uint32_t w) {
     const uint32_t x = (((w & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w) & 0x80808080u;
@@ -225,33 +212,43 @@ __device__ __forceinline__ void store_bits32(uint8_t* p, uint32_t bits) {
     }
 }
 
+// Epilogue, part 0: the old R of this thread's row of the pair tile as bits, CHUNKS x 32 columns from col_base on
+// (chunks at or beyond n_pad: zero). All loads are issued together, before the wait for the tile's accumulator: loaded
+// chunk by chunk after it, 15 dependent rounds to L2 made most of a small product's time (n_pad = 512: 18 us a product,
+// SMALL_NOW us now; n_pad = 2,048: 22 us, MID_NOW us now).
+template <int KIND, int CHUNKS>
+__device__ __forceinline__ void f4_old(const TcParams& p, int64_t row, int64_t col_base, int64_t n_pad,
+                                       uint32_t (&ob)[CHUNKS]) {
+    constexpr int CB = KIND ? 16 : 32;  // bytes of 32 columns
+    const uint8_t* src = p.old_r + row * p.ld + col_base / 32 * CB;
+#pragma unroll
+    for (int c = 0; c < CHUNKS; ++c) ob[c] = col_base + c * 32 < n_pad ? load_bits32<KIND>(src + c * CB) : 0u;
+}
+
+// Epilogue, part 2: R' = R | C for row (mb, quarter, lane) of the pair tile
+// whose first column is col_base: writes R' and, through a 32 x 32 bit
+// transpose in registers, R'^T for every 32-column chunk below n_pad; returns
+// the bits that changed (nonzero in some lane iff R' != R in this warp's rows).
 template <int KIND, int CHUNKS>
 __device__ __forceinline__ uint32_t f4_update(const TcParams& p, int mb, int64_t col_base, int64_t n_pad, int quarter,
-                                              int lane, const uint32_t (&cb)[CHUNKS]) {
+                                              int lane, const uint32_t (&ob)[CHUNKS], const uint32_t (&cb)[CHUNKS]) {
     constexpr int CB = KIND ? 16 : 32;  // bytes of 32 columns
     const int64_t row = static_cast<int64_t>(mb) * TC_BM + quarter * 32 + lane;
     // byte of this warp's 32 rows inside a row of R'^T
     const int64_t rt_col = (static_cast<int64_t>(mb) * TC_BM + quarter * 32) / 32 * CB;
     uint32_t any = 0;
-#pragma unroll 1
+#pragma unroll
     for (int c = 0; c < CHUNKS; ++c) {
         const int64_t col0 = col_base + c * 32;
-        if (col0 >= n_pad) break;
-        const int64_t off = row * p.ld + col0 / 32 * CB;
-        const uint32_t obits = load_bits32<KIND>(p.old_r + off);
-        const uint32_t nbits = obits | f4_pick(cb, c);
-        any |= nbits ^ obits;
-        store_bits32<KIND>(p.out_r + off, nbits);
-        if (p.out_bits != nullptr) p.out_bits[row * p.ldb + col0 / 32] = nbits;
-        // column col0 + j of these 32 rows is row col0 + j of R'^T: lane j gathers it
-        uint32_t mine = 0;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            const uint32_t b = __ballot_sync(0xFFFFFFFFu, (nbits >> j) & 1u);
-            mine = (lane == j) ? b : mine;
+        if (col0 < n_pad) {
+            const uint32_t nbits = ob[c] | cb[c];
+            any |= nbits ^ ob[c];
+            store_bits32<KIND>(p.out_r + row * p.ld + col0 / 32 * CB, nbits);
+            if (p.out_bits != nullptr) p.out_bits[row * p.ldb + col0 / 32] = nbits;
+            const uint32_t mine = warp_transpose32(nbits, lane);  // column col0 + lane of the warp's 32 rows
+            store_bits32<KIND>(p.out_rt + (col0 + lane) * p.ld + rt_col, mine);
+            if (p.out_bits_t != nullptr) p.out_bits_t[(col0 + lane) * p.ldb + rt_col / CB] = mine;
         }
-        store_bits32<KIND>(p.out_rt + (col0 + lane) * p.ld + rt_col, mine);
-        if (p.out_bits_t != nullptr) p.out_bits_t[(col0 + lane) * p.ldb + rt_col / CB] = mine;
     }
     return any;
 }
@@ -458,6 +455,9 @@ tc_duo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             int mp, nb;
             f4_pair_coords(t, m_pairs, p.n_tiles, mp, nb);
             const int mb = 2 * mp + static_cast<int>(rank);
+            uint32_t ob[C::CHUNKS];
+            f4_old<KIND, C::CHUNKS>(p, static_cast<int64_t>(mb) * TC_BM + quarter * 32 + lane,
+                                    static_cast<int64_t>(nb) * C::BN, n_pad, ob);
             if (!f4_wait_lane0(tfull, acc_phase, abort_flag, limit, lane)) {
                 if (lane == 0) atomicCAS(p.error, 0, ERR_D_EPILOGUE);
                 break;
@@ -471,7 +471,7 @@ tc_duo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             mbar_arrive_cluster(tempty_even);
             acc_phase ^= 1u;
             const uint32_t any =
-                f4_update<KIND, C::CHUNKS>(p, mb, static_cast<int64_t>(nb) * C::BN, n_pad, quarter, lane, cb);
+                f4_update<KIND, C::CHUNKS>(p, mb, static_cast<int64_t>(nb) * C::BN, n_pad, quarter, lane, ob, cb);
             if (__any_sync(0xFFFFFFFFu, any != 0) && lane == 0) atomicOr(p.changed, 1);
         }
     }
