@@ -336,6 +336,85 @@ bool tc_skip_enabled() {
     return on;
 }
 
+// Squarings issued before the host first looks at their flags, and from then on. The host's wait, its flag read and the
+// next launch cost about 20 us a squaring when done after each, more than a product of n <= 3,000 (11 to 20 us); a
+// squaring issued in vain leaves at its guard (about 3 us). Uniform random relations of that size close in 5 or 6.
+constexpr int kChainFirst = 6, kChainNext = 3;
+static_assert(kChainFirst <= 8 && kChainNext <= 8, "CTL_STEP holds eight flags");
+
+// Squarings on packed E2M1 R, R^T (Q[0], QT[0], ping-pong with Q[1], QT[1]; bit rows of the new R and R^T into P, PT when
+// not null) until one changes nothing, several at a time: each is guarded by the flag of the one before it and raises
+// its own, so that the ones after the fixpoint do nothing. after(): issued behind every group, before the host waits
+// (the decoding of P, which holds the last R whether or not it is the closure). *cur: the buffer that holds R.
+template <class After>
+bmlp_status rms_f4_chain(bmlp_ctx* ctx, int64_t n_pad, uint8_t* const Q[2], uint8_t* const QT[2], uint64_t* P, uint64_t* PT,
+                         int max_iters, const bmlp_options& o, cudaStream_t s, int* iters, int* cur, After&& after) {
+    NvtxRange nvtx_("tensor-core squarings");
+    const int64_t ld4 = n_pad / 2;
+    CUtensorMap mA[2], mB0[2], mB1[2];
+    for (int b = 0; b < 2; ++b) {
+        ST(make_tmap(ctx, &mA[b], Q[b], n_pad, ld4, ld4, TC_BM));
+        ST(make_tmap(ctx, &mB0[b], QT[b], n_pad, ld4, ld4, TC_BN / 2));
+        ST(make_tmap(ctx, &mB1[b], QT[b], n_pad, ld4, ld4, tc4_b1_rows()));
+    }
+    TcParams p{};
+    p.m_tiles = static_cast<int32_t>(n_pad / TC_BM);
+    p.n_tiles = static_cast<int32_t>((n_pad + tc4_tile_n() - 1) / tc4_tile_n());
+    p.k_blocks = static_cast<int32_t>(n_pad / 256);
+    p.mode = TC_MODE_RMS;
+    p.ld = ld4;
+    p.error = ctx->d_ctl + CTL_ERROR;
+    p.wait_cycles = wait_cycles(ctx, o);
+    p.issued = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_ISSUED);
+    if (P != nullptr) {
+        p.out_bits = reinterpret_cast<uint32_t*>(P);
+        p.out_bits_t = reinterpret_cast<uint32_t*>(PT);
+        p.ldb = n_pad / 32;
+    }
+    *iters = 0;
+    while (*iters < max_iters) {
+        const int c = std::min(max_iters - *iters, *iters == 0 ? kChainFirst : kChainNext);
+        CK(cudaMemsetAsync(ctx->d_ctl + CTL_STEP, 0, static_cast<size_t>(c) * sizeof(int), s), "reset flags");
+        for (int k = 0; k < c; ++k) {
+            const int b = (*iters + k) & 1;
+            p.old_r = Q[b];
+            p.out_r = Q[b ^ 1];
+            p.out_rt = QT[b ^ 1];
+            p.changed = ctx->d_ctl + CTL_STEP + k;
+            p.guard = k > 0 ? ctx->d_ctl + CTL_STEP + k - 1 : nullptr;
+            CK(launch_tc4_product_duo(mA[b], mB0[b], mB1[b], p, ctx->sm_count, s), "tensor-core product launch");
+        }
+        ST(after());
+        ST(read_ctl(ctx, s, nullptr));
+        int ran = 1;  // squaring k ran iff the one before it changed R
+        while (ran < c && ctx->h_ctl[CTL_STEP + ran - 1] != 0) ++ran;
+        const bool done = ctx->h_ctl[CTL_STEP + ran - 1] == 0;
+        *iters += ran;
+        ctx->stats.product_launches += ran;
+        ctx->stats.e2m1_products += ran;
+        ctx->stats.launches += c;
+        *cur = *iters & 1;
+        unsigned long long kbs = 0;
+        memcpy(&kbs, ctx->h_ctl + CTL_ISSUED, sizeof(kbs));
+        ctx->stats.issued_ops = 2.0 * TC_BM * 32.0 * TC_BK * static_cast<double>(kbs);
+        if (done) return BMLP_OK;
+    }
+    return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "no fixpoint within %d products", max_iters);
+}
+
+bool thin_allowed(int64_t n_pad, const bmlp_options& o);
+// Whether the 4-bit squarings of a call are issued several at a time: sizes whose product is cheaper than a host wait
+// (n_pad = 4,096: 33 us), no squaring restricted to zeros among them, and no need of the host between two products (a
+// time budget is checked there, and options.profile times each).
+bool chain_allowed(int64_t n_pad, const bmlp_options& o) {
+    return n_pad <= 4096 && o.profile == 0 && o.budget_ns == 0 && !thin_allowed(n_pad, o);
+}
+
+// Whether squarings on n_pad x n_pad 4-bit operands may run restricted to the rows and columns holding zeros.
+bool thin_allowed(int64_t n_pad, const bmlp_options& o) {
+    return !o.tc_only && thin_enabled() && thin_fixed_s(n_pad) < tc4_product_s(n_pad);
+}
+
 // ------------------------------------------------------------------------
 // Tensor-core squaring fixpoint on E4M3 R / R^T buffers already encoded in
 // (M[0], T[0]). On return *res points at the buffer holding R1+ (and *res_t at
@@ -426,7 +505,7 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
     // Once a 4-bit squaring has run, the next one is first sized on the rows and columns of R that still hold
     // zeros (thin.cu); when those hold few ones, it runs there, on bit rows, at a fraction of a dense product.
     const int64_t ldw_t = n_pad / 64;
-    const bool thin_on = !o.tc_only && thin_enabled() && thin_fixed_s(n_pad) < tc4_product_s(n_pad);
+    const bool thin_on = thin_allowed(n_pad, o);
     bool thin_try = false;  // the last 4-bit squaring left R dense enough (sampled) to size the next one
     // bit rows of R and R^T (n_pad rows each): written by every 4-bit squaring's epilogue when the caller takes the
     // result from them (res_bits), kept by the restricted squarings; bits_current once a squaring has written them
@@ -744,12 +823,16 @@ bmlp_status rms_packed_loop(bmlp_ctx* ctx, int64_t n, int64_t ldw, uint64_t* P[2
     return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "no fixpoint within %d products", max_iters);
 }
 
+// Matrices up to this size run on 4-bit operands whatever their block map: a whole product takes at most 15 us there,
+// less than the map, its read-back and a block-skipping E4M3 squaring (40 us with its maps).
+constexpr int64_t kAlwaysDenseN = 2048;
+
 // Whether R (format fmt; packed rows of ldw words) is dense by its 128 x 128 block map: then a closure starts on
 // 4-bit operands and leaves from them, else on E4M3 with empty K blocks skipped.
 bmlp_status dense_by_blocks(bmlp_ctx* ctx, const Operand& src, int32_t fmt, int64_t ldw, int64_t n, int64_t n_pad,
                             cudaStream_t s, bool* dense) {
     const int64_t kb = n_pad / 128;
-    *dense = !tc_skip_enabled() || kb > 256;
+    *dense = !tc_skip_enabled() || kb > 256 || n_pad <= kAlwaysDenseN;
     if (*dense) return BMLP_OK;
     void* f = nullptr;
     ST(ws_get(ctx, WS_F0, static_cast<size_t>(kb * kb), &f));
@@ -1414,6 +1497,25 @@ static bmlp_status core_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt
             ctx->stats.launches++;
             const uint8_t* q = nullptr;
             const uint64_t* qb = nullptr;
+            if (chain_allowed(n_pad, o)) {
+                // squarings of this size are issued several at a time, the decoding behind them
+                const size_t half = static_cast<size_t>(n_pad) * static_cast<size_t>(ld4);
+                const int64_t ldb = n_pad / 64;
+                uint8_t* const Q[2] = {M[1], M[1] + half};
+                uint8_t* const QT[2] = {T[1], T[1] + half};
+                void* pp = nullptr;
+                ST(ws_get(ctx, WS_THIN_P, static_cast<size_t>(2 * n_pad * ldb * 8), &pp));
+                uint64_t* P = static_cast<uint64_t*>(pp);
+                int cur = 0;
+                st = rms_f4_chain(ctx, n_pad, Q, QT, P, P + n_pad * ldb, max_iters - sp.iters, o, s, &iters, &cur, [&]() {
+                    return packed_out(ctx, P, ldb, n, fmt, ov.dev, o.reflexive, s);
+                });
+                if (st != BMLP_OK && st != BMLP_ERR_NOT_CONVERGED) return st;
+                iters += sp.iters;
+                ctx->stats.iterations = iters;
+                if (iters_out) *iters_out = iters;
+                return st == BMLP_OK ? finish_out(ctx, ov, s) : st;
+            }
             st = rms_tc_loop(ctx, n, n_pad, M, T, max_iters - sp.iters, o, s, &iters, &res, &res_t, &q, &qb);
             if ((st == BMLP_OK || st == BMLP_ERR_NOT_CONVERGED) && qb != nullptr) {
                 // the squarings kept R as bit rows: the result leaves from them
@@ -1650,7 +1752,14 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
             ctx->stats.launches++;
             const uint8_t* q = M[1];  // the closure already, when the bit-row squarings reached it
             st = BMLP_OK;
-            if (!sp.done) {
+            if (!sp.done && chain_allowed(n_pad, o)) {
+                uint8_t* const Q[2] = {M[1], M[1] + half};
+                uint8_t* const QT[2] = {T[1], T[1] + half};
+                int cur = 0;
+                st = rms_f4_chain(ctx, n_pad, Q, QT, nullptr, nullptr, max_iters - sp.iters, o, s, &iters, &cur,
+                                  []() { return BMLP_OK; });
+                q = Q[cur];
+            } else if (!sp.done) {
                 uint8_t *res = nullptr, *res_t = nullptr;
                 st = rms_tc_loop(ctx, n, n_pad, M, T, max_iters - sp.iters, o, s, &iters, &res, &res_t, &q);
             }

@@ -155,7 +155,8 @@ namespace bmlp {
 // a bit-row squaring wrote) two of them and CTL_THIN eight (two ints each, 8-byte aligned).
 enum CtlWord : int {
     CTL_CHANGED = 0, CTL_ERROR = 1, CTL_ITERS = 2, CTL_LEVELS = 3, CTL_QCOUNT = 4, CTL_T0 = 6, CTL_BUDGET = 8,
-    CTL_ISSUED = 10, CTL_COST = 12, CTL_THIN = 16, CTL_BITS = 32, CTL_PSTAT = 34, CTL_WORDS = 38
+    CTL_ISSUED = 10, CTL_COST = 12, CTL_THIN = 16, CTL_BITS = 32, CTL_PSTAT = 34, CTL_STEP = 38,
+    CTL_WORDS = 38 + 8
 };
 // The pinned host mirror has two more ints: CTL_HOST_I64 is a 64-bit slot for values read from elsewhere.
 constexpr int CTL_HOST_I64 = CTL_WORDS;

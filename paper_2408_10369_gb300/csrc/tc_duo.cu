@@ -214,8 +214,8 @@ __device__ __forceinline__ void store_bits32(uint8_t* p, uint32_t bits) {
 
 // Epilogue, part 0: the old R of this thread's row of the pair tile as bits, CHUNKS x 32 columns from col_base on
 // (chunks at or beyond n_pad: zero). All loads are issued together, before the wait for the tile's accumulator: loaded
-// chunk by chunk after it, 15 dependent rounds to L2 made most of a small product's time (n_pad = 512: 18 us a product,
-// SMALL_NOW us now; n_pad = 2,048: 22 us, MID_NOW us now).
+// chunk by chunk after it, 15 dependent rounds to L2 made most of a small product's time (n_pad = 512: 18.1 us a
+// product, 11.6 us now; 2,048: 21.8 and 15.3 us; 5,120: 62 and 54 us).
 template <int KIND, int CHUNKS>
 __device__ __forceinline__ void f4_old(const TcParams& p, int64_t row, int64_t col_base, int64_t n_pad,
                                        uint32_t (&ob)[CHUNKS]) {
