@@ -159,10 +159,12 @@ typedef struct bmlp_stats {
                                   the cluster's shared memory (query batches,
                                   and closures whose columns are skewed)        */
     int32_t thin_squarings;    /* BMLP_RMS_TC: squarings computed only on the
-                                  rows and columns of R that still held zeros
-                                  (few, and holding few ones: R close to its
-                                  closure); counted in iterations, not in
-                                  product_launches                              */
+                                  rows and columns that still held zeros (few,
+                                  and holding few ones: R close to its closure,
+                                  or dense enough that a product over a slice
+                                  of the constants leaves few zeros open);
+                                  counted in iterations, not in
+                                  product_launches or issued_ops                */
     int32_t table_squarings;   /* BMLP_RMS_PACKED: whole-row squarings run on
                                   shared-memory tables of 4-row ORs (Four
                                   Russians; once R's nonzero words hold >= 10

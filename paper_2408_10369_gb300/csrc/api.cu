@@ -132,18 +132,25 @@ constexpr double kClusterClosureSkew = 6.5;
 constexpr int64_t kSlicedMinQueries = 64;
 // Fraction of nonzero 128 x 128 blocks of R below which a squaring skips empty K blocks.
 constexpr double kSkipMaxDensity = 0.5;
-// Fixed device and host time of a squaring restricted to the rows and columns of R that hold zeros: the bit rows of
-// R and R^T (reading both E2M1 matrices, writing both bit-row copies and reading R's again: about 1.4 bytes per
-// entry at about 6 TB/s), the row and column lists and two flag read-backs; the row ORs are costed per word as the
-// bit-row squarings' are.
+// Fixed device and host time of a squaring restricted to the rows and columns that hold zeros: one pass over each bit-row
+// copy (n_pad^2 / 4 bytes at about 4 TB/s), the lists, five launches and two flag read-backs; its row ORs are costed by
+// thin_word_s() and thin_one_s().
 double thin_fixed_s(int64_t n_pad) {
-    return 30e-6 + static_cast<double>(n_pad) * static_cast<double>(n_pad) * 1.4 / 6.0e12;
+    return 35e-6 + static_cast<double>(n_pad) * static_cast<double>(n_pad) * 0.25 / 4.0e12;
 }
+// A squaring whose R is dense in most rows, but not yet saturated, starts with a product over 1 / kSliceParts of k. An
+// entry of R' whose row and column hold fractions dr and dc of ones stays open after it with probability
+// (1 - dr dc)^(n / kSliceParts), so a row with dr dc n / kSliceParts >= kSliceMinHits (dc: the mean of the sampled rows)
+// is taken to be filled, and the others to be left to the restricted squaring; the slice is tried when that is predicted
+// to cost less than kSliceMaxCost of a whole product. When more is left than that, the product goes on over the rest of
+// k: nothing is computed twice, at the cost of one more epilogue and the statistics, and the call tries no other slice.
+constexpr int kSliceParts = 8;
+constexpr double kSliceMinHits = 20.0;
+constexpr double kSliceMaxCost = 0.5;
 // The rows and columns holding zeros are sized only after a squaring whose R, in kThinSampleRows rows spread over it,
 // has its rows with at least n / 2 ones within this fraction of n of one another in count (the rows that reach most
 // constants are saturated, their zeros in common columns).
 constexpr double kThinRowSpread = 1.0 / 32.0;
-constexpr int kThinSampleRows = 256;
 
 struct DeviceGuard {
     int prev = -1;
@@ -256,7 +263,7 @@ double now_s() {
 bmlp_status begin_call(bmlp_ctx* ctx, const bmlp_options& o, cudaStream_t s) {
     ctx->t_call = now_s();
     ctx->budget_ns = o.budget_ns;
-    CK(cudaMemsetAsync(ctx->d_ctl, 0, CTL_WORDS * sizeof(int), s), "reset flags");
+    CK(cudaMemsetAsync(ctx->d_ctl, 0, CTL_SAMPLE * sizeof(int), s), "reset flags");
     return BMLP_OK;
 }
 
@@ -265,8 +272,10 @@ Deadline deadline_of(bmlp_ctx* ctx) {
                     ctx->d_ctl + CTL_BUDGET};
 }
 
-bmlp_status read_ctl(bmlp_ctx* ctx, cudaStream_t s, int* changed) {
-    CK(cudaMemcpyAsync(ctx->h_ctl, ctx->d_ctl, CTL_WORDS * sizeof(int), cudaMemcpyDeviceToHost, s), "read flags");
+bmlp_status read_ctl(bmlp_ctx* ctx, cudaStream_t s, int* changed, bool with_sample = false) {
+    CK(cudaMemcpyAsync(ctx->h_ctl, ctx->d_ctl, (with_sample ? CTL_WORDS : CTL_SAMPLE) * sizeof(int), cudaMemcpyDeviceToHost,
+                       s),
+       "read flags");
     CK(host_sync(ctx, s), "synchronise iteration");
     if (ctx->h_ctl[CTL_ERROR] != 0)
         return set_err(ctx, BMLP_ERR_TIMEOUT, "in-kernel wait timed out (code 0x%x)", ctx->h_ctl[CTL_ERROR]);
@@ -506,56 +515,95 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
     // zeros (thin.cu); when those hold few ones, it runs there, on bit rows, at a fraction of a dense product.
     const int64_t ldw_t = n_pad / 64;
     const bool thin_on = thin_allowed(n_pad, o);
-    bool thin_try = false;  // the last 4-bit squaring left R dense enough (sampled) to size the next one
-    // bit rows of R and R^T (n_pad rows each): written by every 4-bit squaring's epilogue when the caller takes the
-    // result from them (res_bits), kept by the restricted squarings; bits_current once a squaring has written them
-    uint64_t* P = nullptr;
-    uint64_t* PT = nullptr;
-    bool bits_current = false;
+    // The two ways are chosen by a sample of R's rows after each product: thin_try (R close to its closure: no product at
+    // all), slice_try (dense, not saturated: a product over a slice of k first).
+    bool thin_try = false, slice_try = false, slice_failed = false;
+    // bit rows of R and R^T (n_pad rows each), written by every 4-bit squaring's epilogue when the caller takes the
+    // result from them (res_bits) or a restricted squaring may need them; two pairs, since a sliced squaring reads R's
+    // while it completes R''s. bits_current: pair bcur holds R. q_current: the E2M1 pair qcur holds R too (a restricted
+    // squaring writes bit rows only; they are converted when a product needs operands again).
+    uint64_t* P[2] = {nullptr, nullptr};
+    uint64_t* PT[2] = {nullptr, nullptr};
+    int bcur = 0;
+    bool bits_current = false, q_current = true;
     if (thin_on || res_bits != nullptr) {
+        const size_t one = static_cast<size_t>(n_pad * ldw_t);
         void* pp = nullptr;
-        ST(ws_get(ctx, WS_THIN_P, static_cast<size_t>(2 * n_pad * ldw_t * 8), &pp));
-        P = static_cast<uint64_t*>(pp);
-        PT = P + n_pad * ldw_t;
+        ST(ws_get(ctx, WS_THIN_P, (thin_on ? 4 : 2) * one * 8, &pp));
+        P[0] = P[1] = static_cast<uint64_t*>(pp);
+        PT[0] = PT[1] = P[0] + one;
+        if (thin_on) {
+            P[1] = PT[0] + one;
+            PT[1] = P[1] + one;
+        }
     }
     if (res_bits != nullptr) *res_bits = nullptr;
-    auto thin_step = [&](bool* ran, int* changed) -> bmlp_status {
+    auto operands_current = [&]() -> bmlp_status {
+        if (q_current) return BMLP_OK;
+        launch_packed_to_e2m1(P[bcur], ldw_t, n, Q[qcur], QT[qcur], n_pad, s);
+        CK(cudaGetLastError(), "E2M1 encode");
+        ctx->stats.launches++;
+        q_current = true;
+        return BMLP_OK;
+    };
+    // The squaring of R (bit pair r) completed from S (bit pair c) on the rows and columns of S that hold zeros, unless
+    // that is predicted to cost more than `limit` seconds. CTL_OPEN is raised when it stops with some zeros open
+    // (launch_thin_squaring); S = R is then left as it is.
+    auto thin_step = [&](int c, int r, double limit, bool* ran) -> bmlp_status {
         *ran = false;
         void* aux = nullptr;
-        const size_t aux_bytes = static_cast<size_t>(2 * n * 8 + (ldw_t + 1) * 8 + 2 * n * 4);
-        ST(ws_get(ctx, WS_THIN_AUX, aux_bytes, &aux));
-        int64_t* rowcnt = static_cast<int64_t*>(aux);
-        int64_t* colcnt = rowcnt + n;
-        uint64_t* Bmask = reinterpret_cast<uint64_t*>(colcnt + n);
-        int32_t* blist = reinterpret_cast<int32_t*>(Bmask + ldw_t + 1);
-        int32_t* rlist = blist + n;
+        ST(ws_get(ctx, WS_THIN_AUX, thin_aux_bytes(n, ldw_t), &aux));
+        const ThinLists lists = thin_lists(aux, n, ldw_t);
         auto* stat = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_THIN);
-        CK(launch_thin_stats(Q[qcur], QT[qcur], ld4, n, P, PT, ldw_t, rowcnt, colcnt, Bmask, blist, rlist, stat,
-                             bits_current, ctx->sm_count, s),
-           "thin squaring statistics");
-        bits_current = true;  // P, PT hold R, R^T from here on (converted, or already there)
-        ctx->stats.launches += 4;
+        CK(launch_thin_stats(n, P[c], PT[c], P[r], PT[r], ldw_t, lists, stat, ctx->sm_count, s), "thin squaring statistics");
+        ctx->stats.launches += 3;
         ST(read_ctl(ctx, s, nullptr));
         unsigned long long st[6];
         memcpy(st, ctx->h_ctl + CTL_THIN, sizeof(st));
-        // the word ORs over the GPU, or one warp's list entry with the most ones, whichever takes longer
+        // the word ORs over the GPU, or one list entry with the most ones, whichever takes longer
         const double words = static_cast<double>(st[2] + st[3]) * static_cast<double>(ldw_t);
-        const double row_words = static_cast<double>(st[4] > st[5] ? st[4] : st[5]) * static_cast<double>(ldw_t);
-        const double t = thin_fixed_s(n_pad) + std::max(words * bitrow_s_per_word(), row_words * bitrow_row_s_per_word());
-        if (t >= tc4_product_s(n_pad)) return BMLP_OK;
-        const int64_t nb = static_cast<int64_t>(st[0]), nr = static_cast<int64_t>(st[1]);
-        void* tt = nullptr;
-        ST(ws_get(ctx, WS_THIN_T, static_cast<size_t>((nb + nr + 1) * ldw_t * 8), &tt));
-        uint64_t* T1 = static_cast<uint64_t*>(tt);
-        CK(launch_thin_squaring(P, PT, ldw_t, blist, nb, rlist, nr, T1, T1 + nb * ldw_t, Q[qcur], QT[qcur], ld4,
-                                ctx->d_ctl + CTL_CHANGED, ctx->sm_count, s),
-           "thin squaring");
-        ctx->stats.launches += 4;
-        ctx->stats.thin_squarings++;
-        ST(read_ctl(ctx, s, changed));
+        const double top = static_cast<double>(st[4] > st[5] ? st[4] : st[5]);
+        if (thin_fixed_s(n_pad) + std::max(words * thin_word_s(), top * thin_one_s()) >= limit) return BMLP_OK;
+        const int64_t entries = static_cast<int64_t>(st[0] + st[1]);
+        if (entries > 0) {
+            void* tt = nullptr;
+            ST(ws_get(ctx, WS_THIN_T, static_cast<size_t>(entries * ldw_t * 8), &tt));
+            CK(launch_thin_squaring(n, P[c], PT[c], P[r], PT[r], ldw_t, lists, stat, entries, static_cast<uint64_t*>(tt),
+                                    nullptr, nullptr, ld4, ctx->d_ctl + CTL_CHANGED, ctx->d_ctl + CTL_OPEN, c == r,
+                                    ctx->sm_count, s),
+               "thin squaring");
+            ctx->stats.launches += 2;
+        }
         *ran = true;
         return BMLP_OK;
     };
+    // A sample of the rows of the new R (bit pair c): read back with the changed flag ...
+    auto* const d_sample = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_THIN) + 6;
+    auto sample = [&](int c) -> bmlp_status {
+        CK(cudaMemsetAsync(d_sample, 0, 2 * sizeof(unsigned long long), s), "reset row sample");
+        CK(launch_thin_sample(P[c], ldw_t, n, kThinSampleRows, d_sample, ctx->d_ctl + CTL_SAMPLE, s), "row sample");
+        ctx->stats.launches++;
+        return BMLP_OK;
+    };
+    // ... and what it says about the next squaring: every zero of a row that reaches most constants must lie in the few
+    // columns of B, so such rows have (nearly) the same count; or most rows are dense.
+    auto judge = [&]() {
+        unsigned long long smp[2];
+        memcpy(smp, ctx->h_ctl + CTL_THIN + 12, sizeof(smp));
+        const int* ones = ctx->h_ctl + CTL_SAMPLE;
+        const double nn = static_cast<double>(n), per_row = nn / kThinSampleRows;
+        thin_try = smp[0] > 0 && static_cast<double>(smp[0]) - (nn - static_cast<double>(smp[1])) <= kThinRowSpread * nn;
+        double mean = 0.0, left = 0.0;
+        for (int r = 0; r < kThinSampleRows; ++r) mean += ones[r] / (nn * kThinSampleRows);
+        for (int r = 0; r < kThinSampleRows; ++r)
+            if (ones[r] * mean < kSliceMinHits * kSliceParts) left += std::min(ones[r], kThinCap) * per_row;
+        // the columns are taken to leave as much as the rows
+        const double t = thin_fixed_s(n_pad) + 2.0 * left * static_cast<double>(ldw_t) * thin_word_s();
+        const double whole = tc4_product_s(n_pad);
+        slice_try = !slice_failed && mean > 0.0 && t + whole / kSliceParts < kSliceMaxCost * whole;
+    };
+    unsigned long long last_kbs = 0;  // the issued count after the last whole product
+    double sliced_kbs = 0.0;          // what slices that were completed by the rest of k issued
     int cur = 0;
     *iters = 0;
     if (res_f4 != nullptr) {
@@ -576,7 +624,7 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
     }
     for (int it = 0; it < max_iters; ++it) {
         const int nxt = cur ^ 1;
-        CK(cudaMemsetAsync(ctx->d_ctl, 0, 2 * sizeof(int), s), "reset flags");
+        CK(cudaMemsetAsync(ctx->d_ctl, 0, 3 * sizeof(int), s), "reset flags");  // CTL_CHANGED, CTL_ERROR, CTL_OPEN
         if (fp4 && !use_maps && !on_f4) {
             sw = cur;
             const size_t half = static_cast<size_t>(n_pad) * static_cast<size_t>(ld4);
@@ -596,25 +644,37 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
             on_f4 = true;
             qcur = 0;
         }
-        if (on_f4 && thin_try) {
-            bool ran = false;
-            int changed = 0;
-            ST(thin_step(&ran, &changed));
-            if (ran) {
-                *iters = it + 1;
-                if (!changed) {  // R is its closure; Q[qcur], QT[qcur] hold it
-                    if (res_f4 != nullptr) {
-                        *res_f4 = Q[qcur];
-                        if (res_bits != nullptr && bits_current) *res_bits = P;
-                        *res = *res_t = nullptr;
-                        return BMLP_OK;
-                    }
-                    return finish_f4(res, res_t);
-                }
-                continue;
-            }
-        }
         if (on_f4) {
+            auto converged = [&](uint8_t** r, uint8_t** rt) -> bmlp_status {  // Q[qcur], QT[qcur] hold the closure
+                if (res_bits != nullptr && bits_current) {
+                    *res_bits = P[bcur];
+                    *res_f4 = nullptr;
+                    *r = *rt = nullptr;
+                    return BMLP_OK;
+                }
+                ST(operands_current());
+                if (res_f4 == nullptr) return finish_f4(r, rt);
+                *res_f4 = Q[qcur];
+                *r = *rt = nullptr;
+                return BMLP_OK;
+            };
+            int changed = 0;
+            if (thin_try && bits_current) {
+                bool ran = false;
+                ST(thin_step(bcur, bcur, tc4_product_s(n_pad), &ran));
+                if (ran) {
+                    ST(read_ctl(ctx, s, &changed));
+                    if (ctx->h_ctl[CTL_OPEN] == 0) {
+                        ctx->stats.thin_squarings++;
+                        *iters = it + 1;
+                        if (!changed) return converged(res, res_t);
+                        q_current = false;
+                        continue;
+                    }
+                    thin_try = false;  // some zeros need more of their rows: R is as it was
+                }
+            }
+            ST(operands_current());
             TcParams p4 = p;
             p4.ld = ld4;
             p4.k_blocks = static_cast<int32_t>(n_pad / 256);
@@ -623,55 +683,67 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
             p4.old_r = Q[qcur];
             p4.out_r = Q[qcur ^ 1];
             p4.out_rt = QT[qcur ^ 1];
-            // the epilogue writes the bit rows too when the result leaves from them, or a restricted squaring may
-            // follow (which then needs no conversion from E2M1)
-            const bool bits_out = P != nullptr && (res_bits != nullptr || thin_on);
-            if (bits_out) {
-                p4.out_bits = reinterpret_cast<uint32_t*>(P);
-                p4.out_bits_t = reinterpret_cast<uint32_t*>(PT);
+            if (P[0] != nullptr) {
+                p4.out_bits = reinterpret_cast<uint32_t*>(P[bcur ^ 1]);
+                p4.out_bits_t = reinterpret_cast<uint32_t*>(PT[bcur ^ 1]);
                 p4.ldb = 2 * ldw_t;
+                if (bits_current) p4.old_bits = reinterpret_cast<uint32_t*>(P[bcur]);
             }
-            ST(tm.begin());
-            CK(launch_tc4_product_duo(mapA4[qcur], mapB4[qcur], mapB4x[qcur], p4, ctx->sm_count, s),
-               "tensor-core product launch");
-            ST(tm.end());
-            ctx->stats.product_launches++;
-            ctx->stats.e2m1_products++;
-            ctx->stats.launches += 2;
-            bits_current = bits_out;
-            auto* sample = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_THIN) + 6;
-            if (thin_on) {
-                // whether the rows of the new R that reach most constants are saturated (a sample of 256 rows),
-                // read back with the changed flag
-                CK(cudaMemsetAsync(sample, 0, 2 * sizeof(unsigned long long), s), "reset row sample");
-                CK(launch_thin_sample(Q[qcur ^ 1], ld4, n, kThinSampleRows, sample, s), "row sample");
+            auto product = [&]() -> bmlp_status {
                 ctx->stats.launches++;
-            }
-            int changed = 0;
-            ST(read_ctl(ctx, s, &changed));
-            ST(tm.collect());
-            unsigned long long kbs = 0;
-            memcpy(&kbs, ctx->h_ctl + CTL_ISSUED, sizeof(kbs));
-            ctx->stats.issued_ops = 2.0 * TC_BM * 32.0 * TC_BK * static_cast<double>(kbs);
-            *iters = it + 1;
-            qcur ^= 1;
-            if (!changed) {
-                if (res_f4 != nullptr) {
-                    *res_f4 = Q[qcur];
-                    if (res_bits != nullptr && bits_current) *res_bits = P;
-                    *res = *res_t = nullptr;
-                    return BMLP_OK;
+                ST(tm.begin());
+                CK(launch_tc4_product_duo(mapA4[qcur], mapB4[qcur], mapB4x[qcur], p4, ctx->sm_count, s),
+                   "tensor-core product launch");
+                ST(tm.end());
+                return BMLP_OK;
+            };
+            bool sliced = false;  // the squaring is a slice completed by a restricted one
+            double slice_share = 0.0;
+            if (slice_try && bits_current) {
+                TcParams whole = p4;
+                const int slice = std::max(1, p4.k_blocks / kSliceParts);
+                p4.k_blocks = slice;
+                p4.issued = nullptr;  // a slice that a restricted squaring completes is in no product count or time
+                p4.out_r = p4.out_rt = nullptr;  // S as bit rows only
+                ST(product());
+                ST(thin_step(bcur ^ 1, bcur, 0.8 * tc4_product_s(n_pad), &sliced));
+                if (sliced) {
+                    ST(sample(bcur ^ 1));
+                    ST(read_ctl(ctx, s, &changed, true));
+                    sliced = ctx->h_ctl[CTL_OPEN] == 0;
                 }
-                return finish_f4(res, res_t);
+                if (!sliced) {  // the rest of k, on top of S in place; slice and rest count as one product
+                    ST(tm.collect());
+                    slice_failed = true;
+                    slice_share = static_cast<double>(slice) / static_cast<double>(whole.k_blocks - slice);
+                    p4 = whole;
+                    p4.old_bits = reinterpret_cast<uint32_t*>(P[bcur ^ 1]);
+                    p4.k_first = slice;
+                    p4.k_blocks -= slice;
+                }
             }
-            if (thin_on) {
-                // every zero of a row that reaches most constants must lie in the few columns of B: such rows have
-                // (nearly) the same count
-                unsigned long long smp[2];
-                memcpy(smp, ctx->h_ctl + CTL_THIN + 12, sizeof(smp));
-                const double spread = static_cast<double>(smp[0]) - (static_cast<double>(n) - static_cast<double>(smp[1]));
-                thin_try = smp[0] > 0 && spread <= kThinRowSpread * static_cast<double>(n);
+            bcur ^= 1;
+            if (sliced) {
+                ctx->stats.thin_squarings++;
+                q_current = false;
+            } else {
+                ST(product());
+                ctx->stats.product_launches++;
+                ctx->stats.e2m1_products++;
+                qcur ^= 1;
+                bits_current = P[0] != nullptr;
+                if (thin_on) ST(sample(bcur));
+                ST(read_ctl(ctx, s, &changed, thin_on));
+                ST(tm.collect());
+                unsigned long long kbs = 0;
+                memcpy(&kbs, ctx->h_ctl + CTL_ISSUED, sizeof(kbs));
+                sliced_kbs += static_cast<double>(kbs - last_kbs) * slice_share;
+                last_kbs = kbs;
+                ctx->stats.issued_ops = 2.0 * TC_BM * 32.0 * TC_BK * (static_cast<double>(kbs) + sliced_kbs);
             }
+            *iters = it + 1;
+            if (!changed) return converged(res, res_t);
+            if (thin_on) judge();
             continue;
         }
         if (use_maps) {
@@ -716,11 +788,16 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
         }
         if (use_maps) ST(sparse_map(F[cur], &use_maps));
     }
-    if (on_f4 && res_f4 != nullptr) {
+    if (on_f4 && res_bits != nullptr && bits_current) {
+        *res_bits = P[bcur];
+        *res_f4 = nullptr;
+        *res = *res_t = nullptr;
+    } else if (on_f4 && res_f4 != nullptr) {
+        ST(operands_current());
         *res_f4 = Q[qcur];
-        if (res_bits != nullptr && bits_current) *res_bits = P;
         *res = *res_t = nullptr;
     } else if (on_f4) {
+        ST(operands_current());
         ST(finish_f4(res, res_t));
     } else {
         *res = M[cur];
@@ -2502,6 +2579,10 @@ double bitrow_s_per_word() { return sparse_s_per_word(); }
 double bitrow_row_s_per_word() { return sparse_row_s_per_word(); }
 double bitrow_step_s() { return kSparseStepS; }
 double tc4_product_s(int64_t n_pad) { return tc_product_s(n_pad); }
+// Row ORs of a restricted squaring: per word over the whole GPU, and per one of an entry (its named rows are read four
+// at a time by one warp per 256 words).
+double thin_word_s() { return 2e-12; }
+double thin_one_s() { return 0.25e-6; }
 // The restricted squaring's fixed cost, switch, sampled rows and row-count spread, for the device-driven pipelines.
 double thin_fixed_seconds(int64_t n_pad) { return thin_fixed_s(n_pad); }
 bool thin_is_enabled() { return thin_enabled(); }

@@ -337,6 +337,7 @@ enum SoloWord : int {
     SW_COST = 8,      // word ORs of the next bit-row squaring: total, largest row (2 x u64)
     SW_THIN_GO = 12,  // the restricted squaring is cheaper than a product (set inside its statistics' IF)
     SW_STOP = 13,     // a restricted squaring ended the loop
+    SW_TOPEN = 14,    // a restricted squaring stopped with zeros open and left R as it was
     SW_SMP = 16,      // the row sample after a product (2 x u64, thin.cu)
     SW_TSTAT = 20,    // the restricted squaring's statistics (6 x u64, thin.cu)
     SW_WORDS = 32
@@ -420,21 +421,21 @@ __global__ void solo_thin_gate_kernel(int* w, int half, int64_t n, double spread
     const int next = half == 0 ? w[SW_G1] : w[SW_GC];
     const double sp = static_cast<double>(sm[0]) - (static_cast<double>(n) - static_cast<double>(sm[1]));
     const bool go = next != 0 && sm[0] > 0 && sp <= spread * static_cast<double>(n);
-    sm[0] = 0;
-    sm[1] = 0;
+    sm[0] = sm[1] = 0;
     w[SW_THIN_GO] = 0;
     cudaGraphSetConditional(hT, go ? 1u : 0u);
 }
 
 // Inside the statistics' IF: the restricted squaring's cost by the bit-row model (the word ORs over the GPU, or one
 // warp's heaviest list entry) against a tensor-core product, as on the host loop.
-__global__ void solo_thin_decide_kernel(int* w, int64_t ldw, double fixed_s, double s_word, double s_row, double limit) {
+__global__ void solo_thin_decide_kernel(int* w, int64_t ldw, double fixed_s, double s_word, double s_one, double limit) {
     const unsigned long long* st = reinterpret_cast<const unsigned long long*>(w + SW_TSTAT);
     const double words = static_cast<double>(st[2] + st[3]) * static_cast<double>(ldw);
-    const double row_words = static_cast<double>(st[4] > st[5] ? st[4] : st[5]) * static_cast<double>(ldw);
-    const double t = fixed_s + fmax(words * s_word, row_words * s_row);
+    const double top = static_cast<double>(st[4] > st[5] ? st[4] : st[5]);
+    const double t = fixed_s + fmax(words * s_word, top * s_one);
     w[SW_THIN_GO] = t < limit ? 1 : 0;
     w[SW_TCHANGED] = 0;
+    w[SW_TOPEN] = 0;
 }
 
 __global__ void solo_thin_arm_kernel(const int* w, cudaGraphConditionalHandle hT2) {
@@ -445,6 +446,8 @@ __global__ void solo_thin_arm_kernel(const int* w, cudaGraphConditionalHandle hT
 // counted; if it changed nothing that buffer holds the closure, and at the cap while changing the loop stops
 // unconverged; either way the guards go off and the loop-control kernel ends the loop.
 __global__ void solo_thin_post_kernel(int* w, int half, int cap) {
+    w[SW_THIN_GO] = 0;
+    if (w[SW_TOPEN]) return;  // R is as it was: the next product squares it
     w[SW_ITERS] += 1;
     bool stop = false;
     if (!w[SW_TCHANGED]) {
@@ -459,7 +462,6 @@ __global__ void solo_thin_post_kernel(int* w, int half, int cap) {
         w[SW_G1] = 0;
         w[SW_STOP] = 1;
     }
-    w[SW_THIN_GO] = 0;
 }
 
 __global__ void solo_loop_ctl_kernel(const int* w, cudaGraphConditionalHandle hC) {
@@ -917,7 +919,7 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
         oTP = take(bits);
         oTPT = take(bits);
         oTT = take(2 * bits);
-        oTAux = take(static_cast<size_t>(2 * nmax * 8 + (ldwt_max + 1) * 8 + 2 * nmax * 4));
+        oTAux = take(thin_aux_bytes(nmax, ldwt_max));
     }
     void* base = nullptr;
     BST(ws_get(ctx, WS_SOLO, total, &base));
@@ -933,11 +935,6 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
     uint64_t* TP = reinterpret_cast<uint64_t*>(b8 + oTP);
     uint64_t* TPT = reinterpret_cast<uint64_t*>(b8 + oTPT);
     uint64_t* TT = reinterpret_cast<uint64_t*>(b8 + oTT);
-    int64_t* t_rowcnt = reinterpret_cast<int64_t*>(b8 + oTAux);
-    int64_t* t_colcnt = t_rowcnt + nmax;
-    uint64_t* t_bmask = reinterpret_cast<uint64_t*>(t_colcnt + nmax);
-    int32_t* t_blist = reinterpret_cast<int32_t*>(t_bmask + ldwt_max + 1);
-    int32_t* t_rlist = t_blist + nmax;
     BCK(cudaMalloc(&c->d_solo, sizeof(int) * SW_WORDS * ns), "cudaMalloc(large-problem state)");
     BCK(cudaMemset(c->d_solo, 0, sizeof(int) * SW_WORDS * ns), "clear large-problem state");
     c->h_solo.assign(static_cast<size_t>(SW_WORDS * ns), 0);
@@ -1038,6 +1035,7 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
         // that still hold zeros: IF nodes inside the loop's body, one for its statistics and one for the squaring
         const int64_t ldw_t = n_pad / 64;
         const bool thin_p = thin_any && thin_fixed_seconds(n_pad) < limit;
+        const ThinLists t_lists = thin_lists(b8 + oTAux, n, ldw_t);
         cudaGraphConditionalHandle hT[2], hT2[2];
         if (thin_p) {
             for (int h = 0; h < 2; ++h) {
@@ -1089,18 +1087,17 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
                 if (thin_p && e == cudaSuccess) {
                     uint8_t* Qn = Q[half ^ 1];
                     uint8_t* QTn = QT[half ^ 1];
-                    e = launch_thin_sample(Qn, ld4, n, thin_sample_rows(), t_smp, cb);
+                    e = launch_thin_sample(TP, ldw_t, n, thin_sample_rows(), t_smp, nullptr, cb);
                     if (e == cudaSuccess) {
                         solo_thin_gate_kernel<<<1, 1, 0, cb>>>(w, half, n, thin_row_spread(), hT[half]);
                         e = cudaGetLastError();
                     }
                     if (e == cudaSuccess)
                         e = capture_if(hT[half], [&]() -> cudaError_t {
-                            cudaError_t e3 = launch_thin_stats(Qn, QTn, ld4, n, TP, TPT, ldw_t, t_rowcnt, t_colcnt,
-                                                               t_bmask, t_blist, t_rlist, t_stat, true, sms, cc);
+                            cudaError_t e3 = launch_thin_stats(n, TP, TPT, TP, TPT, ldw_t, t_lists, t_stat, sms, cc);
                             if (e3 != cudaSuccess) return e3;
-                            solo_thin_decide_kernel<<<1, 1, 0, cc>>>(w, ldw_t, thin_fixed_seconds(n_pad), s_word, s_row,
-                                                                     limit);
+                            solo_thin_decide_kernel<<<1, 1, 0, cc>>>(w, ldw_t, thin_fixed_seconds(n_pad), thin_word_s(),
+                                                                     thin_one_s(), limit);
                             return cudaGetLastError();
                         });
                     if (e == cudaSuccess) {
@@ -1109,8 +1106,9 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
                     }
                     if (e == cudaSuccess)
                         e = capture_if(hT2[half], [&]() -> cudaError_t {
-                            cudaError_t e3 = launch_thin_squaring_dev(TP, TPT, ldw_t, n, t_blist, t_rlist, t_stat, TT,
-                                                                      Qn, QTn, ld4, w + SW_TCHANGED, sms, cc);
+                            // |B| + |Rb| is known on the device only: the grids cover up to n entries at once
+                            cudaError_t e3 = launch_thin_squaring(n, TP, TPT, TP, TPT, ldw_t, t_lists, t_stat, n, TT, Qn,
+                                                                  QTn, ld4, w + SW_TCHANGED, w + SW_TOPEN, true, sms, cc);
                             if (e3 != cudaSuccess) return e3;
                             solo_thin_post_kernel<<<1, 1, 0, cc>>>(w, half, cap);
                             return cudaGetLastError();

@@ -58,6 +58,10 @@ struct TcParams {
     uint32_t* out_bits;
     uint32_t* out_bits_t;
     int64_t ldb;
+    // if not null, R of this iteration as such bit rows, instead of old_r (may be out_bits); out_r may then be null with
+    // out_bits set: R' leaves as bit rows only
+    const uint32_t* old_bits;
+    int32_t k_first;            // squaring kernels on packed operands: first of the k_blocks blocks of K
 };
 
 // One problem of a grouped batch (device copy; built on the host).
@@ -152,11 +156,14 @@ struct bmlp_ctx {
 namespace bmlp {
 
 // CTL_QCOUNT, CTL_T0, CTL_ISSUED and CTL_BITS are 64-bit words, CTL_COST and CTL_PSTAT (the ones and nonzero words
-// a bit-row squaring wrote) two of them and CTL_THIN eight (two ints each, 8-byte aligned).
+// a bit-row squaring wrote) two of them and CTL_THIN eight (two ints each, 8-byte aligned); CTL_STEP the changed flags of up to eight
+// squarings issued together; CTL_SAMPLE the ones of sampled rows. A read of the control words ends before CTL_SAMPLE
+// unless the sample is wanted.
+constexpr int kThinSampleRows = 256;
 enum CtlWord : int {
-    CTL_CHANGED = 0, CTL_ERROR = 1, CTL_ITERS = 2, CTL_LEVELS = 3, CTL_QCOUNT = 4, CTL_T0 = 6, CTL_BUDGET = 8,
-    CTL_ISSUED = 10, CTL_COST = 12, CTL_THIN = 16, CTL_BITS = 32, CTL_PSTAT = 34, CTL_STEP = 38,
-    CTL_WORDS = 38 + 8
+    CTL_CHANGED = 0, CTL_ERROR = 1, CTL_OPEN = 2, CTL_LEVELS = 3, CTL_QCOUNT = 4, CTL_T0 = 6, CTL_BUDGET = 8,
+    CTL_ISSUED = 10, CTL_COST = 12, CTL_THIN = 16, CTL_BITS = 34, CTL_PSTAT = 36, CTL_STEP = 40,
+    CTL_SAMPLE = 48, CTL_WORDS = 48 + kThinSampleRows
 };
 // The pinned host mirror has two more ints: CTL_HOST_I64 is a 64-bit slot for values read from elsewhere.
 constexpr int CTL_HOST_I64 = CTL_WORDS;
@@ -337,29 +344,41 @@ bool smp_cluster_fits(int64_t n, int64_t rows, int sms);
 cudaError_t launch_smp_cluster(const int64_t* wptrT, const int32_t* widxT, const uint64_t* wvalT, int64_t n,
                                const uint64_t* src, int64_t ldw_src, int64_t rows, uint64_t* out, int64_t ldw_out,
                                int reflexive, int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl);
-// ---- a squaring restricted to the rows and columns of R that still hold zeros (thin.cu)
-// launch_thin_stats: bit rows P, PT (n rows of ldw = n_pad / 64 words) of the E2M1 R, R^T (ld4 = n_pad / 2 bytes per
-// row) with their ones (rowcnt, colcnt); with bits_current, P and PT already hold R and R^T (written by the squaring
-// kernel's epilogue and kept by launch_thin_squaring) and only their ones are counted; B = the columns with fewer
-// than n / 2 ones (Bmask, blist) and Rb = the rows with a zero outside B (rlist); stat[0..5] = |B|, |Rb|, ones in B's
-// columns, ones in Rb's rows, the most ones of a column of B and of a row of Rb.
-// launch_thin_sample: of `rows` rows of Q spread over its n rows, those with at least n / 2 ones: stat[0] = the most
-// ones of one, stat[1] = the most zeros of one (stat[0..1] zero beforehand).
-// launch_thin_squaring: R' = R + R R on those columns and rows, the new ones ORed into Q (R) and QT (R^T) and into
-// the bit rows P, PT in place, *changed raised when there are any; T1, T2: nb x ldw and nr x ldw words of scratch.
-cudaError_t launch_thin_stats(const uint8_t* Q, const uint8_t* QT, int64_t ld4, int64_t n, uint64_t* P, uint64_t* PT,
-                              int64_t ldw, int64_t* rowcnt, int64_t* colcnt, uint64_t* Bmask, int32_t* blist,
-                              int32_t* rlist, unsigned long long* stat, bool bits_current, int sms, cudaStream_t s);
-cudaError_t launch_thin_sample(const uint8_t* Q, int64_t ld4, int64_t n, int rows, unsigned long long* stat,
+// ---- a squaring restricted to the rows and columns that still hold zeros (thin.cu)
+// P, PT: bit rows (n_pad rows of ldw = n_pad / 64 words) of a matrix S with R <= S <= R' = R + R R and of S^T; Src, SrcT:
+// those of R and R^T (the same arrays when S = R). All are written by the squaring kernel's epilogue.
+// launch_thin_sample: over `rows` rows of P spread over its n rows, stat[0] = the most ones of one with
+// at least n / 2, stat[1] = the most zeros of such a row (both zero beforehand), ones (or null) = the ones of each.
+// launch_thin_stats: B = the columns with fewer than n / 2 ones in S, or with at most kThinCap in R and a zero in S (Bmask,
+// blist), Rb = the rows with a zero outside B (rlist), Smask the rows of Rb with at most kThinCap ones in R; stat[0..5] = |B|, |Rb|, and, with at most kThinCap counted
+// of each, the ones of R in B's columns and in Rb's rows, the most of one column of B and of one row of Rb.
+// launch_thin_squaring: R' on those columns and rows; the new ones are ORed into P, PT and, where Q is not null, into S
+// and S^T as E2M1 (Q, QT), *changed raised when there are any. An entry with more than kThinCap ones stops once the zeros
+// that it is there for are filled, at the latest after kThinCap named rows, and raises *incomplete when it stops with
+// some open: S then holds some of R' only, or, with all_or_none, is as it was. The counts are read on the device;
+// `entries` (their sum, or a bound) sizes the grids, T: that many rows of ldw words of scratch.
+constexpr int kThinCap = 512;
+struct ThinLists {
+    uint64_t* Bmask;   // ldw words
+    uint64_t* Smask;   // ldw words
+    int32_t* colcnt;   // n
+    int32_t* srccnt;   // n
+    int32_t* blist;    // n
+    int32_t* rlist;    // n
+};
+size_t thin_aux_bytes(int64_t n, int64_t ldw);
+ThinLists thin_lists(void* aux, int64_t n, int64_t ldw);
+cudaError_t launch_thin_sample(const uint64_t* P, int64_t ldw, int64_t n, int rows, unsigned long long* stat, int* ones,
                                cudaStream_t s);
-cudaError_t launch_thin_squaring(uint64_t* P, uint64_t* PT, int64_t ldw, const int32_t* blist, int64_t nb,
-                                 const int32_t* rlist, int64_t nr, uint64_t* T1, uint64_t* T2, uint8_t* Q,
-                                 uint8_t* QT, int64_t ld4, int* changed, int sms, cudaStream_t s);
-// The same with |B| = stat[0] and |Rb| = stat[1] read on the device (T1: 2 n x ldw words; Rb's rows after B's),
-// for device-driven pipelines whose host never sees the counts.
-cudaError_t launch_thin_squaring_dev(uint64_t* P, uint64_t* PT, int64_t ldw, int64_t n, const int32_t* blist,
-                                     const int32_t* rlist, const unsigned long long* stat, uint64_t* T1, uint8_t* Q,
-                                     uint8_t* QT, int64_t ld4, int* changed, int sms, cudaStream_t s);
+cudaError_t launch_thin_stats(int64_t n, const uint64_t* P, const uint64_t* PT, const uint64_t* Src, const uint64_t* SrcT,
+                              int64_t ldw, const ThinLists& t, unsigned long long* stat, int sms, cudaStream_t s);
+cudaError_t launch_thin_squaring(int64_t n, uint64_t* P, uint64_t* PT, const uint64_t* Src, const uint64_t* SrcT,
+                                 int64_t ldw, const ThinLists& t, const unsigned long long* stat, int64_t entries,
+                                 uint64_t* T, uint8_t* Q, uint8_t* QT, int64_t ld4, int* changed, int* incomplete,
+                                 bool all_or_none, int sms, cudaStream_t s);
+// Seconds of the row ORs of such a squaring (api.cu): per word in all, and per one of its largest entry.
+double thin_word_s();
+double thin_one_s();
 double thin_fixed_seconds(int64_t n_pad);
 bool thin_is_enabled();
 int thin_sample_rows();

@@ -220,6 +220,12 @@ template <int KIND, int CHUNKS>
 __device__ __forceinline__ void f4_old(const TcParams& p, int64_t row, int64_t col_base, int64_t n_pad,
                                        uint32_t (&ob)[CHUNKS]) {
     constexpr int CB = KIND ? 16 : 32;  // bytes of 32 columns
+    if (p.old_bits != nullptr) {
+        const uint32_t* bits = p.old_bits + row * p.ldb + col_base / 32;
+#pragma unroll
+        for (int c = 0; c < CHUNKS; ++c) ob[c] = col_base + c * 32 < n_pad ? bits[c] : 0u;
+        return;
+    }
     const uint8_t* src = p.old_r + row * p.ld + col_base / 32 * CB;
 #pragma unroll
     for (int c = 0; c < CHUNKS; ++c) ob[c] = col_base + c * 32 < n_pad ? load_bits32<KIND>(src + c * CB) : 0u;
@@ -243,10 +249,10 @@ __device__ __forceinline__ uint32_t f4_update(const TcParams& p, int mb, int64_t
         if (col0 < n_pad) {
             const uint32_t nbits = ob[c] | cb[c];
             any |= nbits ^ ob[c];
-            store_bits32<KIND>(p.out_r + row * p.ld + col0 / 32 * CB, nbits);
+            if (p.out_r != nullptr) store_bits32<KIND>(p.out_r + row * p.ld + col0 / 32 * CB, nbits);
             if (p.out_bits != nullptr) p.out_bits[row * p.ldb + col0 / 32] = nbits;
             const uint32_t mine = warp_transpose32(nbits, lane);  // column col0 + lane of the warp's 32 rows
-            store_bits32<KIND>(p.out_rt + (col0 + lane) * p.ld + rt_col, mine);
+            if (p.out_r != nullptr) store_bits32<KIND>(p.out_rt + (col0 + lane) * p.ld + rt_col, mine);
             if (p.out_bits_t != nullptr) p.out_bits_t[(col0 + lane) * p.ldb + rt_col / CB] = mine;
         }
     }
@@ -350,11 +356,12 @@ tc_duo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                     const uint32_t bar = mapa_shared(smem_u32(&full[stage]), 0);
                     if (leader) mbar_arrive_expect_tx(&full[stage], tx);
                     uint8_t* sb = sB + stage * C::B_BYTES;
-                    tma_load_2d_2sm(sA + stage * C::A_BYTES, &tmA, kb * F4_BK, mb * TC_BM, bar);
-                    tma_load_2d_2sm(sb, &tmB0, kb * F4_BK,
+                    const int kx = (p.k_first + kb) * F4_BK;
+                    tma_load_2d_2sm(sA + stage * C::A_BYTES, &tmA, kx, mb * TC_BM, bar);
+                    tma_load_2d_2sm(sb, &tmB0, kx,
                                     static_cast<int>(col_base) + static_cast<int>(rank) * C::B0_ROWS, bar);
                     if (has1)
-                        tma_load_2d_2sm(sb + C::B0_BYTES, &tmB1, kb * F4_BK,
+                        tma_load_2d_2sm(sb + C::B0_BYTES, &tmB1, kx,
                                         static_cast<int>(col_base) + TC_BN + static_cast<int>(rank) * C::B1_ROWS,
                                         bar);
                     issued = true;
