@@ -1170,6 +1170,31 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
     const int64_t ldw = round_up(words_of(n), 2);
     if (ldw > smp_packed_max_words())
         return set_err(ctx, BMLP_ERR_UNSUPPORTED, "packed frontier path supports n <= %d", smp_packed_max_words() * 64);
+    // a few query rows: expanded straight from R's rows, each row of a reached constant read once
+    if (const int ctas = square_first ? 0 : smp_rows_ctas(n, q)) {
+        const int64_t wpr = words_of(n);
+        const uint64_t* rows = static_cast<const uint64_t*>(R.dev);
+        if (fmt == BMLP_FMT_U8) {
+            void* p = nullptr;
+            ST(ws_get(ctx, WS_M0, static_cast<size_t>(n * wpr * 8), &p));
+            ST(to_packed(ctx, R, fmt, n, static_cast<uint64_t*>(p), wpr, s));
+            rows = static_cast<const uint64_t*>(p);
+        }
+        ProductTimer tm{ctx, o.profile != 0, s};
+        ST(tm.begin());
+        CK(launch_smp_rows(rows, wpr, n, src, ldw_src, q, out, ldw_out, o.reflexive, ctx->d_ctl + CTL_LEVELS,
+                           static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), ctas, s, deadline_of(ctx)),
+           "query row kernel launch");
+        ST(tm.end());
+        ctx->stats.product_launches++;
+        ctx->stats.launches++;
+        ST(read_ctl(ctx, s, nullptr));
+        ST(tm.collect());
+        *levels = ctx->h_ctl[CTL_LEVELS];
+        const int cap = o.max_iters > 0 ? o.max_iters : static_cast<int>(n + 1);
+        if (*levels > cap) return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "frontier did not empty within %d levels", cap);
+        return BMLP_OK;
+    }
     void *P = nullptr, *wptr = nullptr, *widx = nullptr, *wval = nullptr;
     ST(ws_get(ctx, WS_WPTR, static_cast<size_t>((n + 2) * 8), &wptr));
     ST(ws_get(ctx, WS_WIDX, static_cast<size_t>(n * ldw * 4), &widx));

@@ -344,6 +344,14 @@ bool smp_cluster_fits(int64_t n, int64_t rows, int sms);
 cudaError_t launch_smp_cluster(const int64_t* wptrT, const int32_t* widxT, const uint64_t* wvalT, int64_t n,
                                const uint64_t* src, int64_t ldw_src, int64_t rows, uint64_t* out, int64_t ldw_out,
                                int reflexive, int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl);
+// The expansion of a few query rows straight from R's packed rows (ld_r words, bits at columns >= n ignored), one cluster
+// of smp_rows_ctas() CTAs per row: 16, 8, 4 or 2, or 0 when q rows do not fit the GPU at once (or are more than
+// kRowsMaxQueries) or n is too large. Results and levels as launch_smp_cluster.
+constexpr int64_t kRowsMaxQueries = 63;
+int smp_rows_ctas(int64_t n, int64_t q);
+cudaError_t launch_smp_rows(const uint64_t* R, int64_t ld_r, int64_t n, const uint64_t* src, int64_t ld_src, int64_t q,
+                            uint64_t* out, int64_t ld_out, int reflexive, int* levels, int max_levels, int ctas,
+                            cudaStream_t s, Deadline dl);
 // ---- a squaring restricted to the rows and columns that still hold zeros (thin.cu)
 // P, PT: bit rows (n_pad rows of ldw = n_pad / 64 words) of a matrix S with R <= S <= R' = R + R R and of S^T; Src, SrcT:
 // those of R and R^T (the same arrays when S = R). All are written by the squaring kernel's epilogue.

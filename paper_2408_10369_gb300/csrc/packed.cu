@@ -1643,6 +1643,146 @@ __global__ void __launch_bounds__(kClusterThreads, 1) smp_cluster_kernel(const C
     cluster_sync();  // no CTA leaves while a peer may still read its shared memory
 }
 
+// ---- Algorithm 2 for a few query rows, straight from R's bit rows
+// One cluster of C CTAs per query row (the largest of 16, 8, 4, 2 whose clusters are all resident at once). Every CTA holds the whole frontier D; CTA
+// r ORs the rows of the frontier constants k = r mod C, four in flight per warp, into its own partial N; after a cluster
+// barrier it gathers its share of the words from every CTA's N, removes the visited constants and stores the new words
+// into every CTA's D; a second barrier ends the level. A query reads the row of each constant it reaches once, so it is
+// bound by the two barriers and the row latency per level (about 3 us) or, from some tens of thousands of constants on,
+// by the rows' bytes; no word index, no transpose and no column is needed. One warp per query over the word indexes of R
+// and R^T, which a call has to build first, took 302 us for a call with one query on n = 5,000 constants with 50 facts
+// each, 48 us now; n = 65,536 power law 6.1 ms, 0.55 ms now, and 16 queries 5.2 and 1.29 ms; a grid of n = 20,000 (117
+// levels) 1.63 and 0.57 ms, 16 queries 1.56 and 0.78 ms. For larger batches the indexes are shared and the forms that
+// use them stay.
+constexpr int kRowsThreads = 512;
+constexpr int kRowsWarps = kRowsThreads / 32;
+constexpr int kRowsMaxCtas = 16;
+
+struct RowQueryArgs {
+    const uint64_t* R;  // packed rows (bits at columns >= n ignored)
+    int64_t ld_r;
+    int64_t n;
+    const uint64_t* src;  // query rows
+    int64_t ld_src;
+    uint64_t* out;
+    int64_t ld_out;
+    int* levels_max;
+    int max_levels;
+    int reflexive;
+    Deadline dl;
+};
+
+__global__ void __launch_bounds__(kRowsThreads, 1) smp_rows_kernel(const RowQueryArgs a) {
+    extern __shared__ uint64_t rq_sm[];
+    __shared__ int s_flag[2][kRowsMaxCtas];  // by level parity, written by each CTA: 1 it found new constants, 2 stop
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = static_cast<int>(cluster_ctarank()), ctas = static_cast<int>(cluster_nctarank());
+    const int wpr = static_cast<int>((a.n + 63) >> 6);
+    const int share = (wpr + ctas - 1) / ctas;
+    const int base = rank * share;
+    const int own = base >= wpr ? 0 : min(share, wpr - base);
+    uint64_t* D = rq_sm;
+    uint64_t* N[2] = {rq_sm + wpr, rq_sm + 2 * wpr};
+    uint64_t* V = rq_sm + 3 * wpr;  // visited, own words
+    const uint64_t* src = a.src + static_cast<int64_t>(cluster_id_x()) * a.ld_src;
+    uint64_t* out = a.out + static_cast<int64_t>(cluster_id_x()) * a.ld_out;
+    const auto valid = [&](int w) {
+        const int64_t v = a.n - 64ll * w;
+        return v < 64 ? (1ull << v) - 1ull : ~0ull;
+    };
+    for (int w = tid; w < wpr; w += kRowsThreads) {
+        D[w] = src[w] & valid(w);
+        N[0][w] = N[1][w] = 0ull;
+    }
+    for (int w = tid; w < own; w += kRowsThreads) V[w] = 0ull;
+    uint64_t mine = 0ull;  // this CTA's constants of a word: bits rank, rank + ctas, ... (ctas divides 64)
+    for (int b = rank; b < 64; b += ctas) mine |= 1ull << b;
+    cluster_sync();
+    int lv = 0;
+    while (true) {
+        const int p = lv & 1;
+        uint64_t* Np = N[p];
+        for (int c0 = 0; c0 < wpr; c0 += 256) {  // 256 words of the rows at a time: 8 per lane
+            uint64_t acc[8];
+#pragma unroll
+            for (int v = 0; v < 8; ++v) acc[v] = 0ull;
+            bool any = false;
+            for (int w0 = warp; w0 < wpr; w0 += kRowsThreads) {  // lane l: word w0 + kRowsWarps l
+                const int w = w0 + kRowsWarps * lane;
+                const uint64_t d = w < wpr ? D[w] & mine : 0ull;
+                unsigned m = __ballot_sync(FULL, d != 0ull);
+                any |= m != 0u;
+                uint64_t bits = 0ull;
+                int kb = 0;
+                while (m != 0u || bits != 0ull) {
+                    const uint64_t* row[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        row[q] = nullptr;
+                        if (bits == 0ull && m != 0u) {
+                            const int sl = __ffs(m) - 1;
+                            m &= m - 1u;
+                            bits = __shfl_sync(FULL, d, sl);
+                            kb = (w0 + kRowsWarps * sl) * 64;
+                        }
+                        if (bits != 0ull) {
+                            row[q] = a.R + (kb + __ffsll(static_cast<long long>(bits)) - 1) * a.ld_r + c0 + lane;
+                            bits &= bits - 1ull;
+                        }
+                    }
+                    uint64_t x[4][8];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int v = 0; v < 8; ++v)
+                            x[q][v] = row[q] != nullptr && c0 + 32 * v + lane < wpr ? __ldg(row[q] + 32 * v) : 0ull;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int v = 0; v < 8; ++v) acc[v] |= x[q][v];
+                }
+            }
+            if (any) {
+#pragma unroll
+                for (int v = 0; v < 8; ++v)
+                    if (acc[v] != 0ull)  // zero beyond wpr
+                        atomicOr(reinterpret_cast<unsigned long long*>(&Np[c0 + 32 * v + lane]),
+                                 static_cast<unsigned long long>(acc[v]));
+            }
+        }
+        cluster_sync();  // every CTA's N is complete, and nobody reads D any more
+        bool grew = false;
+        const uint32_t n_s = smem_u32(Np + base), d_s = smem_u32(D + base);
+        for (int i = tid; i < own; i += kRowsThreads) {
+            uint64_t x = 0ull;
+#pragma unroll
+            for (int c = 0; c < kRowsMaxCtas; ++c)
+                if (c < ctas) x |= ld_dsmem_u64(mapa_shared(n_s + 8u * i, c));
+            x &= valid(base + i) & ~V[i];
+            V[i] |= x;
+            grew |= x != 0ull;
+            for (int c = 0; c < ctas; ++c) st_dsmem_u64(mapa_shared(d_s + 8u * i, c), x);
+        }
+        // the other N was last read before the previous barrier; the next level fills it
+        for (int w = tid; w < wpr; w += kRowsThreads) N[p ^ 1][w] = 0ull;
+        const int any = __syncthreads_or(grew);
+        if (tid < ctas) {
+            const int stop = rank == 0 && a.dl.budget_ns && a.dl.past() ? 2 : 0;
+            st_dsmem_s32(mapa_shared(smem_u32(&s_flag[p][rank]), tid), (any ? 1 : 0) | stop);
+        }
+        cluster_sync();  // the new D and the flags are in place
+        int f = 0;
+        for (int c = 0; c < ctas; ++c) f |= s_flag[p][c];
+        ++lv;
+        if ((f & 1) == 0 || (f & 2) != 0 || lv > a.max_levels) break;  // the same in every CTA: no barrier is left open
+    }
+    if (rank == 0 && tid == 0) atomicMax(a.levels_max, lv);
+    for (int i = tid; i < own; i += kRowsThreads)
+        out[base + i] = V[i] | (a.reflexive ? src[base + i] & valid(base + i) : 0ull);
+    if (rank == ctas - 1)
+        for (int64_t w = wpr + tid; w < a.ld_out; w += kRowsThreads) out[w] = 0ull;
+}
+
 inline int warps_grid(int64_t rows, int sms) {
     int64_t blocks = (rows + 7) / 8;  // 8 warps of 256 threads
     const int64_t cap = static_cast<int64_t>(sms) * 8;
@@ -1837,6 +1977,81 @@ cudaError_t launch_smp_cluster(const int64_t* wptrT, const int32_t* widxT, const
     const ClusterArgs a{wptrT, widxT, wvalT, src, ldw_src, n, rows, out, ldw_out, levels, max_levels, reflexive, lg,
                         dl};
     return cudaLaunchKernelEx(&cfg, smp_cluster_kernel, a);
+}
+
+namespace {
+size_t smp_rows_smem(int64_t n, int ctas) {
+    const int64_t wpr = (n + 63) / 64;
+    return static_cast<size_t>(3 * wpr + (wpr + ctas - 1) / ctas) * 8;
+}
+
+cudaLaunchConfig_t smp_rows_config(int64_t n, int64_t q, int ctas, cudaStream_t s, cudaLaunchAttribute* at) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(q * ctas), 1, 1);
+    cfg.blockDim = dim3(kRowsThreads, 1, 1);
+    cfg.dynamicSmemBytes = smp_rows_smem(n, ctas);
+    cfg.stream = s;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = static_cast<unsigned>(ctas);
+    at->val.clusterDim.y = 1;
+    at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+cudaError_t smp_rows_attributes(size_t smem) {
+    cudaError_t e = cudaFuncSetAttribute(smp_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(smem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(smp_rows_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+}  // namespace
+
+int smp_rows_ctas(int64_t n, int64_t q) {
+    // resident clusters by (device, cluster size, shared memory in steps of 16 KiB), asked once each since the query
+    // costs more than the launch (0: not asked; else the count + 1)
+    static unsigned char known[16][4][16] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (q > kRowsMaxQueries) return 0;
+    for (int h = 0; h < 4; ++h) {
+        const int ctas = kRowsMaxCtas >> h;
+        const size_t smem = smp_rows_smem(n, ctas);
+        const size_t step = (smem + 16383) / 16384;
+        if (step >= 14) return 0;  // 224 KiB: more than a CTA's
+        const bool keyed = dev >= 0 && dev < 16;
+        int clusters = keyed ? static_cast<int>(known[dev][h][step]) - 1 : -1;
+        if (clusters < 0) {
+            cudaLaunchAttribute at;
+            cudaLaunchConfig_t cfg = smp_rows_config(n, 1, ctas, nullptr, &at);
+            cfg.dynamicSmemBytes = step * 16384 > smem ? step * 16384 : smem;
+            clusters = 0;
+            if (smp_rows_attributes(cfg.dynamicSmemBytes) != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&clusters, smp_rows_kernel, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                clusters = 0;
+            }
+            if (clusters > 200) clusters = 200;
+            if (keyed) known[dev][h][step] = static_cast<unsigned char>(clusters + 1);
+        }
+        if (q <= clusters) return ctas;
+    }
+    return 0;
+}
+
+cudaError_t launch_smp_rows(const uint64_t* R, int64_t ld_r, int64_t n, const uint64_t* src, int64_t ld_src, int64_t q,
+                            uint64_t* out, int64_t ld_out, int reflexive, int* levels, int max_levels, int ctas,
+                            cudaStream_t s, Deadline dl) {
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = smp_rows_config(n, q, ctas, s, &at);
+    const cudaError_t e = smp_rows_attributes(cfg.dynamicSmemBytes);
+    if (e != cudaSuccess) return e;
+    const RowQueryArgs a{R, ld_r, n, src, ld_src, out, ld_out, levels, max_levels, reflexive, dl};
+    return cudaLaunchKernelEx(&cfg, smp_rows_kernel, a);
 }
 
 cudaError_t launch_square_growth(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, int64_t n,

@@ -118,6 +118,12 @@ __device__ __forceinline__ uint64_t ld_dsmem_u64(uint32_t addr) {
     asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr));
     return v;
 }
+__device__ __forceinline__ void st_dsmem_u64(uint32_t addr, uint64_t v) {
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ void st_dsmem_s32(uint32_t addr, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 __device__ __forceinline__ int ld_dsmem_s32(uint32_t addr) {
     int v;
     asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr));
