@@ -99,8 +99,6 @@ constexpr int WS_PIPE0 = 21, WS_PIPE1 = 22, WS_PIPE2 = 23, WS_VEC0 = 24;
 constexpr int WS_SQP = 27, WS_SQPTR = 28, WS_SQIDX = 29, WS_SQVAL = 30;
 // E4M3 inputs turned into 0 / 1 bytes, and the 0 / 1 result before it becomes E4M3 bytes.
 constexpr int WS_E8_IN0 = 31, WS_E8_IN1 = 32, WS_E8_OUT = 33;
-// Block totals of the prefix over many blocks in a word-index build.
-constexpr int WS_SCAN = 34;
 // Bit rows of R and R^T, their ones, the column mask and the row and column lists, and the computed rows of a
 // squaring restricted to the rows and columns that still hold zeros.
 constexpr int WS_THIN_P = 35, WS_THIN_AUX = 36, WS_THIN_T = 37;
@@ -806,35 +804,34 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
     return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "no fixpoint within %d products", max_iters);
 }
 
-// Device scratch for the prefix of a word-index build (kScanMaxChunks x 2 words).
-int64_t* scan_scratch(bmlp_ctx* ctx) {
-    void* p = nullptr;
-    return ws_get(ctx, WS_SCAN, static_cast<size_t>(kScanMaxChunks) * 2 * sizeof(int64_t), &p) == BMLP_OK
-               ? static_cast<int64_t*>(p)
-               : nullptr;
+// A word index of n rows of ldw words in three workspace slots.
+bmlp_status index_buffers(bmlp_ctx* ctx, int64_t n, int64_t ldw, int slot_ptr, int slot_idx, int slot_val, WordIndex* x) {
+    void *p = nullptr, *i = nullptr, *v = nullptr;
+    ST(ws_get(ctx, slot_ptr, static_cast<size_t>((2 * n + 2) * 8), &p));
+    ST(ws_get(ctx, slot_idx, static_cast<size_t>(n * ldw * 4), &i));
+    ST(ws_get(ctx, slot_val, static_cast<size_t>(n * ldw * 8), &v));
+    *x = WordIndex{static_cast<int64_t*>(p), static_cast<int32_t*>(i), static_cast<uint64_t*>(v)};
+    return BMLP_OK;
 }
 
 // Packed squaring fixpoint on P[0] (n rows x ldw words). *res = R1+. While fewer than half of R's words are
-// nonzero a squaring runs through R's word index (square_rows_kernel: only the nonzero words of the named rows are
+// nonzero a squaring runs through R's word index (indexed_rows_kernel: only the nonzero words of the named rows are
 // ORed in, and the step streams R in and R' out), after that as the whole-row product (product_packed_kernel); a
-// squaring that widens the rows past half their words hands the next ones to the whole-row product.
+// squaring that widens the rows past half their words hands the next ones to the whole-row product. *res_index (when
+// asked for) is the word index of the result when the last squaring was a word-indexed one, else its ptr is null.
 bmlp_status rms_packed_loop(bmlp_ctx* ctx, int64_t n, int64_t ldw, uint64_t* P[2], int max_iters,
-                            const bmlp_options& o, cudaStream_t s, int* iters, uint64_t** res) {
+                            const bmlp_options& o, cudaStream_t s, int* iters, uint64_t** res,
+                            WordIndex* res_index = nullptr) {
     ProductTimer tm{ctx, o.profile != 0, s};
-    void *wptr = nullptr, *widx = nullptr, *wval = nullptr;
-    ST(ws_get(ctx, WS_WPTR, static_cast<size_t>((n + 2) * 8), &wptr));
-    ST(ws_get(ctx, WS_WIDX, static_cast<size_t>(n * ldw * 4), &widx));
-    ST(ws_get(ctx, WS_WVAL, static_cast<size_t>(n * ldw * 8), &wval));
-    const bool index_fits = ldw * 8 <= 200 * 1024;  // square_rows_kernel assembles a row in shared memory
+    WordIndex x;
+    ST(index_buffers(ctx, n, ldw, WS_WPTR, WS_WIDX, WS_WVAL, &x));
+    const bool index_fits = ldw * 8 <= 200 * 1024;  // indexed_rows_kernel assembles a row in shared memory
     bool sparse = index_fits;
     auto index_of = [&](const uint64_t* Pm) -> bmlp_status {
-        CK(launch_wcsr_build(Pm, n, ldw, static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx),
-                             static_cast<uint64_t*>(wval), s, scan_scratch(ctx)),
-           "word index build");
-        CK(cudaMemcpyAsync(ctx->h_ctl + CTL_HOST_I64, static_cast<const int64_t*>(wptr) + n, sizeof(int64_t),
-                           cudaMemcpyDeviceToHost, s),
+        CK(launch_wcsr_build(Pm, n, ldw, x, s), "word index build");
+        CK(cudaMemcpyAsync(ctx->h_ctl + CTL_HOST_I64, x.ptr + 2 * n, sizeof(int64_t), cudaMemcpyDeviceToHost, s),
            "read word count");
-        ctx->stats.launches += 3;
+        ctx->stats.launches++;
         return BMLP_OK;
     };
     auto half_full = [&]() {
@@ -844,6 +841,7 @@ bmlp_status rms_packed_loop(bmlp_ctx* ctx, int64_t n, int64_t ldw, uint64_t* P[2
     };
     int cur = 0;
     *iters = 0;
+    if (res_index != nullptr) res_index->ptr = nullptr;
     if (sparse) {
         ST(index_of(P[0]));
         CK(host_sync(ctx, s), "read word count");
@@ -859,9 +857,7 @@ bmlp_status rms_packed_loop(bmlp_ctx* ctx, int64_t n, int64_t ldw, uint64_t* P[2
         CK(cudaMemsetAsync(pstat, 0, 2 * sizeof(unsigned long long), s), "reset counts");
         ST(tm.begin());
         if (sparse) {
-            CK(launch_square_rows(static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx),
-                                  static_cast<uint64_t*>(wval), P[cur], n, ldw, P[nxt], ctx->sm_count, s,
-                                  ctx->d_ctl + CTL_CHANGED),
+            CK(launch_indexed_rows(x, x, P[cur], n, ldw, P[nxt], ctx->sm_count, s, ctx->d_ctl + CTL_CHANGED),
                "word-indexed squaring launch");
             ctx->stats.sparse_squarings++;
         } else {
@@ -892,6 +888,7 @@ bmlp_status rms_packed_loop(bmlp_ctx* ctx, int64_t n, int64_t ldw, uint64_t* P[2
         cur = nxt;
         if (!changed) {
             *res = P[cur];
+            if (res_index != nullptr && sparse) *res_index = x;
             return BMLP_OK;
         }
         if (sparse) sparse = !half_full();
@@ -988,7 +985,7 @@ constexpr int64_t kSparseMinN = 4096;
 // Fixed device and host time of one bit-row step besides its word ORs: word index, cost pass, flag read-back.
 constexpr double kSparseStepS = 20e-6;
 
-// Device seconds per word OR of square_rows_kernel over the whole GPU, and per word OR of the one warp that
+// Device seconds per word OR of indexed_rows_kernel over the whole GPU, and per word OR of the one warp that
 // assembles a row (BMLP_SPARSE_PS_PER_WORD / BMLP_SPARSE_ROW_PS_PER_WORD in picoseconds override them).
 double sparse_s_per_word() {
     static const double v = [] {
@@ -1012,6 +1009,12 @@ double tc_product_s(int64_t n_pad) {
     return 2.0 * n3 / 7.0e15 + 20e-6;
 }
 
+// Device seconds of a whole-row product of two sparse matrices on the Four Russians tables, which are built for every
+// word of A whatever it holds (measured: n = 14,541 with 15,000 ones, 744 us).
+double table_product_s(int64_t n) {
+    return 2.4e-16 * static_cast<double>(n) * static_cast<double>(n) * static_cast<double>(n);
+}
+
 struct SparseStart {
     uint64_t* P = nullptr;  // packed rows after the squarings on bit rows (nullptr: none ran)
     int64_t ldw = 0;
@@ -1019,7 +1022,7 @@ struct SparseStart {
     bool done = false;      // the last of them changed nothing: P is the closure
 };
 
-// Squarings R <- R + R R on word-indexed bit rows (square_rows_kernel) for as long as the next one costs less than a
+// Squarings R <- R + R R on word-indexed bit rows (indexed_rows_kernel) for as long as the next one costs less than a
 // tensor-core product. Each step is the squaring the tensor cores would run, so the fixpoint and the count of
 // products are the same (R_k covers the paths of length 1 .. 2^k whichever engine squared it); the cost of a step is
 // the word ORs it will issue, summed on the GPU from the word index, and only grows as R gains bits, so the switch
@@ -1029,12 +1032,11 @@ bmlp_status sparse_squarings(bmlp_ctx* ctx, const Operand& in, int32_t fmt, int6
     NvtxRange nvtx_("bit-row squarings");
     const int64_t ldw = round_up(words_of(n), 2);
     if (n < kSparseMinN || ldw > 2048 || max_iters < 2) return BMLP_OK;
-    void *pa = nullptr, *pb = nullptr, *wptr = nullptr, *widx = nullptr, *wval = nullptr;
+    void *pa = nullptr, *pb = nullptr;
+    WordIndex x;
     ST(ws_get(ctx, WS_SQP, static_cast<size_t>(n * ldw * 8), &pa));
     ST(ws_get(ctx, WS_PT, static_cast<size_t>(n * ldw * 8), &pb));
-    ST(ws_get(ctx, WS_SQPTR, static_cast<size_t>((n + 2) * 8), &wptr));
-    ST(ws_get(ctx, WS_SQIDX, static_cast<size_t>(n * ldw * 4), &widx));
-    ST(ws_get(ctx, WS_SQVAL, static_cast<size_t>(n * ldw * 8), &wval));
+    ST(index_buffers(ctx, n, ldw, WS_SQPTR, WS_SQIDX, WS_SQVAL, &x));
     uint64_t* P[2] = {static_cast<uint64_t*>(pa), static_cast<uint64_t*>(pb)};
     // the first pass reads the caller's rows in place when they already have this layout (never written)
     const uint64_t* R0 = in_place_packed(in, fmt, n, ldw);
@@ -1048,14 +1050,10 @@ bmlp_status sparse_squarings(bmlp_ctx* ctx, const Operand& in, int32_t fmt, int6
     int cur = 0;
     for (;;) {
         const uint64_t* Rc = out->iters == 0 ? R0 : P[cur];
-        CK(launch_wcsr_build(Rc, n, ldw, static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx),
-                             static_cast<uint64_t*>(wval), s, scan_scratch(ctx)),
-           "word index build");
+        CK(launch_wcsr_build(Rc, n, ldw, x, s), "word index build");
         CK(cudaMemsetAsync(cost, 0, 2 * sizeof(unsigned long long), s), "reset cost");
-        CK(launch_square_cost(static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx), static_cast<uint64_t*>(wval),
-                              n, cost, ctx->sm_count, s),
-           "squaring cost launch");
-        ctx->stats.launches += 4;
+        CK(launch_indexed_cost(x, x, n, cost, ctx->sm_count, s), "squaring cost launch");
+        ctx->stats.launches += 2;
         int changed = 1;
         ST(read_ctl(ctx, s, &changed));
         if (out->iters > 0) ST(tm.collect());  // the squaring recorded in the previous pass
@@ -1071,8 +1069,7 @@ bmlp_status sparse_squarings(bmlp_ctx* ctx, const Operand& in, int32_t fmt, int6
         if (out->iters + 1 >= max_iters || t > limit) break;
         CK(cudaMemsetAsync(ctx->d_ctl + CTL_CHANGED, 0, sizeof(int), s), "reset flag");
         ST(tm.begin());
-        CK(launch_square_rows(static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx), static_cast<uint64_t*>(wval),
-                              Rc, n, ldw, P[cur ^ 1], ctx->sm_count, s, ctx->d_ctl + CTL_CHANGED),
+        CK(launch_indexed_rows(x, x, Rc, n, ldw, P[cur ^ 1], ctx->sm_count, s, ctx->d_ctl + CTL_CHANGED),
            "squaring launch");
         ST(tm.end());
         ctx->stats.launches++;
@@ -1195,10 +1192,9 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         if (*levels > cap) return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "frontier did not empty within %d levels", cap);
         return BMLP_OK;
     }
-    void *P = nullptr, *wptr = nullptr, *widx = nullptr, *wval = nullptr;
-    ST(ws_get(ctx, WS_WPTR, static_cast<size_t>((n + 2) * 8), &wptr));
-    ST(ws_get(ctx, WS_WIDX, static_cast<size_t>(n * ldw * 4), &widx));
-    ST(ws_get(ctx, WS_WVAL, static_cast<size_t>(n * ldw * 8), &wval));
+    void* P = nullptr;
+    WordIndex x;
+    ST(index_buffers(ctx, n, ldw, WS_WPTR, WS_WIDX, WS_WVAL, &x));
     if (!square_first && fmt == BMLP_FMT_PACKED64 && words_of(n) == ldw && n % 64 == 0) {
         // query rows: R is only read, so packed rows of the working width without padding bits are used where
         // they are
@@ -1207,10 +1203,8 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         ST(ws_get(ctx, WS_M0, static_cast<size_t>(n * ldw * 8), &P));
         ST(to_packed(ctx, R, fmt, n, static_cast<uint64_t*>(P), ldw, s));
     }
-    CK(launch_wcsr_build(static_cast<uint64_t*>(P), n, ldw, static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx),
-                         static_cast<uint64_t*>(wval), s, scan_scratch(ctx)),
-       "word index build");
-    ctx->stats.launches += 3;
+    CK(launch_wcsr_build(static_cast<uint64_t*>(P), n, ldw, x, s), "word index build");
+    ctx->stats.launches++;
     // nonzero words of R (W) and of R + R R (W2, counted from the word index of R without forming R + R R)
     int64_t ones = -1;  // ones of the current R (with its word index), when a growth test has counted them
     auto growth = [&](int64_t* W, int64_t* W2) -> bmlp_status {
@@ -1218,11 +1212,8 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         auto* bits = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_BITS);
         CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), s), "reset counts");
         CK(cudaMemsetAsync(bits, 0, sizeof(unsigned long long), s), "reset ones");
-        CK(launch_square_growth(static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx),
-                                static_cast<uint64_t*>(wval), n, ldw, cnt, ctx->sm_count, s, bits),
-           "squaring growth launch");
-        CK(cudaMemcpyAsync(ctx->h_ctl + CTL_HOST_I64, static_cast<const int64_t*>(wptr) + n, sizeof(int64_t),
-                           cudaMemcpyDeviceToHost, s),
+        CK(launch_square_growth(x, n, ldw, cnt, ctx->sm_count, s, bits), "squaring growth launch");
+        CK(cudaMemcpyAsync(ctx->h_ctl + CTL_HOST_I64, x.ptr + 2 * n, sizeof(int64_t), cudaMemcpyDeviceToHost, s),
            "read word count");
         ST(read_ctl(ctx, s, nullptr));
         ctx->stats.launches++;
@@ -1248,23 +1239,20 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
                 dense_reach = k == 0 && static_cast<double>(W2) > kSlicedMinGrowth * static_cast<double>(W);
                 break;
             }
-            void *P2 = nullptr, *wptr2 = nullptr, *widx2 = nullptr, *wval2 = nullptr;
+            void* P2 = nullptr;
             ST(ws_get(ctx, WS_SQP, static_cast<size_t>(n * ldw * 8), &P2));
-            ST(ws_get(ctx, WS_SQPTR, static_cast<size_t>((n + 2) * 8), &wptr2));
-            ST(ws_get(ctx, WS_SQIDX, static_cast<size_t>(n * ldw * 4), &widx2));
-            ST(ws_get(ctx, WS_SQVAL, static_cast<size_t>(n * ldw * 8), &wval2));
-            CK(launch_square_rows(static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx),
-                                  static_cast<uint64_t*>(wval), static_cast<uint64_t*>(P), n, ldw,
-                                  static_cast<uint64_t*>(P2), ctx->sm_count, s),
+            WordIndex x2;
+            ST(index_buffers(ctx, n, ldw, WS_SQPTR, WS_SQIDX, WS_SQVAL, &x2));
+            if (k & 1) {  // the buffers alternate
+                ST(ws_get(ctx, WS_M0, static_cast<size_t>(n * ldw * 8), &P2));
+                ST(index_buffers(ctx, n, ldw, WS_WPTR, WS_WIDX, WS_WVAL, &x2));
+            }
+            CK(launch_indexed_rows(x, x, static_cast<uint64_t*>(P), n, ldw, static_cast<uint64_t*>(P2), ctx->sm_count, s),
                "squaring launch");
-            CK(launch_wcsr_build(static_cast<uint64_t*>(P2), n, ldw, static_cast<int64_t*>(wptr2),
-                                 static_cast<int32_t*>(widx2), static_cast<uint64_t*>(wval2), s, scan_scratch(ctx)),
-               "word index build");
-            ctx->stats.launches += 4;
-            std::swap(P, P2);
-            std::swap(wptr, wptr2);
-            std::swap(widx, widx2);
-            std::swap(wval, wval2);
+            CK(launch_wcsr_build(static_cast<uint64_t*>(P2), n, ldw, x2, s), "word index build");
+            ctx->stats.launches += 2;
+            P = P2;
+            x = x2;
             ones = -1;  // counted for the R before this squaring
             ctx->stats.frontier_squarings++;
         }
@@ -1277,25 +1265,19 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         dense_reach = W > 0 && static_cast<double>(W2) > kSlicedMinGrowth * static_cast<double>(W);
     }
     // transposed word index for the pull direction (levels whose frontier is large)
-    void *PT = nullptr, *wptrT = nullptr, *widxT = nullptr, *wvalT = nullptr;
+    void* PT = nullptr;
+    WordIndex xT;
     ST(ws_get(ctx, WS_PT, static_cast<size_t>(n * ldw * 8), &PT));
-    ST(ws_get(ctx, WS_WPTRT, static_cast<size_t>((n + 2) * 8), &wptrT));
-    ST(ws_get(ctx, WS_WIDXT, static_cast<size_t>(n * ldw * 4), &widxT));
-    ST(ws_get(ctx, WS_WVALT, static_cast<size_t>(n * ldw * 8), &wvalT));
+    ST(index_buffers(ctx, n, ldw, WS_WPTRT, WS_WIDXT, WS_WVALT, &xT));
     if (ones >= 0 && ones * 16 <= n * ldw) {
         // few ones: R^T scattered from R's word index (clearing n x ldw words and one atomic OR per one) instead
         // of reading and writing every word
-        CK(launch_scatter_transpose(static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx),
-                                    static_cast<uint64_t*>(wval), n, ldw, static_cast<uint64_t*>(PT), ctx->sm_count,
-                                    s),
-           "scatter transpose");
+        CK(launch_scatter_transpose(x, n, ldw, static_cast<uint64_t*>(PT), ctx->sm_count, s), "scatter transpose");
     } else {
         CK(launch_bit_transpose(static_cast<uint64_t*>(P), static_cast<uint64_t*>(PT), n, ldw, s), "bit transpose");
     }
-    CK(launch_wcsr_build(static_cast<uint64_t*>(PT), n, ldw, static_cast<int64_t*>(wptrT),
-                         static_cast<int32_t*>(widxT), static_cast<uint64_t*>(wvalT), s, scan_scratch(ctx)),
-       "transposed word index build");
-    ctx->stats.launches += 4;
+    CK(launch_wcsr_build(static_cast<uint64_t*>(PT), n, ldw, xT, s), "transposed word index build");
+    ctx->stats.launches += 2;
     CK(cudaMemsetAsync(ctx->d_ctl + CTL_LEVELS, 0, 3 * sizeof(int), s), "reset level and query counters");
     ProductTimer tm{ctx, o.profile != 0, s};
     double skew = 0.0;  // largest column's nonzero words over the mean
@@ -1303,7 +1285,7 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         // no hubs among the columns: a pull scans a hub's whole in-list at every level until all active sources
         // reach it (power-law targets), which the one-query-per-warp kernel avoids
         int64_t wt[2] = {0, 0};
-        CK(cudaMemcpyAsync(wt, static_cast<const int64_t*>(wptrT) + n, sizeof(wt), cudaMemcpyDeviceToHost, s),
+        CK(cudaMemcpyAsync(wt, xT.ptr + 2 * n, sizeof(wt), cudaMemcpyDeviceToHost, s),
            "read column word counts");
         CK(host_sync(ctx, s), "read column word counts");
         skew = static_cast<double>(wt[1]) * static_cast<double>(n) / static_cast<double>(wt[0] > 0 ? wt[0] : 1);
@@ -1314,10 +1296,7 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         // 64 rows per thread-block cluster with the frontier in the cluster's shared memory: query rows, or the
         // closure's identity rows
         ST(tm.begin());
-        CK(launch_smp_cluster(static_cast<int64_t*>(wptrT), static_cast<int32_t*>(widxT),
-                              static_cast<uint64_t*>(wvalT), n, src, ldw_src, q, out, ldw_out,
-                              square_first ? 0 : o.reflexive,
-                              ctx->d_ctl + CTL_LEVELS,
+        CK(launch_smp_cluster(xT, n, src, ldw_src, q, out, ldw_out, square_first ? 0 : o.reflexive, ctx->d_ctl + CTL_LEVELS,
                               static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), ctx->sm_count, s,
                               deadline_of(ctx)),
            "cluster frontier kernel launch");
@@ -1338,8 +1317,7 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         void* scratch = nullptr;
         ST(ws_get(ctx, WS_V, static_cast<size_t>(smp_sliced_grid(n, ctx->sm_count) * 3 * n * 8), &scratch));
         ST(tm.begin());
-        CK(launch_smp_sliced(static_cast<int64_t*>(wptrT), static_cast<int32_t*>(widxT), static_cast<uint64_t*>(wvalT),
-                             n, static_cast<uint64_t*>(scratch), out, ldw_out,
+        CK(launch_smp_sliced(xT, n, static_cast<uint64_t*>(scratch), out, ldw_out,
                              reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_QCOUNT), ctx->d_ctl + CTL_LEVELS,
                              static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), ctx->sm_count, s,
                              deadline_of(ctx)),
@@ -1354,10 +1332,8 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         return BMLP_OK;
     }
     ST(tm.begin());
-    CK(launch_smp_packed(static_cast<int64_t*>(wptr), static_cast<int32_t*>(widx), static_cast<uint64_t*>(wval), n, ldw,
-                         src, ldw_src, q, out, ldw_out, ctx->d_ctl + CTL_LEVELS, ctx->d_ctl + CTL_QCOUNT, o.reflexive,
-                         ctx->sm_count, s, deadline_of(ctx), static_cast<int64_t*>(wptrT),
-                         static_cast<int32_t*>(widxT), static_cast<uint64_t*>(wvalT)),
+    CK(launch_smp_packed(x, xT, n, ldw, src, ldw_src, q, out, ldw_out, ctx->d_ctl + CTL_LEVELS, ctx->d_ctl + CTL_QCOUNT,
+                         o.reflexive, ctx->sm_count, s, deadline_of(ctx)),
        "frontier kernel launch");
     ST(tm.end());
     ctx->stats.product_launches++;
@@ -1923,15 +1899,42 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
         uint64_t* X = static_cast<uint64_t*>(bb[3]);
         ST(to_packed(ctx, b, fmt, n, P[0], ldw, s));
         uint64_t* res = nullptr;
-        st = rms_packed_loop(ctx, n, ldw, P, max_iters, o, s, &iters, &res);
+        WordIndex xc;
+        st = rms_packed_loop(ctx, n, ldw, P, max_iters, o, s, &iters, &res, &xc);
         if (st != BMLP_OK) return st;
-        launch_packed_copy(res, ldw, n, n, res, ldw, 1, s);  // I + R2+
         ST(to_packed(ctx, a, fmt, n, A1, ldw, s));
-        CK(cudaMemsetAsync(ctx->d_ctl, 0, 2 * sizeof(int), s), "reset flags");
-        CK(launch_product_packed(res, A1, X, n, ldw, 0, ctx->d_ctl + CTL_CHANGED, ctx->sm_count, s), "product launch");
-        ctx->stats.product_launches++;
-        ctx->stats.launches += 2;
-        ST(read_ctl(ctx, s, nullptr));
+        bool indexed = false;
+        if (xc.ptr != nullptr) {
+            // a sparse closure: R1 + R2+ R1 through the word indexes of R2+ and R1, unless that is predicted to cost more
+            // than the whole-row product, whose tables cost as much for few ones as for many
+            WordIndex xr;
+            ST(index_buffers(ctx, n, ldw, WS_SQPTR, WS_SQIDX, WS_SQVAL, &xr));
+            auto* cost = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_COST);
+            CK(launch_wcsr_build(A1, n, ldw, xr, s), "word index build");
+            CK(cudaMemsetAsync(cost, 0, 2 * sizeof(unsigned long long), s), "reset cost");
+            CK(launch_indexed_cost(xc, xr, n, cost, ctx->sm_count, s), "product cost launch");
+            ctx->stats.launches += 2;
+            ST(read_ctl(ctx, s, nullptr));
+            unsigned long long words = 0, row_words = 0;
+            memcpy(&words, ctx->h_ctl + CTL_COST, sizeof(words));
+            memcpy(&row_words, ctx->h_ctl + CTL_COST + 2, sizeof(row_words));
+            const double t = kSparseStepS + std::max(static_cast<double>(words) * sparse_s_per_word(),
+                                                     static_cast<double>(row_words) * sparse_row_s_per_word());
+            indexed = t < table_product_s(n);
+            if (indexed) {
+                CK(launch_indexed_rows(xc, xr, A1, n, ldw, X, ctx->sm_count, s), "word-indexed product launch");
+                ctx->stats.product_launches++;
+                ctx->stats.launches++;
+            }
+        }
+        if (!indexed) {
+            launch_packed_copy(res, ldw, n, n, res, ldw, 1, s);  // I + R2+
+            CK(cudaMemsetAsync(ctx->d_ctl, 0, 2 * sizeof(int), s), "reset flags");
+            CK(launch_product_packed(res, A1, X, n, ldw, 0, ctx->d_ctl + CTL_CHANGED, ctx->sm_count, s), "product launch");
+            ctx->stats.product_launches++;
+            ctx->stats.launches += 2;
+            ST(read_ctl(ctx, s, nullptr));
+        }
         ST(packed_out(ctx, X, ldw, n, fmt, ov.dev, 0, s));
     }
     ctx->stats.iterations = iters;

@@ -684,7 +684,7 @@ bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count,
             if (g.engine == 2) {  // R^T and the word indexes of R and R^T (entries sized for the dense worst case)
                 offPT[s] = take(bytes);
                 for (int m = 0; m < 2; ++m) {
-                    offPtr[m][s] = take(static_cast<size_t>((p.n + 2) * 8));
+                    offPtr[m][s] = take(static_cast<size_t>((2 * p.n + 2) * 8));
                     offIdx[m][s] = take(static_cast<size_t>(p.n * g.ldw * 4));
                     offVal[m][s] = take(bytes);
                 }
@@ -900,7 +900,7 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
         total += round_up(static_cast<int64_t>(bytes), 1024);
         return o;
     };
-    const size_t oP0 = take(pk), oP1 = take(pk), oPtr = take(static_cast<size_t>((nmax + 2) * 8)),
+    const size_t oP0 = take(pk), oP1 = take(pk), oPtr = take(static_cast<size_t>((2 * nmax + 2) * 8)),
                  oIdx = take(static_cast<size_t>(nmax * ldw_max * 4)), oVal = take(pk);
     size_t oQ[2], oQT[2];
     for (int k = 0; k < 2; ++k) {
@@ -990,9 +990,10 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
             launch_u8_to_packed(static_cast<const uint8_t*>(src), n, P0, ldw, cs);
         else
             launch_packed_copy(static_cast<const uint64_t*>(src), (n + 63) / 64, n, n, P0, ldw, 0, cs);
-        SCK(launch_wcsr_build(P0, n, ldw, wptr, widx, wval, cs), "word index build");
+        const WordIndex x{wptr, widx, wval};
+        SCK(launch_wcsr_build(P0, n, ldw, x, cs), "word index build");
         auto* cost = reinterpret_cast<unsigned long long*>(w + SW_COST);
-        SCK(launch_square_cost(wptr, widx, wval, n, cost, sms, cs), "squaring cost");
+        SCK(launch_indexed_cost(x, x, n, cost, sms, cs), "squaring cost");
         cudaGraph_t g = nullptr;
         cudaStreamCaptureStatus cst;
         SCK(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &g, nullptr, nullptr, nullptr), "capture info");
@@ -1005,14 +1006,14 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
         SCK(cudaStreamBeginCaptureToGraph(cb, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed),
             "begin capture of the bit-row loop");
         {
-            cudaError_t e = launch_square_rows(wptr, widx, wval, P0, n, ldw, P1, sms, cb, w + SW_CHANGED);
+            cudaError_t e = launch_indexed_rows(x, x, P0, n, ldw, P1, sms, cb, w + SW_CHANGED);
             if (e == cudaSuccess) {  // the next step reads P0 (ldw is even: rows are whole 16-byte units)
                 solo_copy_kernel<<<sms * 4, 256, 0, cb>>>(reinterpret_cast<uint4*>(P0),
                                                            reinterpret_cast<const uint4*>(P1), n * ldw / 2);
                 e = cudaGetLastError();
             }
-            if (e == cudaSuccess) e = launch_wcsr_build(P0, n, ldw, wptr, widx, wval, cb);
-            if (e == cudaSuccess) e = launch_square_cost(wptr, widx, wval, n, cost, sms, cb);
+            if (e == cudaSuccess) e = launch_wcsr_build(P0, n, ldw, x, cb);
+            if (e == cudaSuccess) e = launch_indexed_cost(x, x, n, cost, sms, cb);
             if (e == cudaSuccess) {
                 solo_rows_decide_kernel<<<1, 1, 0, cb>>>(w, cap, 0, step_s, s_word, s_row, limit, hA);
                 e = cudaGetLastError();

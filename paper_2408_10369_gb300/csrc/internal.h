@@ -312,27 +312,26 @@ cudaError_t launch_product_packed(const uint64_t* A, const uint64_t* B, uint64_t
                                   int or_a, int* changed, int sms, cudaStream_t s,
                                   Deadline dl = Deadline{0, nullptr, nullptr}, unsigned long long* pstat = nullptr,
                                   bool tables = true);
-// word-CSR of packed rows: counts -> (exclusive scan by caller kernel) -> fill
-// (widx / wval must hold n * ldw entries: the dense worst case; wptr holds n + 2 entries, wptr[n + 1] receives
-// the largest row's count)
-// scan_scratch: kScanMaxChunks x 2 int64 of device memory for a prefix over many blocks (n > 4096), or nullptr
-// for one block; the two may not be shared by calls that overlap in time.
-constexpr int kScanMaxChunks = 512;
-cudaError_t launch_wcsr_build(const uint64_t* P, int64_t n, int64_t ldw, int64_t* wptr, int32_t* widx,
-                              uint64_t* wval, cudaStream_t s, int64_t* scan_scratch = nullptr);
-cudaError_t launch_smp_packed(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, int64_t n,
-                              int64_t ldw, const uint64_t* src, int64_t ldw_src, int64_t q, uint64_t* out,
-                              int64_t ldw_out, int* levels, int* qcounter, int reflexive, int sms, cudaStream_t s,
-                              Deadline dl = Deadline{0, nullptr, nullptr}, const int64_t* wptrT = nullptr,
-                              const int32_t* widxT = nullptr, const uint64_t* wvalT = nullptr);
-// C = P | P P on packed rows through the word index (wptr, widx, wval) of P
-cudaError_t launch_square_rows(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, const uint64_t* P,
-                               int64_t n, int64_t ldw, uint64_t* C, int sms, cudaStream_t s, int* changed = nullptr);
+// Word index of n packed rows: row i's nonzero words are entries ptr[2 i] .. ptr[2 i + 1] - 1 (word index and value, in
+// increasing order; the rows' ranges lie in any order), ptr[2 n] = the entries in all, ptr[2 n + 1] = the
+// largest row's. ptr holds 2 n + 2 words (16-byte aligned), idx and val n * ldw entries (the dense worst case).
+struct WordIndex {
+    int64_t* ptr;
+    int32_t* idx;
+    uint64_t* val;
+};
+cudaError_t launch_wcsr_build(const uint64_t* P, int64_t n, int64_t ldw, const WordIndex& x, cudaStream_t s);
+cudaError_t launch_smp_packed(const WordIndex& x, const WordIndex& T, int64_t n, int64_t ldw, const uint64_t* src,
+                              int64_t ldw_src, int64_t q, uint64_t* out, int64_t ldw_out, int* levels, int* qcounter,
+                              int reflexive, int sms, cudaStream_t s, Deadline dl);
+// C = P | A B on packed rows through the word indexes of A and B (A = B = P: a squaring step); *changed (or null) is
+// raised when C != P
+cudaError_t launch_indexed_rows(const WordIndex& A, const WordIndex& B, const uint64_t* P, int64_t n, int64_t ldw,
+                                uint64_t* C, int sms, cudaStream_t s, int* changed = nullptr);
 // Full closure rows by 64-source bit-sliced frontier expansion over the word index of R^T (rows 0 .. n-1 of out,
 // ldw_out words each). scratch: smp_sliced_grid(n, sms) x 3 n words; *bcounter = 0 and *levels = 0 beforehand.
 int64_t smp_sliced_grid(int64_t n, int sms);
-cudaError_t launch_smp_sliced(const int64_t* wptrT, const int32_t* widxT, const uint64_t* wvalT, int64_t n,
-                              uint64_t* scratch, uint64_t* out, int64_t ldw_out, unsigned long long* bcounter,
+cudaError_t launch_smp_sliced(const WordIndex& T, int64_t n, uint64_t* scratch, uint64_t* out, int64_t ldw_out, unsigned long long* bcounter,
                               int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl);
 // The same expansion for query rows, with the frontier of each 64-row batch in the distributed shared memory of a
 // thread-block cluster (one cluster per batch, n <= 65,536): rows 0 .. rows - 1 of out (ldw_out words each) are
@@ -341,8 +340,7 @@ cudaError_t launch_smp_sliced(const int64_t* wptrT, const int32_t* widxT, const 
 // cluster.
 bool smp_cluster_shape(int64_t n, int64_t batches, int sms, int* ctas, int* log2_chunk);
 bool smp_cluster_fits(int64_t n, int64_t rows, int sms);
-cudaError_t launch_smp_cluster(const int64_t* wptrT, const int32_t* widxT, const uint64_t* wvalT, int64_t n,
-                               const uint64_t* src, int64_t ldw_src, int64_t rows, uint64_t* out, int64_t ldw_out,
+cudaError_t launch_smp_cluster(const WordIndex& T, int64_t n, const uint64_t* src, int64_t ldw_src, int64_t rows, uint64_t* out, int64_t ldw_out,
                                int reflexive, int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl);
 // The expansion of a few query rows straight from R's packed rows (ld_r words, bits at columns >= n ignored), one cluster
 // of smp_rows_ctas() CTAs per row: 16, 8, 4 or 2, or 0 when q rows do not fit the GPU at once (or are more than
@@ -394,18 +392,16 @@ double thin_row_spread();
 // nonzero words of R + R R (out[0] += their total) and the word ORs of that squaring (out[1] += their total), from
 // the word index of R (ldw words per row, at most 49,152), without forming R + R R; bits_out (if not null) += the
 // ones of R
-cudaError_t launch_square_growth(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, int64_t n,
-                                 int64_t ldw, unsigned long long* out, int sms, cudaStream_t s,
+cudaError_t launch_square_growth(const WordIndex& x, int64_t n, int64_t ldw, unsigned long long* out, int sms, cudaStream_t s,
                                  unsigned long long* bits_out = nullptr);
 // R^T's bit rows (n x ldw words) from R's word index: cleared, then every set bit (i, j) of R sets bit i of row j
 // by a 64-bit atomic OR. Work in proportion to the ones of R, against n x ldw words read and written by
 // launch_bit_transpose.
-cudaError_t launch_scatter_transpose(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, int64_t n,
-                                     int64_t ldw, uint64_t* out, int sms, cudaStream_t s);
-// word ORs of the next squaring step (sum over the set bits k of a row of the nonzero words of row k):
+cudaError_t launch_scatter_transpose(const WordIndex& x, int64_t n, int64_t ldw, uint64_t* out, int sms, cudaStream_t s);
+// word ORs of launch_indexed_rows (sum over the set bits k of a row of A of the nonzero words of row k of B):
 // cost[0] += their total over all rows, cost[1] = max(cost[1], the largest row's)
-cudaError_t launch_square_cost(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, int64_t n,
-                               unsigned long long* cost, int sms, cudaStream_t s);
+cudaError_t launch_indexed_cost(const WordIndex& A, const WordIndex& B, int64_t n, unsigned long long* cost, int sms,
+                                cudaStream_t s);
 // (R+ + {(u, v)})+ in place on a transitive R+ (n packed rows of ldw words)
 cudaError_t launch_insert_fact(uint64_t* P, int64_t n, int64_t ldw, int64_t u, int64_t v, int sms, cudaStream_t s);
 // The same for m <= kInsertChunk facts at once (pairs: m x 2 constants in device memory, checked by the caller) through
@@ -421,7 +417,7 @@ int smp_packed_max_words();
 struct FrontierJob {
     const uint64_t* P;     // R as packed rows (n x ldw words, padding bits and words zero)
     uint64_t* PT;          // R^T, written by the launch
-    int64_t* wptr;         // word index of R ((n + 2) offsets; entries sized for the dense worst case)
+    int64_t* wptr;         // word index of R (as WordIndex)
     int32_t* widx;
     uint64_t* wval;
     int64_t* wptrT;        // word index of R^T

@@ -20,8 +20,10 @@
 //                 (queries are independent, so no grid-wide step is needed;
 //                 a warp takes the next query from a global counter when its
 //                 query has converged).
-//  * square_rows  R + R R through the word index, before the frontier closure
-//                 of a path-like relation (same closure, fewer levels).
+//  * indexed_rows P + A B through the word indexes of A and B: the sparse first
+//                 squarings of a closure (A = B = P), a sparse composition's product.
+//  * smp_rows     Algorithm 2 for a few query rows straight from R's rows, one
+//                 thread-block cluster per row.
 //  * smp_cluster  Algorithm 2 for 64 sources or 64 query rows at once,
 //                 bit-sliced, with the frontier spread over the shared
 //                 memory of a thread-block cluster (read through DSMEM).
@@ -292,232 +294,117 @@ __global__ void __launch_bounds__(kM4Threads, 2) product_m4rm_kernel(const uint6
 }
 
 // ---- word-CSR of packed rows
-// Word x of a row of an n x n matrix with its bits at columns >= n cleared (a caller's padding bits are not
-// columns; words past ceil(n / 64) are padding too).
-__device__ __forceinline__ uint64_t wcsr_columns(uint64_t w, int64_t x, int64_t n) {
-    const int64_t nw = (n + 63) >> 6;
-    if (x < nw - 1) return w;
-    if (x > nw - 1) return 0ull;
-    return (n & 63) ? (w & ((1ull << (n & 63)) - 1ull)) : w;
+// Entries of row k of a word index: [x, y).
+__device__ __forceinline__ longlong2 wcsr_row(const int64_t* __restrict__ wptr, int64_t k) {
+    return *reinterpret_cast<const longlong2*>(wptr + 2 * k);
 }
 
-// Rows warp_id, warp_id + nwarps, ... of P: their counts of nonzero words into wptr[i + 1].
-__device__ __forceinline__ void wcsr_count_rows(const uint64_t* __restrict__ P, int64_t n, int64_t ldw,
-                                                int64_t* __restrict__ wptr, int64_t warp_id, int64_t nwarps,
-                                                int lane) {
-    for (int64_t i = warp_id; i < n; i += nwarps) {
-        const uint64_t* row = P + i * ldw;
-        int64_t c = 0;
-        int64_t wb = 0;
-        for (; wb + 128 <= ldw; wb += 128) {  // four loads in flight per lane
-            uint64_t w[4];
+// The word index of P in one launch: a warp per row, eight rows per block and step. A pass over the row's words keeps
+// only which of them are nonzero (bit k of a lane's mask: word 32 k + lane of a chunk of 1,024); the counts give the
+// row's place among the block's eight, whose entries start where the running total ptr[2 n] stood (zero beforehand, as
+// ptr[2 n + 1], which receives the largest row's count). The nonzero words are then read again, from L2, and written in
+// order. The ranges of the steps lie in the order in which the blocks came: every reader goes by a row's own range, so
+// no prefix over all rows is needed. Bound by HBM, one read of P. Counts, a prefix over them and a second whole read of P
+// took four launches and 62 us at n = 32,768 (134 MB), 24 us at 14,541, 183 us at 65,536; this kernel 47, 9 and 99 us
+// (5.2 TB/s). Holding the rows in registers between the two passes was slower (203 us at 65,536: two blocks per SM),
+// and a fixed place for every eight rows instead of the running total did not help that form (220 us).
+constexpr int kIndexChunk = 1024;  // words whose nonzero mask a lane holds
+
+__device__ __forceinline__ uint32_t wcsr_mask(const uint64_t* __restrict__ row, int64_t c0, int64_t wpr, uint64_t last,
+                                              int lane) {
+    uint32_t nz = 0;
+    for (int k0 = 0; k0 < 32 && c0 + 32 * k0 < wpr; k0 += 8) {  // eight loads in flight per lane
+        uint64_t v[8];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) w[k] = row[wb + 32 * k + lane];
+        for (int q = 0; q < 8; ++q) {
+            const int64_t x = c0 + 32 * (k0 + q) + lane;
+            v[q] = x < wpr ? row[x] : 0ull;
+        }
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                c += __popc(__ballot_sync(FULL, wcsr_columns(w[k], wb + 32 * k + lane, n) != 0ull));
+        for (int q = 0; q < 8; ++q) {
+            if (c0 + 32 * (k0 + q) + lane == wpr - 1) v[q] &= last;
+            nz |= (v[q] != 0ull ? 1u : 0u) << (k0 + q);
         }
-        for (; wb < ldw; wb += 32) {
-            const uint64_t w = (wb + lane < ldw) ? wcsr_columns(row[wb + lane], wb + lane, n) : 0ull;
-            c += __popc(__ballot_sync(FULL, w != 0ull));
-        }
-        if (lane == 0) wptr[i + 1] = c;
-        if (i == 0 && lane == 0) wptr[0] = 0;
     }
+    return nz;
 }
 
-__global__ void wcsr_count_kernel(const uint64_t* __restrict__ P, int64_t n, int64_t ldw, int64_t* __restrict__ wptr) {
-    const int64_t warp_id = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    wcsr_count_rows(P, n, ldw, wptr, warp_id, nwarps, threadIdx.x & 31);
-}
-
-// In-place inclusive scan of wptr[1..n] by one block of 1024 threads, in tiles of 4,096 counts (4 consecutive
-// counts per thread, so a warp reads 1 KB contiguously); wptr[n + 1] = the largest count.
-__device__ __forceinline__ void scan_block(int64_t* __restrict__ wptr, int64_t n) {
-    __shared__ int64_t warp_tot[32];
-    __shared__ int64_t carry;
-    __shared__ unsigned long long top;
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    if (t == 0) {
-        carry = 0;
-        top = 0ull;
-    }
-    __syncthreads();
-    int64_t mx = 0;
-    for (int64_t base = 1; base <= n; base += 4096) {
-        int64_t v[4];
-        int64_t s = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int64_t x = base + 4 * t + k;
-            const int64_t c = x <= n ? wptr[x] : 0;
-            mx = c > mx ? c : mx;
-            s += c;
-            v[k] = s;  // inclusive within the thread
-        }
-        int64_t ws = s;  // inclusive over the warp's threads
-        for (int off = 1; off < 32; off <<= 1) {
-            const int64_t y = __shfl_up_sync(FULL, ws, off);
-            if (lane >= off) ws += y;
-        }
-        if (lane == 31) warp_tot[wid] = ws;
-        __syncthreads();
-        if (wid == 0) {
-            int64_t x = warp_tot[lane];  // inclusive over the block's warps
-            for (int off = 1; off < 32; off <<= 1) {
-                const int64_t y = __shfl_up_sync(FULL, x, off);
-                if (lane >= off) x += y;
-            }
-            warp_tot[lane] = x;
-        }
-        __syncthreads();
-        const int64_t before = carry + (wid > 0 ? warp_tot[wid - 1] : 0) + (ws - s);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int64_t x = base + 4 * t + k;
-            if (x <= n) wptr[x] = before + v[k];
-        }
-        __syncthreads();  // every thread has read carry and warp_tot
-        if (t == 0) carry += warp_tot[31];
-        __syncthreads();
-    }
-    atomicMax(&top, static_cast<unsigned long long>(mx));
-    __syncthreads();
-    if (t == 0) wptr[n + 1] = static_cast<int64_t>(top);
-}
-
-__global__ void __launch_bounds__(1024) scan_kernel(int64_t* __restrict__ wptr, int64_t n) { scan_block(wptr, n); }
-
-// The same prefix over many blocks. Pass 1: chunk b, the counts wptr[1 + 4096 b .. 4096 (b + 1)], is scanned in
-// place (inclusive within the chunk); sums[b] = its total and sums[chunks + b] = its largest count.
-constexpr int kScanChunk = 4096;
-__global__ void __launch_bounds__(1024) scan_chunks_kernel(int64_t* __restrict__ wptr, int64_t n,
-                                                           int64_t* __restrict__ sums, int chunks) {
-    __shared__ int64_t warp_tot[32];
-    __shared__ int64_t warp_max[32];
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    const int64_t base = 1 + static_cast<int64_t>(blockIdx.x) * kScanChunk + 4 * t;
-    int64_t v[4];
-    int64_t s = 0, mx = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int64_t c = base + k <= n ? wptr[base + k] : 0;
-        mx = c > mx ? c : mx;
-        s += c;
-        v[k] = s;
-    }
-    int64_t ws = s;
-    for (int off = 1; off < 32; off <<= 1) {
-        const int64_t y = __shfl_up_sync(FULL, ws, off);
-        if (lane >= off) ws += y;
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        const int64_t y = __shfl_xor_sync(FULL, mx, off);
-        mx = y > mx ? y : mx;
-    }
-    if (lane == 31) warp_tot[wid] = ws;
-    if (lane == 0) warp_max[wid] = mx;
-    __syncthreads();
-    if (wid == 0) {
-        int64_t x = warp_tot[lane], m = warp_max[lane];
-        for (int off = 1; off < 32; off <<= 1) {
-            const int64_t y = __shfl_up_sync(FULL, x, off);
-            if (lane >= off) x += y;
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            const int64_t y = __shfl_xor_sync(FULL, m, off);
-            m = y > m ? y : m;
-        }
-        warp_tot[lane] = x;
-        if (lane == 31) {
-            sums[blockIdx.x] = x;
-            sums[chunks + blockIdx.x] = m;
-        }
-    }
-    __syncthreads();
-    const int64_t before = (wid > 0 ? warp_tot[wid - 1] : 0) + (ws - s);
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (base + k <= n) wptr[base + k] = before + v[k];
-}
-
-// Pass 2: chunk b gains the totals of the chunks before it; block 0 writes wptr[0] = 0 and wptr[n + 1] = the
-// largest count.
-__global__ void __launch_bounds__(1024) scan_add_kernel(int64_t* __restrict__ wptr, int64_t n,
-                                                        const int64_t* __restrict__ sums, int chunks) {
-    __shared__ int64_t offset;
-    const int t = threadIdx.x, lane = t & 31;
-    if (t < 32) {
-        int64_t o = 0, m = 0;
-        for (int b = lane; b < chunks; b += 32) {
-            if (b < static_cast<int>(blockIdx.x)) o += sums[b];
-            m = sums[chunks + b] > m ? sums[chunks + b] : m;
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            o += __shfl_xor_sync(FULL, o, off);
-            const int64_t y = __shfl_xor_sync(FULL, m, off);
-            m = y > m ? y : m;
-        }
-        if (t == 0) {
-            offset = o;
-            if (blockIdx.x == 0) {
-                wptr[0] = 0;
-                wptr[n + 1] = m;
-            }
-        }
-    }
-    __syncthreads();
-    if (blockIdx.x == 0) return;  // the first chunk's prefix is already final
-    const int64_t base = 1 + static_cast<int64_t>(blockIdx.x) * kScanChunk + 4 * t;
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (base + k <= n) wptr[base + k] += offset;
-}
-
-__device__ __forceinline__ void wcsr_fill_rows(const uint64_t* __restrict__ P, int64_t n, int64_t ldw,
-                                               const int64_t* __restrict__ wptr, int32_t* __restrict__ widx,
-                                               uint64_t* __restrict__ wval, int64_t warp_id, int64_t nwarps, int lane) {
+__device__ __forceinline__ void wcsr_build_rows(const uint64_t* __restrict__ P, int64_t n, int64_t ldw,
+                                                int64_t* __restrict__ wptr, int32_t* __restrict__ widx,
+                                                uint64_t* __restrict__ wval, int64_t block, int64_t blocks) {
+    __shared__ int s_cnt[8];
+    __shared__ unsigned long long s_base;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1u;
-    for (int64_t i = warp_id; i < n; i += nwarps) {
+    const int64_t wpr = (n + 63) >> 6;
+    const uint64_t last = (n & 63) ? (1ull << (n & 63)) - 1ull : ~0ull;  // columns < n of a row's last word
+    for (int64_t i0 = block * 8; i0 < n; i0 += blocks * 8) {  // the same steps in all warps of the block
+        const int64_t i = i0 + warp;
         const uint64_t* row = P + i * ldw;
-        int64_t o = wptr[i];
-        int64_t wb = 0;
-        for (; wb + 128 <= ldw; wb += 128) {  // four loads in flight per lane
-            uint64_t w[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) w[k] = row[wb + 32 * k + lane];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) w[k] = wcsr_columns(w[k], wb + 32 * k + lane, n);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const unsigned m = __ballot_sync(FULL, w[k] != 0ull);
-                if (w[k]) {
-                    const int64_t at = o + __popc(m & below);
-                    widx[at] = static_cast<int32_t>(wb + 32 * k + lane);
-                    wval[at] = w[k];
-                }
-                o += __popc(m);
+        uint32_t nz = 0;
+        int c = 0;
+        if (i < n) {
+            if (wpr <= kIndexChunk) {
+                nz = wcsr_mask(row, 0, wpr, last, lane);
+                c = __popc(nz);
+            } else {
+                for (int64_t c0 = 0; c0 < wpr; c0 += kIndexChunk) c += __popc(wcsr_mask(row, c0, wpr, last, lane));
             }
         }
-        for (; wb < ldw; wb += 32) {
-            const uint64_t w = (wb + lane < ldw) ? wcsr_columns(row[wb + lane], wb + lane, n) : 0ull;
-            const unsigned m = __ballot_sync(FULL, w != 0ull);
-            if (w) {
-                const int64_t at = o + __popc(m & below);
-                widx[at] = static_cast<int32_t>(wb + lane);
-                wval[at] = w;
+        const int count = static_cast<int>(__reduce_add_sync(FULL, static_cast<unsigned>(c)));
+        if (lane == 0) s_cnt[warp] = count;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int total = 0, top = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                total += s_cnt[k];
+                top = max(top, s_cnt[k]);
             }
-            o += __popc(m);
+            auto* totals = reinterpret_cast<unsigned long long*>(wptr + 2 * n);
+            s_base = total > 0 ? atomicAdd(totals, static_cast<unsigned long long>(total)) : 0ull;
+            if (top > 0) atomicMax(totals + 1, static_cast<unsigned long long>(top));
+        }
+        __syncthreads();
+        int64_t o = static_cast<int64_t>(s_base);
+        for (int k = 0; k < warp; ++k) o += s_cnt[k];
+        __syncthreads();  // the counts are rewritten in the next step
+        if (i >= n) continue;
+        if (lane == 0) *reinterpret_cast<longlong2*>(wptr + 2 * i) = make_longlong2(o, o + count);
+        for (int64_t c0 = 0; c0 < wpr; c0 += kIndexChunk) {
+            if (wpr > kIndexChunk) nz = wcsr_mask(row, c0, wpr, last, lane);
+            uint32_t any = __reduce_or_sync(FULL, nz);  // groups of 32 words that hold a nonzero one
+            while (any) {                               // four of them at a time
+                int g[4];
+                uint64_t v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    g[q] = any ? __ffs(any) - 1 : -1;
+                    any &= any - 1u;
+                    const int64_t x = c0 + 32 * g[q] + lane;
+                    v[q] = g[q] >= 0 && ((nz >> g[q]) & 1u) ? row[x] : 0ull;
+                    if (x == wpr - 1) v[q] &= last;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (g[q] < 0) break;  // uniform
+                    const unsigned m = __ballot_sync(FULL, v[q] != 0ull);
+                    if (v[q]) {
+                        const int64_t e = o + __popc(m & below);
+                        widx[e] = static_cast<int32_t>(c0 + 32 * g[q] + lane);
+                        wval[e] = v[q];
+                    }
+                    o += __popc(m);
+                }
+            }
         }
     }
 }
 
-__global__ void wcsr_fill_kernel(const uint64_t* __restrict__ P, int64_t n, int64_t ldw, const int64_t* __restrict__ wptr,
-                                 int32_t* __restrict__ widx, uint64_t* __restrict__ wval) {
-    const int64_t warp_id = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    wcsr_fill_rows(P, n, ldw, wptr, widx, wval, warp_id, nwarps, threadIdx.x & 31);
+__global__ void __launch_bounds__(256) wcsr_build_kernel(const uint64_t* __restrict__ P, int64_t n, int64_t ldw,
+                                                         int64_t* __restrict__ wptr, int32_t* __restrict__ widx,
+                                                         uint64_t* __restrict__ wval) {
+    wcsr_build_rows(P, n, ldw, wptr, widx, wval, blockIdx.x, gridDim.x);
 }
 
 // Bit-matrix transpose of n x n packed rows (ldw words each), one 64 x 64
@@ -612,9 +499,9 @@ __device__ __forceinline__ void push_rows(const int64_t (&k)[NQ], int lane, cons
     int64_t e0[NQ], e1[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const int64_t kk = k[q] >= 0 ? k[q] : 0;  // an in-range index even where the value is dropped
-        e0[q] = k[q] >= 0 ? wptr[kk] : 0;
-        e1[q] = k[q] >= 0 ? wptr[kk + 1] : 0;
+        const longlong2 r = wcsr_row(wptr, k[q] >= 0 ? k[q] : 0);  // an in-range index even where the value is dropped
+        e0[q] = k[q] >= 0 ? r.x : 0;
+        e1[q] = k[q] >= 0 ? r.y : 0;
     }
     bool light[NQ];
 #pragma unroll
@@ -765,8 +652,8 @@ __device__ __forceinline__ int smp_expand_row(SrcWord srcw, uint64_t* __restrict
     while ((int64_t(64) << gshift) < wpr) ++gshift;
     const int ngroups = static_cast<int>((wpr + (int64_t(1) << gshift) - 1) >> gshift);
     const uint64_t all_groups = ngroups >= 64 ? ~0ull : (1ull << ngroups) - 1ull;
-    const float w_out = wptrT != nullptr ? static_cast<float>(wptr[n]) / static_cast<float>(n) : 0.f;
-    const float w_in = wptrT != nullptr ? static_cast<float>(wptrT[n]) / static_cast<float>(n) : 0.f;
+    const float w_out = wptrT != nullptr ? static_cast<float>(wptr[2 * n]) / static_cast<float>(n) : 0.f;
+    const float w_in = wptrT != nullptr ? static_cast<float>(wptrT[2 * n]) / static_cast<float>(n) : 0.f;
     // D = sources; FL = their nonzero words (ballot compaction); V = 0
     int fcount = 0;
     for (int64_t w0 = 0; w0 < ldw; w0 += 32) {
@@ -818,8 +705,9 @@ __device__ __forceinline__ int smp_expand_row(SrcWord srcw, uint64_t* __restrict
 #pragma unroll
                         for (int q = 0; q < 2; ++q) {
                             const int64_t j = w * 64 + (bs[q] < 0 ? 0 : bs[q]);
-                            s0[q] = bs[q] < 0 ? 0 : wptrT[j];
-                            s1[q] = bs[q] < 0 ? 0 : wptrT[j + 1];
+                            const longlong2 r = wcsr_row(wptrT, j);
+                            s0[q] = bs[q] < 0 ? 0 : r.x;
+                            s1[q] = bs[q] < 0 ? 0 : r.y;
                         }
                         int xi[2][2];
                         uint64_t xv[2][2];
@@ -940,39 +828,25 @@ __global__ void __launch_bounds__(256, 4) smp_packed_kernel(const int64_t* __res
 }
 
 // ---- closures by frontier expansion of many small relations in one launch (grouped batch)
-// Transpose and word index of R and of R^T for every job: blockIdx.y = job; blockIdx.z = 0 builds the
-// transpose, then (separate launches, stage 1-3) the word indexes of both matrices (blockIdx.z = matrix).
+// Transpose and word index of R and of R^T for every job: blockIdx.y = job; one launch builds the transposes, the next
+// the word indexes of both matrices (blockIdx.z = matrix).
 __global__ void __launch_bounds__(64) frontier_transpose_kernel(const FrontierJob* __restrict__ jobs) {
     __shared__ uint64_t t[64];
     const FrontierJob& J = jobs[blockIdx.y];
     const int64_t wpr = (J.n + 63) / 64;
     for (int64_t tile = blockIdx.x; tile < wpr * wpr; tile += gridDim.x)
         bit_transpose_tile(J.P, J.PT, J.n, J.ldw, tile / wpr, tile % wpr, t);
-    // padding words of the transpose's rows
+    // the totals of the two word indexes that the next launch builds, and padding words of the transpose's rows
+    if (blockIdx.x == 0 && threadIdx.x < 2) J.wptr[2 * J.n + threadIdx.x] = J.wptrT[2 * J.n + threadIdx.x] = 0;
     for (int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; r < J.n;
          r += static_cast<int64_t>(gridDim.x) * blockDim.x)
         for (int64_t w = wpr; w < J.ldw; ++w) J.PT[r * J.ldw + w] = 0ull;
 }
 
-__global__ void __launch_bounds__(256) frontier_wcsr_count_kernel(const FrontierJob* __restrict__ jobs) {
+__global__ void __launch_bounds__(256) frontier_wcsr_kernel(const FrontierJob* __restrict__ jobs) {
     const FrontierJob& J = jobs[blockIdx.y];
-    const int64_t warp_id = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    if (blockIdx.z == 0) wcsr_count_rows(J.P, J.n, J.ldw, J.wptr, warp_id, nwarps, threadIdx.x & 31);
-    else wcsr_count_rows(J.PT, J.n, J.ldw, J.wptrT, warp_id, nwarps, threadIdx.x & 31);
-}
-
-__global__ void __launch_bounds__(1024) frontier_scan_kernel(const FrontierJob* __restrict__ jobs) {
-    const FrontierJob& J = jobs[blockIdx.y];
-    scan_block(blockIdx.z == 0 ? J.wptr : J.wptrT, J.n);
-}
-
-__global__ void __launch_bounds__(256) frontier_wcsr_fill_kernel(const FrontierJob* __restrict__ jobs) {
-    const FrontierJob& J = jobs[blockIdx.y];
-    const int64_t warp_id = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    if (blockIdx.z == 0) wcsr_fill_rows(J.P, J.n, J.ldw, J.wptr, J.widx, J.wval, warp_id, nwarps, threadIdx.x & 31);
-    else wcsr_fill_rows(J.PT, J.n, J.ldw, J.wptrT, J.widxT, J.wvalT, warp_id, nwarps, threadIdx.x & 31);
+    if (blockIdx.z == 0) wcsr_build_rows(J.P, J.n, J.ldw, J.wptr, J.widx, J.wval, blockIdx.x, gridDim.x);
+    else wcsr_build_rows(J.PT, J.n, J.ldw, J.wptrT, J.widxT, J.wvalT, blockIdx.x, gridDim.x);
 }
 
 // Every row of every job as one query: the rows of all jobs are numbered job by job (job j owns rows
@@ -1138,30 +1012,28 @@ __global__ void __launch_bounds__(kInsertWarps * 32) insert_rows_kernel(uint64_t
     }
 }
 
-// ---- one squaring step on packed rows through the word index of R:
-// C_i = R_i | OR_{k in R_i} R_k, where row k contributes only its nonzero
-// words (push_balanced), so the cost follows the index, not n / 64 words per k.
-// Warp per row; the row is assembled in shared memory (ldw words per warp).
-__global__ void __launch_bounds__(256) square_rows_kernel(const int64_t* __restrict__ wptr,
-                                                          const int32_t* __restrict__ widx,
-                                                          const uint64_t* __restrict__ wval,
-                                                          const uint64_t* __restrict__ P, int64_t n, int64_t ldw,
-                                                          uint64_t* __restrict__ C, int* __restrict__ changed) {
+// ---- one product on packed rows through word indexes: C_i = P_i | OR_{k in A_i} B_k, where row k contributes only its
+// nonzero words (push_balanced), so the cost follows the indexes, not n / 64 words per k. With A = B = P = R that is one
+// squaring step. Warp per row; the row is assembled in shared memory (ldw words per warp). *changed (or null) is raised
+// when C_i != P_i.
+__global__ void __launch_bounds__(256) indexed_rows_kernel(const WordIndex A, const WordIndex B,
+                                                           const uint64_t* __restrict__ P, int64_t n, int64_t ldw,
+                                                           uint64_t* __restrict__ C, int* __restrict__ changed) {
     extern __shared__ uint64_t sq_sm[];
     const int lane = threadIdx.x & 31;
     uint64_t* S = sq_sm + static_cast<int64_t>(threadIdx.x >> 5) * ldw;
     const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
+        const longlong2 range = wcsr_row(A.ptr, i);
         for (int64_t w = lane; w < ldw; w += 32) S[w] = P[i * ldw + w];
         __syncwarp();
         uint64_t tm = 0;  // word groups are not needed here
-        const int64_t e0 = wptr[i], e1 = wptr[i + 1];
-        for (int64_t b0 = e0; b0 < e1; b0 += 32) {
+        for (int64_t b0 = range.x; b0 < range.y; b0 += 32) {
             const int64_t e = b0 + lane;
-            const int64_t ee = e < e1 ? e : 0;
-            const uint64_t d = e < e1 ? wval[ee] : 0ull;
-            const int64_t w = e < e1 ? widx[ee] : 0;
-            push_balanced(d, w, lane, wptr, widx, wval, S, 30, tm);
+            const int64_t ee = e < range.y ? e : range.x;
+            const uint64_t d = e < range.y ? A.val[ee] : 0ull;
+            const int64_t w = e < range.y ? A.idx[ee] : 0;
+            push_balanced(d, w, lane, B.ptr, B.idx, B.val, S, 30, tm);
         }
         __syncwarp();
         bool grew = false;
@@ -1175,29 +1047,26 @@ __global__ void __launch_bounds__(256) square_rows_kernel(const int64_t* __restr
     }
 }
 
-// ---- the work of the next squaring step through the word index: for every
-// set bit k of every row, the nonzero words of row k (what square_rows_kernel
-// ORs into that row). cost[0] += the total, cost[1] = max over rows (one warp
-// assembles a row, so the largest row bounds the step from below). Warp per
-// row, two 64-bit atomics per warp. Bits at or beyond n are zero in every
-// row, so k < n.
-__global__ void __launch_bounds__(256) square_cost_kernel(const int64_t* __restrict__ wptr,
-                                                          const int32_t* __restrict__ widx,
-                                                          const uint64_t* __restrict__ wval, int64_t n,
-                                                          unsigned long long* __restrict__ cost) {
+// ---- the work of such a product: for every set bit k of every row of A, the nonzero words of row k of B (what
+// indexed_rows_kernel ORs into that row). cost[0] += the total, cost[1] = max over rows (one warp assembles a row, so the
+// largest row bounds the step from below). Warp per row, two 64-bit atomics per warp. Bits at or beyond n are zero in
+// every row, so k < n.
+__global__ void __launch_bounds__(256) indexed_cost_kernel(const WordIndex A, const WordIndex B, int64_t n,
+                                                           unsigned long long* __restrict__ cost) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
     unsigned long long total = 0, top = 0;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
         unsigned long long c = 0;
-        const int64_t e1 = wptr[i + 1];
-        for (int64_t e = wptr[i] + lane; e < e1; e += 32) {
-            uint64_t d = wval[e];
-            const int64_t base = static_cast<int64_t>(widx[e]) << 6;
+        const longlong2 range = wcsr_row(A.ptr, i);
+        for (int64_t e = range.x + lane; e < range.y; e += 32) {
+            uint64_t d = A.val[e];
+            const int64_t base = static_cast<int64_t>(A.idx[e]) << 6;
             while (d) {
                 const int64_t k = base + (__ffsll(static_cast<long long>(d)) - 1);
                 d &= d - 1ull;
-                c += static_cast<unsigned long long>(wptr[k + 1] - wptr[k]);
+                const longlong2 r = wcsr_row(B.ptr, k);
+                c += static_cast<unsigned long long>(r.y - r.x);
             }
         }
         for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(FULL, c, off);
@@ -1227,8 +1096,8 @@ __global__ void __launch_bounds__(256) square_growth_kernel(const int64_t* __res
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
         for (int j = lane; j < bw; j += 32) bm[j] = 0u;
         __syncwarp();
-        const int64_t e1 = wptr[i + 1];
-        for (int64_t e = wptr[i] + lane; e < e1; e += 32) {
+        const longlong2 range = wcsr_row(wptr, i);
+        for (int64_t e = range.x + lane; e < range.y; e += 32) {
             const int x = widx[e];
             atomicOr(&bm[x >> 5], 1u << (x & 31));
             uint64_t d = wval[e];
@@ -1237,8 +1106,8 @@ __global__ void __launch_bounds__(256) square_growth_kernel(const int64_t* __res
             while (d) {
                 const int64_t k = base + (__ffsll(static_cast<long long>(d)) - 1);
                 d &= d - 1ull;
-                const int64_t f1 = wptr[k + 1];
-                for (int64_t f = wptr[k]; f < f1; ++f) {
+                const longlong2 r = wcsr_row(wptr, k);
+                for (int64_t f = r.x; f < r.y; ++f) {
                     const int y = widx[f];
                     atomicOr(&bm[y >> 5], 1u << (y & 31));
                     ++ors;
@@ -1273,8 +1142,8 @@ __global__ void __launch_bounds__(256) scatter_transpose_kernel(const int64_t* _
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
         const unsigned long long bit = 1ull << (i & 63);
         const int64_t wi = i >> 6;
-        const int64_t e1 = wptr[i + 1];
-        for (int64_t e = wptr[i] + lane; e < e1; e += 32) {
+        const longlong2 range = wcsr_row(wptr, i);
+        for (int64_t e = range.x + lane; e < range.y; e += 32) {
             uint64_t d = wval[e];
             const int64_t base = static_cast<int64_t>(widx[e]) << 6;
             while (d) {
@@ -1346,12 +1215,14 @@ __global__ void __launch_bounds__(kSlicedThreads) smp_sliced_kernel(const int64_
                 uint64_t acca = 0ull, accb = 0ull;
                 int64_t ea = 0, ea1 = 0, eb = 0, eb1 = 0;
                 if (needa) {
-                    ea = wptrT[wa];
-                    ea1 = wptrT[wa + 1];
+                    const longlong2 r = wcsr_row(wptrT, wa);
+                    ea = r.x;
+                    ea1 = r.y;
                 }
                 if (needb) {
-                    eb = wptrT[wb];
-                    eb1 = wptrT[wb + 1];
+                    const longlong2 r = wcsr_row(wptrT, wb);
+                    eb = r.x;
+                    eb1 = r.y;
                 }
                 while (true) {
                     const bool ta = ea < ea1 && (acca & needa) != needa;
@@ -1565,8 +1436,9 @@ __global__ void __launch_bounds__(kClusterThreads, 1) smp_cluster_kernel(const C
             const uint64_t need = act & ~vw;  // active rows that have not reached w = base + i
             int es = 0, c = 0;
             if (need) {
-                es = static_cast<int>(a.wptrT[base + i]);
-                c = static_cast<int>(a.wptrT[base + i + 1]) - es;
+                const longlong2 r = wcsr_row(a.wptrT, base + i);
+                es = static_cast<int>(r.x);
+                c = static_cast<int>(r.y - r.x);
             }
             acc_s[lane] = 0ull;
             __syncwarp();
@@ -1841,30 +1713,23 @@ cudaError_t launch_insert_chunk(uint64_t* P, int64_t n, int64_t ldw, const int32
     return cudaGetLastError();
 }
 
-cudaError_t launch_wcsr_build(const uint64_t* P, int64_t n, int64_t ldw, int64_t* wptr, int32_t* widx, uint64_t* wval,
-                              cudaStream_t s, int64_t* scan_scratch) {
-    const int grid = warps_grid(n, 152);
-    wcsr_count_kernel<<<grid, 256, 0, s>>>(P, n, ldw, wptr);
-    const int64_t chunks = (n + kScanChunk - 1) / kScanChunk;
-    if (scan_scratch != nullptr && chunks > 1 && chunks <= kScanMaxChunks) {
-        scan_chunks_kernel<<<static_cast<unsigned>(chunks), 1024, 0, s>>>(wptr, n, scan_scratch, static_cast<int>(chunks));
-        scan_add_kernel<<<static_cast<unsigned>(chunks), 1024, 0, s>>>(wptr, n, scan_scratch, static_cast<int>(chunks));
-    } else {
-        scan_kernel<<<1, 1024, 0, s>>>(wptr, n);
-    }
-    wcsr_fill_kernel<<<grid, 256, 0, s>>>(P, n, ldw, wptr, widx, wval);
+cudaError_t launch_wcsr_build(const uint64_t* P, int64_t n, int64_t ldw, const WordIndex& x, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(x.ptr + 2 * n, 0, 2 * sizeof(int64_t), s);
+    if (e != cudaSuccess) return e;
+    const int64_t blocks = (n + 7) / 8;  // one step each: the next block's reads overlap this one's writes
+    wcsr_build_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(P, n, ldw, x.ptr, x.idx, x.val);
     return cudaGetLastError();
 }
 
 int smp_packed_max_words() { return 7168; }
 
-cudaError_t launch_square_rows(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, const uint64_t* P,
-                               int64_t n, int64_t ldw, uint64_t* C, int sms, cudaStream_t s, int* changed) {
+cudaError_t launch_indexed_rows(const WordIndex& A, const WordIndex& B, const uint64_t* P, int64_t n, int64_t ldw,
+                                uint64_t* C, int sms, cudaStream_t s, int* changed) {
     int warps = 8;
     while (warps > 1 && warps * ldw * 8 > 32 * 1024) warps >>= 1;
     const size_t smem = static_cast<size_t>(warps) * static_cast<size_t>(ldw) * 8;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(square_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(indexed_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(smem));
         if (e != cudaSuccess) return e;
     }
@@ -1872,7 +1737,7 @@ cudaError_t launch_square_rows(const int64_t* wptr, const int32_t* widx, const u
     const int64_t cap = static_cast<int64_t>(sms) * 16;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    square_rows_kernel<<<static_cast<int>(blocks), warps * 32, smem, s>>>(wptr, widx, wval, P, n, ldw, C, changed);
+    indexed_rows_kernel<<<static_cast<int>(blocks), warps * 32, smem, s>>>(A, B, P, n, ldw, C, changed);
     return cudaGetLastError();
 }
 
@@ -1882,11 +1747,10 @@ int64_t smp_sliced_grid(int64_t n, int sms) {
     return nbatch < cap ? nbatch : cap;
 }
 
-cudaError_t launch_smp_sliced(const int64_t* wptrT, const int32_t* widxT, const uint64_t* wvalT, int64_t n,
-                              uint64_t* scratch, uint64_t* out, int64_t ldw_out, unsigned long long* bcounter,
+cudaError_t launch_smp_sliced(const WordIndex& T, int64_t n, uint64_t* scratch, uint64_t* out, int64_t ldw_out, unsigned long long* bcounter,
                               int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl) {
     const int64_t grid = smp_sliced_grid(n, sms);
-    smp_sliced_kernel<<<static_cast<int>(grid), kSlicedThreads, 0, s>>>(wptrT, widxT, wvalT, n, (n + 63) / 64, scratch, out,
+    smp_sliced_kernel<<<static_cast<int>(grid), kSlicedThreads, 0, s>>>(T.ptr, T.idx, T.val, n, (n + 63) / 64, scratch, out,
                                                              ldw_out, bcounter, levels, max_levels, dl);
     return cudaGetLastError();
 }
@@ -1963,8 +1827,7 @@ static bool smp_cluster_fits_query(int ctas, int lg) {
     return clusters > 0;
 }
 
-cudaError_t launch_smp_cluster(const int64_t* wptrT, const int32_t* widxT, const uint64_t* wvalT, int64_t n,
-                               const uint64_t* src, int64_t ldw_src, int64_t rows, uint64_t* out, int64_t ldw_out,
+cudaError_t launch_smp_cluster(const WordIndex& T, int64_t n, const uint64_t* src, int64_t ldw_src, int64_t rows, uint64_t* out, int64_t ldw_out,
                                int reflexive, int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl) {
     const int64_t batches = (rows + 63) / 64;
     int ctas = 0, lg = 0;
@@ -1974,7 +1837,7 @@ cudaError_t launch_smp_cluster(const int64_t* wptrT, const int32_t* widxT, const
     cudaError_t e = cudaFuncSetAttribute(smp_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(cfg.dynamicSmemBytes));
     if (e != cudaSuccess) return e;
-    const ClusterArgs a{wptrT, widxT, wvalT, src, ldw_src, n, rows, out, ldw_out, levels, max_levels, reflexive, lg,
+    const ClusterArgs a{T.ptr, T.idx, T.val, src, ldw_src, n, rows, out, ldw_out, levels, max_levels, reflexive, lg,
                         dl};
     return cudaLaunchKernelEx(&cfg, smp_cluster_kernel, a);
 }
@@ -2054,35 +1917,32 @@ cudaError_t launch_smp_rows(const uint64_t* R, int64_t ld_r, int64_t n, const ui
     return cudaLaunchKernelEx(&cfg, smp_rows_kernel, a);
 }
 
-cudaError_t launch_square_growth(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, int64_t n,
-                                 int64_t ldw, unsigned long long* out, int sms, cudaStream_t s,
+cudaError_t launch_square_growth(const WordIndex& x, int64_t n, int64_t ldw, unsigned long long* out, int sms, cudaStream_t s,
                                  unsigned long long* bits_out) {
     const size_t smem = static_cast<size_t>(8) * ((ldw + 31) / 32) * 4;
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
-    square_growth_kernel<<<warps_grid(n, sms), 256, smem, s>>>(wptr, widx, wval, n, ldw, out, bits_out);
+    square_growth_kernel<<<warps_grid(n, sms), 256, smem, s>>>(x.ptr, x.idx, x.val, n, ldw, out, bits_out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_transpose(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, int64_t n,
-                                     int64_t ldw, uint64_t* out, int sms, cudaStream_t s) {
+cudaError_t launch_scatter_transpose(const WordIndex& x, int64_t n, int64_t ldw, uint64_t* out, int sms, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(out, 0, static_cast<size_t>(n) * static_cast<size_t>(ldw) * 8, s);
     if (e != cudaSuccess) return e;
-    scatter_transpose_kernel<<<warps_grid(n, sms), 256, 0, s>>>(wptr, widx, wval, n, ldw,
+    scatter_transpose_kernel<<<warps_grid(n, sms), 256, 0, s>>>(x.ptr, x.idx, x.val, n, ldw,
                                                                 reinterpret_cast<unsigned long long*>(out));
     return cudaGetLastError();
 }
 
-cudaError_t launch_square_cost(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, int64_t n,
-                               unsigned long long* cost, int sms, cudaStream_t s) {
-    square_cost_kernel<<<warps_grid(n, sms), 256, 0, s>>>(wptr, widx, wval, n, cost);
+cudaError_t launch_indexed_cost(const WordIndex& A, const WordIndex& B, int64_t n, unsigned long long* cost, int sms,
+                                cudaStream_t s) {
+    indexed_cost_kernel<<<warps_grid(n, sms), 256, 0, s>>>(A, B, n, cost);
     return cudaGetLastError();
 }
 
-cudaError_t launch_smp_packed(const int64_t* wptr, const int32_t* widx, const uint64_t* wval, int64_t n, int64_t ldw,
-                              const uint64_t* src, int64_t ldw_src, int64_t q, uint64_t* out, int64_t ldw_out,
-                              int* levels, int* qcounter, int reflexive, int sms, cudaStream_t s, Deadline dl,
-                              const int64_t* wptrT, const int32_t* widxT, const uint64_t* wvalT) {
+cudaError_t launch_smp_packed(const WordIndex& x, const WordIndex& T, int64_t n, int64_t ldw, const uint64_t* src,
+                              int64_t ldw_src, int64_t q, uint64_t* out, int64_t ldw_out, int* levels, int* qcounter,
+                              int reflexive, int sms, cudaStream_t s, Deadline dl) {
     // blocks of 1-8 warps, chosen so that as many warps as possible fit an SM's shared memory
     const int64_t per_warp = smp_warp_bytes(ldw);
     if (per_warp > 200 * 1024) return cudaErrorInvalidValue;
@@ -2099,8 +1959,8 @@ cudaError_t launch_smp_packed(const int64_t* wptr, const int32_t* widx, const ui
     if (blocks < 1) blocks = 1;
     const int max_levels = static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF);
     smp_packed_kernel<<<static_cast<int>(blocks), warps * 32, smem, s>>>(
-        wptr, widx, wval, n, ldw, src, ldw_src, q, out, ldw_out, levels,
-        reinterpret_cast<unsigned long long*>(qcounter), reflexive, max_levels, dl, wptrT, widxT, wvalT);
+        x.ptr, x.idx, x.val, n, ldw, src, ldw_src, q, out, ldw_out, levels,
+        reinterpret_cast<unsigned long long*>(qcounter), reflexive, max_levels, dl, T.ptr, T.idx, T.val);
     return cudaGetLastError();
 }
 
@@ -2122,9 +1982,7 @@ cudaError_t launch_frontier_group(const FrontierJob* jobs, int njobs, int64_t ma
     if (tb > 4096) tb = 4096;
     frontier_transpose_kernel<<<dim3(static_cast<unsigned>(tb < 1 ? 1 : tb), nj), 64, 0, s>>>(jobs);
     const int rows_grid = warps_grid(max_n, sms) / 8 + 1;  // the jobs of a launch share the GPU
-    frontier_wcsr_count_kernel<<<dim3(static_cast<unsigned>(rows_grid), nj, 2), 256, 0, s>>>(jobs);
-    frontier_scan_kernel<<<dim3(1, nj, 2), 1024, 0, s>>>(jobs);
-    frontier_wcsr_fill_kernel<<<dim3(static_cast<unsigned>(rows_grid), nj, 2), 256, 0, s>>>(jobs);
+    frontier_wcsr_kernel<<<dim3(static_cast<unsigned>(rows_grid), nj, 2), 256, 0, s>>>(jobs);
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
     int warps = 8;
