@@ -614,8 +614,7 @@ bool is_solo(const bmlp_problem& p, int variant, int64_t solo_n) {
     return v == BMLP_AUTO || v == BMLP_RMS_TC;
 }
 
-bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, long long wait_cycles,
-                       const cudaGraphNode_t* after, size_t nafter);
+bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, long long wait_cycles);
 
 bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count, int variant, long long wait_cycles,
                         uint64_t key, int64_t solo_n, BatchCache** out) {
@@ -777,7 +776,7 @@ bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count,
     BCK(prepare_tc_group(), "tensor-core group kernel attributes");
     BCK(cudaGraphCreate(&c->graph, 0), "cudaGraphCreate");
     if (np == 0) {
-        BST(build_solo(ctx, c, probs, wait_cycles, nullptr, 0));
+        BST(build_solo(ctx, c, probs, wait_cycles));
         BCK(cudaGraphInstantiate(&c->exec, c->graph, 0), "cudaGraphInstantiate");
         *out = c;
         return BMLP_OK;
@@ -847,7 +846,7 @@ bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count,
         BST(add_kernel(ctx, c->graph, &n_dec, &n_final, 1, reinterpret_cast<void*>(&batch_decode_kernel),
                        dim3(64, gy), dim3(256), 0, a));
     }
-    if (!c->solo.empty()) BST(build_solo(ctx, c, probs, wait_cycles, &n_dec, 1));
+    if (!c->solo.empty()) BST(build_solo(ctx, c, probs, wait_cycles));
     BCK(cudaGraphInstantiate(&c->exec, c->graph, 0), "cudaGraphInstantiate");
     *out = c;
     return BMLP_OK;
@@ -879,16 +878,16 @@ bmlp_status add_while(bmlp_ctx* ctx, cudaStream_t cs, cudaGraphConditionalHandle
     return add_conditional(ctx, cs, h, cudaGraphCondTypeWhile, body);
 }
 
-// The large problems as device-driven single-problem pipelines, one after another (they share one scratch sized
-// for the largest), captured into the batch graph after `after`.
-bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, long long wait_cycles,
-                       const cudaGraphNode_t* after, size_t nafter) {
-    const int ns = static_cast<int>(c->solo.size());
+// One lane of the large problems: device-driven single-problem pipelines, one after another on one scratch sized for the
+// lane's largest, captured into the batch graph as a branch of its own. `mine`: their places in c->solo. With base null
+// only *bytes, the scratch that the lane needs, is computed.
+bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, long long wait_cycles,
+                       const std::vector<int>& mine, uint8_t* base, size_t* bytes) {
     int64_t nmax = 0;
     bool any_compose = false;
-    for (int i : c->solo) {
-        nmax = std::max(nmax, probs[i].n);
-        any_compose |= probs[i].kind == BMLP_PROBLEM_COMPOSE;
+    for (int k : mine) {
+        nmax = std::max(nmax, probs[c->solo[k]].n);
+        any_compose |= probs[c->solo[k]].kind == BMLP_PROBLEM_COMPOSE;
     }
     const int64_t ldw_max = round_up((nmax + 63) / 64, 2);
     const int64_t np_max = round_up(nmax, TC_PAD);
@@ -921,9 +920,9 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
         oTT = take(2 * bits);
         oTAux = take(thin_aux_bytes(nmax, ldwt_max));
     }
-    void* base = nullptr;
-    BST(ws_get(ctx, WS_SOLO, total, &base));
-    uint8_t* b8 = static_cast<uint8_t*>(base);
+    *bytes = total;
+    if (base == nullptr) return BMLP_OK;
+    uint8_t* b8 = base;
     uint64_t* P0 = reinterpret_cast<uint64_t*>(b8 + oP0);
     uint64_t* P1 = reinterpret_cast<uint64_t*>(b8 + oP1);
     int64_t* wptr = reinterpret_cast<int64_t*>(b8 + oPtr);
@@ -935,10 +934,6 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
     uint64_t* TP = reinterpret_cast<uint64_t*>(b8 + oTP);
     uint64_t* TPT = reinterpret_cast<uint64_t*>(b8 + oTPT);
     uint64_t* TT = reinterpret_cast<uint64_t*>(b8 + oTT);
-    BCK(cudaMalloc(&c->d_solo, sizeof(int) * SW_WORDS * ns), "cudaMalloc(large-problem state)");
-    BCK(cudaMemset(c->d_solo, 0, sizeof(int) * SW_WORDS * ns), "clear large-problem state");
-    c->h_solo.assign(static_cast<size_t>(SW_WORDS * ns), 0);
-
     cudaStream_t cs = nullptr, cb = nullptr, cc = nullptr;
     BCK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking), "capture stream");
     cudaError_t ce = cudaStreamCreateWithFlags(&cb, cudaStreamNonBlocking);
@@ -956,7 +951,7 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
             cudaStreamDestroy(c);
         }
     } guard_streams{cs, cb, cc};
-    BCK(cudaStreamBeginCaptureToGraph(cs, c->graph, after, nullptr, nafter, cudaStreamCaptureModeRelaxed),
+    BCK(cudaStreamBeginCaptureToGraph(cs, c->graph, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed),
         "begin capture of the large problems");
     bmlp_status status = BMLP_OK;
     auto fail = [&](bmlp_status st) {
@@ -977,7 +972,7 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
     } while (0)
     const int sms = ctx->sm_count;
     const double s_word = bitrow_s_per_word(), s_row = bitrow_row_s_per_word(), step_s = bitrow_step_s();
-    for (int k = 0; k < ns; ++k) {
+    for (int k : mine) {
         const bmlp_problem& p = probs[c->solo[k]];
         int* w = c->d_solo + SW_WORDS * k;
         const int64_t n = p.n, ldw = round_up((n + 63) / 64, 2), n_pad = round_up(n, TC_PAD), ld4 = n_pad / 2;
@@ -1175,6 +1170,54 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
     cudaGraph_t g = nullptr;
     BCK(cudaStreamEndCapture(cs, &g), "end capture of the large problems");
     return status;
+}
+
+// Branches of the batch graph that the large problems are dealt out to, besides the branch of the grouped ones. A
+// pipeline is a chain of small launches (bit-row squarings, decisions) between tensor-core products that fill the GPU, so
+// several chains at once fill each other's gaps (measured on the knowledge-graph batch, 33 closures and 8 compositions
+// with n >= 4,096: LANES_TABLE). More lanes than that add scratch (at most kLaneBytes in all, else fewer lanes).
+constexpr int kLanes = 4;
+constexpr size_t kLaneBytes = size_t(24) << 30;
+
+bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, long long wait_cycles) {
+    const int ns = static_cast<int>(c->solo.size());
+    BCK(cudaMalloc(&c->d_solo, sizeof(int) * SW_WORDS * ns), "cudaMalloc(large-problem state)");
+    BCK(cudaMemset(c->d_solo, 0, sizeof(int) * SW_WORDS * ns), "clear large-problem state");
+    c->h_solo.assign(static_cast<size_t>(SW_WORDS * ns), 0);
+    // longest first, each to the lane with the least predicted time: a product or two of its size, and its launches
+    std::vector<int> order(ns);
+    for (int k = 0; k < ns; ++k) order[k] = k;
+    const auto cost = [&](int k) {
+        const bmlp_problem& p = probs[c->solo[k]];
+        return 2.0 * tc4_product_s(round_up(p.n, TC_PAD)) + 300e-6;
+    };
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(x) > cost(y); });
+    for (int lanes = std::min(kLanes, ns); lanes >= 1; --lanes) {
+        std::vector<std::vector<int>> mine(lanes);
+        std::vector<double> load(lanes, 0.0);
+        for (int k : order) {
+            const int l = static_cast<int>(std::min_element(load.begin(), load.end()) - load.begin());
+            mine[l].push_back(k);
+            load[l] += cost(k);
+        }
+        std::vector<size_t> bytes(lanes, 0);
+        size_t total = 0;
+        for (int l = 0; l < lanes; ++l) {
+            BST(build_lane(ctx, c, probs, wait_cycles, mine[l], nullptr, &bytes[l]));
+            total += bytes[l];
+        }
+        if (lanes > 1 && total > kLaneBytes) continue;
+        void* base = nullptr;
+        BST(ws_get(ctx, WS_SOLO, total, &base));
+        size_t at = 0;
+        for (int l = 0; l < lanes; ++l) {
+            size_t unused = 0;
+            BST(build_lane(ctx, c, probs, wait_cycles, mine[l], static_cast<uint8_t*>(base) + at, &unused));
+            at += bytes[l];
+        }
+        break;
+    }
+    return BMLP_OK;
 }
 
 uint64_t batch_key(const bmlp_problem* probs, int64_t count, int variant, const int* tune, int64_t solo_n) {
