@@ -38,20 +38,10 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int TILE = 64;
 
 // ------------------------------------------------------------ encoding --
-__device__ __forceinline__ uint32_t src_bits16(const void* in, int fmt, int64_t n, int64_t r, int64_t c0) {
+// Columns c0 .. c0 + 15 of row r of n packed rows (padding bits zero).
+__device__ __forceinline__ uint32_t src_bits16(const uint64_t* in, int64_t ldw, int64_t n, int64_t r, int64_t c0) {
     if (r >= n || c0 >= n) return 0;
-    uint32_t m = 0;
-    if (fmt == BMLP_FMT_U8) {
-        const uint8_t* row = static_cast<const uint8_t*>(in) + r * n;
-        for (int x = 0; x < 16; ++x)
-            if (c0 + x < n && row[c0 + x] != 0) m |= 1u << x;
-    } else {
-        const uint64_t w = static_cast<const uint64_t*>(in)[r * ((n + 63) / 64) + (c0 >> 6)];
-        m = static_cast<uint32_t>((w >> (c0 & 63)) & 0xFFFFu);
-        const int64_t valid = n - c0;
-        if (valid < 16) m &= (1u << valid) - 1u;
-    }
-    return m;
+    return static_cast<uint32_t>((in[r * ldw + (c0 >> 6)] >> (c0 & 63)) & 0xFFFFu);
 }
 
 __device__ __forceinline__ uint4 expand16(uint32_t m) {
@@ -66,16 +56,16 @@ __device__ __forceinline__ uint4 expand16(uint32_t m) {
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// R and R^T (ld x ld E4M3 bytes, zero padding) of one caller matrix, tiles
+// R and R^T (ld x ld E4M3 bytes, zero padding) of n packed rows, tiles
 // strided over the blocks of this problem.
-__device__ void encode_e4m3(const void* in, int fmt, int64_t n, uint8_t* R, uint8_t* RT, int64_t ld,
+__device__ void encode_e4m3(const uint64_t* in, int64_t ldw, int64_t n, uint8_t* R, uint8_t* RT, int64_t ld,
                             uint16_t (*masks)[TILE / 16 + 1]) {
     const int tid = threadIdx.x;
     const int r = tid >> 2, cseg = (tid & 3) * 16;
     const int64_t tiles1 = ld / TILE;
     for (int64_t t = blockIdx.x; t < tiles1 * tiles1; t += gridDim.x) {
         const int64_t row0 = (t / tiles1) * TILE, col0 = (t % tiles1) * TILE;
-        const uint32_t m = src_bits16(in, fmt, n, row0 + r, col0 + cseg);
+        const uint32_t m = src_bits16(in, ldw, n, row0 + r, col0 + cseg);
         masks[r][tid & 3] = static_cast<uint16_t>(m);
         *reinterpret_cast<uint4*>(R + (row0 + r) * ld + col0 + cseg) = expand16(m);
         __syncthreads();
@@ -87,41 +77,76 @@ __device__ void encode_e4m3(const void* in, int fmt, int64_t n, uint8_t* R, uint
     }
 }
 
-// blockIdx.y = problem. 256 threads.
-__global__ void __launch_bounds__(256) batch_encode_kernel(const GroupProblem* probs) {
-    __shared__ uint16_t masks[TILE][TILE / 16 + 1];
-    const GroupProblem& g = probs[blockIdx.y];
-    if (g.n == 0) return;
-    if (g.engine == 0) {
-        encode_e4m3(g.kind == 1 ? g.in2 : g.in1, g.fmt, g.n, g.M[0], g.T[0], g.ld, masks);
-        if (g.kind == 1) encode_e4m3(g.in1, g.fmt, g.n, g.X, g.R1T, g.ld, masks);  // X is scratch here
-    } else {
-        const int64_t wpr = (g.n + 63) / 64;
-        const int64_t total = g.n * g.ldw;
-        for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < total;
-             t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-            const int64_t r = t / g.ldw, w = t % g.ldw;
+// A caller matrix as n packed rows of ldw words (a warp per row, padding bits and words zero); its ones are added into
+// *ones and the most of one row goes into *top (null: not counted).
+__device__ void pack_rows(const void* in, int fmt, int64_t n, uint64_t* P, int64_t ldw, unsigned long long* ones,
+                          int* top) {
+    const int lane = threadIdx.x & 31;
+    const int64_t wpr = (n + 63) / 64;
+    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
+    unsigned long long sum = 0;
+    unsigned most = 0;
+    for (int64_t r = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n; r += warps) {
+        unsigned c = 0;
+        for (int64_t w0 = 0; w0 < ldw; w0 += 32) {
             uint64_t bits = 0;
-            if (w < wpr) {
-                if (g.fmt == BMLP_FMT_U8) {
-                    const uint8_t* row = static_cast<const uint8_t*>(g.in1) + r * g.n + w * 64;
-                    const int64_t valid = g.n - w * 64 < 64 ? g.n - w * 64 : 64;
-                    for (int k = 0; k < valid; ++k)
-                        if (row[k]) bits |= 1ull << k;
-                } else {
-                    bits = static_cast<const uint64_t*>(g.in1)[r * wpr + w];
-                    const int64_t valid = g.n - w * 64;
-                    if (valid < 64) bits &= (1ull << valid) - 1ull;
+            const int64_t w = w0 + lane;
+            if (fmt == BMLP_FMT_U8) {
+                const uint8_t* row = static_cast<const uint8_t*>(in) + r * n;
+                for (int64_t x = w0; x < w0 + 32 && x < wpr; ++x) {  // 64 bytes of the row per step, a byte per lane
+                    const int64_t j = x * 64 + lane;
+                    const unsigned lo = __ballot_sync(FULL, j < n && row[j] != 0);
+                    const unsigned hi = __ballot_sync(FULL, j + 32 < n && row[j + 32] != 0);
+                    if (x == w) bits = static_cast<uint64_t>(lo) | (static_cast<uint64_t>(hi) << 32);
                 }
+            } else if (w < wpr) {
+                bits = static_cast<const uint64_t*>(in)[r * wpr + w];
+                const int64_t valid = n - w * 64;
+                if (valid < 64) bits &= (1ull << valid) - 1ull;
             }
-            g.P[0][t] = bits;
+            if (w < ldw) P[r * ldw + w] = bits;
+            c += __popcll(bits);
         }
+        c = __reduce_add_sync(FULL, c);
+        sum += c;
+        most = c > most ? c : most;
+    }
+    if (ones != nullptr && lane == 0 && sum != 0ull) {
+        atomicAdd(ones, sum);
+        atomicMax(top, static_cast<int>(most));
     }
 }
 
+// blockIdx.y = problem. 256 threads. Every problem starts as packed rows.
+__global__ void __launch_bounds__(256) batch_encode_kernel(const GroupProblem* probs, const GroupState* st) {
+    const GroupProblem& g = probs[blockIdx.y];
+    if (g.n == 0) return;
+    pack_rows(g.kind == 1 ? g.in2 : g.in1, g.fmt, g.n, g.P[0], g.ldw, &st->ones[blockIdx.y], &st->top[blockIdx.y]);
+    if (g.kind == 1) pack_rows(g.in1, g.fmt, g.n, g.PR1, g.ldw, nullptr, nullptr);
+}
+
+// Tensor-core operands of the problems that the bit rows handed over.
+__global__ void __launch_bounds__(256) batch_operands_kernel(const GroupProblem* probs, const GroupState* st) {
+    __shared__ uint16_t masks[TILE][TILE / 16 + 1];
+    const GroupProblem& g = probs[blockIdx.y];
+    if (g.n == 0 || st->phase[blockIdx.y] == 0) return;
+    encode_e4m3(g.P[st->ppar[blockIdx.y]], g.ldw, g.n, g.M[0], g.T[0], g.ld, masks);
+    if (g.kind == 1) encode_e4m3(g.PR1, g.ldw, g.n, g.X, g.R1T, g.ld, masks);  // X is scratch here
+}
+
 // ------------------------------------------------------------- planner --
-// mode 0: start of the loop (every problem active); mode 1: after a product
-// (retire, flip parity, count); mode 2: final products of compositions.
+// Whether the next squaring of a tensor-core problem is cheaper on its bit rows: every one of R names a row of ldw words
+// (L2 reads over the whole GPU), and the row with the most ones is one warp's work; against its share of a grouped
+// tensor-core product (ld^3 at the E4M3 kernel's rate). Relations of a knowledge graph with fewer constants than triples
+// stay sparse up to their closure: their dense products were 7.2 ms of a batch, their bit rows are 0.5 ms.
+__device__ __forceinline__ bool rows_cheaper(const GroupProblem& g, unsigned long long ones, int top) {
+    const double ld = static_cast<double>(g.ld);
+    return top <= 192 && static_cast<double>(ones) * static_cast<double>(g.ldw) * 1.5e-12 < 2.0 * ld * ld * ld / 2.4e15;
+}
+
+// mode 0: start (every squaring problem on bit rows, except the tensor-core ones whose bit rows are too full); mode 1:
+// after a bit-row squaring; mode 3: start of the tensor-core loop (the problems handed over); mode 4: after a tensor-core
+// product (1 and 4: retire, flip parity, count; 1 also hands over); mode 2: final products of compositions.
 __global__ void __launch_bounds__(1024) batch_plan_kernel(const GroupProblem* probs, const GroupState* st, int nprob,
                                                           int mode, cudaGraphConditionalHandle h, int set_cond) {
     __shared__ int part_tc[1024], part_pk[1024];
@@ -137,8 +162,9 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(const GroupProblem* pr
             st->parity[p] = g.engine == 2 ? 1 : 0;
             st->iters[p] = 0;
             st->notconv[p] = 0;
-            st->active[p] = (g.n > 0 && g.engine != 2) ? 1 : 0;
-        } else if (mode == 1) {
+            st->phase[p] = g.n > 0 && g.engine == 0 && !rows_cheaper(g, st->ones[p], st->top[p]) ? 1 : 0;
+            st->active[p] = (g.n > 0 && g.engine != 2 && st->phase[p] == 0) ? 1 : 0;
+        } else if (mode == 1 || mode == 4) {
             if (st->active[p]) {
                 st->iters[p] += 1;
                 st->parity[p] ^= 1;
@@ -147,15 +173,26 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(const GroupProblem* pr
                 } else if (st->iters[p] >= g.cap) {
                     st->active[p] = 0;
                     st->notconv[p] = 1;
+                } else if (mode == 1 && g.engine == 0 && !rows_cheaper(g, st->ones[p], st->top[p])) {
+                    st->active[p] = 0;
+                    st->phase[p] = 1;
                 }
             }
+        } else if (mode == 3) {
+            st->ppar[p] = st->parity[p];
+            st->active[p] = st->phase[p];
+            if (st->phase[p]) st->parity[p] = 0;
         } else {
-            st->active[p] = (g.kind == 1 && g.n > 0) ? 1 : 0;
+            st->active[p] = (g.kind == 1 && g.n > 0 && st->phase[p] == 1) ? 1 : 0;
+        }
+        if (mode <= 1) {
+            st->ones[p] = 0ull;
+            st->top[p] = 0;
         }
         st->changed[p] = 0;
         const int act = st->active[p];
-        const int ctc = (act && (mode == 2 || g.engine == 0)) ? g.m_tiles * g.n_tiles : 0;
-        const int cpk = (act && mode != 2 && g.engine == 1) ? static_cast<int>(g.n) : 0;
+        const int ctc = (act && mode >= 2) ? g.m_tiles * g.n_tiles : 0;
+        const int cpk = (act && mode <= 1) ? static_cast<int>(g.n) : 0;
         st->tc_offs[p] = ctc;
         st->pk_offs[p] = cpk;
         stc += ctc;
@@ -191,81 +228,108 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(const GroupProblem* pr
 }
 
 // ------------------------------------------------ packed squaring step --
-// One warp per active row of every packed-engine problem:
-// C_i = R_i | OR_{k : R_ik = 1} R_k, chunks of 32 lanes x VEC x 2 words.
-template <int VEC>
+// C_i = A_i' | OR_{k : A_ik = 1} B_k for one row, by a whole warp (A_i' = init, a row of ldw words), in chunks of 64 words
+// (two per lane), four named rows in flight. Returns the ones written; *grew: C_i != init.
+__device__ __forceinline__ unsigned gather_row(const uint64_t* __restrict__ arow, const uint64_t* __restrict__ B,
+                                               const uint64_t* __restrict__ init, uint64_t* __restrict__ out, int64_t ldw,
+                                               int lane, bool* grew) {
+    unsigned ones = 0;
+    uint32_t any = 0;
+    for (int64_t c0 = 0; c0 < ldw; c0 += 64) {
+        const int64_t w = c0 + 2 * lane;
+        const bool in = w < ldw;  // ldw is even: both words
+        const uint4 old = in ? *reinterpret_cast<const uint4*>(init + w) : make_uint4(0, 0, 0, 0);
+        uint4 acc = old;
+        for (int64_t wb = 0; wb < ldw; wb += 32) {
+            const uint64_t aw = wb + lane < ldw ? arow[wb + lane] : 0ull;
+            unsigned m = __ballot_sync(FULL, aw != 0ull);
+            uint64_t bits = 0ull;
+            int64_t kb = 0;
+            while (m != 0u || bits != 0ull) {
+                uint4 x[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (bits == 0ull && m != 0u) {
+                        const int sl = __ffs(m) - 1;
+                        m &= m - 1u;
+                        bits = __shfl_sync(FULL, aw, sl);
+                        kb = (wb + sl) * 64;
+                    }
+                    x[q] = make_uint4(0, 0, 0, 0);
+                    if (bits != 0ull) {
+                        const int64_t k = kb + __ffsll(static_cast<long long>(bits)) - 1;
+                        bits &= bits - 1ull;
+                        if (in) x[q] = *reinterpret_cast<const uint4*>(B + k * ldw + w);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    acc.x |= x[q].x;
+                    acc.y |= x[q].y;
+                    acc.z |= x[q].z;
+                    acc.w |= x[q].w;
+                }
+            }
+        }
+        if (in) *reinterpret_cast<uint4*>(out + w) = acc;
+        any |= (old.x ^ acc.x) | (old.y ^ acc.y) | (old.z ^ acc.z) | (old.w ^ acc.w);
+        ones += __popc(acc.x) + __popc(acc.y) + __popc(acc.z) + __popc(acc.w);
+    }
+    *grew = __any_sync(FULL, any != 0u) != 0;
+    return __reduce_add_sync(FULL, ones);
+}
+
+// One warp per active row of every problem on bit rows: R' = R | R R.
 __global__ void __launch_bounds__(256) packed_group_kernel(const GroupProblem* probs, const GroupState* st, int nprob) {
     const int lane = threadIdx.x & 31;
     const int64_t warp_id = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
     const int total = *st->pk_total;
     const int* offs = st->pk_offs;
-    constexpr int64_t chunk_words = 64 * VEC;
-    for (int64_t item = warp_id; item < total; item += nwarps) {
-        int lo = 0, hi = nprob - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (offs[mid] <= item) lo = mid; else hi = mid - 1;
-        }
+    // a run of consecutive rows per warp, so that the problem of the first is searched for once
+    const int64_t per = (total + nwarps - 1) / nwarps;
+    const int64_t first = warp_id * per, end = first + per < total ? first + per : total;
+    if (first >= end) return;
+    int lo = 0, hi = nprob - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (offs[mid] <= first) lo = mid; else hi = mid - 1;
+    }
+    for (int64_t item = first; item < end; ++item) {
+        while (offs[lo + 1] <= item) ++lo;  // offs[nprob] = total > item
         const GroupProblem& g = probs[lo];
         const int par = st->parity[lo];
         const int64_t i = item - offs[lo];
-        const int64_t ldw = g.ldw;
         const uint64_t* src = g.P[par];
-        uint64_t* dst = g.P[par ^ 1];
-        const uint64_t* arow = src + i * ldw;
-        uint32_t any = 0;
-        for (int64_t c0 = 0; c0 < ldw; c0 += chunk_words) {
-            uint4 acc[VEC];
-#pragma unroll
-            for (int v = 0; v < VEC; ++v) {
-                const int64_t w = c0 + 2 * (lane + 32 * v);
-                acc[v] = (w < ldw) ? *reinterpret_cast<const uint4*>(arow + w) : make_uint4(0, 0, 0, 0);
-            }
-            for (int64_t wb = 0; wb < ldw; wb += 32) {
-                const uint64_t aw = (wb + lane < ldw) ? arow[wb + lane] : 0ull;
-                unsigned m = __ballot_sync(FULL, aw != 0ull);
-                while (m) {
-                    const int sl = __ffs(m) - 1;
-                    m &= m - 1;
-                    uint64_t bits = __shfl_sync(FULL, aw, sl);
-                    const int64_t kbase = (wb + sl) * 64;
-                    while (bits) {
-                        const int b0 = __ffsll(static_cast<long long>(bits)) - 1;
-                        bits &= bits - 1;
-                        const uint64_t* r0 = src + (kbase + b0) * ldw + c0;
-#pragma unroll
-                        for (int v = 0; v < VEC; ++v) {
-                            const int64_t w = 2 * (lane + 32 * v);
-                            if (c0 + w < ldw) {
-                                const uint4 x = *reinterpret_cast<const uint4*>(r0 + w);
-                                acc[v].x |= x.x;
-                                acc[v].y |= x.y;
-                                acc[v].z |= x.z;
-                                acc[v].w |= x.w;
-                            }
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int v = 0; v < VEC; ++v) {
-                const int64_t w = c0 + 2 * (lane + 32 * v);
-                if (w < ldw) {
-                    const uint4 o = *reinterpret_cast<const uint4*>(arow + w);
-                    any |= (o.x ^ acc[v].x) | (o.y ^ acc[v].y) | (o.z ^ acc[v].z) | (o.w ^ acc[v].w);
-                    *reinterpret_cast<uint4*>(dst + i * ldw + w) = acc[v];
-                }
+        bool grew = false;
+        const unsigned ones = gather_row(src + i * g.ldw, src, src + i * g.ldw, g.P[par ^ 1] + i * g.ldw, g.ldw, lane, &grew);
+        if (lane == 0) {
+            if (grew) atomicOr(&st->changed[lo], 1);
+            if (ones != 0u) {
+                atomicAdd(&st->ones[lo], static_cast<unsigned long long>(ones));
+                atomicMax(&st->top[lo], static_cast<int>(ones));
             }
         }
-        if (__any_sync(FULL, any != 0) && lane == 0) atomicOr(&st->changed[lo], 1);
+    }
+}
+
+// Compositions whose closure ended on bit rows: (I + R2+) R1 into the other packed buffer, a warp per row.
+__global__ void __launch_bounds__(256) batch_compose_rows_kernel(const GroupProblem* probs, const GroupState* st) {
+    const GroupProblem& g = probs[blockIdx.y];
+    if (g.kind != 1 || g.n == 0 || st->phase[blockIdx.y] != 0) return;
+    const int lane = threadIdx.x & 31;
+    const int par = st->ppar[blockIdx.y];
+    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < g.n; i += warps) {
+        bool grew = false;
+        gather_row(g.P[par] + i * g.ldw, g.PR1, g.PR1 + i * g.ldw, g.P[par ^ 1] + i * g.ldw, g.ldw, lane, &grew);
     }
 }
 
 // I + R2+ for the compositions (diagonal of the closure buffer).
 __global__ void batch_compose_prep_kernel(const GroupProblem* probs, const GroupState* st) {
     const GroupProblem& g = probs[blockIdx.y];
-    if (g.kind != 1 || g.n == 0) return;
+    if (g.kind != 1 || g.n == 0 || st->phase[blockIdx.y] == 0) return;
     uint8_t* R = g.M[st->parity[blockIdx.y]];
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < g.n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x)
@@ -278,46 +342,38 @@ __global__ void __launch_bounds__(256) batch_decode_kernel(const GroupProblem* p
     if (g.n == 0) return;
     const int64_t n = g.n, wpr = (n + 63) / 64;
     const int refl = (g.kind == 0) ? g.reflexive : 0;
-    const int par = st->parity[blockIdx.y];
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (g.engine == 0) {
-        const uint8_t* src = (g.kind == 1) ? g.X : g.M[par];
+    const int lane = threadIdx.x & 31;
+    const bool tc = st->phase[blockIdx.y] == 1;
+    const uint8_t* M = (g.kind == 1) ? g.X : g.M[st->parity[blockIdx.y]];
+    const uint64_t* P = g.P[st->ppar[blockIdx.y] ^ (g.kind == 1 ? 1 : 0)];
+    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
+    // a warp per row: words of 64 columns, or bytes, from the E4M3 bytes of a row or from its words
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
         if (g.fmt == BMLP_FMT_U8) {
-            uint8_t* out = static_cast<uint8_t*>(g.out);
-            for (int64_t t = t0; t < n * n; t += stride) {
-                const int64_t i = t / n, j = t % n;
-                out[t] = (src[i * g.ld + j] != 0 || (refl && i == j)) ? 1 : 0;
+            uint8_t* out = static_cast<uint8_t*>(g.out) + i * n;
+            for (int64_t j = lane; j < n; j += 32) {
+                const bool b = tc ? M[i * g.ld + j] != 0 : ((P[i * g.ldw + (j >> 6)] >> (j & 63)) & 1ull) != 0ull;
+                out[j] = (b || (refl && i == j)) ? 1 : 0;
             }
         } else {
-            uint64_t* out = static_cast<uint64_t*>(g.out);
-            for (int64_t t = t0; t < n * wpr; t += stride) {
-                const int64_t i = t / wpr, w = t % wpr;
-                const uint8_t* row = src + i * g.ld + w * 64;
+            uint64_t* out = static_cast<uint64_t*>(g.out) + i * wpr;
+            for (int64_t w0 = 0; w0 < wpr; w0 += 32) {
+                const int64_t w = w0 + lane;
                 uint64_t bits = 0;
-                for (int k = 0; k < 64; ++k)
-                    if (row[k]) bits |= 1ull << k;
-                const int64_t valid = n - w * 64;
-                if (valid < 64) bits &= (1ull << valid) - 1ull;
+                if (!tc) {
+                    bits = w < wpr ? P[i * g.ldw + w] : 0ull;
+                } else {
+                    for (int64_t x = w0; x < w0 + 32 && x < wpr; ++x) {  // ld is a multiple of 256: both bytes exist
+                        const uint8_t* b = M + i * g.ld + x * 64 + lane;
+                        const unsigned lo = __ballot_sync(FULL, b[0] != 0);
+                        const unsigned hi = __ballot_sync(FULL, b[32] != 0);
+                        if (x == w) bits = static_cast<uint64_t>(lo) | (static_cast<uint64_t>(hi) << 32);
+                    }
+                    const int64_t valid = n - w * 64;
+                    if (valid < 64) bits &= valid > 0 ? (1ull << valid) - 1ull : 0ull;
+                }
                 if (refl && (i >> 6) == w) bits |= 1ull << (i & 63);
-                out[t] = bits;
-            }
-        }
-    } else {
-        const uint64_t* P = g.P[par];
-        if (g.fmt == BMLP_FMT_U8) {
-            uint8_t* out = static_cast<uint8_t*>(g.out);
-            for (int64_t t = t0; t < n * n; t += stride) {
-                const int64_t i = t / n, j = t % n;
-                out[t] = (((P[i * g.ldw + (j >> 6)] >> (j & 63)) & 1ull) || (refl && i == j)) ? 1 : 0;
-            }
-        } else {
-            uint64_t* out = static_cast<uint64_t*>(g.out);
-            for (int64_t t = t0; t < n * wpr; t += stride) {
-                const int64_t i = t / wpr, w = t % wpr;
-                uint64_t bits = P[i * g.ldw + w];
-                if (refl && (i >> 6) == w) bits |= 1ull << (i & 63);
-                out[t] = bits;
+                if (w < wpr) out[w] = bits;
             }
         }
     }
@@ -518,7 +574,8 @@ struct BatchCache {
     std::vector<int> order;          // device slot -> caller index
     GroupProblem* d_probs = nullptr;
     GroupState* d_st = nullptr;
-    int* d_ints = nullptr;           // parity | active | iters | changed | notconv | tc_offs | pk_offs | totals
+    int* d_ints = nullptr;           // ones (u64) | top | parity | active | iters | changed | notconv | tc_offs |
+                                      // pk_offs | totals | phase | ppar
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     size_t ws_bytes = 0;
@@ -641,7 +698,7 @@ bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count,
         return o;
     };
     std::vector<size_t> offM0(np), offM1(np), offT0(np), offT1(np), offX(np), offR1T(np), offP0(np), offP1(np);
-    std::vector<size_t> offPT(np), offPtr[2], offIdx[2], offVal[2];
+    std::vector<size_t> offPT(np), offPR1(np), offPtr[2], offIdx[2], offVal[2];
     for (int m = 0; m < 2; ++m) {
         offPtr[m].resize(np);
         offIdx[m].resize(np);
@@ -675,11 +732,13 @@ bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count,
                 offX[s] = take(mat);
                 offR1T[s] = take(mat);
             }
-        } else {
-            g.ldw = round_up((p.n + 63) / 64, 2);
-            const size_t bytes = static_cast<size_t>(p.n * g.ldw * 8);
-            offP0[s] = take(bytes);
-            offP1[s] = take(bytes);
+        }
+        g.ldw = round_up((p.n + 63) / 64, 2);
+        const size_t bytes = static_cast<size_t>(p.n * g.ldw * 8);
+        offP0[s] = take(bytes);
+        offP1[s] = take(bytes);
+        if (p.kind == BMLP_PROBLEM_COMPOSE) offPR1[s] = take(bytes);
+        {
             if (g.engine == 2) {  // R^T and the word indexes of R and R^T (entries sized for the dense worst case)
                 offPT[s] = take(bytes);
                 for (int m = 0; m < 2; ++m) {
@@ -711,10 +770,10 @@ bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count,
                 g.R1T = b8 + offR1T[s];
                 BST(make_tmap(ctx, &g.mapBF, g.R1T, g.ld, g.ld, g.ld, TC_BN));
             }
-        } else {
-            g.P[0] = reinterpret_cast<uint64_t*>(b8 + offP0[s]);
-            g.P[1] = reinterpret_cast<uint64_t*>(b8 + offP1[s]);
         }
+        g.P[0] = reinterpret_cast<uint64_t*>(b8 + offP0[s]);
+        g.P[1] = reinterpret_cast<uint64_t*>(b8 + offP1[s]);
+        if (g.kind == 1) g.PR1 = reinterpret_cast<uint64_t*>(b8 + offPR1[s]);
     }
     // frontier jobs (engine 2): every row of the closure as one query, all jobs in one launch
     std::vector<FrontierJob> jobs;
@@ -744,11 +803,13 @@ bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count,
     // device copies
     BCK(cudaMalloc(&c->d_probs, sizeof(GroupProblem) * (np > 0 ? np : 1)), "cudaMalloc(batch problems)");
     BCK(cudaMemcpy(c->d_probs, hp.data(), sizeof(GroupProblem) * np, cudaMemcpyHostToDevice), "copy batch problems");
-    const size_t nints = static_cast<size_t>(5 * np + 2 * (np + 1) + 2);
+    const size_t nints = static_cast<size_t>(10 * np + 2 * (np + 1) + 2);
     BCK(cudaMalloc(&c->d_ints, sizeof(int) * nints), "cudaMalloc(batch state)");
     BCK(cudaMemset(c->d_ints, 0, sizeof(int) * nints), "clear batch state");
     GroupState hs;
-    int* q = c->d_ints;
+    hs.ones = reinterpret_cast<unsigned long long*>(c->d_ints);  // the counts that a launch starts from: cleared by it
+    hs.top = c->d_ints + 2 * np;
+    int* q = c->d_ints + 3 * np;
     hs.parity = q; q += np;
     hs.active = q; q += np;
     hs.iters = q; q += np;
@@ -758,6 +819,8 @@ bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count,
     hs.pk_offs = q; q += np + 1;
     hs.tc_total = q; q += 1;
     hs.pk_total = q; q += 1;
+    hs.phase = q; q += np;
+    hs.ppar = q; q += np;
     BCK(cudaMalloc(&c->d_st, sizeof(GroupState)), "cudaMalloc(batch state)");
     BCK(cudaMemcpy(c->d_st, &hs, sizeof(GroupState), cudaMemcpyHostToDevice), "copy batch state");
     if (!jobs.empty()) {
@@ -781,71 +844,79 @@ bmlp_status build_batch(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t count,
         *out = c;
         return BMLP_OK;
     }
-    cudaGraphConditionalHandle h;
-    BCK(cudaGraphConditionalHandleCreate(&h, c->graph, 1, cudaGraphCondAssignDefault), "conditional handle");
+    cudaGraphConditionalHandle hA, hB;  // the bit-row loop and the tensor-core loop
+    BCK(cudaGraphConditionalHandleCreate(&hA, c->graph, 0, cudaGraphCondAssignDefault), "conditional handle");
+    BCK(cudaGraphConditionalHandleCreate(&hB, c->graph, 0, cudaGraphCondAssignDefault), "conditional handle");
     GroupProblem* dp = c->d_probs;
     GroupState* ds = c->d_st;
     int nprob = np;
     int* err = ctx->d_ctl + CTL_ERROR;
     long long wc = wait_cycles;
-    int mode0 = 0, mode1 = 1, mode2 = 2, phase0 = 0, phase1 = 1, set0 = 0, set1 = 1;
+    int phase0 = 0, phase1 = 1;
     const int sms = ctx->sm_count;
     const unsigned gy = static_cast<unsigned>(np > 0 ? np : 1);
-    cudaGraphNode_t n_enc, n_init, n_while, n_prep, n_plan2, n_final, n_dec;
-    {
-        void* a[] = {&dp};
-        BST(add_kernel(ctx, c->graph, &n_enc, nullptr, 0, reinterpret_cast<void*>(&batch_encode_kernel),
-                       dim3(64, gy), dim3(256), 0, a));
-    }
-    {
-        void* a[] = {&dp, &ds, &nprob, &mode0, &h, &set0};
-        BST(add_kernel(ctx, c->graph, &n_init, &n_enc, 1, reinterpret_cast<void*>(&batch_plan_kernel), dim3(1),
-                       dim3(1024), 0, a));
-    }
+    bool any_compose = false;
+    for (const GroupProblem& g : hp) any_compose |= g.kind == 1 && g.n > 0;
+    // a node with the problem list and state as its arguments, one block row per problem
+    const auto per_problem = [&](cudaGraphNode_t* node, const cudaGraphNode_t* dep, size_t ndep, void* fn, unsigned gx) {
+        void* a[] = {&dp, &ds};
+        return add_kernel(ctx, c->graph, node, dep, ndep, fn, dim3(gx, gy), dim3(256), 0, a);
+    };
+    const auto plan = [&](cudaGraph_t g, cudaGraphNode_t* node, const cudaGraphNode_t* dep, size_t ndep, int mode,
+                          cudaGraphConditionalHandle h, int set_cond) {
+        void* a[] = {&dp, &ds, &nprob, &mode, &h, &set_cond};
+        return add_kernel(ctx, g, node, dep, ndep, reinterpret_cast<void*>(&batch_plan_kernel), dim3(1), dim3(1024), 0, a);
+    };
+    const auto loop = [&](cudaGraphNode_t* node, const cudaGraphNode_t* dep, size_t ndep, cudaGraphConditionalHandle h,
+                          cudaGraph_t* body) {
+        cudaGraphNodeParams cp = {};
+        cp.type = cudaGraphNodeTypeConditional;
+        cp.conditional.handle = h;
+        cp.conditional.type = cudaGraphCondTypeWhile;
+        cp.conditional.size = 1;
+        BCK(cudaGraphAddNode(node, c->graph, dep, nullptr, ndep, &cp), "while node");
+        *body = cp.conditional.phGraph_out[0];
+        return BMLP_OK;
+    };
+    cudaGraphNode_t n_enc, n_init, n_rows, n_hand, n_ops, n_tc, n_last;
+    cudaGraph_t body_rows = nullptr, body_tc = nullptr;
+    BST(per_problem(&n_enc, nullptr, 0, reinterpret_cast<void*>(&batch_encode_kernel), 32));
+    BST(plan(c->graph, &n_init, &n_enc, 1, 0, hA, 1));
     // the closures by frontier expansion: one chain of grouped launches after the planner's start
     std::vector<cudaGraphNode_t> before_while{n_init};
     if (!jobs.empty()) BST(add_frontier_chain(ctx, c, static_cast<int>(jobs.size()), fr_max_n, fr_max_ldw, fr_total,
                                               n_init, &before_while));
-    cudaGraphNodeParams cp = {};
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = h;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    BCK(cudaGraphAddNode(&n_while, c->graph, before_while.data(), nullptr, before_while.size(), &cp), "while node");
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
+    BST(loop(&n_rows, before_while.data(), before_while.size(), hA, &body_rows));
     {
-        // the two engines touch disjoint problems, so their launches may overlap
-        cudaGraphNode_t n_eng[2], n_plan;
-        void* a[] = {&dp, &ds, &nprob, &phase0, &err, &wc};
-        BST(add_kernel(ctx, body, &n_eng[0], nullptr, 0, tc_group_kernel_ptr(), dim3(sms), dim3(TC_THREADS),
-                       tc_smem_bytes(), a));
+        cudaGraphNode_t n_sq, n_plan;
         void* b[] = {&dp, &ds, &nprob};
-        BST(add_kernel(ctx, body, &n_eng[1], nullptr, 0, reinterpret_cast<void*>(&packed_group_kernel<4>),
-                       dim3(sms * 8), dim3(256), 0, b));
-        void* d[] = {&dp, &ds, &nprob, &mode1, &h, &set1};
-        BST(add_kernel(ctx, body, &n_plan, n_eng, 2, reinterpret_cast<void*>(&batch_plan_kernel), dim3(1),
-                       dim3(1024), 0, d));
+        BST(add_kernel(ctx, body_rows, &n_sq, nullptr, 0, reinterpret_cast<void*>(&packed_group_kernel), dim3(sms * 8),
+                       dim3(256), 0, b));
+        BST(plan(body_rows, &n_plan, &n_sq, 1, 1, hA, 1));
     }
+    BST(plan(c->graph, &n_hand, &n_rows, 1, 3, hB, 1));
+    BST(per_problem(&n_ops, &n_hand, 1, reinterpret_cast<void*>(&batch_operands_kernel), 64));
+    BST(loop(&n_tc, &n_ops, 1, hB, &body_tc));
     {
-        void* a[] = {&dp, &ds};
-        BST(add_kernel(ctx, c->graph, &n_prep, &n_while, 1, reinterpret_cast<void*>(&batch_compose_prep_kernel),
-                       dim3(8, gy), dim3(256), 0, a));
+        cudaGraphNode_t n_sq, n_plan;
+        void* a[] = {&dp, &ds, &nprob, &phase0, &err, &wc};
+        BST(add_kernel(ctx, body_tc, &n_sq, nullptr, 0, tc_group_kernel_ptr(), dim3(sms), dim3(TC_THREADS),
+                       tc_smem_bytes(), a));
+        BST(plan(body_tc, &n_plan, &n_sq, 1, 4, hB, 1));
     }
-    {
-        void* a[] = {&dp, &ds, &nprob, &mode2, &h, &set0};
-        BST(add_kernel(ctx, c->graph, &n_plan2, &n_prep, 1, reinterpret_cast<void*>(&batch_plan_kernel), dim3(1),
-                       dim3(1024), 0, a));
-    }
-    {
+    n_last = n_tc;
+    if (any_compose) {
+        cudaGraphNode_t n_prep, n_prod, n_plan2, n_final;
+        BST(per_problem(&n_prep, &n_last, 1, reinterpret_cast<void*>(&batch_compose_prep_kernel), 8));
+        BST(per_problem(&n_prod, &n_prep, 1, reinterpret_cast<void*>(&batch_compose_rows_kernel), 32));
+        BST(plan(c->graph, &n_plan2, &n_prod, 1, 2, hB, 0));
         void* a[] = {&dp, &ds, &nprob, &phase1, &err, &wc};
         BST(add_kernel(ctx, c->graph, &n_final, &n_plan2, 1, tc_group_kernel_ptr(), dim3(sms), dim3(TC_THREADS),
                        tc_smem_bytes(), a));
+        n_last = n_final;
     }
-    {
-        void* a[] = {&dp, &ds};
-        BST(add_kernel(ctx, c->graph, &n_dec, &n_final, 1, reinterpret_cast<void*>(&batch_decode_kernel),
-                       dim3(64, gy), dim3(256), 0, a));
-    }
+    cudaGraphNode_t n_dec;
+    BST(per_problem(&n_dec, &n_last, 1, reinterpret_cast<void*>(&batch_decode_kernel), 32));
     if (!c->solo.empty()) BST(build_solo(ctx, c, probs, wait_cycles));
     BCK(cudaGraphInstantiate(&c->exec, c->graph, 0), "cudaGraphInstantiate");
     *out = c;
@@ -1175,7 +1246,7 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
 // Branches of the batch graph that the large problems are dealt out to, besides the branch of the grouped ones. A
 // pipeline is a chain of small launches (bit-row squarings, decisions) between tensor-core products that fill the GPU, so
 // several chains at once fill each other's gaps (measured on the knowledge-graph batch, 33 closures and 8 compositions
-// with n >= 4,096: LANES_TABLE). More lanes than that add scratch (at most kLaneBytes in all, else fewer lanes).
+// with n >= 4,096: 37.4 ms on one branch, 32.2 on two, 30.4 on four, 30.4 on twelve). More lanes than that add scratch (at most kLaneBytes in all, else fewer lanes).
 constexpr int kLanes = 4;
 constexpr size_t kLaneBytes = size_t(24) << 30;
 
@@ -1256,9 +1327,9 @@ bmlp_status batch_run_impl(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t cou
     ctx->stats.n_pad = static_cast<int64_t>(c->ws_bytes);
     BCK(cudaGraphLaunch(c->exec, s), "cudaGraphLaunch");
     const int np = c->nprob;
-    BCK(cudaMemcpyAsync(c->h_iters.data(), c->d_ints + 2 * np, sizeof(int) * np, cudaMemcpyDeviceToHost, s),
+    BCK(cudaMemcpyAsync(c->h_iters.data(), c->d_ints + 5 * np, sizeof(int) * np, cudaMemcpyDeviceToHost, s),
         "read iterations");
-    BCK(cudaMemcpyAsync(c->h_notconv.data(), c->d_ints + 4 * np, sizeof(int) * np, cudaMemcpyDeviceToHost, s),
+    BCK(cudaMemcpyAsync(c->h_notconv.data(), c->d_ints + 7 * np, sizeof(int) * np, cudaMemcpyDeviceToHost, s),
         "read convergence");
     const int ns = static_cast<int>(c->solo.size());
     if (ns > 0)

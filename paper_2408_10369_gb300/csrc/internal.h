@@ -73,13 +73,14 @@ struct GroupProblem {  // aligned as CUtensorMap (TMA descriptors must be 64-byt
     uint8_t* T[2];         // E4M3 R^T ping-pong
     uint8_t* X;            // composition: final product
     uint8_t* R1T;          // composition: E4M3 R1^T
-    uint64_t* P[2];        // packed ping-pong (packed engine)
+    uint64_t* P[2];        // packed ping-pong (packed engine, and the tensor-core engine's bit-row start)
+    uint64_t* PR1;         // composition: packed R1
     const void* in1;       // caller's R1 (closure input, or composition r1)
     const void* in2;       // caller's R2 (composition r2)
     void* out;             // caller's output
     int64_t n;
     int64_t ld;            // n_pad (tensor-core engine)
-    int64_t ldw;           // words per packed row (packed engine)
+    int64_t ldw;           // words per packed row
     int32_t m_tiles, n_tiles, k_blocks;
     int32_t kind;          // 0 closure, 1 composition
     int32_t engine;        // 0 tensor cores, 1 packed
@@ -90,6 +91,10 @@ struct GroupProblem {  // aligned as CUtensorMap (TMA descriptors must be 64-byt
 
 // Per-problem loop state of a grouped batch (device memory).
 struct GroupState {
+    unsigned long long* ones;  // ones of the current R while on bit rows
+    int* top;        // and the most of one row
+    int* phase;      // 0: on bit rows, 1: handed over to the tensor cores
+    int* ppar;       // packed buffer that held R when the bit-row squarings ended
     int* parity;     // buffer holding the current R
     int* active;     // still iterating
     int* iters;      // products issued
