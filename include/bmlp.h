@@ -145,19 +145,18 @@ typedef struct bmlp_stats {
     int32_t sliced_closures;   /* BMLP_SMP_PACKED closures, and query batches
                                   of >= 64 rows (n >= 4096), whose relation
                                   widens the rows fast (R + R R has > 2.8 x
-                                  the words of R): expanded 64 rows at a time
-                                  (bit-sliced frontiers, one thread-block
-                                  cluster per 64 rows for n <= 65,536)          */
+                                  the words of R): expanded 16 to 64 rows at a
+                                  time with bit-sliced frontiers (for
+                                  n <= 65,536 in one SM's shared memory)        */
     double sparse_ms;          /* their summed device time (options.profile)    */
     double sparse_words;       /* the word ORs they issued                      */
     int32_t host_syncs;        /* times the host waited for the device during
                                   the call to read back a flag, a decision or
                                   the results (1 for a batch that ran as one
                                   device-driven graph: the final read)          */
-    int32_t cluster_frontiers; /* of sliced_closures, those run one thread-block
-                                  cluster per 64 rows with the frontier in
-                                  the cluster's shared memory (query batches,
-                                  and closures whose columns are skewed)        */
+    int32_t cluster_frontiers; /* of sliced_closures with n <= 65,536, the query
+                                  batches and the closures whose columns are
+                                  skewed (largest in-degree > 6.5 x the mean)   */
     int32_t thin_squarings;    /* BMLP_RMS_TC: squarings computed only on the
                                   rows and columns that still held zeros (few,
                                   and holding few ones: R close to its closure,
@@ -205,7 +204,7 @@ bmlp_status bmlp_get_stats(const bmlp_ctx* ctx, bmlp_stats* out);
  * Variants: BMLP_RMS_TC (n >= 4096: bit-row squarings while R is sparse,
  * see options.tc_only; then tensor cores), BMLP_RMS_PACKED, BMLP_SMP_PACKED
  * (all n rows as frontiers: path-like R is squared first and expanded one
- * row per warp, R whose rows widen fast is expanded 64 rows per CTA), BMLP_SMP_TC,
+ * row per warp, R whose rows widen fast is expanded up to 64 rows per CTA), BMLP_SMP_TC,
  * BMLP_AUTO (the learned dispatcher once trained or loaded, else BMLP_RMS_TC).
  */
 bmlp_status bmlp_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt, void* out,
@@ -239,8 +238,9 @@ bmlp_status bmlp_rms_alg1(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt, 
  * layout. A source is in its own output row only if it lies on a cycle.
  * R is n x n in format fmt. *iters_out receives the deepest frontier level.
  * Variants: BMLP_SMP_PACKED, BMLP_SMP_TC, BMLP_AUTO. BMLP_SMP_PACKED expands
- * one query row per warp, or, for batches of >= 64 rows over a relation whose
- * rows widen fast (n >= 4096), 64 rows at a time with bit-sliced frontiers.
+ * up to 63 rows one per thread-block cluster straight from R; larger batches
+ * one row per warp, or, over a relation whose rows widen fast (n >= 4096), 16
+ * to 64 rows at a time with bit-sliced frontiers.
  */
 bmlp_status bmlp_smp(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt,
                      const uint64_t* src_rows, int64_t nq, uint64_t* out_rows,

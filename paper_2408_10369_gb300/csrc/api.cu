@@ -121,12 +121,9 @@ constexpr double kSlicedMinGrowth = 2.8;
 // ... and no column of R has more than this many times the mean nonzero words of a column (a pull rescans a hub's
 // in-list at every level until every active source reaches it).
 constexpr double kSlicedMaxSkew = 16.0;
-// Closures whose largest column holds more than this many times the mean nonzero words of a column run on the
-// cluster kernel, whose warps walk many constants' in-lists together (measured on the corpus at n = 22,535-32,629:
-// power-law targets, column skew 7.8-15.6, 0.71-0.93 of the global-memory kernel's time; ER and SBM, skew 2.9-5.3,
-// 0.99-1.33 of it).
-constexpr double kClusterClosureSkew = 6.5;
-// Query batches of at least this many rows take the same test (a batch of 64 rows is one cluster's work).
+// Largest in-degree over the mean above which a sliced closure's columns count as skewed (bmlp_stats).
+constexpr double kSkewedColumns = 6.5;
+// Query batches of at least this many rows take the same test.
 constexpr int64_t kSlicedMinQueries = 64;
 // Fraction of nonzero 128 x 128 blocks of R below which a squaring skips empty K blocks.
 constexpr double kSkipMaxDensity = 0.5;
@@ -1156,10 +1153,21 @@ void reset_stats(bmlp_ctx* ctx, int variant, int64_t n_pad) {
 // Without a trained dispatcher the fixed choice is squaring on the tensor cores.
 int pick_variant_rms(int64_t) { return BMLP_RMS_TC; }
 
+// The identity as n packed rows of ldw words.
+bmlp_status identity_rows(bmlp_ctx* ctx, int64_t n, int64_t ldw, cudaStream_t s, const uint64_t** rows) {
+    void* p = nullptr;
+    ST(ws_get(ctx, WS_SRC, static_cast<size_t>(n * ldw * 8), &p));
+    launch_identity_packed(static_cast<uint64_t*>(p), ldw, n, s);
+    CK(cudaGetLastError(), "identity launch");
+    ctx->stats.launches++;
+    *rows = static_cast<const uint64_t*>(p);
+    return BMLP_OK;
+}
+
 // Frontier expansion (Algorithm 2) on packed rows for the sources `src`
 // (device, q x ldw_src words). out: device, q x ldw_out words. square_first:
-// a full closure (src = the identity, q = n), which may square R first
-// (path-like R) or expand 64 sources at a time (rows that widen fast).
+// a full closure (src null: the identity's rows, q = n), which may square R
+// first (path-like R) or expand many sources at a time (rows that widen fast).
 bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t n, const uint64_t* src,
                            int64_t ldw_src, int64_t q, uint64_t* out, int64_t ldw_out, const bmlp_options& o,
                            cudaStream_t s, int* levels, bool square_first = false) {
@@ -1264,6 +1272,36 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         ST(growth(&W, &W2));
         dense_reach = W > 0 && static_cast<double>(W2) > kSlicedMinGrowth * static_cast<double>(W);
     }
+    const int width = dense_reach && smp_sliced_enabled() && ones >= 0 ? smp_tile_width(n, q, ctx->sm_count) : 0;
+    if (width > 0) {
+        // batches of rows with their frontier in one SM's shared memory: query rows, or the closure's identity rows
+        void* scratch = nullptr;
+        ST(ws_get(ctx, WS_V, smp_tile_bytes(n, ones, width, ctx->sm_count), &scratch));
+        CK(cudaMemsetAsync(ctx->d_ctl + CTL_LEVELS, 0, 3 * sizeof(int), s), "reset level and query counters");
+        ProductTimer tm{ctx, o.profile != 0, s};
+        ST(tm.begin());
+        CK(launch_smp_tiles(x, n, ones, square_first ? nullptr : src, ldw_src, q, out, ldw_out,
+                            square_first ? 0 : o.reflexive, width, scratch,
+                            reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_QCOUNT), ctx->d_ctl + CTL_LEVELS,
+                            static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), ctx->sm_count, s, deadline_of(ctx)),
+           "tile frontier kernel launch");
+        ST(tm.end());
+        ctx->stats.product_launches++;
+        ctx->stats.launches += 7;
+        ctx->stats.sliced_closures++;
+        CK(cudaMemcpyAsync(ctx->h_ctl + CTL_HOST_I64, smp_tile_top_degree(scratch, n), sizeof(int), cudaMemcpyDeviceToHost, s),
+           "read largest in-degree");
+        ST(read_ctl(ctx, s, nullptr));
+        ST(tm.collect());
+        const double skew = static_cast<double>(ctx->h_ctl[CTL_HOST_I64]) * static_cast<double>(n) /
+                            static_cast<double>(ones > 0 ? ones : 1);
+        if (!square_first || skew > kSkewedColumns) ctx->stats.cluster_frontiers++;
+        *levels = ctx->h_ctl[CTL_LEVELS];
+        const int cap = o.max_iters > 0 ? o.max_iters : static_cast<int>(n + 1);
+        if (*levels > cap) return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "frontier did not empty within %d levels", cap);
+        return BMLP_OK;
+    }
+    if (!square_first) dense_reach = false;  // larger relations: query rows one per warp
     // transposed word index for the pull direction (levels whose frontier is large)
     void* PT = nullptr;
     WordIndex xT;
@@ -1280,7 +1318,6 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
     ctx->stats.launches += 2;
     CK(cudaMemsetAsync(ctx->d_ctl + CTL_LEVELS, 0, 3 * sizeof(int), s), "reset level and query counters");
     ProductTimer tm{ctx, o.profile != 0, s};
-    double skew = 0.0;  // largest column's nonzero words over the mean
     if (dense_reach && smp_sliced_enabled()) {
         // no hubs among the columns: a pull scans a hub's whole in-list at every level until all active sources
         // reach it (power-law targets), which the one-query-per-warp kernel avoids
@@ -1288,29 +1325,8 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         CK(cudaMemcpyAsync(wt, xT.ptr + 2 * n, sizeof(wt), cudaMemcpyDeviceToHost, s),
            "read column word counts");
         CK(host_sync(ctx, s), "read column word counts");
-        skew = static_cast<double>(wt[1]) * static_cast<double>(n) / static_cast<double>(wt[0] > 0 ? wt[0] : 1);
+        const double skew = static_cast<double>(wt[1]) * static_cast<double>(n) / static_cast<double>(wt[0] > 0 ? wt[0] : 1);
         dense_reach = skew <= kSlicedMaxSkew;
-    }
-    if (dense_reach && smp_sliced_enabled() && (!square_first || skew > kClusterClosureSkew) &&
-        smp_cluster_fits(n, q, ctx->sm_count)) {
-        // 64 rows per thread-block cluster with the frontier in the cluster's shared memory: query rows, or the
-        // closure's identity rows
-        ST(tm.begin());
-        CK(launch_smp_cluster(xT, n, src, ldw_src, q, out, ldw_out, square_first ? 0 : o.reflexive, ctx->d_ctl + CTL_LEVELS,
-                              static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), ctx->sm_count, s,
-                              deadline_of(ctx)),
-           "cluster frontier kernel launch");
-        ST(tm.end());
-        ctx->stats.product_launches++;
-        ctx->stats.launches++;
-        ctx->stats.sliced_closures++;
-        ctx->stats.cluster_frontiers++;
-        ST(read_ctl(ctx, s, nullptr));
-        ST(tm.collect());
-        *levels = ctx->h_ctl[CTL_LEVELS];
-        const int cap = o.max_iters > 0 ? o.max_iters : static_cast<int>(n + 1);
-        if (*levels > cap) return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "frontier did not empty within %d levels", cap);
-        return BMLP_OK;
     }
     if (dense_reach && smp_sliced_enabled() && square_first) {
         // every row of the closure (src = the identity), 64 sources per CTA over the word index of R^T
@@ -1331,6 +1347,7 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         *levels = ctx->h_ctl[CTL_LEVELS];
         return BMLP_OK;
     }
+    if (src == nullptr) ST(identity_rows(ctx, n, ldw_src, s, &src));
     ST(tm.begin());
     CK(launch_smp_packed(x, xT, n, ldw, src, ldw_src, q, out, ldw_out, ctx->d_ctl + CTL_LEVELS, ctx->d_ctl + CTL_QCOUNT,
                          o.reflexive, ctx->sm_count, s, deadline_of(ctx)),
@@ -1627,10 +1644,7 @@ static bmlp_status core_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt
     } else if (variant == BMLP_SMP_PACKED || variant == BMLP_SMP_TC) {
         // the full closure as n selective queries, one per constant
         const int64_t ldw_src = words_of(n);
-        void *src = nullptr, *dst = nullptr;
-        ST(ws_get(ctx, WS_SRC, static_cast<size_t>(n * ldw_src * 8), &src));
-        launch_identity_packed(static_cast<uint64_t*>(src), ldw_src, n, s);
-        ctx->stats.launches++;
+        void* dst = nullptr;
         uint64_t* outp = nullptr;
         if (fmt == BMLP_FMT_PACKED64) {
             outp = static_cast<uint64_t*>(ov.dev);
@@ -1641,11 +1655,13 @@ static bmlp_status core_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt
         bmlp_options o2 = o;
         o2.reflexive = 0;
         o2.max_iters = 0;
-        if (variant == BMLP_SMP_PACKED)
-            st = smp_packed_run(ctx, in, fmt, n, static_cast<uint64_t*>(src), ldw_src, n, outp, ldw_src, o2, s, &iters,
-                                true);
-        else
-            st = smp_tc_run(ctx, in, fmt, n, static_cast<uint64_t*>(src), ldw_src, n, outp, ldw_src, o2, s, &iters);
+        if (variant == BMLP_SMP_PACKED) {
+            st = smp_packed_run(ctx, in, fmt, n, nullptr, ldw_src, n, outp, ldw_src, o2, s, &iters, true);
+        } else {
+            const uint64_t* src = nullptr;
+            ST(identity_rows(ctx, n, ldw_src, s, &src));
+            st = smp_tc_run(ctx, in, fmt, n, src, ldw_src, n, outp, ldw_src, o2, s, &iters);
+        }
         if (st == BMLP_OK) {
             if (fmt == BMLP_FMT_U8)
                 launch_packed_to_u8(outp, ldw_src, n, static_cast<uint8_t*>(ov.dev), o.reflexive, s);

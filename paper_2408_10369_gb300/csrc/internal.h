@@ -338,18 +338,20 @@ cudaError_t launch_indexed_rows(const WordIndex& A, const WordIndex& B, const ui
 int64_t smp_sliced_grid(int64_t n, int sms);
 cudaError_t launch_smp_sliced(const WordIndex& T, int64_t n, uint64_t* scratch, uint64_t* out, int64_t ldw_out, unsigned long long* bcounter,
                               int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl);
-// The same expansion for query rows, with the frontier of each 64-row batch in the distributed shared memory of a
-// thread-block cluster (one cluster per batch, n <= 65,536): rows 0 .. rows - 1 of out (ldw_out words each) are
-// v_q R+ for the query rows in src (ldw_src words each), OR-ed with v_q when reflexive. *levels = 0 beforehand
-// receives the largest level count. smp_cluster_fits: the shape exists for n and the device can hold one such
-// cluster.
-bool smp_cluster_shape(int64_t n, int64_t batches, int sms, int* ctas, int* log2_chunk);
-bool smp_cluster_fits(int64_t n, int64_t rows, int sms);
-cudaError_t launch_smp_cluster(const WordIndex& T, int64_t n, const uint64_t* src, int64_t ldw_src, int64_t rows, uint64_t* out, int64_t ldw_out,
-                               int reflexive, int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl);
+// The same expansion with the whole frontier of a batch in one SM's shared memory (frontier.cu; n <= 65,536): the rows
+// of src (ld_src words each), or of the identity when src is null, into out (ld_out words each), OR-ed with the source row
+// when reflexive. x: the word index of R, ones: its ones. smp_tile_width: rows per batch (0: n is too large);
+// smp_tile_bytes: scratch. *counter = 0 and *levels = 0 beforehand; *levels receives the largest level count, and
+// *smp_tile_top_degree the largest in-degree.
+int smp_tile_width(int64_t n, int64_t rows, int sms);
+size_t smp_tile_bytes(int64_t n, int64_t ones, int width, int sms);
+const int* smp_tile_top_degree(void* scratch, int64_t n);
+cudaError_t launch_smp_tiles(const WordIndex& x, int64_t n, int64_t ones, const uint64_t* src, int64_t ld_src, int64_t rows,
+                             uint64_t* out, int64_t ld_out, int reflexive, int width, void* scratch,
+                             unsigned long long* counter, int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl);
 // The expansion of a few query rows straight from R's packed rows (ld_r words, bits at columns >= n ignored), one cluster
 // of smp_rows_ctas() CTAs per row: 16, 8, 4 or 2, or 0 when q rows do not fit the GPU at once (or are more than
-// kRowsMaxQueries) or n is too large. Results and levels as launch_smp_cluster.
+// kRowsMaxQueries) or n is too large. Results and levels as launch_smp_tiles.
 constexpr int64_t kRowsMaxQueries = 63;
 int smp_rows_ctas(int64_t n, int64_t q);
 cudaError_t launch_smp_rows(const uint64_t* R, int64_t ld_r, int64_t n, const uint64_t* src, int64_t ld_src, int64_t q,
