@@ -60,15 +60,18 @@ Lists lists_of(void* scratch, int64_t n) {
     return l;
 }
 
-// fn(i, j) for every one (i, j) of the indexed relation: a warp per row, a lane per nonzero word (eight lanes per row took
-// twice as long on power-law rows).
+// fn(i, j) for every one (i, j) of the indexed relation: a warp per row, a lane per nonzero word; rows of more than kLong
+// words by the whole block afterwards (a power-law row of a thousand facts kept its warp busy for the whole pass: the list
+// fill of one took 46 us at n = 20,011 and 58 at 65,536, and takes 14 and 21).
+constexpr int kLong = 64, kLongQueue = 64;
 template <class Fn>
 __device__ __forceinline__ void for_ones(const WordIndex& x, int64_t n, Fn&& fn) {
+    __shared__ int s_queue[kLongQueue];
+    __shared__ int s_queued;
     const int lane = threadIdx.x & 31;
     const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-        const longlong2 r = *reinterpret_cast<const longlong2*>(x.ptr + 2 * i);
-        for (int64_t e = r.x + lane; e < r.y; e += 32) {
+    const auto row = [&](int64_t i, const longlong2& r, int64_t first, int64_t step) {
+        for (int64_t e = r.x + first; e < r.y; e += step) {
             uint64_t d = x.val[e];
             const int base = x.idx[e] << 6;
             while (d) {
@@ -76,7 +79,27 @@ __device__ __forceinline__ void for_ones(const WordIndex& x, int64_t n, Fn&& fn)
                 d &= d - 1ull;
             }
         }
+    };
+    if (threadIdx.x == 0) s_queued = 0;
+    __syncthreads();
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
+        const longlong2 r = *reinterpret_cast<const longlong2*>(x.ptr + 2 * i);
+        if (r.y - r.x > kLong) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&s_queued, 1);
+            at = __shfl_sync(FULL, at, 0);
+            if (at < kLongQueue) {
+                if (lane == 0) s_queue[at] = static_cast<int>(i);
+                continue;
+            }
+        }
+        row(i, r, lane, 32);
     }
+    __syncthreads();
+    const int queued = min(s_queued, kLongQueue);
+    for (int k = 0; k < queued; ++k)
+        row(s_queue[k], *reinterpret_cast<const longlong2*>(x.ptr + 2 * static_cast<int64_t>(s_queue[k])), threadIdx.x,
+            blockDim.x);
 }
 
 __global__ void __launch_bounds__(kPrepThreads) lists_degree_kernel(const WordIndex x, int64_t n, Lists l) {

@@ -471,75 +471,81 @@ __host__ __device__ __forceinline__ int64_t smp_warp_bytes(int64_t ldw) {
     return (18 * ldw + 64 + 16 + 15) & ~int64_t(15);
 }
 
+// N[x] |= v in shared memory, as its nonzero 32-bit halves: OR without return value is one instruction there at 32 bits
+// and a compare-and-swap loop at 64, and most words of a sparse relation have one bit.
+__device__ __forceinline__ void or_word(uint64_t* N, int64_t x, uint64_t v) {
+    unsigned* at = reinterpret_cast<unsigned*>(N + x);
+    const unsigned lo = static_cast<unsigned>(v), hi = static_cast<unsigned>(v >> 32);
+    if (lo) atomicOr(at, lo);
+    if (hi) atomicOr(at + 1, hi);
+}
+
 // Rows of up to NQ frontier constants per lane (k < 0: none) ORed into N:
 // their nonzero words, by shared-memory atomics without return value. The row
-// ranges and the first four entries of every light row (<= 16 nonzero words)
-// are loaded before the first atomic; heavy rows are walked by the whole warp.
-// tm collects the word groups written (bit x >> gshift for word x).
-template <int NQ>
-__device__ __forceinline__ void push_rows(const int64_t (&k)[NQ], int lane, const int64_t* __restrict__ wptr,
+// ranges and the first four entries of every light row (<= kLightRow nonzero words)
+// are loaded before the first atomic; heavy rows are walked by the whole warp, four entries a lane in flight.
+// tm collects the word groups written (bit x >> gshift for word x) unless the caller has no use for them.
+constexpr int kLightRow = 16;
+template <int NQ, bool kGroups = true>
+__device__ __forceinline__ void push_rows(const int (&k)[NQ], int lane, const int64_t* __restrict__ wptr,
                                           const int32_t* __restrict__ widx, const uint64_t* __restrict__ wval,
                                           uint64_t* N, int gshift, uint64_t& tm) {
-    int64_t e0[NQ], e1[NQ];
+    int64_t e0[NQ];
+    int len[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         const longlong2 r = wcsr_row(wptr, k[q] >= 0 ? k[q] : 0);  // an in-range index even where the value is dropped
-        e0[q] = k[q] >= 0 ? r.x : 0;
-        e1[q] = k[q] >= 0 ? r.y : 0;
+        e0[q] = r.x;
+        len[q] = k[q] >= 0 ? static_cast<int>(r.y - r.x) : 0;
     }
-    bool light[NQ];
+    // entries e, e + step, ... (four; those at or beyond `left` are not the row's)
+    const auto four = [&](int64_t e, int step, int left) {
+        int y[4];
+        uint64_t yv[4];
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) light[q] = k[q] >= 0 && (e1[q] - e0[q]) <= 16;
+        for (int j = 0; j < 4; ++j) {
+            const bool in = step * j < left;
+            y[j] = in ? widx[e + step * j] : -1;
+            yv[j] = in ? wval[e + step * j] : 0ull;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (y[j] >= 0) {
+                or_word(N, y[j], yv[j]);
+                if (kGroups) tm |= 1ull << (y[j] >> gshift);
+            }
+    };
     int x[NQ][4];
     uint64_t val[NQ][4];
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const bool in = light[q] && e0[q] + j < e1[q];
-            const int64_t ee = in ? e0[q] + j : 0;
-            x[q][j] = in ? widx[ee] : -1;
-            val[q][j] = in ? wval[ee] : 0ull;
+            const bool in = len[q] <= kLightRow && j < len[q];
+            x[q][j] = in ? widx[e0[q] + j] : -1;
+            val[q][j] = in ? wval[e0[q] + j] : 0ull;
         }
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             if (x[q][j] >= 0) {
-                atomicOr(reinterpret_cast<unsigned long long*>(&N[x[q][j]]), static_cast<unsigned long long>(val[q][j]));
-                tm |= 1ull << (x[q][j] >> gshift);
+                or_word(N, x[q][j], val[q][j]);
+                if (kGroups) tm |= 1ull << (x[q][j] >> gshift);
             }
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
-        if (light[q])
-            for (int64_t e = e0[q] + 4; e < e1[q]; e += 4) {
-                int y[4];
-                uint64_t yv[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int64_t ee = e + j < e1[q] ? e + j : 0;
-                    y[j] = e + j < e1[q] ? widx[ee] : -1;
-                    yv[j] = e + j < e1[q] ? wval[ee] : 0ull;
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (y[j] >= 0) {
-                        atomicOr(reinterpret_cast<unsigned long long*>(&N[y[j]]), static_cast<unsigned long long>(yv[j]));
-                        tm |= 1ull << (y[j] >> gshift);
-                    }
-            }
+        if (len[q] <= kLightRow)
+            for (int f = 4; f < len[q]; f += 4) four(e0[q] + f, 1, len[q] - f);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        unsigned hm = __ballot_sync(FULL, k[q] >= 0 && !light[q]);
+        unsigned hm = __ballot_sync(FULL, len[q] > kLightRow);
         while (hm) {
             const int sl = __ffs(hm) - 1;
             hm &= hm - 1;
-            const int64_t h0 = __shfl_sync(FULL, e0[q], sl), h1 = __shfl_sync(FULL, e1[q], sl);
-            for (int64_t e = h0 + lane; e < h1; e += 32) {
-                const int xx = widx[e];
-                atomicOr(reinterpret_cast<unsigned long long*>(&N[xx]), static_cast<unsigned long long>(wval[e]));
-                tm |= 1ull << (xx >> gshift);
-            }
+            const int64_t h0 = __shfl_sync(FULL, e0[q], sl);
+            const int hl = __shfl_sync(FULL, len[q], sl);
+            for (int f = lane; f < hl; f += 128) four(h0 + f, 32, hl - f);
         }
     }
 }
@@ -549,14 +555,14 @@ template <int NQ>
 __device__ __forceinline__ void push_step(uint64_t& d, int64_t w, int lane, const int64_t* __restrict__ wptr,
                                           const int32_t* __restrict__ widx, const uint64_t* __restrict__ wval,
                                           uint64_t* N, int gshift, uint64_t& tm) {
-    int64_t k[NQ];
+    int k[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         k[q] = -1;
         if (d) {
             const int b = __ffsll(static_cast<long long>(d)) - 1;
             d &= d - 1;
-            k[q] = w * 64 + b;
+            k[q] = static_cast<int>(w) * 64 + b;
         }
     }
     push_rows<NQ>(k, lane, wptr, widx, wval, N, gshift, tm);
@@ -587,7 +593,8 @@ __device__ __forceinline__ int select_bit(uint64_t x, int r) {
 // Push of a chunk of frontier words (lane l holds word d of index w) with the set bits dealt out to the
 // lanes in rank order, two per lane per step: a word with many bits (a band of a squared path, a dense
 // frontier) is shared by the whole warp instead of being walked by one lane.
-__device__ __forceinline__ void push_balanced(uint64_t d, int64_t w, int lane, const int64_t* __restrict__ wptr,
+template <int NQ, bool kGroups = true>
+__device__ __forceinline__ void push_balanced(uint64_t d, int w, int lane, const int64_t* __restrict__ wptr,
                                               const int32_t* __restrict__ widx, const uint64_t* __restrict__ wval,
                                               uint64_t* N, int gshift, uint64_t& tm) {
     const int c = __popcll(d);
@@ -599,10 +606,10 @@ __device__ __forceinline__ void push_balanced(uint64_t d, int64_t w, int lane, c
     }
     const int total = __shfl_sync(FULL, incl, 31);
     const int excl = incl - c;
-    for (int base = 0; base < total; base += 64) {
-        int64_t k[2];
+    for (int base = 0; base < total; base += 32 * NQ) {
+        int k[NQ];
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < NQ; ++q) {
             const int r = base + q * 32 + lane;
             int owner = 0;  // the lane whose bits hold rank r: the first with inclusive count > r
 #pragma unroll
@@ -611,11 +618,11 @@ __device__ __forceinline__ void push_balanced(uint64_t d, int64_t w, int lane, c
                 if (v <= r) owner += st;
             }
             const uint64_t od = __shfl_sync(FULL, d, owner);
-            const int64_t ow = __shfl_sync(FULL, w, owner);
+            const int ow = __shfl_sync(FULL, w, owner);
             const int oex = __shfl_sync(FULL, excl, owner);
             k[q] = r < total ? ow * 64 + select_bit(od, r - oex) : -1;
         }
-        push_rows<2>(k, lane, wptr, widx, wval, N, gshift, tm);
+        push_rows<NQ, kGroups>(k, lane, wptr, widx, wval, N, gshift, tm);
     }
 }
 
@@ -726,7 +733,7 @@ __device__ __forceinline__ int smp_expand_row(SrcWord srcw, uint64_t* __restrict
                 if (__reduce_max_sync(FULL, static_cast<unsigned>(__popcll(d))) <= 2u)
                     push_step<2>(d, w, lane, wptr, widx, wval, N, gshift, tm);
                 else
-                    push_balanced(d, w, lane, wptr, widx, wval, N, gshift, tm);
+                    push_balanced<2>(d, w, lane, wptr, widx, wval, N, gshift, tm);
             }
             gm = static_cast<uint64_t>(__reduce_or_sync(FULL, static_cast<unsigned>(tm))) |
                  (static_cast<uint64_t>(__reduce_or_sync(FULL, static_cast<unsigned>(tm >> 32))) << 32);
@@ -996,122 +1003,218 @@ __global__ void __launch_bounds__(kInsertWarps * 32) insert_rows_kernel(uint64_t
     }
 }
 
+// ---- passes over a word index with a warp per row
+// Rows are dealt to the warps of all blocks; a row with many times the mean of entries (a power-law relation's, a thousand
+// against three) would keep one warp busy long after the others are done, so a block puts such rows into a queue and walks
+// them with all of its warps at the end (a full queue: the warp walks the row after all). Measured on power-law relations,
+// with a warp for every row and with the queue (one pass):
+//                                  n = 14,000        20,011          65,536
+//     square_growth_kernel                 -       98 -> 46 us    131 -> 80 us
+//     indexed_rows_kernel       364 -> 69 us            (two products of a closure; 8 x and 64 against 16 x and 192:
+//     indexed_cost_kernel        54 -> 26 us             2,317 against 2,376 us for that closure)
+constexpr int kRowQueue = 64;
+
+// Entries of a row from which it is queued: eight times the mean, at least 64.
+__device__ __forceinline__ int64_t long_row(const WordIndex& A, int64_t n) {
+    const int64_t mean8 = 8 * A.ptr[2 * n] / n;
+    return mean8 > 64 ? mean8 : 64;
+}
+
+// Calls row(i, range, false) for this warp's rows that are not queued, then row(i, range, true) with all warps of the block
+// in step for the queued ones. One call site: the body is large, and two copies of it took more registers than fit.
+template <class Row>
+__device__ __forceinline__ void rows_of_index(const WordIndex& A, int64_t n, Row&& row) {
+    __shared__ int s_queue[kRowQueue];
+    __shared__ int s_queued;
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = blockDim.x >> 5, warps = static_cast<int64_t>(gridDim.x) * nw;
+    if (threadIdx.x == 0) s_queued = 0;
+    __syncthreads();
+    const int64_t limit = long_row(A, n);
+    int64_t next = static_cast<int64_t>(blockIdx.x) * nw + (threadIdx.x >> 5);
+    bool together = false;
+    for (int queued = 0, k = 0;;) {
+        int64_t i;
+        longlong2 range;
+        if (!together) {
+            if (next >= n) {
+                __syncthreads();
+                together = true;
+                queued = s_queued < kRowQueue ? s_queued : kRowQueue;
+                continue;
+            }
+            i = next;
+            next += warps;
+            range = wcsr_row(A.ptr, i);
+            if (range.y - range.x > limit) {
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&s_queued, 1);
+                at = __shfl_sync(FULL, at, 0);
+                if (at < kRowQueue) {
+                    if (lane == 0) s_queue[at] = static_cast<int>(i);
+                    continue;
+                }
+            }
+        } else {
+            if (k >= queued) break;
+            i = s_queue[k++];
+            range = wcsr_row(A.ptr, i);
+        }
+        row(i, range, together);
+    }
+}
+
+__device__ __forceinline__ void sync_row(bool together) {
+    if (together) __syncthreads();
+    else __syncwarp();
+}
+
 // ---- one product on packed rows through word indexes: C_i = P_i | OR_{k in A_i} B_k, where row k contributes only its
 // nonzero words (push_balanced), so the cost follows the indexes, not n / 64 words per k. With A = B = P = R that is one
-// squaring step. Warp per row; the row is assembled in shared memory (ldw words per warp). *changed (or null) is raised
-// when C_i != P_i.
-__global__ void __launch_bounds__(256) indexed_rows_kernel(const WordIndex A, const WordIndex B,
+// squaring step. The row is assembled in shared memory (ldw words per warp). The kernel waits for L2 (a range, then its
+// words, at random), so it is as fast as it has loads in flight: 32-bit lengths and one named row a lane at a time leave 48
+// registers and five blocks an SM (n = 14,000, 1.5 entries a row, the four products of a closure: 801 us with two rows a
+// lane, 64 registers and 64-bit shared-memory atomics; 602, 563 and 535 us at four, five and six blocks, of which the last
+// spills and loses on power-law relations). *changed (or null) is raised when C_i != P_i.
+__global__ void __launch_bounds__(256, 5) indexed_rows_kernel(const WordIndex A, const WordIndex B,
                                                            const uint64_t* __restrict__ P, int64_t n, int64_t ldw,
                                                            uint64_t* __restrict__ C, int* __restrict__ changed) {
     extern __shared__ uint64_t sq_sm[];
     const int lane = threadIdx.x & 31;
-    uint64_t* S = sq_sm + static_cast<int64_t>(threadIdx.x >> 5) * ldw;
-    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-        const longlong2 range = wcsr_row(A.ptr, i);
-        for (int64_t w = lane; w < ldw; w += 32) S[w] = P[i * ldw + w];
-        __syncwarp();
+    bool grew = false;
+    rows_of_index(A, n, [&](int64_t i, const longlong2& range, bool together) {
+        const int nw = together ? blockDim.x >> 5 : 1, warp = threadIdx.x >> 5;  // together: the warps take entries in turn
+        const int first = together ? threadIdx.x : lane, step = 32 * nw;
+        uint64_t* S = together ? sq_sm : sq_sm + warp * ldw;
+        for (int64_t w = first; w < ldw; w += step) S[w] = P[i * ldw + w];
+        sync_row(together);
         uint64_t tm = 0;  // word groups are not needed here
-        for (int64_t b0 = range.x; b0 < range.y; b0 += 32) {
-            const int64_t e = b0 + lane;
+        for (int64_t b0 = range.x; b0 < range.y; b0 += step) {
+            const int64_t e = b0 + (together ? lane * nw + warp : lane);
             const int64_t ee = e < range.y ? e : range.x;
             const uint64_t d = e < range.y ? A.val[ee] : 0ull;
-            const int64_t w = e < range.y ? A.idx[ee] : 0;
-            push_balanced(d, w, lane, B.ptr, B.idx, B.val, S, 30, tm);
+            const int w = e < range.y ? A.idx[ee] : 0;
+            push_balanced<1, false>(d, w, lane, B.ptr, B.idx, B.val, S, 30, tm);
         }
-        __syncwarp();
-        bool grew = false;
-        for (int64_t w = lane; w < ldw; w += 32) {
+        sync_row(together);
+        for (int64_t w = first; w < ldw; w += step) {
             const uint64_t c = S[w];
             grew |= c != P[i * ldw + w];
             C[i * ldw + w] = c;
         }
-        if (changed != nullptr && __any_sync(FULL, grew) && lane == 0) atomicOr(changed, 1);
-        __syncwarp();
-    }
+        sync_row(together);
+    });
+    if (changed != nullptr && __any_sync(FULL, grew) && lane == 0) atomicOr(changed, 1);
+}
+
+// Sum over the block (every thread calls it; thread 0 gets it).
+__device__ __forceinline__ unsigned long long block_sum(unsigned long long x) {
+    __shared__ unsigned long long part[32];
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(FULL, x, off);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = x;
+    __syncthreads();
+    x = 0;
+    if (threadIdx.x == 0)
+        for (int k = 0; k < static_cast<int>(blockDim.x >> 5); ++k) x += part[k];
+    __syncthreads();
+    return x;
 }
 
 // ---- the work of such a product: for every set bit k of every row of A, the nonzero words of row k of B (what
-// indexed_rows_kernel ORs into that row). cost[0] += the total, cost[1] = max over rows (one warp assembles a row, so the
-// largest row bounds the step from below). Warp per row, two 64-bit atomics per warp. Bits at or beyond n are zero in
-// every row, so k < n.
+// indexed_rows_kernel ORs into that row). cost[0] += the total, cost[1] = max over rows (one warp or block assembles a
+// row, so the largest row bounds the step from below). Two 64-bit atomics per block. Bits at or beyond n are zero in every
+// row, so k < n.
 __global__ void __launch_bounds__(256) indexed_cost_kernel(const WordIndex A, const WordIndex B, int64_t n,
                                                            unsigned long long* __restrict__ cost) {
     const int lane = threadIdx.x & 31;
-    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
-    unsigned long long total = 0, top = 0;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
+    unsigned long long total = 0, top = 0;  // lane 0's (a queued row: thread 0's)
+    const auto words_of = [&](int64_t e) {
         unsigned long long c = 0;
-        const longlong2 range = wcsr_row(A.ptr, i);
-        for (int64_t e = range.x + lane; e < range.y; e += 32) {
-            uint64_t d = A.val[e];
-            const int64_t base = static_cast<int64_t>(A.idx[e]) << 6;
-            while (d) {
-                const int64_t k = base + (__ffsll(static_cast<long long>(d)) - 1);
-                d &= d - 1ull;
-                const longlong2 r = wcsr_row(B.ptr, k);
-                c += static_cast<unsigned long long>(r.y - r.x);
+        uint64_t d = A.val[e];
+        const int64_t base = static_cast<int64_t>(A.idx[e]) << 6;
+        while (d) {  // up to four rows' ranges in flight
+            longlong2 r[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                r[q] = make_longlong2(0, 0);
+                if (d) {
+                    r[q] = wcsr_row(B.ptr, base + (__ffsll(static_cast<long long>(d)) - 1));
+                    d &= d - 1ull;
+                }
             }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) c += static_cast<unsigned long long>(r[q].y - r[q].x);
         }
-        for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(FULL, c, off);
-        total += c;
-        top = c > top ? c : top;
-    }
-    if (lane == 0 && total != 0ull) {
-        atomicAdd(cost, total);
-        atomicMax(cost + 1, top);
-    }
+        return c;
+    };
+    rows_of_index(A, n, [&](int64_t, const longlong2& range, bool together) {
+        unsigned long long c = 0;
+        const int first = together ? threadIdx.x : lane, step = together ? blockDim.x : 32;
+        for (int64_t e = range.x + first; e < range.y; e += step) c += words_of(e);
+        if (together) {
+            c = block_sum(c);
+            if (threadIdx.x != 0) c = 0;
+        } else {
+            for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(FULL, c, off);
+        }
+        if (lane == 0) {
+            total += c;
+            top = c > top ? c : top;
+        }
+    });
+    if (lane == 0 && total != 0ull) atomicMax(cost + 1, top);
+    total = block_sum(total);
+    if (threadIdx.x == 0 && total != 0ull) atomicAdd(cost, total);
 }
 
-// ---- the next squaring step's nonzero words without forming it: per row (one warp), the union of the row's own
-// word indices and those of every row k it names (R + R R), in a shared-memory bitmap of ldw bits.
+// ---- the next squaring step's nonzero words without forming it: per row, the union of the row's own word indices and
+// those of every row k it names (R + R R), in a shared-memory bitmap of ldw bits.
 // out[0] += the total nonzero words of R + R R, out[1] += the word ORs the squaring would issue.
-__global__ void __launch_bounds__(256) square_growth_kernel(const int64_t* __restrict__ wptr,
-                                                            const int32_t* __restrict__ widx,
-                                                            const uint64_t* __restrict__ wval, int64_t n, int64_t ldw,
+__global__ void __launch_bounds__(256, 6) square_growth_kernel(const WordIndex A, int64_t n, int64_t ldw,
                                                             unsigned long long* __restrict__ out,
                                                             unsigned long long* __restrict__ bits_out) {
     extern __shared__ uint32_t growth_bm[];
     const int lane = threadIdx.x & 31;
     const int bw = static_cast<int>((ldw + 31) / 32);  // bitmap words per warp
-    uint32_t* bm = growth_bm + (threadIdx.x >> 5) * bw;
-    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
     unsigned long long words = 0, ors = 0, ones = 0;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-        for (int j = lane; j < bw; j += 32) bm[j] = 0u;
-        __syncwarp();
-        const longlong2 range = wcsr_row(wptr, i);
-        for (int64_t e = range.x + lane; e < range.y; e += 32) {
-            const int x = widx[e];
-            atomicOr(&bm[x >> 5], 1u << (x & 31));
-            uint64_t d = wval[e];
-            ones += static_cast<unsigned long long>(__popcll(d));
-            const int64_t base = static_cast<int64_t>(x) << 6;
-            while (d) {
-                const int64_t k = base + (__ffsll(static_cast<long long>(d)) - 1);
-                d &= d - 1ull;
-                const longlong2 r = wcsr_row(wptr, k);
-                for (int64_t f = r.x; f < r.y; ++f) {
-                    const int y = widx[f];
-                    atomicOr(&bm[y >> 5], 1u << (y & 31));
-                    ++ors;
-                }
+    const auto mark = [&](uint32_t* bm, int64_t e) {
+        const int x = A.idx[e];
+        atomicOr(&bm[x >> 5], 1u << (x & 31));
+        uint64_t d = A.val[e];
+        ones += static_cast<unsigned long long>(__popcll(d));
+        const int64_t base = static_cast<int64_t>(x) << 6;
+        while (d) {
+            const longlong2 r = wcsr_row(A.ptr, base + (__ffsll(static_cast<long long>(d)) - 1));
+            d &= d - 1ull;
+            ors += static_cast<unsigned long long>(r.y - r.x);
+            for (int64_t f = r.x; f < r.y; f += 4) {  // four of the named row's entries in flight
+                int y[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) y[q] = f + q < r.y ? A.idx[f + q] : -1;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (y[q] >= 0) atomicOr(&bm[y[q] >> 5], 1u << (y[q] & 31));
             }
         }
-        __syncwarp();
-        for (int j = lane; j < bw; j += 32) words += static_cast<unsigned long long>(__popc(bm[j]));
-        __syncwarp();  // the bitmap is cleared for the next row
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        words += __shfl_xor_sync(FULL, words, off);
-        ors += __shfl_xor_sync(FULL, ors, off);
-        ones += __shfl_xor_sync(FULL, ones, off);
-    }
-    if (lane == 0 && (words | ors) != 0ull) {
+    };
+    rows_of_index(A, n, [&](int64_t, const longlong2& range, bool together) {
+        uint32_t* bm = together ? growth_bm : growth_bm + (threadIdx.x >> 5) * bw;
+        const int first = together ? threadIdx.x : lane, step = together ? blockDim.x : 32;
+        for (int j = first; j < bw; j += step) bm[j] = 0u;
+        sync_row(together);
+        for (int64_t e = range.x + first; e < range.y; e += step) mark(bm, e);
+        sync_row(together);
+        for (int j = first; j < bw; j += step) words += static_cast<unsigned long long>(__popc(bm[j]));
+        sync_row(together);  // the bitmap is cleared for the next row
+    });
+    words = block_sum(words);
+    ors = block_sum(ors);
+    ones = block_sum(ones);
+    if (threadIdx.x == 0 && (words | ors) != 0ull) {
         atomicAdd(out, words);
         atomicAdd(out + 1, ors);
     }
-    if (lane == 0 && bits_out != nullptr && ones != 0ull) atomicAdd(bits_out, ones);
+    if (threadIdx.x == 0 && bits_out != nullptr && ones != 0ull) atomicAdd(bits_out, ones);
 }
 
 // Bit rows of R^T from the word index of R (out cleared beforehand): warp per row i of R, a lane per nonzero word;
@@ -1602,7 +1705,7 @@ cudaError_t launch_square_growth(const WordIndex& x, int64_t n, int64_t ldw, uns
                                  unsigned long long* bits_out) {
     const size_t smem = static_cast<size_t>(8) * ((ldw + 31) / 32) * 4;
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
-    square_growth_kernel<<<warps_grid(n, sms), 256, smem, s>>>(x.ptr, x.idx, x.val, n, ldw, out, bits_out);
+    square_growth_kernel<<<warps_grid(n, sms), 256, smem, s>>>(x, n, ldw, out, bits_out);
     return cudaGetLastError();
 }
 
