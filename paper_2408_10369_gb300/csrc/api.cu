@@ -425,11 +425,13 @@ bool thin_allowed(int64_t n_pad, const bmlp_options& o) {
 // its transpose). With res_f4 set, the caller has instead encoded R / R^T as
 // packed E2M1 into the halves of M[1] / T[1]; every squaring then runs on
 // 4-bit operands and *res_f4 receives the E2M1 result (row stride n_pad / 2);
-// the squarings also keep R as bit rows, and *res_bits receives them (n_pad
-// rows of n_pad / 64 words), or null if no squaring ran.
+// the squarings also keep R and R^T as bit rows (n_pad rows of n_pad / 64
+// words), which *res_bits and *res_bits_t receive; *res_f4 is null then if the
+// last squarings left the E2M1 operands behind.
 bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], uint8_t* T[2], int max_iters,
                         const bmlp_options& o, cudaStream_t s, int* iters, uint8_t** res, uint8_t** res_t,
-                        const uint8_t** res_f4 = nullptr, const uint64_t** res_bits = nullptr) {
+                        const uint8_t** res_f4 = nullptr, const uint64_t** res_bits = nullptr,
+                        const uint64_t** res_bits_t = nullptr) {
     NvtxRange nvtx_("tensor-core squarings");
     CUtensorMap mapA[2], mapB[2], mapBh[2];
     for (int b = 0; b < 2; ++b) {
@@ -643,7 +645,8 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
             auto converged = [&](uint8_t** r, uint8_t** rt) -> bmlp_status {  // Q[qcur], QT[qcur] hold the closure
                 if (res_bits != nullptr && bits_current) {
                     *res_bits = P[bcur];
-                    *res_f4 = nullptr;
+                    if (res_bits_t != nullptr) *res_bits_t = PT[bcur];
+                    *res_f4 = q_current ? Q[qcur] : nullptr;
                     *r = *rt = nullptr;
                     return BMLP_OK;
                 }
@@ -785,7 +788,8 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
     }
     if (on_f4 && res_bits != nullptr && bits_current) {
         *res_bits = P[bcur];
-        *res_f4 = nullptr;
+        if (res_bits_t != nullptr) *res_bits_t = PT[bcur];
+        *res_f4 = q_current ? Q[qcur] : nullptr;
         *res = *res_t = nullptr;
     } else if (on_f4 && res_f4 != nullptr) {
         ST(operands_current());
@@ -1075,20 +1079,44 @@ bmlp_status sparse_squarings(bmlp_ctx* ctx, const Operand& in, int32_t fmt, int6
         out->iters++;
         cur ^= 1;
     }
-    if (out->iters > 0) {
-        out->P = P[cur];
+    if (out->iters > 0 || R0 == P[0]) {  // also without a squaring, where R had to be copied: bit rows are read faster
+        out->P = P[cur];                 // than the caller's bytes
         out->ldw = ldw;
     }
     return BMLP_OK;
 }
 
-// X = A B thresholded to 0/1 for packed E2M1 operands (A row-major, B given as B^T, both n_pad x n_pad / 2 bytes), on
-// the 4-bit squaring kernel with a zero old R (Z, cleared here), so that its R' is the product; its R'^T goes to XT
-// (scratch). Raises the call's error on an in-kernel timeout.
-bmlp_status e2m1_product(bmlp_ctx* ctx, const uint8_t* A, const uint8_t* BT, int64_t n_pad, uint8_t* Z, uint8_t* X,
-                         uint8_t* XT, const bmlp_options& o, cudaStream_t s) {
+// Device and host time of a composition's product by row ORs besides them and its passes over bit rows: launches, waits.
+constexpr double kGatherFixedS = 25e-6;
+
+// E2M1 R and R^T (n_pad) of a caller matrix or of bit rows of ldw_in words. Bytes go through bit rows in `bits` (n rows of
+// ceil(n / 64) words) above kAlwaysDenseN: the byte pass then reads whole aligned lines and the transposing one an eighth
+// of the bytes (n = 5,000: 23 us in one pass, 9 + 5 in two; n = 300: 2 and 4).
+bmlp_status to_e2m1(bmlp_ctx* ctx, const Operand& in, int32_t fmt, int64_t ldw_in, int64_t n, uint8_t* R, uint8_t* RT,
+                    int64_t n_pad, cudaStream_t s) {
+    if (fmt == BMLP_FMT_U8 && n > kAlwaysDenseN) {
+        void* bits = nullptr;
+        const int64_t ldw = words_of(n);
+        ST(ws_get(ctx, WS_SQP, static_cast<size_t>(n * ldw * 8), &bits));
+        launch_u8_to_packed(static_cast<const uint8_t*>(in.dev), n, static_cast<uint64_t*>(bits), ldw, s);
+        launch_packed_to_e2m1(static_cast<const uint64_t*>(bits), ldw, n, R, RT, n_pad, s);
+        ctx->stats.launches++;
+    } else if (fmt == BMLP_FMT_U8) {
+        launch_u8_to_e2m1(static_cast<const uint8_t*>(in.dev), n, R, RT, n_pad, s);
+    } else {
+        launch_packed_to_e2m1(static_cast<const uint64_t*>(in.dev), ldw_in, n, R, RT, n_pad, s);
+    }
+    CK(cudaGetLastError(), "E2M1 encode");
+    ctx->stats.launches++;
+    return BMLP_OK;
+}
+
+// X = A B thresholded to 0/1 for packed E2M1 operands (A row-major, B given as B^T, both n_pad x n_pad / 2 bytes), as bit
+// rows (n_pad rows of n_pad / 64 words), on the 4-bit squaring kernel without an old R. Raises the call's error on an
+// in-kernel timeout.
+bmlp_status e2m1_product(bmlp_ctx* ctx, const uint8_t* A, const uint8_t* BT, int64_t n_pad, uint64_t* X,
+                         const bmlp_options& o, cudaStream_t s) {
     const int64_t ld4 = n_pad / 2;
-    CK(cudaMemsetAsync(Z, 0, static_cast<size_t>(n_pad) * static_cast<size_t>(ld4), s), "clear old R");
     CUtensorMap fa, fb0, fb1;
     ST(make_tmap(ctx, &fa, A, n_pad, ld4, ld4, TC_BM));
     ST(make_tmap(ctx, &fb0, BT, n_pad, ld4, ld4, TC_BN / 2));
@@ -1099,16 +1127,15 @@ bmlp_status e2m1_product(bmlp_ctx* ctx, const uint8_t* A, const uint8_t* BT, int
     pp.k_blocks = static_cast<int32_t>(n_pad / 256);
     pp.mode = TC_MODE_RMS;
     pp.ld = ld4;
-    pp.old_r = Z;
-    pp.out_r = X;
-    pp.out_rt = XT;
+    pp.out_bits = reinterpret_cast<uint32_t*>(X);
+    pp.ldb = n_pad / 32;
     pp.changed = ctx->d_ctl + CTL_CHANGED;
     pp.error = ctx->d_ctl + CTL_ERROR;
     pp.wait_cycles = wait_cycles(ctx, o);
     CK(launch_tc4_product_duo(fa, fb0, fb1, pp, ctx->sm_count, s), "4-bit product launch");
     ctx->stats.product_launches++;
     ctx->stats.e2m1_products++;
-    ctx->stats.launches += 2;
+    ctx->stats.launches++;
     return read_ctl(ctx, s, nullptr);
 }
 
@@ -1584,12 +1611,7 @@ static bmlp_status core_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt
         if (o.e4m3_only == 0) ST(dense_by_blocks(ctx, src, sfmt, sldw, n, n_pad, s, &direct));
         if (direct) {
             const int64_t ld4 = n_pad / 2;
-            if (sfmt == BMLP_FMT_U8)
-                launch_u8_to_e2m1(static_cast<const uint8_t*>(src.dev), n, M[1], T[1], n_pad, s);
-            else
-                launch_packed_to_e2m1(static_cast<const uint64_t*>(src.dev), sldw, n, M[1], T[1], n_pad, s);
-            CK(cudaGetLastError(), "E2M1 encode");
-            ctx->stats.launches++;
+            ST(to_e2m1(ctx, src, sfmt, sldw, n, M[1], T[1], n_pad, s));
             const uint8_t* q = nullptr;
             const uint64_t* qb = nullptr;
             if (chain_allowed(n_pad, o)) {
@@ -1612,17 +1634,9 @@ static bmlp_status core_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt
                 return st == BMLP_OK ? finish_out(ctx, ov, s) : st;
             }
             st = rms_tc_loop(ctx, n, n_pad, M, T, max_iters - sp.iters, o, s, &iters, &res, &res_t, &q, &qb);
-            if ((st == BMLP_OK || st == BMLP_ERR_NOT_CONVERGED) && qb != nullptr) {
-                // the squarings kept R as bit rows: the result leaves from them
+            // the squarings kept R as bit rows: the result leaves from them
+            if (st == BMLP_OK || st == BMLP_ERR_NOT_CONVERGED)
                 ST(packed_out(ctx, qb, n_pad / 64, n, fmt, ov.dev, o.reflexive, s));
-            } else if (st == BMLP_OK || st == BMLP_ERR_NOT_CONVERGED) {
-                if (fmt == BMLP_FMT_U8)
-                    launch_e2m1_to_u8(q, ld4, n, static_cast<uint8_t*>(ov.dev), o.reflexive, s);
-                else
-                    launch_e2m1_to_packed(q, ld4, n, static_cast<uint64_t*>(ov.dev), words_of(n), o.reflexive, s);
-                CK(cudaGetLastError(), "E2M1 decode");
-                ctx->stats.launches++;
-            }
         } else {
             ST(to_e4m3(ctx, src, sfmt, n, M[0], T[0], n_pad, s, sldw));
             st = rms_tc_loop(ctx, n, n_pad, M, T, max_iters - sp.iters, o, s, &iters, &res, &res_t);
@@ -1817,9 +1831,64 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
         uint8_t* M[2] = {static_cast<uint8_t*>(bb[0]), static_cast<uint8_t*>(bb[1])};
         uint8_t* T[2] = {static_cast<uint8_t*>(bb[2]), static_cast<uint8_t*>(bb[3])};
         uint8_t* X = static_cast<uint8_t*>(bb[4]);
+        // R1 as bit rows and its number of ones, read along with the closure's flags
+        const int64_t ldx = n_pad / 64;
+        uint64_t* const A1 = reinterpret_cast<uint64_t*>(X);
+        const bool bits_r1 = n >= kSparseMinN && !o.tc_only && o.e4m3_only == 0;
+        if (bits_r1) {
+            auto* const ones = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_BITS);
+            CK(cudaMemsetAsync(ones, 0, sizeof(*ones), s), "reset count");
+            ST(to_packed(ctx, a, fmt, n, A1, ldx, s));
+            CK(launch_packed_ones(A1, n * ldx, ones, ctx->sm_count, s), "count ones");
+            ctx->stats.launches++;
+        }
+        // (I + R2+) R1 from bit rows of R2+ (ld words) or of its transpose: R1^T names few rows of R2+^T, so the product is
+        // formed transposed, as so many row ORs, when they are predicted to take less than a product on the tensor cores
+        // (a composition of byte matrices, n = 9,001, 2 and 3 facts a row: 1,430 us with the product, R1's encoding and the
+        // decoding of its 4-bit result, 975 us so)
+        auto gather = [&](const uint64_t* P, const uint64_t* PT, int64_t ld, bool* ran) -> bmlp_status {
+            *ran = false;
+            if (!bits_r1) return BMLP_OK;
+            unsigned long long ones = 0;
+            memcpy(&ones, ctx->h_ctl + CTL_BITS, sizeof(ones));
+            const double bytes = static_cast<double>(n) * static_cast<double>(ldx) * 8.0;
+            if (kGatherFixedS + 6.0 * bytes / 4.0e12 + static_cast<double>(ones) * static_cast<double>(ldx) * thin_word_s() >=
+                tc4_product_s(n_pad))
+                return BMLP_OK;
+            uint64_t* const W[3] = {reinterpret_cast<uint64_t*>(M[0]), reinterpret_cast<uint64_t*>(T[0]),
+                                    reinterpret_cast<uint64_t*>(T[0]) + n * ldx};
+            if (PT == nullptr) {
+                if (ld != ldx) {
+                    launch_packed_copy(P, ld, n, n, W[0], ldx, 0, s);
+                    P = W[0];
+                }
+                CK(launch_bit_transpose(P, W[2], n, ldx, s), "transpose launch");
+                PT = W[2];
+                ctx->stats.launches += 2;
+            }
+            CK(launch_bit_transpose(A1, W[1], n, ldx, s), "transpose launch");
+            CK(launch_product_packed(W[1], PT, W[0], n, ldx, 1, ctx->d_ctl + CTL_CHANGED, ctx->sm_count, s, Deadline{}, nullptr,
+                                     false),
+               "product launch");
+            CK(launch_bit_transpose(W[0], A1, n, ldx, s), "transpose launch");
+            ctx->stats.launches += 3;
+            ctx->stats.product_launches++;
+            ST(packed_out(ctx, A1, ldx, n, fmt, ov.dev, 0, s));
+            *ran = true;
+            return BMLP_OK;
+        };
+        bool out_done = false;
         // R2+ as in bmlp_rms: squarings on bit rows while R2 is sparse, then on the tensor cores
         SparseStart sp;
         if (!o.tc_only) ST(sparse_squarings(ctx, b, fmt, n, n_pad, max_iters, o, s, &sp));
+        if (sp.done) {
+            ST(gather(sp.P, nullptr, sp.ldw, &out_done));
+            if (out_done) {
+                ctx->stats.iterations = iters = sp.iters;
+                if (iters_out) *iters_out = iters;
+                return finish_out(ctx, ov, s);
+            }
+        }
         Operand src = b;
         int32_t sfmt = fmt;
         int64_t sldw = words_of(n);
@@ -1834,17 +1903,12 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
         if (direct) {
             // dense R2: its closure on packed E2M1 operands in the halves of M[1], T[1] (as bmlp_rms), then
             // (I + R2+) R1 on the same 4-bit squaring kernel: A = I + R2+ (diagonal set in place), B^T = R1^T
-            // (R1 and R1^T encoded into the first halves of M[0], T[0]) and a zero old R (M[0]'s second half), so
-            // that the kernel's R' is C > 0 (into X; R'^T into T[0]'s second half)
+            // (R1 and R1^T encoded into the first halves of M[0], T[0])
             const int64_t ld4 = n_pad / 2;
             const size_t half = static_cast<size_t>(n_pad) * static_cast<size_t>(ld4);
-            if (sfmt == BMLP_FMT_U8)
-                launch_u8_to_e2m1(static_cast<const uint8_t*>(src.dev), n, M[1], T[1], n_pad, s);
-            else
-                launch_packed_to_e2m1(static_cast<const uint64_t*>(src.dev), sldw, n, M[1], T[1], n_pad, s);
-            CK(cudaGetLastError(), "E2M1 encode");
-            ctx->stats.launches++;
+            ST(to_e2m1(ctx, src, sfmt, sldw, n, M[1], T[1], n_pad, s));
             const uint8_t* q = M[1];  // the closure already, when the bit-row squarings reached it
+            const uint64_t *qb = nullptr, *qbt = nullptr;
             st = BMLP_OK;
             if (!sp.done && chain_allowed(n_pad, o)) {
                 uint8_t* const Q[2] = {M[1], M[1] + half};
@@ -1855,25 +1919,27 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
                 q = Q[cur];
             } else if (!sp.done) {
                 uint8_t *res = nullptr, *res_t = nullptr;
-                st = rms_tc_loop(ctx, n, n_pad, M, T, max_iters - sp.iters, o, s, &iters, &res, &res_t, &q);
+                st = rms_tc_loop(ctx, n, n_pad, M, T, max_iters - sp.iters, o, s, &iters, &res, &res_t, &q, &qb, &qbt);
             }
             iters += sp.iters;
             if (st != BMLP_OK) return st;
-            uint8_t* A = const_cast<uint8_t*>(q);  // a half of M[1], this call's workspace
-            launch_set_diag_e2m1(A, ld4, n, s);
-            if (fmt == BMLP_FMT_U8)
-                launch_u8_to_e2m1(static_cast<const uint8_t*>(a.dev), n, M[0], T[0], n_pad, s);
-            else
-                launch_packed_to_e2m1(static_cast<const uint64_t*>(a.dev), words_of(n), n, M[0], T[0], n_pad, s);
-            CK(cudaGetLastError(), "E2M1 encode of R1");
-            ctx->stats.launches += 2;
-            ST(e2m1_product(ctx, A, T[0], n_pad, M[0] + half, X, T[0] + half, o, s));
-            if (fmt == BMLP_FMT_U8)
-                launch_e2m1_to_u8(X, ld4, n, static_cast<uint8_t*>(ov.dev), 0, s);
-            else
-                launch_e2m1_to_packed(X, ld4, n, static_cast<uint64_t*>(ov.dev), words_of(n), 0, s);
-            CK(cudaGetLastError(), "E2M1 decode");
-            ctx->stats.launches++;
+            if (qb != nullptr) ST(gather(qb, qbt, ldx, &out_done));
+            if (!out_done) {
+                uint8_t* A = const_cast<uint8_t*>(q);  // a half of M[1], this call's workspace
+                if (A == nullptr) {
+                    A = M[1];
+                    launch_packed_to_e2m1(qb, ldx, n, M[1], T[1], n_pad, s);
+                    CK(cudaGetLastError(), "E2M1 encode");
+                    ctx->stats.launches++;
+                }
+                launch_set_diag_e2m1(A, ld4, n, s);
+                ctx->stats.launches++;
+                Operand r1 = a;
+                if (bits_r1) r1.dev = A1;
+                ST(to_e2m1(ctx, r1, bits_r1 ? BMLP_FMT_PACKED64 : fmt, bits_r1 ? ldx : words_of(n), n, M[0], T[0], n_pad, s));
+                ST(e2m1_product(ctx, A, T[0], n_pad, A1, o, s));
+                ST(packed_out(ctx, A1, ldx, n, fmt, ov.dev, 0, s));
+            }
         } else {
             if (sp.P) {
                 Operand pk;
@@ -2014,22 +2080,13 @@ static bmlp_status core_rms_alg1(bmlp_ctx* ctx, const void* R, int64_t n, int32_
     for (int k = 0; k < 5; ++k) B8[k] = static_cast<uint8_t*>(bb[k]);
     if (o.e4m3_only == 0) {
         // on 4-bit operands: A = I + R1+ and R1 (with R1^T) as packed E2M1 in the first halves of the buffers
-        const int64_t ld4 = n_pad / 2;
-        const size_t half = static_cast<size_t>(n_pad) * static_cast<size_t>(ld4);
         launch_packed_to_e2m1(static_cast<const uint64_t*>(q), ldw, n, B8[0], B8[2], n_pad, s);
-        if (fmt == BMLP_FMT_U8)
-            launch_u8_to_e2m1(static_cast<const uint8_t*>(a.dev), n, B8[1], B8[3], n_pad, s);
-        else
-            launch_packed_to_e2m1(static_cast<const uint64_t*>(a.dev), ldw, n, B8[1], B8[3], n_pad, s);
         CK(cudaGetLastError(), "E2M1 encode");
-        ctx->stats.launches += 2;
-        ST(e2m1_product(ctx, B8[0], B8[3], n_pad, B8[0] + half, B8[4], B8[2] + half, o, s));
-        if (fmt == BMLP_FMT_U8)
-            launch_e2m1_to_u8(B8[4], ld4, n, static_cast<uint8_t*>(ov.dev), o.reflexive, s);
-        else
-            launch_e2m1_to_packed(B8[4], ld4, n, static_cast<uint64_t*>(ov.dev), words_of(n), o.reflexive, s);
-        CK(cudaGetLastError(), "E2M1 decode");
         ctx->stats.launches++;
+        ST(to_e2m1(ctx, a, fmt, ldw, n, B8[1], B8[3], n_pad, s));
+        uint64_t* X = reinterpret_cast<uint64_t*>(B8[4]);
+        ST(e2m1_product(ctx, B8[0], B8[3], n_pad, X, o, s));
+        ST(packed_out(ctx, X, n_pad / 64, n, fmt, ov.dev, o.reflexive, s));
     } else {
         Operand qs;
         qs.dev = q;

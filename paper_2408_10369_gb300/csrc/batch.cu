@@ -1198,19 +1198,23 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
         }
         // ---- results: Q[0] holds the closure (a product that changed nothing left both buffers equal)
         if (p.kind == BMLP_PROBLEM_CLOSURE) {
-            if (p.fmt == BMLP_FMT_U8)
-                launch_e2m1_to_u8(Q[0], ld4, n, static_cast<uint8_t*>(p.out), p.reflexive, cs);
-            else
+            if (p.fmt == BMLP_FMT_U8) {  // bytes leave through bit rows, in the places of the bit-row squarings
+                launch_e2m1_to_packed(Q[0], ld4, n, P0, ldw, 0, cs);
+                launch_packed_to_u8(P0, ldw, n, static_cast<uint8_t*>(p.out), p.reflexive, cs);
+            } else {
                 launch_e2m1_to_packed(Q[0], ld4, n, static_cast<uint64_t*>(p.out), (n + 63) / 64, p.reflexive, cs);
+            }
         } else {
             // out = (I + R2+) R1 on 4-bit operands, on the squaring kernel: A = I + R2+ (Q[0], diagonal set),
             // B^T = R1^T (encoded with R1 into the free pair Q[1], QT[1]), and a zero "old R" (QT[0]), so that the
             // kernel's R' is C > 0; R' goes to Q[1] (R1 is no longer needed), R'^T to the scratch
             launch_set_diag_e2m1(Q[0], ld4, n, cs);
-            if (p.fmt == BMLP_FMT_U8)
-                launch_u8_to_e2m1(static_cast<const uint8_t*>(p.R1), n, Q[1], QT[1], n_pad, cs);
-            else
+            if (p.fmt == BMLP_FMT_U8) {
+                launch_u8_to_packed(static_cast<const uint8_t*>(p.R1), n, P0, ldw, cs);
+                launch_packed_to_e2m1(P0, ldw, n, Q[1], QT[1], n_pad, cs);
+            } else {
                 launch_packed_to_e2m1(static_cast<const uint64_t*>(p.R1), (n + 63) / 64, n, Q[1], QT[1], n_pad, cs);
+            }
             SCK(cudaMemsetAsync(QT[0], 0, static_cast<size_t>(n_pad) * static_cast<size_t>(ld4), cs), "clear old R");
             CUtensorMap fa, fb0, fb1;
             SST(make_tmap(ctx, &fa, Q[0], n_pad, ld4, ld4, TC_BM));
@@ -1229,10 +1233,12 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
             pp.error = ctx->d_ctl + CTL_ERROR;
             pp.wait_cycles = wait_cycles;
             SCK(launch_tc4_product_duo(fa, fb0, fb1, pp, sms, cs), "final product");
-            if (p.fmt == BMLP_FMT_U8)
-                launch_e2m1_to_u8(Q[1], ld4, n, static_cast<uint8_t*>(p.out), 0, cs);
-            else
+            if (p.fmt == BMLP_FMT_U8) {  // bytes leave through bit rows, in the places of the bit-row squarings
+                launch_e2m1_to_packed(Q[1], ld4, n, P0, ldw, 0, cs);
+                launch_packed_to_u8(P0, ldw, n, static_cast<uint8_t*>(p.out), 0, cs);
+            } else {
                 launch_e2m1_to_packed(Q[1], ld4, n, static_cast<uint64_t*>(p.out), (n + 63) / 64, 0, cs);
+            }
         }
         SCK(cudaGetLastError(), "large-problem launches");
     }

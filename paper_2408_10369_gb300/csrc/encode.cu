@@ -189,31 +189,6 @@ __global__ void __launch_bounds__(256) packed_to_e2m1_kernel(const uint64_t* __r
     }
 }
 
-// Packed E2M1 rows -> u8 0/1 rows (n x n, + I if reflexive); 16 outputs per thread.
-__global__ void e2m1_to_u8_kernel(const uint8_t* __restrict__ Q, int64_t ld4, int64_t n, uint8_t* __restrict__ out,
-                                  int reflexive, bool vec_out) {
-    const int64_t segs = (n + 15) / 16;
-    const int64_t total = n * segs;
-    for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < total;
-         t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t i = t / segs, j0 = (t % segs) * 16;
-        const uint2 v = *reinterpret_cast<const uint2*>(Q + i * ld4 + j0 / 2);
-        uint32_t bits = nib_gather8(v.x) | (nib_gather8(v.y) << 8);
-        if (reflexive && i >= j0 && i < j0 + 16) bits |= 1u << (i - j0);
-        uint8_t* o = out + i * n + j0;
-        if (vec_out && j0 + 16 <= n) {
-            uint32_t q[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                q[k] = ((bits >> (4 * k)) & 1u) | (((bits >> (4 * k + 1)) & 1u) << 8) |
-                       (((bits >> (4 * k + 2)) & 1u) << 16) | (((bits >> (4 * k + 3)) & 1u) << 24);
-            *reinterpret_cast<uint4*>(o) = make_uint4(q[0], q[1], q[2], q[3]);
-        } else {
-            for (int k = 0; k < 16 && j0 + k < n; ++k) o[k] = (bits >> k) & 1u;
-        }
-    }
-}
-
 // Packed E2M1 rows -> packed bit rows (ldw_out words, + I if reflexive); one output word per thread.
 __global__ void e2m1_to_packed_kernel(const uint8_t* __restrict__ Q, int64_t ld4, int64_t n,
                                       uint64_t* __restrict__ out, int64_t ldw_out, int reflexive) {
@@ -688,11 +663,6 @@ void launch_packed_to_e2m1(const uint64_t* in, int64_t ldw_in, int64_t n, uint8_
     const bool vec = (ldw_in % 2 == 0) && ((reinterpret_cast<uintptr_t>(in) & 15) == 0);
     dim3 grid(static_cast<unsigned>(n_pad / 256), static_cast<unsigned>(n_pad / 256));
     packed_to_e2m1_kernel<<<grid, 256, 0, s>>>(in, ldw_in, n, R, RT, n_pad / 2, vec);
-}
-
-void launch_e2m1_to_u8(const uint8_t* Q, int64_t ld4, int64_t n, uint8_t* out, int reflexive, cudaStream_t s) {
-    const bool vec = (n % 16 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
-    e2m1_to_u8_kernel<<<grid_for(n * ((n + 15) / 16), 256), 256, 0, s>>>(Q, ld4, n, out, reflexive, vec);
 }
 
 void launch_e2m1_to_packed(const uint8_t* Q, int64_t ld4, int64_t n, uint64_t* out, int64_t ldw_out, int reflexive,

@@ -58,8 +58,8 @@ struct TcParams {
     uint32_t* out_bits;
     uint32_t* out_bits_t;
     int64_t ldb;
-    // if not null, R of this iteration as such bit rows, instead of old_r (may be out_bits); out_r may then be null with
-    // out_bits set: R' leaves as bit rows only
+    // if not null, R of this iteration as such bit rows, instead of old_r (may be out_bits). out_r may be null with out_bits
+    // set: R' leaves as bit rows only; without old_r and old_bits R' is the product alone
     const uint32_t* old_bits;
     int32_t k_first;            // squaring kernels on packed operands: first of the k_blocks blocks of K
 };
@@ -247,7 +247,6 @@ void launch_u8_to_e2m1(const uint8_t* in, int64_t n, uint8_t* R, uint8_t* RT, in
 void launch_packed_to_e2m1(const uint64_t* in, int64_t ldw_in, int64_t n, uint8_t* R, uint8_t* RT, int64_t n_pad,
                            cudaStream_t s);
 // packed E2M1 rows (ld4 bytes) -> u8 n x n / packed rows of ldw_out words (+ I if reflexive)
-void launch_e2m1_to_u8(const uint8_t* Q, int64_t ld4, int64_t n, uint8_t* out, int reflexive, cudaStream_t s);
 void launch_e2m1_to_packed(const uint8_t* Q, int64_t ld4, int64_t n, uint64_t* out, int64_t ldw_out, int reflexive,
                            cudaStream_t s);
 // 1 per nonzero 128 x 128 block of an n x n matrix (fmt u8 with rows of n bytes, or packed with rows of
@@ -418,6 +417,8 @@ int64_t insert_chunk_words(int64_t ldw);
 cudaError_t launch_insert_chunk(uint64_t* P, int64_t n, int64_t ldw, const int32_t* pairs, int m, uint64_t* scratch,
                                 int sms, cudaStream_t s);
 // out = in^T on n x n packed rows of ldw words (every word of out written, padding words with zeros)
+// *ones += the ones of `words` 64-bit words (16-byte aligned, an even number).
+cudaError_t launch_packed_ones(const uint64_t* P, int64_t words, unsigned long long* ones, int sms, cudaStream_t s);
 cudaError_t launch_bit_transpose(const uint64_t* in, uint64_t* out, int64_t n, int64_t ldw, cudaStream_t s);
 int smp_packed_max_words();
 // One closure by frontier expansion inside a grouped batch (device copy): every row of R1+ as one query row.

@@ -1217,6 +1217,18 @@ __global__ void __launch_bounds__(256, 6) square_growth_kernel(const WordIndex A
     if (threadIdx.x == 0 && bits_out != nullptr && ones != 0ull) atomicAdd(bits_out, ones);
 }
 
+// Ones of a run of words, 16 bytes a lane.
+__global__ void __launch_bounds__(256) packed_ones_kernel(const uint64_t* __restrict__ P, int64_t words,
+                                                          unsigned long long* __restrict__ out) {
+    unsigned long long c = 0;
+    for (int64_t k = blockIdx.x * 256ll + threadIdx.x; 2 * k < words; k += gridDim.x * 256ll) {
+        const uint4 v = reinterpret_cast<const uint4*>(P)[k];
+        c += static_cast<unsigned long long>(__popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w));
+    }
+    c = block_sum(c);
+    if (threadIdx.x == 0 && c) atomicAdd(out, c);
+}
+
 // Bit rows of R^T from the word index of R (out cleared beforehand): warp per row i of R, a lane per nonzero word;
 // each set bit (i, j) ORs bit i into word i / 64 of row j. Rows i of one 64-row group hit the same words of R^T,
 // on different bits.
@@ -1745,6 +1757,11 @@ cudaError_t launch_smp_packed(const WordIndex& x, const WordIndex& T, int64_t n,
     smp_packed_kernel<<<static_cast<int>(blocks), warps * 32, smem, s>>>(
         x.ptr, x.idx, x.val, n, ldw, src, ldw_src, q, out, ldw_out, levels,
         reinterpret_cast<unsigned long long*>(qcounter), reflexive, max_levels, dl, T.ptr, T.idx, T.val);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_packed_ones(const uint64_t* P, int64_t words, unsigned long long* ones, int sms, cudaStream_t s) {
+    packed_ones_kernel<<<static_cast<int>(std::min<int64_t>((words + 511) / 512, sms * 8)), 256, 0, s>>>(P, words, ones);
     return cudaGetLastError();
 }
 

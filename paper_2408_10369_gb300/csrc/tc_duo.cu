@@ -226,6 +226,11 @@ __device__ __forceinline__ void f4_old(const TcParams& p, int64_t row, int64_t c
         for (int c = 0; c < CHUNKS; ++c) ob[c] = col_base + c * 32 < n_pad ? bits[c] : 0u;
         return;
     }
+    if (p.old_r == nullptr) {
+#pragma unroll
+        for (int c = 0; c < CHUNKS; ++c) ob[c] = 0u;
+        return;
+    }
     const uint8_t* src = p.old_r + row * p.ld + col_base / 32 * CB;
 #pragma unroll
     for (int c = 0; c < CHUNKS; ++c) ob[c] = col_base + c * 32 < n_pad ? load_bits32<KIND>(src + c * CB) : 0u;
