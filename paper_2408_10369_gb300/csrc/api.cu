@@ -419,6 +419,31 @@ bool thin_allowed(int64_t n_pad, const bmlp_options& o) {
     return !o.tc_only && thin_enabled() && thin_fixed_s(n_pad) < tc4_product_s(n_pad);
 }
 
+// Whether a call by the tensor-core variant runs as one launch on bit rows: small relations whose call asks for nothing that
+// needs the tensor cores or the host between two products.
+bool small_allowed(int64_t n, const bmlp_options& o) {
+    return n <= kSmallN && !o.tc_only && o.e4m3_only == 0 && o.profile == 0 && o.budget_ns == 0;
+}
+
+// The closure of `in`, or with r1 the composition (I + in+) r1, by that launch.
+bmlp_status small_closure(bmlp_ctx* ctx, const Operand& in, const void* r1, int64_t n, int32_t fmt, void* out, int reflexive,
+                          int max_iters, const bmlp_options& o, cudaStream_t s, int* iters) {
+    void* scratch = nullptr;
+    ST(ws_get(ctx, WS_SMALL, small_closure_bytes(n), &scratch));
+    CK(launch_small_closure(in.dev, r1, out, n, fmt == BMLP_FMT_U8, reflexive, max_iters, scratch,
+                            reinterpret_cast<unsigned*>(ctx->d_ctl + CTL_THIN), ctx->d_ctl + CTL_STEP, ctx->d_ctl + CTL_ERROR, wait_cycles(ctx, o), ctx->sm_count, s),
+       "small closure launch");
+    ctx->stats.launches++;
+    ST(read_ctl(ctx, s, nullptr));
+    *iters = ctx->h_ctl[CTL_STEP];
+    ctx->stats.product_launches += *iters;
+    ctx->stats.iterations = *iters;
+    if (ctx->h_ctl[CTL_STEP + 1] != 0)
+        return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "no fixpoint within %d products", max_iters);
+    if (r1 != nullptr) ctx->stats.product_launches++;
+    return BMLP_OK;
+}
+
 // ------------------------------------------------------------------------
 // Tensor-core squaring fixpoint on E4M3 R / R^T buffers already encoded in
 // (M[0], T[0]). On return *res points at the buffer holding R1+ (and *res_t at
@@ -1577,6 +1602,9 @@ static bmlp_status core_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt
         int32_t it = 0;
         st = batch_run_impl(ctx, &pr, 1, variant, wait_cycles(ctx, o), &it, s, batch_solo_n());
         iters = it;
+    } else if (variant == BMLP_RMS_TC && small_allowed(n, o)) {
+        ctx->stats.n_pad = round_up(n, TC_PAD);
+        st = small_closure(ctx, in, nullptr, n, fmt, ov.dev, o.reflexive, max_iters, o, s, &iters);
     } else if (variant == BMLP_RMS_TC) {
         const int64_t n_pad = round_up(n, TC_PAD);
         ctx->stats.n_pad = n_pad;
@@ -1818,7 +1846,10 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
     ST(stage_out(ctx, out, fmt_bytes(fmt, n, n), WS_OUT, &ov));
     int iters = 0;
     bmlp_status st;
-    if (variant == BMLP_RMS_TC) {
+    if (variant == BMLP_RMS_TC && small_allowed(n, o)) {
+        ctx->stats.n_pad = round_up(n, TC_PAD);
+        ST(small_closure(ctx, b, a.dev, n, fmt, ov.dev, 0, max_iters, o, s, &iters));
+    } else if (variant == BMLP_RMS_TC) {
         const int64_t n_pad = round_up(n, TC_PAD);
         ctx->stats.n_pad = n_pad;
         const size_t bytes = static_cast<size_t>(n_pad * n_pad);

@@ -174,6 +174,8 @@ enum CtlWord : int {
 constexpr int CTL_HOST_I64 = CTL_WORDS;
 constexpr int CTL_HOST_WORDS = CTL_WORDS + 2;
 
+// Bit rows and the barrier of the one-launch closures (small.cu).
+constexpr int WS_SMALL = 40;
 // Workspace slots of the grouped batch and of its device-driven large problems (the others are private to api.cu).
 constexpr int WS_BATCH = 15;
 constexpr int WS_SOLO = 25;
@@ -417,6 +419,13 @@ int64_t insert_chunk_words(int64_t ldw);
 cudaError_t launch_insert_chunk(uint64_t* P, int64_t n, int64_t ldw, const int32_t* pairs, int m, uint64_t* scratch,
                                 int sms, cudaStream_t s);
 // out = in^T on n x n packed rows of ldw words (every word of out written, padding words with zeros)
+// ---- small relations (small.cu): closure of `in`, or with r1 the composition (I + in+) r1, in one cooperative launch.
+// *arrived must be zero; result[0] = products, result[1] = 1 if the last of max_iters still changed R (a composition is then not written).
+constexpr int64_t kSmallN = 1024;
+size_t small_closure_bytes(int64_t n);
+cudaError_t launch_small_closure(const void* in, const void* r1, void* out, int64_t n, bool bytes, int reflexive,
+                                 int max_iters, void* scratch, unsigned* arrived, int* result, int* error,
+                                 long long wait_cycles, int sms, cudaStream_t s);
 // *ones += the ones of `words` 64-bit words (16-byte aligned, an even number).
 cudaError_t launch_packed_ones(const uint64_t* P, int64_t words, unsigned long long* ones, int sms, cudaStream_t s);
 cudaError_t launch_bit_transpose(const uint64_t* in, uint64_t* out, int64_t n, int64_t ldw, cudaStream_t s);
