@@ -1267,7 +1267,17 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
     ctx->stats.launches++;
     // nonzero words of R (W) and of R + R R (W2, counted from the word index of R without forming R + R R)
     int64_t ones = -1;  // ones of the current R (with its word index), when a growth test has counted them
-    auto growth = [&](int64_t* W, int64_t* W2) -> bmlp_status {
+    // the tiled frontier's counts, taken along: constants that something reaches, rows to expand (all, under a time budget:
+    // a row that follows from another one is formed at the end)
+    auto* const tile_counts = ctx->d_ctl + CTL_PSTAT;
+    const bool derive = square_first && ctx->budget_ns == 0;
+    void* prep = nullptr;
+    auto growth = [&](int64_t* W, int64_t* W2, bool tiles) -> bmlp_status {
+        if (tiles && n <= 65536 && smp_sliced_enabled()) {
+            ST(ws_get(ctx, WS_TILE_PREP, smp_tile_prep_bytes(n), &prep));
+            CK(launch_smp_tile_prep(x, n, prep, tile_counts, derive, ctx->sm_count, s), "frontier preparation launch");
+            ctx->stats.launches += 2;
+        }
         auto* cnt = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_COST);
         auto* bits = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_BITS);
         CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), s), "reset counts");
@@ -1293,7 +1303,7 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         // it saves in levels, and that squaring is not formed.
         for (int k = 0; k < kSquareMaxSteps; ++k) {
             int64_t W = 0, W2 = 0;
-            ST(growth(&W, &W2));
+            ST(growth(&W, &W2, k == 0));
             if (static_cast<double>(W2) > kSquareMaxGrowth * static_cast<double>(W)) {
                 // the first squaring widens the rows fast: closure rows fill up within a few levels
                 dense_reach = k == 0 && static_cast<double>(W2) > kSlicedMinGrowth * static_cast<double>(W);
@@ -1321,31 +1331,41 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         // query rows 64 at a time (bit-sliced) when the rows of R widen fast, the closures' test; R itself is used
         // as it is (the levels stay those of R)
         int64_t W = 0, W2 = 0;
-        ST(growth(&W, &W2));
+        ST(growth(&W, &W2, true));
         dense_reach = W > 0 && static_cast<double>(W2) > kSlicedMinGrowth * static_cast<double>(W);
     }
-    const int width = dense_reach && smp_sliced_enabled() && ones >= 0 ? smp_tile_width(n, q, ctx->sm_count) : 0;
+    const int64_t n1 = ctx->h_ctl[CTL_PSTAT], expand = square_first ? ctx->h_ctl[CTL_PSTAT + 1] : q;
+    const int width = dense_reach && prep != nullptr && ones >= 0 ? smp_tile_width(n1, expand, ctx->sm_count) : 0;
     if (width > 0) {
-        // batches of rows with their frontier in one SM's shared memory: query rows, or the closure's identity rows
+        // batches of rows with their frontier in one SM's shared memory: query rows, or the closure's rows
         void* scratch = nullptr;
-        ST(ws_get(ctx, WS_V, smp_tile_bytes(n, ones, width, ctx->sm_count), &scratch));
+        ST(ws_get(ctx, WS_V, smp_tile_bytes(n, n1, ones, width, ctx->sm_count), &scratch));
         CK(cudaMemsetAsync(ctx->d_ctl + CTL_LEVELS, 0, 3 * sizeof(int), s), "reset level and query counters");
         ProductTimer tm{ctx, o.profile != 0, s};
         ST(tm.begin());
-        CK(launch_smp_tiles(x, n, ones, square_first ? nullptr : src, ldw_src, q, out, ldw_out,
-                            square_first ? 0 : o.reflexive, width, scratch,
-                            reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_QCOUNT), ctx->d_ctl + CTL_LEVELS,
-                            static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), ctx->sm_count, s, deadline_of(ctx)),
-           "tile frontier kernel launch");
+        const auto tiles = [&](bool again) {
+            return launch_smp_tiles(x, n, n1, ones, square_first ? nullptr : src, ldw_src, expand, out, ldw_out,
+                                    square_first ? 0 : o.reflexive, width, prep, scratch, derive, again, tile_counts,
+                                    reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_QCOUNT),
+                                    ctx->d_ctl + CTL_LEVELS, static_cast<int>(n + 1), ctx->sm_count, s, deadline_of(ctx));
+        };
+        CK(tiles(false), "tile frontier kernel launch");
         ST(tm.end());
         ctx->stats.product_launches++;
         ctx->stats.launches += 7;
         ctx->stats.sliced_closures++;
-        CK(cudaMemcpyAsync(ctx->h_ctl + CTL_HOST_I64, smp_tile_top_degree(scratch, n), sizeof(int), cudaMemcpyDeviceToHost, s),
+        CK(cudaMemcpyAsync(ctx->h_ctl + CTL_HOST_I64, smp_tile_top_degree(prep, n), sizeof(int), cudaMemcpyDeviceToHost, s),
            "read largest in-degree");
         ST(read_ctl(ctx, s, nullptr));
         ST(tm.collect());
-        const double skew = static_cast<double>(ctx->h_ctl[CTL_HOST_I64]) * static_cast<double>(n) /
+        const int top_degree = ctx->h_ctl[CTL_HOST_I64];
+        if (derive && ctx->h_ctl[CTL_PSTAT + 2] > ctx->h_ctl[CTL_LEVELS]) {
+            // derived rows whose level count is not certain could be the deepest ones
+            CK(tiles(true), "tile frontier kernel launch");
+            ctx->stats.launches += 2;
+            ST(read_ctl(ctx, s, nullptr));
+        }
+        const double skew = static_cast<double>(top_degree) * static_cast<double>(n) /
                             static_cast<double>(ones > 0 ? ones : 1);
         if (!square_first || skew > kSkewedColumns) ctx->stats.cluster_frontiers++;
         *levels = ctx->h_ctl[CTL_LEVELS];
