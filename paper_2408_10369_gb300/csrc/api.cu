@@ -363,7 +363,7 @@ bmlp_status rms_f4_chain(bmlp_ctx* ctx, int64_t n_pad, uint8_t* const Q[2], uint
     }
     TcParams p{};
     p.m_tiles = static_cast<int32_t>(n_pad / TC_BM);
-    p.n_tiles = static_cast<int32_t>((n_pad + tc4_tile_n() - 1) / tc4_tile_n());
+    p.n_tiles = tc4_tiles(n_pad, ctx->sm_count);
     p.k_blocks = static_cast<int32_t>(n_pad / 256);
     p.mode = TC_MODE_RMS;
     p.ld = ld4;
@@ -701,7 +701,7 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
             TcParams p4 = p;
             p4.ld = ld4;
             p4.k_blocks = static_cast<int32_t>(n_pad / 256);
-            p4.n_tiles = static_cast<int32_t>((n_pad + tc4_tile_n() - 1) / tc4_tile_n());
+            p4.n_tiles = tc4_tiles(n_pad, ctx->sm_count);
             p4.fmap = p4.fmapT = p4.fmap_next = p4.fmapT_next = nullptr;
             p4.old_r = Q[qcur];
             p4.out_r = Q[qcur ^ 1];
@@ -1148,7 +1148,7 @@ bmlp_status e2m1_product(bmlp_ctx* ctx, const uint8_t* A, const uint8_t* BT, int
     ST(make_tmap(ctx, &fb1, BT, n_pad, ld4, ld4, tc4_b1_rows()));
     TcParams pp{};
     pp.m_tiles = static_cast<int32_t>(n_pad / TC_BM);
-    pp.n_tiles = static_cast<int32_t>((n_pad + tc4_tile_n() - 1) / tc4_tile_n());
+    pp.n_tiles = tc4_tiles(n_pad, ctx->sm_count);
     pp.k_blocks = static_cast<int32_t>(n_pad / 256);
     pp.mode = TC_MODE_RMS;
     pp.ld = ld4;

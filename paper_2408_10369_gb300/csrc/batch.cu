@@ -1130,7 +1130,7 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
             for (int half = 0; half < 2 && e == cudaSuccess; ++half) {
                 TcParams p4{};
                 p4.m_tiles = static_cast<int32_t>(n_pad / TC_BM);
-                p4.n_tiles = static_cast<int32_t>((n_pad + tc4_tile_n() - 1) / tc4_tile_n());
+                p4.n_tiles = tc4_tiles(n_pad, sms);
                 p4.k_blocks = static_cast<int32_t>(n_pad / 256);
                 p4.mode = TC_MODE_RMS;
                 p4.ld = ld4;
@@ -1222,7 +1222,7 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
             SST(make_tmap(ctx, &fb1, QT[1], n_pad, ld4, ld4, tc4_b1_rows()));
             TcParams pp{};
             pp.m_tiles = static_cast<int32_t>(n_pad / TC_BM);
-            pp.n_tiles = static_cast<int32_t>((n_pad + tc4_tile_n() - 1) / tc4_tile_n());
+            pp.n_tiles = tc4_tiles(n_pad, sms);
             pp.k_blocks = static_cast<int32_t>(n_pad / 256);
             pp.mode = TC_MODE_RMS;
             pp.ld = ld4;

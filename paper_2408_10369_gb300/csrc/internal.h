@@ -286,10 +286,10 @@ cudaError_t launch_tc_product(const CUtensorMap& a, const CUtensorMap& b, const 
                               cudaStream_t s);
 // squaring step (RMS mode only) on packed E2M1 operands (n_pad x n_pad / 2 bytes, p.ld = n_pad / 2,
 // p.k_blocks = n_pad / 256) as M = 256 MMAs per CTA pair (tcgen05 .cta_group::2, 2-CTA clusters) on pair tiles
-// of 256 rows x tc4_tile_n() columns (p.n_tiles = ceil(n_pad / tc4_tile_n())); maps over R (A, box 128 rows)
+// of 256 rows x 480 columns, or 256 columns for small n_pad (p.n_tiles = tc4_tiles(n_pad, sms)); maps over R (A, box 128 rows)
 // and R^T (b0: box 128 rows; b1: box tc4_b1_rows() rows), 128 bytes wide. p.issued counts 128 x 32 x 128
 // multiply-add units.
-int tc4_tile_n();
+int tc4_tiles(int64_t n_pad, int sms);
 int tc4_b1_rows();
 // the same squaring step on E4M3 operands (n_pad x n_pad bytes, p.ld = n_pad, p.k_blocks = n_pad / 128) as
 // kind::f8f6f4 M = 256 MMAs per CTA pair on pair tiles of 256 x tc8_tile_n() (p.n_tiles = ceil(n_pad / that));

@@ -557,12 +557,27 @@ cudaError_t launch_duo(const CUtensorMap& a, const CUtensorMap& b0, const CUtens
     return cudaGetLastError();
 }
 
-int tc4_tile_n() { return Duo<1, TC4_N1>::BN; }
+// Columns of a pair tile. Up to about n_pad = 4,000 a product takes as long as its rounds of tiles over the SM pairs, and a
+// round of 256-column tiles has half the MMAs and half the epilogue of one of 480-column tiles: 256 where that takes fewer
+// than 1.55 times the rounds (for large n the ratio of their times per tile, 1.875 x 7.33 / 8.88). A product of uniform
+// random relations, 480 and 256 columns: n_pad = 1,280: 14.1 and 10.5 us; 2,048: 15.8 and 11.7; 2,304 (1 and 2 rounds): 17.0
+// and 18.4; 3,072 (2 and 2): 31.5 and 21.2; 3,840 (2 and 3): 30.9 and 28.4.
+static int tile_columns(int64_t n_pad, int sms) {
+    const int64_t m_pairs = n_pad / (2 * TC_BM), pairs = sms / 2 > 0 ? sms / 2 : 1;
+    const auto rounds = [&](int64_t bn) { return (m_pairs * ((n_pad + bn - 1) / bn) + pairs - 1) / pairs; };
+    return 100 * rounds(Duo<1, 0>::BN) < 155 * rounds(Duo<1, TC4_N1>::BN) ? Duo<1, 0>::BN : Duo<1, TC4_N1>::BN;
+}
+int tc4_tiles(int64_t n_pad, int sms) {
+    const int bn = tile_columns(n_pad, sms);
+    return static_cast<int>((n_pad + bn - 1) / bn);
+}
 int tc4_b1_rows() { return Duo<1, TC4_N1>::B1_ROWS; }
 int tc8_tile_n() { return Duo<0, TC8_N1>::BN; }
 
 cudaError_t launch_tc4_product_duo(const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1,
                                    const TcParams& p, int sms, cudaStream_t s) {
+    if (tile_columns(static_cast<int64_t>(p.m_tiles) * TC_BM, sms) == Duo<1, 0>::BN)
+        return launch_duo<1, 0>(a, b0, b0, p, sms, s);
     return launch_duo<1, TC4_N1>(a, b0, b1, p, sms, s);
 }
 
