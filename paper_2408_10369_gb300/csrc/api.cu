@@ -406,12 +406,15 @@ bmlp_status rms_f4_chain(bmlp_ctx* ctx, int64_t n_pad, uint8_t* const Q[2], uint
     return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "no fixpoint within %d products", max_iters);
 }
 
-bool thin_allowed(int64_t n_pad, const bmlp_options& o);
 // Whether the 4-bit squarings of a call are issued several at a time: sizes whose product is cheaper than a host wait
-// (n_pad = 4,096: 33 us), no squaring restricted to zeros among them, and no need of the host between two products (a
-// time budget is checked there, and options.profile times each).
-bool chain_allowed(int64_t n_pad, const bmlp_options& o) {
-    return n_pad <= 4096 && o.profile == 0 && o.budget_ns == 0 && !thin_allowed(n_pad, o);
+// (n_pad = 4,096: 33 us), or up to kChainMaxN those of a relation that was sparse enough for a bit-row start (a dense one
+// has one or two products left, and the last is cheaper restricted to zeros); and no need of the host between two products
+// (a time budget is checked there, and options.profile times each). In turn with restricted squarings, which the host
+// sizes, and issued together: n = 3,700 with 2 facts a row 413 and 266 us; 5,000: 493 and 444; power-law 4,600: 548 and
+// 438; 5,600: 737 and 626; 6,600: 901 and 800; uniform 6,600, 3 a row: 681 and 663; 5,000 with 500 a row: 235 and 252.
+constexpr int64_t kChainMaxN = 6656;
+bool chain_allowed(int64_t n_pad, const bmlp_options& o, bool sparse_start) {
+    return n_pad <= (sparse_start ? kChainMaxN : 4096) && o.profile == 0 && o.budget_ns == 0;
 }
 
 // Whether squarings on n_pad x n_pad 4-bit operands may run restricted to the rows and columns holding zeros.
@@ -1662,7 +1665,7 @@ static bmlp_status core_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt
             ST(to_e2m1(ctx, src, sfmt, sldw, n, M[1], T[1], n_pad, s));
             const uint8_t* q = nullptr;
             const uint64_t* qb = nullptr;
-            if (chain_allowed(n_pad, o)) {
+            if (chain_allowed(n_pad, o, sp.iters > 0)) {
                 // squarings of this size are issued several at a time, the decoding behind them
                 const size_t half = static_cast<size_t>(n_pad) * static_cast<size_t>(ld4);
                 const int64_t ldb = n_pad / 64;
@@ -1885,7 +1888,7 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
         // R1 as bit rows and its number of ones, read along with the closure's flags
         const int64_t ldx = n_pad / 64;
         uint64_t* const A1 = reinterpret_cast<uint64_t*>(X);
-        const bool bits_r1 = n >= kSparseMinN && !o.tc_only && o.e4m3_only == 0;
+        const bool bits_r1 = n > kAlwaysDenseN && !o.tc_only && o.e4m3_only == 0;
         if (bits_r1) {
             auto* const ones = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_BITS);
             CK(cudaMemsetAsync(ones, 0, sizeof(*ones), s), "reset count");
@@ -1961,11 +1964,19 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
             const uint8_t* q = M[1];  // the closure already, when the bit-row squarings reached it
             const uint64_t *qb = nullptr, *qbt = nullptr;
             st = BMLP_OK;
-            if (!sp.done && chain_allowed(n_pad, o)) {
+            if (!sp.done && chain_allowed(n_pad, o, sp.iters > 0)) {
                 uint8_t* const Q[2] = {M[1], M[1] + half};
                 uint8_t* const QT[2] = {T[1], T[1] + half};
                 int cur = 0;
-                st = rms_f4_chain(ctx, n_pad, Q, QT, nullptr, nullptr, max_iters - sp.iters, o, s, &iters, &cur,
+                uint64_t* P = nullptr;
+                if (bits_r1) {  // bit rows for the product by row ORs
+                    void* pp = nullptr;
+                    ST(ws_get(ctx, WS_THIN_P, static_cast<size_t>(2 * n_pad * ldx * 8), &pp));
+                    P = static_cast<uint64_t*>(pp);
+                    qb = P;
+                    qbt = P + n_pad * ldx;
+                }
+                st = rms_f4_chain(ctx, n_pad, Q, QT, P, const_cast<uint64_t*>(qbt), max_iters - sp.iters, o, s, &iters, &cur,
                                   []() { return BMLP_OK; });
                 q = Q[cur];
             } else if (!sp.done) {
