@@ -21,9 +21,10 @@
 //               tcgen05.mma.cta_group::2 kind::mxf4 of M=256, N=256 into TMEM
 //               columns 0..255 and one of M=256, N=224 into columns 256..479
 //               (in each CTA); the unit scale factors fill columns 480..511;
-//   warps 2..5  epilogue (both CTAs): loads the tile's old R while the MMAs
-//               run, drains the accumulator into registers as bits and frees
-//               it at once, then computes R' = R | [C > 0], writes R' and R'^T
+//   warps 2..9  epilogue (both CTAs), two warps per 32 rows, each half of the
+//               tile's columns: loads the tile's old R while the MMAs run,
+//               drains the accumulator into registers as bits and frees it at
+//               once, then computes R' = R | [C > 0], writes R' and R'^T
 //               (transposed in registers) and raises `changed` if R' != R.
 // Every mbarrier wait is bounded; on expiry the CTA records an error code,
 // waits (bounded) for its own copies and MMAs in flight, frees TMEM and exits.
@@ -39,6 +40,8 @@ constexpr int F4_BK = 128;                     // bytes of K per stage (256 elem
 constexpr int F4_UMMA_K_BYTES = 32;            // 64 E2M1 elements per MMA
 constexpr int F4_TMEM_COLS = 512;
 constexpr uint32_t F4_UE8M0_ONE4 = 0x7F7F7F7Fu;  // four UE8M0 scales of 2^0
+
+constexpr int DUO_THREADS = 320;
 
 constexpr int F4_GROUP_M = 8;  // raster: 8 row-block pairs share B tiles in L2
 
@@ -120,18 +123,23 @@ struct Duo {
     static constexpr int B1_BYTES = B1_ROWS * F4_BK;
     static constexpr int B_BYTES = B0_BYTES + B1_BYTES;
     static constexpr int STAGES = N1 ? 4 : 6;
-    static constexpr int CHUNKS = BN / 32;              // 32-column chunks of the epilogue
+    static constexpr int CHUNKS = (BN / 32 + 1) / 2;    // 32-column chunks of an epilogue warp (the second half of the
+                                                        // columns may have one less)
     static constexpr int SFA_COL = N1 ? 480 : 256;      // E2M1 scale factors (all 2^0; with N1 both operands
     static constexpr int SFB_COL = N1 ? 480 : 384;      // read the same filled columns)
     static constexpr int SF_FILL = N1 ? 32 : 0;         // N1: columns 480..511 hold 2^0 scales
     static constexpr int OFF_A = 0;
     static constexpr int OFF_B = OFF_A + STAGES * A_BYTES;
-    static constexpr int OFF_BAR = OFF_B + STAGES * B_BYTES;
-    static constexpr int NUM_BARS = 2 * STAGES + 3;     // full[], empty[], tfull, tempty, done
+    static constexpr int ROW_PITCH = CHUNKS | 1;        // words of a row of the epilogue's bits (odd: no bank conflicts)
+    static constexpr int OFF_ROWS = OFF_B + STAGES * B_BYTES;
+    static constexpr int OFF_COLS = OFF_ROWS + 2 * TC_BM * ROW_PITCH * 4;
+    static constexpr int OFF_BAR = OFF_COLS + 2 * CHUNKS * 32 * (TC_BM / 32) * 4;
+    static constexpr int NUM_BARS = 2 * STAGES + 7;     // full[], empty[], tfull, tempty, done, put[2], got[2]
     static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;
     static constexpr int SMEM_BYTES = OFF_MISC + 16 + 1024;
     static_assert(N1 == 0 || (N1 % 32 == 0 && N1 <= (KIND ? 224 : 256)), "second MMA width");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
+    static_assert(OFF_BAR % 16 == 0, "alignment");
     static_assert(B_BYTES % 1024 == 0 && A_BYTES % 1024 == 0, "swizzle atoms stay 1024-byte aligned");
 };
 
@@ -212,62 +220,95 @@ __device__ __forceinline__ void store_bits32(uint8_t* p, uint32_t bits) {
     }
 }
 
-// Epilogue, part 0: the old R of this thread's row of the pair tile as bits, CHUNKS x 32 columns from col_base on
-// (chunks at or beyond n_pad: zero). All loads are issued together, before the wait for the tile's accumulator: loaded
-// chunk by chunk after it, 15 dependent rounds to L2 made most of a small product's time (n_pad = 512: 18.1 us a
-// product, 11.6 us now; 2,048: 21.8 and 15.3 us; 5,120: 62 and 54 us).
-template <int KIND, int CHUNKS>
-__device__ __forceinline__ void f4_old(const TcParams& p, int64_t row, int64_t col_base, int64_t n_pad,
-                                       uint32_t (&ob)[CHUNKS]) {
+// The epilogue's accesses to R. A thread has a row of the tile (its TMEM lane), but a warp instruction that reads or writes
+// 16 bytes in each of 32 rows takes 32 steps of the load-store unit; with those a tile's epilogue took 10 k cycles after
+// its last MMA, and most of the time of a small product or of one over few K blocks. So the bits of a warp's 32 rows go
+// through shared memory: piece idx = 32 i + lane of them (32 columns of a row) is row idx / CHUNKS, and the lanes of an
+// instruction cover a few whole rows of the tile. The columns of R'^T are collected from four warps, 128 bits each. Eight
+// warps share the work since it then waits for instructions of one warp per scheduler (eight without the staging gained
+// nothing, four with it a third). A product, before and now: n_pad = 5,120 54.9 and 46.7 us; 7,680 147 and 132, its slice
+// over an eighth of K 52 and 42; 2,048 11.7 and 10.9; 32,768 7,760 and 7,700.
+// Part 0: the old R of this thread's row of the pair tile as bits, CHUNKS x 32 columns from col_base on (chunks at or beyond
+// column `end`: zero). row0: the warp's first row; rows: its 32 x ROW_PITCH words of shared memory. All loads are issued together,
+// before the wait for the tile's accumulator.
+template <int KIND, int CHUNKS, int PITCH>
+__device__ __forceinline__ void f4_old(const TcParams& p, int64_t row0, int64_t col_base, int64_t end, int lane,
+                                       uint32_t* rows, uint32_t (&ob)[CHUNKS]) {
     constexpr int CB = KIND ? 16 : 32;  // bytes of 32 columns
-    if (p.old_bits != nullptr) {
-        const uint32_t* bits = p.old_bits + row * p.ldb + col_base / 32;
-#pragma unroll
-        for (int c = 0; c < CHUNKS; ++c) ob[c] = col_base + c * 32 < n_pad ? bits[c] : 0u;
-        return;
-    }
-    if (p.old_r == nullptr) {
+    if (p.old_bits == nullptr && p.old_r == nullptr) {
 #pragma unroll
         for (int c = 0; c < CHUNKS; ++c) ob[c] = 0u;
         return;
     }
-    const uint8_t* src = p.old_r + row * p.ld + col_base / 32 * CB;
 #pragma unroll
-    for (int c = 0; c < CHUNKS; ++c) ob[c] = col_base + c * 32 < n_pad ? load_bits32<KIND>(src + c * CB) : 0u;
+    for (int i = 0; i < CHUNKS; ++i) {
+        const int idx = i * 32 + lane, r = idx / CHUNKS, c = idx % CHUNKS;
+        ob[i] = 0u;
+        if (col_base + c * 32 < end)
+            ob[i] = p.old_bits != nullptr ? p.old_bits[(row0 + r) * p.ldb + col_base / 32 + c]
+                                          : load_bits32<KIND>(p.old_r + (row0 + r) * p.ld + (col_base / 32 + c) * CB);
+    }
+    __syncwarp();  // the rows of the tile before have been read
+#pragma unroll
+    for (int i = 0; i < CHUNKS; ++i) rows[((i * 32 + lane) / CHUNKS) * PITCH + (i * 32 + lane) % CHUNKS] = ob[i];
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < CHUNKS; ++c) ob[c] = rows[lane * PITCH + c];
 }
 
-// Epilogue, part 2: R' = R | C for row (mb, quarter, lane) of the pair tile
-// whose first column is col_base: writes R' and, through a 32 x 32 bit
-// transpose in registers, R'^T for every 32-column chunk below n_pad; returns
-// the bits that changed (nonzero in some lane iff R' != R in this warp's rows).
-template <int KIND, int CHUNKS>
-__device__ __forceinline__ uint32_t f4_update(const TcParams& p, int mb, int64_t col_base, int64_t n_pad, int quarter,
-                                              int lane, const uint32_t (&ob)[CHUNKS], const uint32_t (&cb)[CHUNKS]) {
-    constexpr int CB = KIND ? 16 : 32;  // bytes of 32 columns
-    const int64_t row = static_cast<int64_t>(mb) * TC_BM + quarter * 32 + lane;
-    // byte of this warp's 32 rows inside a row of R'^T
-    const int64_t rt_col = (static_cast<int64_t>(mb) * TC_BM + quarter * 32) / 32 * CB;
+// Part 2: R' = R | C for the warp's 32 rows: their bits into `rows`, their transposed bits (column 32 c + lane, word
+// `quarter`) into `cols`, and R' from there to global memory. Returns the bits that changed (nonzero in some lane iff
+// R' != R in this warp's rows).
+template <int KIND, int CHUNKS, int PITCH>
+__device__ __forceinline__ uint32_t f4_update(const TcParams& p, int64_t row0, int64_t col_base, int64_t end, int quarter,
+                                              int lane, uint32_t* rows, uint32_t* cols, const uint32_t (&ob)[CHUNKS],
+                                              const uint32_t (&cb)[CHUNKS]) {
+    constexpr int CB = KIND ? 16 : 32;
     uint32_t any = 0;
+    __syncwarp();  // every lane has its old bits
 #pragma unroll
     for (int c = 0; c < CHUNKS; ++c) {
-        const int64_t col0 = col_base + c * 32;
-        if (col0 < n_pad) {
-            const uint32_t nbits = ob[c] | cb[c];
-            any |= nbits ^ ob[c];
-            if (p.out_r != nullptr) store_bits32<KIND>(p.out_r + row * p.ld + col0 / 32 * CB, nbits);
-            if (p.out_bits != nullptr) p.out_bits[row * p.ldb + col0 / 32] = nbits;
-            const uint32_t mine = warp_transpose32(nbits, lane);  // column col0 + lane of the warp's 32 rows
-            if (p.out_r != nullptr) store_bits32<KIND>(p.out_rt + (col0 + lane) * p.ld + rt_col, mine);
-            if (p.out_bits_t != nullptr) p.out_bits_t[(col0 + lane) * p.ldb + rt_col / CB] = mine;
+        const bool in = col_base + c * 32 < end;
+        const uint32_t nbits = in ? ob[c] | cb[c] : 0u;
+        any |= in ? nbits ^ ob[c] : 0u;
+        rows[lane * PITCH + c] = nbits;
+        cols[(c * 32 + lane) * 4 + quarter] = warp_transpose32(nbits, lane);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < CHUNKS; ++i) {
+        const int idx = i * 32 + lane, r = idx / CHUNKS, c = idx % CHUNKS;
+        if (col_base + c * 32 < end) {
+            const uint32_t w = rows[r * PITCH + c];
+            if (p.out_r != nullptr) store_bits32<KIND>(p.out_r + (row0 + r) * p.ld + (col_base / 32 + c) * CB, w);
+            if (p.out_bits != nullptr) p.out_bits[(row0 + r) * p.ldb + col_base / 32 + c] = w;
         }
     }
     return any;
 }
 
+// Part 3, when all four warps of a half have put their columns: R'^T of it, thread t of 128 (four threads a column).
+template <int KIND, int CHUNKS>
+__device__ __forceinline__ void f4_columns(const TcParams& p, int mb, int64_t col_base, int64_t end, int t,
+                                           const uint32_t* cols) {
+    constexpr int CB = KIND ? 16 : 32;
+    if (p.out_r == nullptr && p.out_bits_t == nullptr) return;
+#pragma unroll
+    for (int i = 0; i < CHUNKS; ++i) {
+        const int idx = i * 128 + t;
+        const int64_t col = col_base + (idx >> 2), word = static_cast<int64_t>(mb) * (TC_BM / 32) + (idx & 3);
+        if (col < end) {
+            const uint32_t w = cols[idx];
+            if (p.out_r != nullptr) store_bits32<KIND>(p.out_rt + col * p.ld + word * CB, w);
+            if (p.out_bits_t != nullptr) p.out_bits_t[col * p.ldb + word] = w;
+        }
+    }
+}
+
 // tmA: A = R (box 128 rows x 128 bytes); tmB0 / tmB1: B^T = R^T (boxes of
 // B0_ROWS / B1_ROWS rows x 128 bytes; tmB1 unused when N1 = 0).
 template <int KIND, int N1>
-__global__ void __launch_bounds__(TC_THREADS, 1) __cluster_dims__(2, 1, 1)
+__global__ void __launch_bounds__(DUO_THREADS, 1) __cluster_dims__(2, 1, 1)
 tc_duo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                const __grid_constant__ CUtensorMap tmB1, const TcParams p) {
     using C = Duo<KIND, N1>;
@@ -284,6 +325,8 @@ tc_duo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     uint64_t* tfull = bars + 2 * C::STAGES; // each CTA: the accumulator holds a finished tile
     uint64_t* tempty = tfull + 1;           // even CTA: both CTAs' epilogues drained the accumulator
     uint64_t* done = tempty + 1;            // even CTA: every MMA it issued has completed
+    uint64_t* put = done + 1;               // each CTA, each half of the columns: its four warps have put a tile's columns
+    uint64_t* got = put + 2;                // and have read them
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
 
@@ -306,8 +349,12 @@ tc_duo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             mbar_init(&empty[s], 1);
         }
         mbar_init(tfull, 1);
-        mbar_init(tempty, 256);
+        mbar_init(tempty, 512);
         mbar_init(done, 1);
+        for (int h = 0; h < 2; ++h) {
+            mbar_init(&put[h], 4);
+            mbar_init(&got[h], 4);
+        }
         *abort_flag = 0;
         fence_mbar_init();
     }
@@ -319,7 +366,7 @@ tc_duo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    if (KIND == 1 && warp >= 2) {
+    if (KIND == 1 && warp >= 2 && warp < 6) {
         // every scale factor of A and B is 2^0, in all 128 lanes of this CTA
         const uint32_t lanes = static_cast<uint32_t>((warp & 3) * 32) << 16;
         const uint32_t ones[8] = {F4_UE8M0_ONE4, F4_UE8M0_ONE4, F4_UE8M0_ONE4, F4_UE8M0_ONE4,
@@ -462,29 +509,49 @@ tc_duo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         const int quarter = warp & 3;
         const uint32_t lanes = static_cast<uint32_t>(quarter * 32) << 16;
         const uint32_t tempty_even = mapa_shared(smem_u32(tempty), 0);
+        const int half = warp < 6 ? 0 : 1, off = half * C::CHUNKS * 32;  // this warp's first column of the tile
+        uint32_t* rows = reinterpret_cast<uint32_t*>(smem + C::OFF_ROWS) + (warp - 2) * 32 * C::ROW_PITCH;
+        uint32_t* cols = reinterpret_cast<uint32_t*>(smem + C::OFF_COLS) + off * (TC_BM / 32);
         uint32_t acc_phase = 0;
         for (int t = first; t < num_pairs; t += step) {
             int mp, nb;
             f4_pair_coords(t, m_pairs, p.n_tiles, mp, nb);
             const int mb = 2 * mp + static_cast<int>(rank);
+            const int64_t row0 = static_cast<int64_t>(mb) * TC_BM + quarter * 32;
+            const int64_t col = static_cast<int64_t>(nb) * C::BN + off, next = static_cast<int64_t>(nb + 1) * C::BN;
+            const int64_t end = next < n_pad ? next : n_pad;
             uint32_t ob[C::CHUNKS];
-            f4_old<KIND, C::CHUNKS>(p, static_cast<int64_t>(mb) * TC_BM + quarter * 32 + lane,
-                                    static_cast<int64_t>(nb) * C::BN, n_pad, ob);
+            f4_old<KIND, C::CHUNKS, C::ROW_PITCH>(p, row0, col, end, lane, rows, ob);
             if (!f4_wait_lane0(tfull, acc_phase, abort_flag, limit, lane)) {
                 if (lane == 0) atomicCAS(p.error, 0, ERR_D_EPILOGUE);
                 break;
             }
             tc_fence_after();
             // drain C > 0 into registers, then free the accumulator for the next tile's MMAs (columns of a
-            // tile that got no second MMA hold stale counts; f4_update stops before them)
+            // tile that got no second MMA hold stale counts, those behind an odd number of chunks the scale factors;
+            // f4_update stops before them)
             uint32_t cb[C::CHUNKS];
-            f4_drain<C::CHUNKS>(tmem_base + lanes, cb);
+            f4_drain<C::CHUNKS>(tmem_base + lanes + static_cast<uint32_t>(off), cb);
             tc_fence_before();
             mbar_arrive_cluster(tempty_even);
-            acc_phase ^= 1u;
+            // the columns of the tile before have been read (the first wait, of the other parity, returns at once)
+            if (!f4_wait_lane0(&got[half], acc_phase ^ 1u, abort_flag, limit, lane)) {
+                if (lane == 0) atomicCAS(p.error, 0, ERR_D_EPILOGUE);
+                break;
+            }
             const uint32_t any =
-                f4_update<KIND, C::CHUNKS>(p, mb, static_cast<int64_t>(nb) * C::BN, n_pad, quarter, lane, ob, cb);
+                f4_update<KIND, C::CHUNKS, C::ROW_PITCH>(p, row0, col, end, quarter, lane, rows, cols, ob, cb);
             if (__any_sync(0xFFFFFFFFu, any != 0) && lane == 0) atomicOr(p.changed, 1);
+            if (lane == 0) mbar_arrive(&put[half]);
+            if (!f4_wait_lane0(&put[half], acc_phase, abort_flag, limit, lane)) {
+                if (lane == 0) atomicCAS(p.error, 0, ERR_D_EPILOGUE);
+                break;
+            }
+            __syncwarp();
+            f4_columns<KIND, C::CHUNKS>(p, mb, col, end, quarter * 32 + lane, cols);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&got[half]);
+            acc_phase ^= 1u;
         }
     }
 
@@ -553,15 +620,15 @@ cudaError_t launch_duo(const CUtensorMap& a, const CUtensorMap& b0, const CUtens
     int clusters = sms / 2;
     if (clusters > pairs) clusters = pairs;
     if (clusters < 1) clusters = 1;
-    tc_duo_kernel<KIND, N1><<<2 * clusters, TC_THREADS, Duo<KIND, N1>::SMEM_BYTES, s>>>(a, b0, b1, p);
+    tc_duo_kernel<KIND, N1><<<2 * clusters, DUO_THREADS, Duo<KIND, N1>::SMEM_BYTES, s>>>(a, b0, b1, p);
     return cudaGetLastError();
 }
 
 // Columns of a pair tile. Up to about n_pad = 4,000 a product takes as long as its rounds of tiles over the SM pairs, and a
 // round of 256-column tiles has half the MMAs and half the epilogue of one of 480-column tiles: 256 where that takes fewer
 // than 1.55 times the rounds (for large n the ratio of their times per tile, 1.875 x 7.33 / 8.88). A product of uniform
-// random relations, 480 and 256 columns: n_pad = 1,280: 14.1 and 10.5 us; 2,048: 15.8 and 11.7; 2,304 (1 and 2 rounds): 17.0
-// and 18.4; 3,072 (2 and 2): 31.5 and 21.2; 3,840 (2 and 3): 30.9 and 28.4.
+// random relations, 480 and 256 columns: n_pad = 2,048 (1 round each): 14.6 and 10.9 us; 3,072 (2 and 2): 25.3 and 18.6;
+// 3,840 (2 and 3): 28.7 and 27.5; 2,304 (1 and 2; with the epilogue before) 17.0 and 18.4.
 static int tile_columns(int64_t n_pad, int sms) {
     const int64_t m_pairs = n_pad / (2 * TC_BM), pairs = sms / 2 > 0 ? sms / 2 : 1;
     const auto rounds = [&](int64_t bn) { return (m_pairs * ((n_pad + bn - 1) / bn) + pairs - 1) / pairs; };
