@@ -205,7 +205,8 @@ bmlp_status bmlp_get_stats(const bmlp_ctx* ctx, bmlp_stats* out);
  * see options.tc_only; then tensor cores), BMLP_RMS_PACKED, BMLP_SMP_PACKED
  * (all n rows as frontiers: path-like R is squared first and expanded one
  * row per warp, R whose rows widen fast is expanded up to 64 rows per CTA), BMLP_SMP_TC,
- * BMLP_AUTO (the learned dispatcher once trained or loaded, else BMLP_RMS_TC).
+ * BMLP_AUTO (the learned dispatcher once trained or loaded, else BMLP_RMS_TC;
+ * where that is the choice and n <= 1024, one launch on bit rows).
  */
 bmlp_status bmlp_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt, void* out,
                      const bmlp_options* opts, int32_t* iters_out, cudaStream_t stream);
@@ -220,8 +221,7 @@ bmlp_status bmlp_rms(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt, void*
  * last product). *iters_out receives the squarings plus 1: ceil(log2 L0) + 2,
  * with L0 the longest shortest path between two different constants (2 when
  * L0 <= 1). The squarings run as bmlp_rms with BMLP_RMS_TC (bit-row start,
- * operand forms, options.tc_only), the final product on the tensor cores
- * with E4M3 operands. Variants: BMLP_RMS_TC or BMLP_AUTO (the same). R and
+ * operand forms, options.tc_only), the final product on the tensor cores. Variants: BMLP_RMS_TC or BMLP_AUTO (the same). R and
  * out as in bmlp_rms; options.reflexive gives I + R1+.
  */
 bmlp_status bmlp_rms_alg1(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt, void* out,
@@ -251,8 +251,9 @@ bmlp_status bmlp_smp(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt,
  * setting of paper Sec. 7): given closure = R1+ (any transitive relation,
  * e.g. the output of bmlp_rms), add the facts r1(u_k, v_k) of `pairs` (m
  * pairs of int32 constants, device or host memory) and update closure in
- * place to (R1 + E)+. Each fact is one rank-1 update: every constant that
- * reaches u_k (and u_k) gains v_k and everything v_k reaches. closure is
+ * place to (R1 + E)+. Each fact is a rank-1 update: every constant that
+ * reaches u_k (and u_k) gains v_k and everything v_k reaches; three or more
+ * facts are taken together, up to 1,024 a pass over the rows. closure is
  * n x n in format fmt (device or host memory). Facts already derivable cost
  * one word read. Constants outside [0, n) give BMLP_ERR_INVALID_ARG before
  * anything changes. Deleting facts is not incremental: recompute with
@@ -382,8 +383,8 @@ typedef struct bmlp_problem {
  * count is the deepest level + 1.
  * Problems large enough to fill the GPU alone (n >= 4096 by default, the
  * environment variable BMLP_BATCH_SOLO_N changes it, 0 = never) that are not
- * forced onto packed rows run in the same graph, one after another, as
- * device-driven single-problem pipelines: squarings on word-indexed bit rows
+ * forced onto packed rows run in the same graph, on up to four parallel
+ * branches, as device-driven single-problem pipelines: squarings on word-indexed bit rows
  * while the next one is predicted cheaper than a tensor-core product (a
  * one-thread decision kernel sets the condition of a WHILE node), then
  * squarings on packed E2M1 operands on the tensor cores (a second WHILE

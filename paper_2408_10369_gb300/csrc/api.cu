@@ -422,10 +422,10 @@ bool thin_allowed(int64_t n_pad, const bmlp_options& o) {
     return !o.tc_only && thin_enabled() && thin_fixed_s(n_pad) < tc4_product_s(n_pad);
 }
 
-// Whether a call by the tensor-core variant runs as one launch on bit rows: small relations whose call asks for nothing that
-// needs the tensor cores or the host between two products.
+// Whether a call runs as one launch on bit rows: small relations, no variant named (BMLP_RMS_TC asked for by name stays on
+// the tensor cores), and nothing that needs those or the host between two products.
 bool small_allowed(int64_t n, const bmlp_options& o) {
-    return n <= kSmallN && !o.tc_only && o.e4m3_only == 0 && o.profile == 0 && o.budget_ns == 0;
+    return o.variant == BMLP_AUTO && n <= kSmallN && !o.tc_only && o.e4m3_only == 0 && o.profile == 0 && o.budget_ns == 0;
 }
 
 // The closure of `in`, or with r1 the composition (I + in+) r1, by that launch.

@@ -50,12 +50,14 @@ def test_closures(ctx, n, fmt):
         L = oracle.longest_shortest_path(n, *csr)
         for reflexive in (False, True):
             R = operand(n, csr, fmt)
-            it = ctx.rms(R, n, R, fmt=FMT[fmt], variant="rms_tc", reflexive=reflexive)  # in place
+            it = ctx.rms(R, n, R, fmt=FMT[fmt], reflexive=reflexive)  # in place
             ref = want.copy()
             if reflexive:
                 np.fill_diagonal(ref, 1)
             np.testing.assert_array_equal(bits(R, n, fmt), ref)
-            assert it == oracle.rms_iterations(L) == ctx.stats()["product_launches"]
+            st = ctx.stats()
+            assert it == oracle.rms_iterations(L) == st["product_launches"]
+            assert st["e2m1_products"] == (0 if n <= 1024 else it)
 
 
 @pytest.mark.parametrize("n", [1, 40, 257, 640, 1024])
@@ -77,7 +79,7 @@ def test_limits(ctx):
     R, out = operand(n, csr, "u8"), torch.zeros((n, n), dtype=torch.uint8, device="cuda")
     for kwargs, status in (({"max_iters": 3}, bmlp.BMLP_ERR_NOT_CONVERGED), ({"timeout_ns": 1}, bmlp.BMLP_ERR_TIMEOUT)):
         with pytest.raises(bmlp.BmlpError) as e:
-            ctx.rms(R, n, out, variant="rms_tc", **kwargs)
+            ctx.rms(R, n, out, **kwargs)
         assert e.value.status == status
-        assert ctx.rms(R, n, out, variant="rms_tc") == oracle.rms_iterations(n - 1)
+        assert ctx.rms(R, n, out) == oracle.rms_iterations(n - 1)
         np.testing.assert_array_equal(out.cpu().numpy(), oracle.closure(n, *csr))
