@@ -2,20 +2,21 @@
 // sizes (closures, paper Sec. 3.3 program P2, and two-relation compositions,
 // Sec. 3.4 Thm. 1) evaluated together.
 //
-// Per iteration, ONE persistent tensor-core launch (tc_group_kernel) runs the
-// squaring step R <- R + R R of every unconverged tensor-core problem over a
-// device work list of (problem, tile) items, and one packed launch does the
-// same for the problems the autotuner put on packed rows. A single-block
-// planner then retires problems whose changed flag stayed 0 (or that reached
-// their cap), flips the ping-pong parity of the others, rebuilds both work
-// lists and sets the condition of the CUDA graph WHILE node that holds the
-// iteration. Encoding, the iteration, the final products of compositions and
-// decoding are one graph launch; the host reads back the per-problem
-// iteration counts once at the end.
+// Two CUDA graph WHILE nodes hold the squaring steps R <- R + R R. In the
+// first ONE launch per iteration (packed_group_kernel) squares, on bit rows,
+// the problems that the autotuner put there and every other one for as long as
+// that is cheaper than its share of a grouped tensor-core product; in the
+// second ONE persistent tensor-core launch (tc_group_kernel) squares the
+// problems handed over, over a device work list of (problem, tile) items. A
+// single-block planner after each retires problems whose changed flag stayed 0
+// (or that reached their cap), flips the ping-pong parity of the others,
+// rebuilds the work lists and sets the node's condition. Encoding, the
+// iterations, the final products of compositions and decoding are one graph
+// launch; the host reads back the per-problem iteration counts once at the end.
 //
 // Problems large enough to fill the GPU on their own (n >= solo_n) run in the
-// same graph as device-driven single-problem pipelines, one after another:
-// squarings on word-indexed bit rows while the next one costs less than a
+// same graph as device-driven single-problem pipelines, on up to four
+// parallel branches: squarings on word-indexed bit rows while the next one costs less than a
 // tensor-core product (the same cost model and the same switch as the
 // single-problem path, decided by a one-thread kernel that sets the
 // condition of a WHILE node), then squarings on packed E2M1 operands on the
@@ -149,8 +150,8 @@ __device__ __forceinline__ bool rows_cheaper(const GroupProblem& g, unsigned lon
 // product (1 and 4: retire, flip parity, count; 1 also hands over); mode 2: final products of compositions.
 __global__ void __launch_bounds__(1024) batch_plan_kernel(const GroupProblem* probs, const GroupState* st, int nprob,
                                                           int mode, cudaGraphConditionalHandle h, int set_cond) {
-    __shared__ int part_tc[1024], part_pk[1024];
-    const int t = threadIdx.x;
+    __shared__ unsigned long long warp_sum[32];
+    const int t = threadIdx.x, lane = t & 31;
     const int per = (nprob + 1023) / 1024;
     const int a = t * per, b = min(a + per, nprob);
     int stc = 0, spk = 0;
@@ -198,18 +199,29 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(const GroupProblem* pr
         stc += ctc;
         spk += cpk;
     }
-    part_tc[t] = stc;
-    part_pk[t] = spk;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const int vt = t >= off ? part_tc[t - off] : 0;
-        const int vp = t >= off ? part_pk[t - off] : 0;
-        __syncthreads();
-        part_tc[t] += vt;
-        part_pk[t] += vp;
-        __syncthreads();
+    // exclusive prefixes over the threads, both at once (each total is below 2^31): in registers, since the plan runs between
+    // any two steps of all problems and a scan through shared memory with its twenty barriers was a third of its 5 us
+    const unsigned long long mine = (static_cast<unsigned long long>(stc) << 32) | static_cast<unsigned>(spk);
+    unsigned long long incl = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const unsigned long long v = __shfl_up_sync(FULL, incl, off);
+        if (lane >= off) incl += v;
     }
-    int rt = t > 0 ? part_tc[t - 1] : 0, rp = t > 0 ? part_pk[t - 1] : 0;
+    if (lane == 31) warp_sum[t >> 5] = incl;
+    __syncthreads();
+    if (t < 32) {
+        unsigned long long w = warp_sum[lane];
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned long long v = __shfl_up_sync(FULL, w, off);
+            if (lane >= off) w += v;
+        }
+        warp_sum[lane] = w;
+    }
+    __syncthreads();
+    const unsigned long long before = incl - mine + (t >= 32 ? warp_sum[(t >> 5) - 1] : 0ull);
+    int rt = static_cast<int>(before >> 32), rp = static_cast<int>(before & 0xFFFFFFFFull);
     for (int p = a; p < b; ++p) {
         const int ct = st->tc_offs[p], cp = st->pk_offs[p];
         st->tc_offs[p] = rt;
@@ -218,7 +230,7 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(const GroupProblem* pr
         rp += cp;
     }
     if (t == 0) {
-        const int tt = part_tc[1023], tp = part_pk[1023];
+        const int tt = static_cast<int>(warp_sum[31] >> 32), tp = static_cast<int>(warp_sum[31] & 0xFFFFFFFFull);
         st->tc_offs[nprob] = tt;
         st->pk_offs[nprob] = tp;
         *st->tc_total = tt;
@@ -229,30 +241,44 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(const GroupProblem* pr
 
 // ------------------------------------------------ packed squaring step --
 // C_i = A_i' | OR_{k : A_ik = 1} B_k for one row, by a whole warp (A_i' = init, a row of ldw words), in chunks of 64 words
-// (two per lane), four named rows in flight. Returns the ones written; *grew: C_i != init.
+// (two per lane), four named rows in flight. A row of up to 16 or 32 words takes a quarter or half of the lanes, so the
+// warp's groups of 8 or 16 take its nonzero words in turn (a batch of 1,000 entities: six launches of 226 us in all, 128 now;
+// the batch 594 and 494 us). Returns the ones written; *grew: C_i != init.
 __device__ __forceinline__ unsigned gather_row(const uint64_t* __restrict__ arow, const uint64_t* __restrict__ B,
                                                const uint64_t* __restrict__ init, uint64_t* __restrict__ out, int64_t ldw,
                                                int lane, bool* grew) {
     unsigned ones = 0;
     uint32_t any = 0;
+    const int gs = ldw <= 16 ? 8 : ldw <= 32 ? 16 : 32, groups = 32 / gs, group = lane / gs;
     for (int64_t c0 = 0; c0 < ldw; c0 += 64) {
-        const int64_t w = c0 + 2 * lane;
+        const int64_t w = c0 + 2 * (lane & (gs - 1));
         const bool in = w < ldw;  // ldw is even: both words
         const uint4 old = in ? *reinterpret_cast<const uint4*>(init + w) : make_uint4(0, 0, 0, 0);
         uint4 acc = old;
         for (int64_t wb = 0; wb < ldw; wb += 32) {
             const uint64_t aw = wb + lane < ldw ? arow[wb + lane] : 0ull;
             unsigned m = __ballot_sync(FULL, aw != 0ull);
+            if (groups > 1) {  // this group's share of the nonzero words (at most 32 words: one pass)
+                const int turn = __popc(m & ((1u << lane) - 1u)) & (groups - 1);
+                unsigned share = 0;
+                for (int q = 0; q < groups; ++q) {
+                    const unsigned x = __ballot_sync(FULL, aw != 0ull && turn == q);
+                    if (q == group) share = x;
+                }
+                m = share;
+            }
             uint64_t bits = 0ull;
             int64_t kb = 0;
-            while (m != 0u || bits != 0ull) {
+            while (__any_sync(FULL, m != 0u || bits != 0ull)) {
                 uint4 x[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    if (bits == 0ull && m != 0u) {
-                        const int sl = __ffs(m) - 1;
+                    const bool word = bits == 0ull && m != 0u;
+                    const int sl = word ? __ffs(static_cast<int>(m)) - 1 : 0;
+                    const uint64_t next = __shfl_sync(FULL, aw, sl);
+                    if (word) {
                         m &= m - 1u;
-                        bits = __shfl_sync(FULL, aw, sl);
+                        bits = next;
                         kb = (wb + sl) * 64;
                     }
                     x[q] = make_uint4(0, 0, 0, 0);
@@ -271,9 +297,17 @@ __device__ __forceinline__ unsigned gather_row(const uint64_t* __restrict__ arow
                 }
             }
         }
-        if (in) *reinterpret_cast<uint4*>(out + w) = acc;
-        any |= (old.x ^ acc.x) | (old.y ^ acc.y) | (old.z ^ acc.z) | (old.w ^ acc.w);
-        ones += __popc(acc.x) + __popc(acc.y) + __popc(acc.z) + __popc(acc.w);
+        for (int off = gs; off < 32; off <<= 1) {
+            acc.x |= __shfl_xor_sync(FULL, acc.x, off);
+            acc.y |= __shfl_xor_sync(FULL, acc.y, off);
+            acc.z |= __shfl_xor_sync(FULL, acc.z, off);
+            acc.w |= __shfl_xor_sync(FULL, acc.w, off);
+        }
+        if (in && group == 0) {
+            *reinterpret_cast<uint4*>(out + w) = acc;
+            any |= (old.x ^ acc.x) | (old.y ^ acc.y) | (old.z ^ acc.z) | (old.w ^ acc.w);
+            ones += __popc(acc.x) + __popc(acc.y) + __popc(acc.z) + __popc(acc.w);
+        }
     }
     *grew = __any_sync(FULL, any != 0u) != 0;
     return __reduce_add_sync(FULL, ones);
@@ -1205,9 +1239,9 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
                 launch_e2m1_to_packed(Q[0], ld4, n, static_cast<uint64_t*>(p.out), (n + 63) / 64, p.reflexive, cs);
             }
         } else {
-            // out = (I + R2+) R1 on 4-bit operands, on the squaring kernel: A = I + R2+ (Q[0], diagonal set),
-            // B^T = R1^T (encoded with R1 into the free pair Q[1], QT[1]), and a zero "old R" (QT[0]), so that the
-            // kernel's R' is C > 0; R' goes to Q[1] (R1 is no longer needed), R'^T to the scratch
+            // out = (I + R2+) R1 on 4-bit operands, on the squaring kernel without an old R: A = I + R2+ (Q[0], diagonal
+            // set), B^T = R1^T (encoded with R1 into the free pair Q[1], QT[1]); R' = C > 0 goes to Q[1] (R1 is no longer
+            // needed), R'^T to the scratch
             launch_set_diag_e2m1(Q[0], ld4, n, cs);
             if (p.fmt == BMLP_FMT_U8) {
                 launch_u8_to_packed(static_cast<const uint8_t*>(p.R1), n, P0, ldw, cs);
@@ -1215,7 +1249,6 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
             } else {
                 launch_packed_to_e2m1(static_cast<const uint64_t*>(p.R1), (n + 63) / 64, n, Q[1], QT[1], n_pad, cs);
             }
-            SCK(cudaMemsetAsync(QT[0], 0, static_cast<size_t>(n_pad) * static_cast<size_t>(ld4), cs), "clear old R");
             CUtensorMap fa, fb0, fb1;
             SST(make_tmap(ctx, &fa, Q[0], n_pad, ld4, ld4, TC_BM));
             SST(make_tmap(ctx, &fb0, QT[1], n_pad, ld4, ld4, TC_BN / 2));
@@ -1226,7 +1259,6 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
             pp.k_blocks = static_cast<int32_t>(n_pad / 256);
             pp.mode = TC_MODE_RMS;
             pp.ld = ld4;
-            pp.old_r = QT[0];
             pp.out_r = Q[1];
             pp.out_rt = M0;
             pp.changed = w + SW_CHANGED;
@@ -1252,7 +1284,8 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
 // Branches of the batch graph that the large problems are dealt out to, besides the branch of the grouped ones. A
 // pipeline is a chain of small launches (bit-row squarings, decisions) between tensor-core products that fill the GPU, so
 // several chains at once fill each other's gaps (measured on the knowledge-graph batch, 33 closures and 8 compositions
-// with n >= 4,096: 37.4 ms on one branch, 32.2 on two, 30.4 on four, 30.4 on twelve). More lanes than that add scratch (at most kLaneBytes in all, else fewer lanes).
+// with n >= 4,096: 37.4 ms on one branch, 32.2 on two, 30.4 on four, 30.4 on twelve). More lanes than that add scratch
+// (at most kLaneBytes in all, else fewer lanes).
 constexpr int kLanes = 4;
 constexpr size_t kLaneBytes = size_t(24) << 30;
 
