@@ -480,11 +480,19 @@ __device__ __forceinline__ void or_word(uint64_t* N, int64_t x, uint64_t v) {
     if (hi) atomicOr(at + 1, hi);
 }
 
+// The same, and grew = 1 if N[x] lacks one of the bits: looked at until this lane has found one. (A bit that is missing when
+// it is looked for was missing from the start, and whoever finds it missing sets it, so the answers of all lanes together
+// say whether a word grew.)
+__device__ __forceinline__ void or_grow(uint64_t* N, int64_t x, uint64_t v, uint64_t& grew) {
+    if (grew == 0ull && (v & ~N[x]) != 0ull) grew = 1ull;
+    or_word(N, x, v);
+}
+
 // Rows of up to NQ frontier constants per lane (k < 0: none) ORed into N:
 // their nonzero words, by shared-memory atomics without return value. The row
 // ranges and the first four entries of every light row (<= kLightRow nonzero words)
 // are loaded before the first atomic; heavy rows are walked by the whole warp, four entries a lane in flight.
-// tm collects the word groups written (bit x >> gshift for word x) unless the caller has no use for them.
+// tm collects the word groups written (bit x >> gshift for word x), or without kGroups whether a word grew (1).
 constexpr int kLightRow = 16;
 template <int NQ, bool kGroups = true>
 __device__ __forceinline__ void push_rows(const int (&k)[NQ], int lane, const int64_t* __restrict__ wptr,
@@ -511,8 +519,12 @@ __device__ __forceinline__ void push_rows(const int (&k)[NQ], int lane, const in
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             if (y[j] >= 0) {
-                or_word(N, y[j], yv[j]);
-                if (kGroups) tm |= 1ull << (y[j] >> gshift);
+                if (kGroups) {
+                    or_word(N, y[j], yv[j]);
+                    tm |= 1ull << (y[j] >> gshift);
+                } else {
+                    or_grow(N, y[j], yv[j], tm);
+                }
             }
     };
     int x[NQ][4];
@@ -530,8 +542,12 @@ __device__ __forceinline__ void push_rows(const int (&k)[NQ], int lane, const in
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             if (x[q][j] >= 0) {
-                or_word(N, x[q][j], val[q][j]);
-                if (kGroups) tm |= 1ull << (x[q][j] >> gshift);
+                if (kGroups) {
+                    or_word(N, x[q][j], val[q][j]);
+                    tm |= 1ull << (x[q][j] >> gshift);
+                } else {
+                    or_grow(N, x[q][j], val[q][j], tm);
+                }
             }
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
@@ -1074,21 +1090,27 @@ __device__ __forceinline__ void sync_row(bool together) {
 // squaring step. The row is assembled in shared memory (ldw words per warp). The kernel waits for L2 (a range, then its
 // words, at random), so it is as fast as it has loads in flight: 32-bit lengths and one named row a lane at a time leave 48
 // registers and five blocks an SM (n = 14,000, 1.5 entries a row, the four products of a closure: 801 us with two rows a
-// lane, 64 registers and 64-bit shared-memory atomics; 602, 563 and 535 us at four, five and six blocks, of which the last
-// spills and loses on power-law relations). *changed (or null) is raised when C_i != P_i.
+// lane, 64 registers and 64-bit shared-memory atomics, 532 now; six blocks spill and lose on power-law relations). *changed (or null) is raised when C_i != P_i.
 __global__ void __launch_bounds__(256, 5) indexed_rows_kernel(const WordIndex A, const WordIndex B,
                                                            const uint64_t* __restrict__ P, int64_t n, int64_t ldw,
                                                            uint64_t* __restrict__ C, int* __restrict__ changed) {
-    extern __shared__ uint64_t sq_sm[];
+    extern __shared__ __align__(16) uint64_t sq_sm[];
     const int lane = threadIdx.x & 31;
-    bool grew = false;
+    uint64_t tm = 0;  // whether a row grew
     rows_of_index(A, n, [&](int64_t i, const longlong2& range, bool together) {
         const int nw = together ? blockDim.x >> 5 : 1, warp = threadIdx.x >> 5;  // together: the warps take entries in turn
         const int first = together ? threadIdx.x : lane, step = 32 * nw;
         uint64_t* S = together ? sq_sm : sq_sm + warp * ldw;
-        for (int64_t w = first; w < ldw; w += step) S[w] = P[i * ldw + w];
+        // the row in 16-byte pieces (ldw is even) by asynchronous copies, all in flight without registers: one word at a time
+        // through them a row of few entries took twice the time of its bytes (n = 32,768, 4 entries a row, 268 MB: 99 us,
+        // 52 now)
+        const ulonglong2* Pi = reinterpret_cast<const ulonglong2*>(P + i * ldw);
+        ulonglong2* Si = reinterpret_cast<ulonglong2*>(S);
+        const int pieces = static_cast<int>(ldw >> 1);
+        for (int v = first; v < pieces; v += step)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(Si + v)), "l"(Pi + v) : "memory");
+        asm volatile("cp.async.wait_all;" ::: "memory");
         sync_row(together);
-        uint64_t tm = 0;  // word groups are not needed here
         for (int64_t b0 = range.x; b0 < range.y; b0 += step) {
             const int64_t e = b0 + (together ? lane * nw + warp : lane);
             const int64_t ee = e < range.y ? e : range.x;
@@ -1097,14 +1119,11 @@ __global__ void __launch_bounds__(256, 5) indexed_rows_kernel(const WordIndex A,
             push_balanced<1, false>(d, w, lane, B.ptr, B.idx, B.val, S, 30, tm);
         }
         sync_row(together);
-        for (int64_t w = first; w < ldw; w += step) {
-            const uint64_t c = S[w];
-            grew |= c != P[i * ldw + w];
-            C[i * ldw + w] = c;
-        }
+        ulonglong2* Ci = reinterpret_cast<ulonglong2*>(C + i * ldw);
+        for (int v = first; v < pieces; v += step) Ci[v] = Si[v];
         sync_row(together);
     });
-    if (changed != nullptr && __any_sync(FULL, grew) && lane == 0) atomicOr(changed, 1);
+    if (changed != nullptr && __any_sync(FULL, tm != 0) && lane == 0) atomicOr(changed, 1);
 }
 
 // Sum over the block (every thread calls it; thread 0 gets it).
@@ -1608,6 +1627,9 @@ int smp_packed_max_words() { return 7168; }
 
 cudaError_t launch_indexed_rows(const WordIndex& A, const WordIndex& B, const uint64_t* P, int64_t n, int64_t ldw,
                                 uint64_t* C, int sms, cudaStream_t s, int* changed) {
+    // rows are read and written in 16-byte pieces
+    if ((ldw & 1) != 0 || ((reinterpret_cast<uintptr_t>(P) | reinterpret_cast<uintptr_t>(C)) & 15) != 0)
+        return cudaErrorInvalidValue;
     int warps = 8;
     while (warps > 1 && warps * ldw * 8 > 32 * 1024) warps >>= 1;
     const size_t smem = static_cast<size_t>(warps) * static_cast<size_t>(ldw) * 8;
@@ -1617,7 +1639,9 @@ cudaError_t launch_indexed_rows(const WordIndex& A, const WordIndex& B, const ui
         if (e != cudaSuccess) return e;
     }
     int64_t blocks = (n + warps - 1) / warps;
-    const int64_t cap = static_cast<int64_t>(sms) * 16;
+    // one round of resident blocks, whose rows then end together (10 or 16 blocks an SM: n = 32,768, 4 entries a row 55 and
+    // 57 us against 52; n = 16,000 23 and 25 against 21)
+    const int64_t cap = static_cast<int64_t>(sms) * 5;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     indexed_rows_kernel<<<static_cast<int>(blocks), warps * 32, smem, s>>>(A, B, P, n, ldw, C, changed);
