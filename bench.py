@@ -362,7 +362,7 @@ def run_extras(args, ctx, stream, n, ip, ix, R, FMT, out_main, bf16, hbm, check)
     del o2
 
     # -- one bit-row squaring R <- R + R R (rms_packed) on the sparse input (ER mean out-degree 4; through the word
-    # index, square_rows_kernel) and on a dense one (the closure of the n = 8,192 graph; whole rows, Four Russians
+    # index, indexed_rows_kernel) and on a dense one (the closure of the n = 8,192 graph; whole rows, Four Russians
     # tables, product_m4rm_kernel)
     pk = {}
 
@@ -376,7 +376,7 @@ def run_extras(args, ctx, stream, n, ip, ix, R, FMT, out_main, bf16, hbm, check)
                 if e.status != bmlp.BMLP_ERR_NOT_CONVERGED:
                     raise
             tms.append(ctx.stats()["product_ms"])
-        kern = "square_rows_kernel" if ctx.stats()["sparse_squarings"] else "product_m4rm_kernel"
+        kern = "indexed_rows_kernel" if ctx.stats()["sparse_squarings"] else "product_m4rm_kernel"
         return statistics.median(tms[1:]) / 1e3, kern
 
     dense8k = None
@@ -432,12 +432,12 @@ def run_extras(args, ctx, stream, n, ip, ix, R, FMT, out_main, bf16, hbm, check)
     del expanded
     st = ctx.stats()
     ex["powerlaw_smp"] = {"queries_per_s": q / ms * 1e3, "ms_per_batch": ms,
-                          "kernel": "smp_cluster_kernel" if st["cluster_frontiers"] else "smp_packed_kernel",
+                          "kernel": "smp_tile_kernel" if st["cluster_frontiers"] else "smp_packed_kernel",
                           "kernel_ms": kms, "levels": st["iterations"], "algorithmic_bytes": alg_bytes,
                           "effective_gbs": alg_bytes / kms / 1e6,
                           "note": "bytes a query-at-a-time expansion reads, over the kernel time; the bit-sliced "
-                                  "kernel reads each in-list once per level for 64 rows, and the word index of "
-                                  "R^T (about 3 MB) stays in L2, so this is an effective rate, not HBM traffic"}
+                                  "kernel reads each in-list once per level for 16 to 64 rows, and those lists "
+                                  "(about 2 MB) stay in L2, so this is an effective rate, not HBM traffic"}
     pl = (nq, pip, pix, srch, got)
     del P, src, qo
 
