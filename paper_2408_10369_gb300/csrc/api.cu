@@ -1542,7 +1542,8 @@ bmlp_status bmlp_ctx_create(bmlp_ctx** out, int32_t device) {
     cudaDeviceGetAttribute(&ctx->clock_khz, cudaDevAttrClockRate, device);
     if (cudaMalloc(&ctx->d_ctl, CTL_WORDS * sizeof(int)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_ctl, CTL_HOST_WORDS * sizeof(int)) != cudaSuccess ||
-        cudaEventCreate(&ctx->ev[0]) != cudaSuccess || cudaEventCreate(&ctx->ev[1]) != cudaSuccess) {
+        cudaEventCreate(&ctx->ev[0]) != cudaSuccess || cudaEventCreate(&ctx->ev[1]) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_insert, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         bmlp_ctx_destroy(ctx);
         return BMLP_ERR_OOM;
@@ -1564,6 +1565,7 @@ bmlp_status bmlp_ctx_destroy(bmlp_ctx* ctx) {
     if (ctx->h_ctl) cudaFreeHost(ctx->h_ctl);
     for (auto& e : ctx->ev)
         if (e) cudaEventDestroy(e);
+    if (ctx->ev_insert) cudaEventDestroy(ctx->ev_insert);
     delete ctx;
     return BMLP_OK;
 }
@@ -1785,9 +1787,17 @@ static bmlp_status core_insert(bmlp_ctx* ctx, void* closure, int64_t n, int32_t 
             ctx->stats.launches++;
         }
     } else {
+        // The call returns while its launches still read the two workspaces, and the next insertion may come on another
+        // stream: it waits on the device for the last one's (1 us of host time; no wait on the same stream).
         void *dp = nullptr, *scratch = nullptr;
         ST(ws_get(ctx, WS_INS_FACTS, hp.size() * sizeof(int32_t), &dp));
         ST(ws_get(ctx, WS_INS_SCRATCH, static_cast<size_t>(insert_chunk_words(ldw)) * 8, &scratch));
+        CK(cudaStreamWaitEvent(s, ctx->ev_insert, 0), "order insertions");
+        struct Record {  // also when a launch fails after others have been issued
+            cudaEvent_t e;
+            cudaStream_t s;
+            ~Record() { cudaEventRecord(e, s); }
+        } record{ctx->ev_insert, s};
         CK(cudaMemcpyAsync(dp, hp.data(), hp.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s), "copy facts");
         for (int64_t k = 0; k < m; k += kInsertChunk) {
             const int c = static_cast<int>(m - k < kInsertChunk ? m - k : kInsertChunk);

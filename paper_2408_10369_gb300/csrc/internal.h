@@ -151,6 +151,7 @@ struct bmlp_ctx {
     int* d_ctl = nullptr;        // device control words (see CTL_* below)
     int* h_ctl = nullptr;        // pinned host mirror
     cudaEvent_t ev[2] = {nullptr, nullptr};
+    cudaEvent_t ev_insert = nullptr;  // after the last insertion's use of its workspaces, whatever its stream
     bmlp_stats stats{};
     void* encode_fn = nullptr;   // cuTensorMapEncodeTiled from the driver
     double t_call = 0.0;         // host time at the start of the current call (s)
