@@ -1781,7 +1781,11 @@ static bmlp_status core_insert(bmlp_ctx* ctx, void* closure, int64_t n, int32_t 
         P = static_cast<uint64_t*>(p);
         ST(to_packed(ctx, in, fmt, n, P, ldw, s));
     }
-    if (m < kInsertChunkMin) {
+    // a capture records launches only: the facts travel as their arguments, since the copy of a chunk's would be replayed
+    // from host memory that is gone by then, and its workspaces belong to whichever call comes next
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (m >= kInsertChunkMin && cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+    if (m < kInsertChunkMin || capture != cudaStreamCaptureStatusNone) {
         for (int64_t k = 0; k < m; ++k) {
             CK(launch_insert_fact(P, n, ldw, hp[2 * k], hp[2 * k + 1], ctx->sm_count, s), "insert launch");
             ctx->stats.launches++;

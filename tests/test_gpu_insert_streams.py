@@ -1,5 +1,7 @@
 """Insertions whose launches are still running when the next one comes: on other streams of one context (the calls share the
-context's workspace)."""
+context's workspace), and recorded in a graph that is replayed after the facts' host memory is gone."""
+import gc
+
 import numpy as np
 import pytest
 import torch
@@ -36,5 +38,31 @@ def test_insertions_on_streams_of_one_context():
             torch.cuda.synchronize()
             for got, (_, _, want) in zip(mats, cases):
                 np.testing.assert_array_equal(wl.unpack_rows(got.cpu().numpy().view(np.uint64), len(got)), want)
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("m", [2, 3, 300])
+def test_insertion_in_a_graph(m):
+    n = 1100
+    before, e, want = grown(n, 0.7, m, 4)
+    other, e2, want2 = grown(900, 0.7, 500, 5)
+    ctx = pkg.Context(0)
+    try:
+        mat, stream = before.clone(), torch.cuda.Stream()
+        facts = e.copy()
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=stream):
+            ctx.insert(mat, n, facts, fmt=PACKED, stream=stream)
+        assert torch.equal(mat, before)
+        facts[:] = 0
+        del facts
+        gc.collect()
+        ctx.insert(other, 900, e2, fmt=PACKED)  # takes the workspaces
+        graph.replay()
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(wl.unpack_rows(mat.cpu().numpy().view(np.uint64), n), want)
+        np.testing.assert_array_equal(wl.unpack_rows(other.cpu().numpy().view(np.uint64), 900), want2)
     finally:
         ctx.close()
