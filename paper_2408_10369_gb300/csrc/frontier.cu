@@ -737,8 +737,7 @@ int tile_kept(int64_t n, int width) {
 
 template <int W>
 cudaError_t launch_tiles(const TileArgs& a, int grid, size_t smem, cudaStream_t s) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(smp_tile_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const cudaError_t e = allow_smem(smp_tile_kernel<W>, kTileSmem);
     if (e != cudaSuccess) return e;
     smp_tile_kernel<W><<<grid, kThreads, smem, s>>>(a);
     return cudaGetLastError();

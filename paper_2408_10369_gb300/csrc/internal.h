@@ -132,6 +132,14 @@ struct Deadline {
 #endif
 };
 
+// A kernel's limit of dynamic shared memory belongs to the kernel on the device, not to a context or a thread: set to what
+// one launch needs, it could be lowered by another thread's smaller launch between this one's setting and its launch, which
+// is then refused. So every setting of a kernel raises the limit to the same value, the most that any of its launches needs.
+template <class K>
+inline cudaError_t allow_smem(K* kernel, size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
+
 // Grow-only device buffer owned by a context.
 struct DevBuf {
     void* p = nullptr;

@@ -27,6 +27,8 @@
 //  * smp_sliced   Algorithm 2 for 64 sources at once, bit-sliced, for relations
 //                 too large for the tile form of frontier.cu.
 //  * insert_fact  one new fact into a transitive closure (rank-1 update).
+#include <atomic>
+
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -1582,8 +1584,7 @@ cudaError_t launch_product_packed(const uint64_t* A, const uint64_t* B, uint64_t
         return cudaGetLastError();
     }
     const int64_t grid = ((n + kM4Rows - 1) / kM4Rows) * ((ldw + kM4Cols - 1) / kM4Cols);
-    cudaError_t e = cudaFuncSetAttribute(product_m4rm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kM4Smem));
+    const cudaError_t e = allow_smem(product_m4rm_kernel, kM4Smem);
     if (e != cudaSuccess) return e;
     product_m4rm_kernel<<<static_cast<unsigned>(grid), kM4Threads, kM4Smem, s>>>(A, B, dst, n, ldw, or_a, changed,
                                                                                    dl, pstat);
@@ -1605,8 +1606,7 @@ cudaError_t launch_insert_chunk(uint64_t* P, int64_t n, int64_t ldw, const int32
     uint64_t* G = scratch;
     uint64_t* W = scratch + kInsertChunk * (kInsertChunk / 64);
     const int smem = m * mw * 8;  // at most 128 KiB
-    cudaError_t e = cudaFuncSetAttribute(insert_reach_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kInsertChunk * (kInsertChunk / 64) * 8);
+    const cudaError_t e = allow_smem(insert_reach_kernel, kInsertChunk * (kInsertChunk / 64) * 8);
     if (e != cudaSuccess) return e;
     insert_links_kernel<<<m, kInsertWarps * 32, 0, s>>>(P, ldw, pairs, m, mw, reinterpret_cast<uint32_t*>(G));
     insert_reach_kernel<<<(m + kInsertWarps - 1) / kInsertWarps, kInsertWarps * 32, smem, s>>>(P, n, ldw, pairs, m, mw, G,
@@ -1625,6 +1625,9 @@ cudaError_t launch_wcsr_build(const uint64_t* P, int64_t n, int64_t ldw, const W
 
 int smp_packed_max_words() { return 7168; }
 
+// Most shared memory of a warp's arrays, and so of a block of the kernels that choose their warps by it.
+constexpr size_t kMostWarpSmem = 200 * 1024;
+
 cudaError_t launch_indexed_rows(const WordIndex& A, const WordIndex& B, const uint64_t* P, int64_t n, int64_t ldw,
                                 uint64_t* C, int sms, cudaStream_t s, int* changed) {
     // rows are read and written in 16-byte pieces
@@ -1633,9 +1636,9 @@ cudaError_t launch_indexed_rows(const WordIndex& A, const WordIndex& B, const ui
     int warps = 8;
     while (warps > 1 && warps * ldw * 8 > 32 * 1024) warps >>= 1;
     const size_t smem = static_cast<size_t>(warps) * static_cast<size_t>(ldw) * 8;
+    if (smem > kMostWarpSmem) return cudaErrorInvalidValue;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(indexed_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem));
+        const cudaError_t e = allow_smem(indexed_rows_kernel, kMostWarpSmem);
         if (e != cudaSuccess) return e;
     }
     int64_t blocks = (n + warps - 1) / warps;
@@ -1683,18 +1686,19 @@ cudaLaunchConfig_t smp_rows_config(int64_t n, int64_t q, int ctas, cudaStream_t 
     return cfg;
 }
 
-cudaError_t smp_rows_attributes(size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(smp_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(smp_rows_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    return e;
+// Shared memory of a CTA in steps of kRowsSmemStep, of which it has at most kRowsSmemSteps.
+constexpr size_t kRowsSmemStep = 16384, kRowsSmemSteps = 13;
+
+cudaError_t smp_rows_attributes() {
+    const cudaError_t e = allow_smem(smp_rows_kernel, kRowsSmemStep * kRowsSmemSteps);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(smp_rows_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 }  // namespace
 
 int smp_rows_ctas(int64_t n, int64_t q) {
-    // resident clusters by (device, cluster size, shared memory in steps of 16 KiB), asked once each since the query
-    // costs more than the launch (0: not asked; else the count + 1)
-    static unsigned char known[16][4][16] = {};
+    // resident clusters by (device, cluster size, steps of shared memory), asked once each since the query costs more than
+    // the launch (0: not asked; else the count + 1); written by any thread, always with the same value
+    static std::atomic<unsigned char> known[16][4][kRowsSmemSteps + 1] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
@@ -1703,23 +1707,22 @@ int smp_rows_ctas(int64_t n, int64_t q) {
     if (q > kRowsMaxQueries) return 0;
     for (int h = 0; h < 4; ++h) {
         const int ctas = kRowsMaxCtas >> h;
-        const size_t smem = smp_rows_smem(n, ctas);
-        const size_t step = (smem + 16383) / 16384;
-        if (step >= 14) return 0;  // 224 KiB: more than a CTA's
+        const size_t step = (smp_rows_smem(n, ctas) + kRowsSmemStep - 1) / kRowsSmemStep;
+        if (step > kRowsSmemSteps) return 0;
         const bool keyed = dev >= 0 && dev < 16;
-        int clusters = keyed ? static_cast<int>(known[dev][h][step]) - 1 : -1;
+        int clusters = keyed ? static_cast<int>(known[dev][h][step].load(std::memory_order_relaxed)) - 1 : -1;
         if (clusters < 0) {
             cudaLaunchAttribute at;
             cudaLaunchConfig_t cfg = smp_rows_config(n, 1, ctas, nullptr, &at);
-            cfg.dynamicSmemBytes = step * 16384 > smem ? step * 16384 : smem;
+            cfg.dynamicSmemBytes = step * kRowsSmemStep;
             clusters = 0;
-            if (smp_rows_attributes(cfg.dynamicSmemBytes) != cudaSuccess ||
+            if (smp_rows_attributes() != cudaSuccess ||
                 cudaOccupancyMaxActiveClusters(&clusters, smp_rows_kernel, &cfg) != cudaSuccess) {
                 cudaGetLastError();
-                clusters = 0;
+                continue;  // asked again by the next call
             }
             if (clusters > 200) clusters = 200;
-            if (keyed) known[dev][h][step] = static_cast<unsigned char>(clusters + 1);
+            if (keyed) known[dev][h][step].store(static_cast<unsigned char>(clusters + 1), std::memory_order_relaxed);
         }
         if (q <= clusters) return ctas;
     }
@@ -1731,7 +1734,7 @@ cudaError_t launch_smp_rows(const uint64_t* R, int64_t ld_r, int64_t n, const ui
                             cudaStream_t s, Deadline dl) {
     cudaLaunchAttribute at;
     const cudaLaunchConfig_t cfg = smp_rows_config(n, q, ctas, s, &at);
-    const cudaError_t e = smp_rows_attributes(cfg.dynamicSmemBytes);
+    const cudaError_t e = smp_rows_attributes();
     if (e != cudaSuccess) return e;
     const RowQueryArgs a{R, ld_r, n, src, ld_src, out, ld_out, levels, max_levels, reflexive, dl};
     return cudaLaunchKernelEx(&cfg, smp_rows_kernel, a);
@@ -1765,12 +1768,11 @@ cudaError_t launch_smp_packed(const WordIndex& x, const WordIndex& T, int64_t n,
                               int reflexive, int sms, cudaStream_t s, Deadline dl) {
     // blocks of 1-8 warps, chosen so that as many warps as possible fit an SM's shared memory
     const int64_t per_warp = smp_warp_bytes(ldw);
-    if (per_warp > 200 * 1024) return cudaErrorInvalidValue;
+    if (per_warp > static_cast<int64_t>(kMostWarpSmem)) return cudaErrorInvalidValue;
     int warps = 8;
     while (warps > 1 && warps * per_warp > 32 * 1024) warps >>= 1;
     const size_t smem = static_cast<size_t>(warps) * per_warp;
-    cudaError_t e = cudaFuncSetAttribute(smp_packed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
+    const cudaError_t e = allow_smem(smp_packed_kernel, kMostWarpSmem);
     if (e != cudaSuccess) return e;
     int64_t blocks = (q + warps - 1) / warps;
     int per_sm = static_cast<int>((220 * 1024) / (smem + 1024));
@@ -1800,7 +1802,7 @@ cudaError_t launch_frontier_group(const FrontierJob* jobs, int njobs, int64_t ma
                                   unsigned long long* counter, int sms, cudaStream_t s) {
     if (njobs <= 0) return cudaSuccess;
     const int64_t per_warp = smp_warp_bytes(max_ldw);
-    if (per_warp > 200 * 1024 || njobs > 65535) return cudaErrorInvalidValue;
+    if (per_warp > static_cast<int64_t>(kMostWarpSmem) || njobs > 65535) return cudaErrorInvalidValue;
     const unsigned nj = static_cast<unsigned>(njobs);
     const int64_t wpr = (max_n + 63) / 64;
     int64_t tb = wpr * wpr;
@@ -1813,7 +1815,7 @@ cudaError_t launch_frontier_group(const FrontierJob* jobs, int njobs, int64_t ma
     int warps = 8;
     while (warps > 1 && warps * per_warp > 32 * 1024) warps >>= 1;
     const size_t smem = static_cast<size_t>(warps) * per_warp;
-    e = cudaFuncSetAttribute(frontier_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    e = allow_smem(frontier_group_kernel, kMostWarpSmem);
     if (e != cudaSuccess) return e;
     int per_sm = static_cast<int>((220 * 1024) / (smem + 1024));
     if (per_sm < 1) per_sm = 1;

@@ -21,6 +21,7 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int kThreads = 1024;
 constexpr int kPieces = 4;   // 16-byte pieces of a matrix that a thread has in flight
 constexpr int kWarps = kThreads / 32;
+constexpr size_t kMostSmem = 220 * 1024;  // of 227 KiB, beside the lists (n = 1,024 on 152 SMs: 131 KiB)
 
 struct SmallArgs {
     const void* in;       // n x n bytes, or bit rows of words64 64-bit words
@@ -312,8 +313,8 @@ cudaError_t launch_small_closure(const void* in, const void* r1, void* out, int6
     a.wait_cycles = wait_cycles;
     const int grid = static_cast<int>((n + a.rows_per - 1) / a.rows_per);
     const size_t smem = (static_cast<size_t>(n) + 3 * static_cast<size_t>(a.rows_per)) * a.pitch * 4;
-    cudaError_t e = cudaFuncSetAttribute(small_closure_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
+    if (smem > kMostSmem) return cudaErrorInvalidValue;
+    const cudaError_t e = allow_smem(small_closure_kernel, kMostSmem);
     if (e != cudaSuccess) return e;
     void* args[] = {&a};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(small_closure_kernel), dim3(static_cast<unsigned>(grid)),
