@@ -1284,8 +1284,8 @@ bmlp_status build_lane(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
 // Branches of the batch graph that the large problems are dealt out to, besides the branch of the grouped ones. A
 // pipeline is a chain of small launches (bit-row squarings, decisions) between tensor-core products that fill the GPU, so
 // several chains at once fill each other's gaps (measured on the knowledge-graph batch, 33 closures and 8 compositions
-// with n >= 4,096: 37.4 ms on one branch, 32.2 on two, 30.4 on four, 30.4 on twelve). More lanes than that add scratch
-// (at most kLaneBytes in all, else fewer lanes).
+// with n >= 4,096: 37.4 ms on one branch, 32.2 on two, 30.4 on four, 30.4 on twelve). Every lane adds scratch: fewer of
+// them where that would be more than kLaneBytes in all, or more than the device has left.
 constexpr int kLanes = 4;
 constexpr size_t kLaneBytes = size_t(24) << 30;
 
@@ -1318,7 +1318,9 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
         }
         if (lanes > 1 && total > kLaneBytes) continue;
         void* base = nullptr;
-        BST(ws_get(ctx, WS_SOLO, total, &base));
+        const bmlp_status got = ws_get(ctx, WS_SOLO, total, &base);
+        if (got == BMLP_ERR_OOM && lanes > 1) continue;
+        BST(got);
         size_t at = 0;
         for (int l = 0; l < lanes; ++l) {
             size_t unused = 0;

@@ -1,0 +1,48 @@
+"""Calls on a device whose memory is mostly held by the caller: the forms that want more workspace give way to those that
+need less, and a call that did not fit runs once there is room."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as wl
+
+pkg = pytest.importorskip("paper_2408_10369_gb300")
+from paper_2408_10369_gb300 import bmlp  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+PACKED = bmlp.BMLP_FMT_PACKED64
+
+
+def hold_all_but(free):
+    """Device memory held so that about `free` bytes are left."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.empty(torch.cuda.mem_get_info()[0] - free, dtype=torch.uint8, device="cuda")
+
+
+@pytest.fixture(scope="module")
+def large_problems():
+    n = 12000
+    csr = wl.er_graph(n, 3.0, 11)
+    R = torch.from_numpy(wl.csr_to_packed(n, *csr).view(np.int64)).cuda()
+    with pkg.Context(0) as ctx:  # kernels and graphs are loaded while there is room
+        r = torch.from_numpy(wl.csr_to_packed(4096, *wl.er_graph(4096, 3.0, 1)).view(np.int64)).cuda()
+        ctx.batch_run([dict(n=4096, R1=r, out=torch.zeros_like(r), fmt=PACKED) for _ in range(4)])
+    return n, R, wl.pack_rows(oracle.closure(n, *csr))
+
+
+def test_batch_branches_give_way_to_memory(large_problems):
+    """Four problems of 12,000 constants on four branches take 1.9 GB of scratch, on two 1.0 GB."""
+    n, R, want = large_problems
+    outs = [torch.zeros_like(R) for _ in range(4)]
+    with pkg.Context(0) as ctx:
+        held = hold_all_but(1300 << 20)
+        try:
+            ctx.batch_run([dict(n=n, R1=R, out=o, fmt=PACKED) for o in outs])
+            torch.cuda.synchronize()
+        finally:
+            del held
+            torch.cuda.empty_cache()
+    for o in outs:
+        np.testing.assert_array_equal(o.cpu().numpy().view(np.uint64), want)
