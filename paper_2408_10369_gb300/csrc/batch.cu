@@ -1363,7 +1363,13 @@ bmlp_status batch_run_impl(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t cou
     if (count > (int64_t(1) << 20)) return set_err(ctx, BMLP_ERR_UNSUPPORTED, "more than 2^20 problems");
     const uint64_t key = batch_key(probs, count, variant, ctx->tune, solo_n);
     BatchCache* c = static_cast<BatchCache*>(ctx->batch);
-    if (c == nullptr || c->key != key) BST(build_batch(ctx, probs, count, variant, wait_cycles, key, solo_n, &c));
+    if (c == nullptr || c->key != key) {
+        const bmlp_status built = build_batch(ctx, probs, count, variant, wait_cycles, key, solo_n, &c);
+        if (built != BMLP_OK) {  // nothing half built is left to be found under the key by the next call
+            batch_cache_free(ctx);
+            return built;
+        }
+    }
     BCK(cudaMemsetAsync(ctx->d_ctl, 0, CTL_WORDS * sizeof(int), s), "reset flags");
     ctx->stats.n_pad = static_cast<int64_t>(c->ws_bytes);
     BCK(cudaGraphLaunch(c->exec, s), "cudaGraphLaunch");

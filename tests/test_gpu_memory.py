@@ -46,3 +46,22 @@ def test_batch_branches_give_way_to_memory(large_problems):
             torch.cuda.empty_cache()
     for o in outs:
         np.testing.assert_array_equal(o.cpu().numpy().view(np.uint64), want)
+
+
+def test_batch_runs_once_there_is_room(large_problems):
+    n, R, want = large_problems
+    out = torch.zeros_like(R)
+    items = pkg.Context.problems([dict(n=n, R1=R, out=out, fmt=PACKED)])
+    with pkg.Context(0) as ctx:
+        held = hold_all_but(200 << 20)
+        try:
+            for _ in range(2):
+                with pytest.raises(bmlp.BmlpError) as e:
+                    ctx.batch_run(items)
+                assert e.value.status == bmlp.BMLP_ERR_OOM
+        finally:
+            del held
+            torch.cuda.empty_cache()
+        ctx.batch_run(items)
+        torch.cuda.synchronize()
+    np.testing.assert_array_equal(out.cpu().numpy().view(np.uint64), want)
