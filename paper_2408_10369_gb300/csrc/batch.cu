@@ -1332,8 +1332,10 @@ bmlp_status build_solo(bmlp_ctx* ctx, BatchCache* c, const bmlp_problem* probs, 
     return BMLP_OK;
 }
 
-uint64_t batch_key(const bmlp_problem* probs, int64_t count, int variant, const int* tune, int64_t solo_n) {
+uint64_t batch_key(const bmlp_problem* probs, int64_t count, int variant, long long wait_cycles, const int* tune,
+                   int64_t solo_n) {
     uint64_t h = 1469598103934665603ull;
+    h = fnv(h, &wait_cycles, sizeof(wait_cycles));  // the bound is an argument of the graph's tensor-core kernels
     h = fnv(h, &count, sizeof(count));
     h = fnv(h, &variant, sizeof(variant));
     h = fnv(h, &solo_n, sizeof(solo_n));
@@ -1361,7 +1363,7 @@ bmlp_status batch_run_impl(bmlp_ctx* ctx, const bmlp_problem* probs, int64_t cou
             return set_err(ctx, BMLP_ERR_INVALID_ARG, "problem %lld: matrices must be device memory", (long long)i);
     }
     if (count > (int64_t(1) << 20)) return set_err(ctx, BMLP_ERR_UNSUPPORTED, "more than 2^20 problems");
-    const uint64_t key = batch_key(probs, count, variant, ctx->tune, solo_n);
+    const uint64_t key = batch_key(probs, count, variant, wait_cycles, ctx->tune, solo_n);
     BatchCache* c = static_cast<BatchCache*>(ctx->batch);
     if (c == nullptr || c->key != key) {
         const bmlp_status built = build_batch(ctx, probs, count, variant, wait_cycles, key, solo_n, &c);
