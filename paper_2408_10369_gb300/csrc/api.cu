@@ -698,6 +698,7 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
                         continue;
                     }
                     thin_try = false;  // some zeros need more of their rows: R is as it was
+                    CK(cudaMemsetAsync(ctx->d_ctl + CTL_OPEN, 0, sizeof(int), s), "reset flag");  // a slice may follow
                 }
             }
             ST(operands_current());
