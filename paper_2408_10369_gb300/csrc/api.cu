@@ -102,6 +102,8 @@ constexpr int WS_E8_IN0 = 31, WS_E8_IN1 = 32, WS_E8_OUT = 33;
 // Bit rows of R and R^T, their ones, the column mask and the row and column lists, and the computed rows of a
 // squaring restricted to the rows and columns that still hold zeros.
 constexpr int WS_THIN_P = 35, WS_THIN_AUX = 36, WS_THIN_T = 37;
+// The second pair of bit rows, of calls that try a slice.
+constexpr int WS_THIN_P2 = 42;
 // The facts of an insertion (checked copy) and the chunk kernels' scratch.
 constexpr int WS_INS_FACTS = 38, WS_INS_SCRATCH = 39;
 // Facts from which an insertion runs in chunks of three launches instead of one launch per fact (n = 14,541: 19.5 us
@@ -544,23 +546,20 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
     // all), slice_try (dense, not saturated: a product over a slice of k first).
     bool thin_try = false, slice_try = false, slice_failed = false;
     // bit rows of R and R^T (n_pad rows each), written by every 4-bit squaring's epilogue when the caller takes the
-    // result from them (res_bits) or a restricted squaring may need them; two pairs, since a sliced squaring reads R's
-    // while it completes R''s. bits_current: pair bcur holds R. q_current: the E2M1 pair qcur holds R too (a restricted
-    // squaring writes bit rows only; they are converted when a product needs operands again).
+    // result from them (res_bits) or a restricted squaring may need them, in place until a slice is tried: it reads R's
+    // while it completes R''s, so a second pair is taken then, where the device has room for it. bits_current: pair bcur
+    // holds R. q_current: the E2M1 pair qcur holds R too (a restricted squaring writes bit rows only; they are converted
+    // when a product needs operands again).
+    const size_t pair_words = static_cast<size_t>(n_pad * ldw_t);
     uint64_t* P[2] = {nullptr, nullptr};
     uint64_t* PT[2] = {nullptr, nullptr};
     int bcur = 0;
     bool bits_current = false, q_current = true;
     if (thin_on || res_bits != nullptr) {
-        const size_t one = static_cast<size_t>(n_pad * ldw_t);
         void* pp = nullptr;
-        ST(ws_get(ctx, WS_THIN_P, (thin_on ? 4 : 2) * one * 8, &pp));
+        ST(ws_get(ctx, WS_THIN_P, 2 * pair_words * 8, &pp));
         P[0] = P[1] = static_cast<uint64_t*>(pp);
-        PT[0] = PT[1] = P[0] + one;
-        if (thin_on) {
-            P[1] = PT[0] + one;
-            PT[1] = P[1] + one;
-        }
+        PT[0] = PT[1] = P[0] + pair_words;
     }
     if (res_bits != nullptr) *res_bits = nullptr;
     auto operands_current = [&]() -> bmlp_status {
@@ -702,6 +701,18 @@ bmlp_status rms_tc_loop(bmlp_ctx* ctx, int64_t n, int64_t n_pad, uint8_t* M[2], 
                 }
             }
             ST(operands_current());
+            if (slice_try && bits_current && P[0] == P[1]) {
+                void* pp = nullptr;
+                const bmlp_status got = ws_get(ctx, WS_THIN_P2, 2 * pair_words * 8, &pp);
+                if (got != BMLP_OK && got != BMLP_ERR_OOM) return got;
+                if (got == BMLP_ERR_OOM) {
+                    slice_try = false;
+                    slice_failed = true;
+                } else {
+                    P[bcur ^ 1] = static_cast<uint64_t*>(pp);
+                    PT[bcur ^ 1] = P[bcur ^ 1] + pair_words;
+                }
+            }
             TcParams p4 = p;
             p4.ld = ld4;
             p4.k_blocks = static_cast<int32_t>(n_pad / 256);

@@ -65,3 +65,39 @@ def test_batch_runs_once_there_is_room(large_problems):
         ctx.batch_run(items)
         torch.cuda.synchronize()
     np.testing.assert_array_equal(out.cpu().numpy().view(np.uint64), want)
+
+
+def workspace_of(R, n, out, **opt):
+    """Bytes that a context takes for this closure, and its statistics."""
+    out.zero_()
+    torch.cuda.synchronize()
+    with pkg.Context(0) as ctx:
+        before = torch.cuda.mem_get_info()[0]
+        ctx.rms(R, n, out, **opt)
+        torch.cuda.synchronize()
+        return before - torch.cuda.mem_get_info()[0], ctx.stats()
+
+
+def test_second_pair_of_bit_rows_only_for_slices():
+    """A dense closure of 9,216 constants takes one pair of bit rows (21 MB); a second one when a slice is tried, and none is
+    tried where that does not fit."""
+    n = 9216
+    R = torch.ones((n, n), dtype=torch.uint8, device="cuda")
+    R[:, 1500] = 0
+    R[n - 100:, 1500] = 1
+    out = torch.zeros_like(R)
+    one, st = workspace_of(R, n, out, variant="rms_tc")  # one product fills the column
+    assert int(out.min()) == 1 and st["e2m1_products"] == 1
+    R[:801, n - 100:] = 0
+    two, st = workspace_of(R, n, out, variant="rms_tc")  # a product, and a slice
+    assert int(out.min()) == 1 and st["e2m1_products"] == 1 and st["thin_squarings"] == 2
+    pair = 2 * n * (n // 64) * 8
+    assert two - one > 0.9 * pair
+    held = hold_all_but(one + pair // 2 + (6 << 20))
+    try:
+        some, st = workspace_of(R, n, out, variant="rms_tc")
+        assert int(out.min()) == 1 and st["e2m1_products"] == 2
+        assert some < two - pair // 2
+    finally:
+        del held
+        torch.cuda.empty_cache()
