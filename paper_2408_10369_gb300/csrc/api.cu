@@ -1797,7 +1797,15 @@ static bmlp_status core_insert(bmlp_ctx* ctx, void* closure, int64_t n, int32_t 
     // from host memory that is gone by then, and its workspaces belong to whichever call comes next
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (m >= kInsertChunkMin && cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
-    if (m < kInsertChunkMin || capture != cudaStreamCaptureStatusNone) {
+    bool chunks = m >= kInsertChunkMin && capture == cudaStreamCaptureStatusNone;
+    void *dp = nullptr, *scratch = nullptr;
+    if (chunks) {
+        bmlp_status got = ws_get(ctx, WS_INS_FACTS, hp.size() * sizeof(int32_t), &dp);
+        if (got == BMLP_OK) got = ws_get(ctx, WS_INS_SCRATCH, static_cast<size_t>(insert_chunk_words(ldw)) * 8, &scratch);
+        if (got != BMLP_OK && got != BMLP_ERR_OOM) return got;
+        chunks = got == BMLP_OK;  // no room: a launch per fact needs none
+    }
+    if (!chunks) {
         for (int64_t k = 0; k < m; ++k) {
             CK(launch_insert_fact(P, n, ldw, hp[2 * k], hp[2 * k + 1], ctx->sm_count, s), "insert launch");
             ctx->stats.launches++;
@@ -1805,9 +1813,6 @@ static bmlp_status core_insert(bmlp_ctx* ctx, void* closure, int64_t n, int32_t 
     } else {
         // The call returns while its launches still read the two workspaces, and the next insertion may come on another
         // stream: it waits on the device for the last one's (1 us of host time; no wait on the same stream).
-        void *dp = nullptr, *scratch = nullptr;
-        ST(ws_get(ctx, WS_INS_FACTS, hp.size() * sizeof(int32_t), &dp));
-        ST(ws_get(ctx, WS_INS_SCRATCH, static_cast<size_t>(insert_chunk_words(ldw)) * 8, &scratch));
         CK(cudaStreamWaitEvent(s, ctx->ev_insert, 0), "order insertions");
         struct Record {  // also when a launch fails after others have been issued
             cudaEvent_t e;

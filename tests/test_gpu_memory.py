@@ -101,3 +101,22 @@ def test_second_pair_of_bit_rows_only_for_slices():
     finally:
         del held
         torch.cuda.empty_cache()
+
+
+def test_insertion_without_room_for_a_chunk():
+    n = 131072  # 17 MB of scratch
+    P = torch.zeros((n, wl.words(n)), dtype=torch.int64, device="cuda")
+    facts = np.array([[1, 2], [5, 6], [3, 4], [9, 8], [7, 0], [2, 100000], [100000, 3]], np.int32)
+    with pkg.Context(0) as ctx:
+        want = P.clone()
+        for f in facts:
+            ctx.insert(want, n, f[None], fmt=PACKED)
+        held = hold_all_but(8 << 20)
+        try:
+            ctx.insert(P, n, facts, fmt=PACKED)
+            assert ctx.stats()["launches"] == len(facts)
+            torch.cuda.synchronize()
+        finally:
+            del held
+            torch.cuda.empty_cache()
+        assert torch.equal(P, want) and bool(P[1, 0] & 0x1C == 0x1C)
