@@ -2083,19 +2083,22 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
             // a sparse closure: R1 + R2+ R1 through the word indexes of R2+ and R1, unless that is predicted to cost more
             // than the whole-row product, whose tables cost as much for few ones as for many
             WordIndex xr;
-            ST(index_buffers(ctx, n, ldw, WS_SQPTR, WS_SQIDX, WS_SQVAL, &xr));
-            auto* cost = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_COST);
-            CK(launch_wcsr_build(A1, n, ldw, xr, s), "word index build");
-            CK(cudaMemsetAsync(cost, 0, 2 * sizeof(unsigned long long), s), "reset cost");
-            CK(launch_indexed_cost(xc, xr, n, cost, ctx->sm_count, s), "product cost launch");
-            ctx->stats.launches += 2;
-            ST(read_ctl(ctx, s, nullptr));
-            unsigned long long words = 0, row_words = 0;
-            memcpy(&words, ctx->h_ctl + CTL_COST, sizeof(words));
-            memcpy(&row_words, ctx->h_ctl + CTL_COST + 2, sizeof(row_words));
-            const double t = kSparseStepS + std::max(static_cast<double>(words) * sparse_s_per_word(),
-                                                     static_cast<double>(row_words) * sparse_row_s_per_word());
-            indexed = t < table_product_s(n);
+            const bmlp_status got = index_buffers(ctx, n, ldw, WS_SQPTR, WS_SQIDX, WS_SQVAL, &xr);
+            if (got != BMLP_OK && got != BMLP_ERR_OOM) return got;
+            if (got == BMLP_OK) {  // no room for it: the whole-row product needs none
+                auto* cost = reinterpret_cast<unsigned long long*>(ctx->d_ctl + CTL_COST);
+                CK(launch_wcsr_build(A1, n, ldw, xr, s), "word index build");
+                CK(cudaMemsetAsync(cost, 0, 2 * sizeof(unsigned long long), s), "reset cost");
+                CK(launch_indexed_cost(xc, xr, n, cost, ctx->sm_count, s), "product cost launch");
+                ctx->stats.launches += 2;
+                ST(read_ctl(ctx, s, nullptr));
+                unsigned long long words = 0, row_words = 0;
+                memcpy(&words, ctx->h_ctl + CTL_COST, sizeof(words));
+                memcpy(&row_words, ctx->h_ctl + CTL_COST + 2, sizeof(row_words));
+                const double t = kSparseStepS + std::max(static_cast<double>(words) * sparse_s_per_word(),
+                                                         static_cast<double>(row_words) * sparse_row_s_per_word());
+                indexed = t < table_product_s(n);
+            }
             if (indexed) {
                 CK(launch_indexed_rows(xc, xr, A1, n, ldw, X, ctx->sm_count, s), "word-indexed product launch");
                 ctx->stats.product_launches++;

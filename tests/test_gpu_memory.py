@@ -120,3 +120,29 @@ def test_insertion_without_room_for_a_chunk():
             del held
             torch.cuda.empty_cache()
         assert torch.equal(P, want) and bool(P[1, 0] & 0x1C == 0x1C)
+
+
+def test_packed_composition_without_room_for_a_second_index():
+    n = 9001
+    a, b = wl.er_graph(n, 2.0, 5), wl.er_graph(n, 0.8, 6)
+    A, B = (torch.from_numpy(wl.csr_to_packed(n, *x).view(np.int64)).cuda() for x in (a, b))
+    out, again = torch.zeros_like(A), torch.zeros_like(A)
+    torch.cuda.synchronize()
+    with pkg.Context(0) as ctx:
+        before = torch.cuda.mem_get_info()[0]
+        ctx.compose(A, B, n, out, fmt=PACKED, variant="rms_packed")
+        torch.cuda.synchronize()
+        used = before - torch.cuda.mem_get_info()[0]
+        launches = ctx.stats()["launches"]
+    held = hold_all_but(used - n * (n // 64) * 8 // 2)
+    try:
+        with pkg.Context(0) as ctx:
+            ctx.compose(A, B, n, again, fmt=PACKED, variant="rms_packed")
+            torch.cuda.synchronize()
+            assert ctx.stats()["launches"] < launches  # no index of R1 and no pass over its cost
+    finally:
+        del held
+        torch.cuda.empty_cache()
+    assert torch.equal(out, again)
+    rows = np.arange(0, n, 97, dtype=np.int32)
+    np.testing.assert_array_equal(wl.unpack_rows(out.cpu().numpy().view(np.uint64), n)[rows], oracle.compose_rows(n, a, b, rows))
