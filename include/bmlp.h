@@ -243,9 +243,10 @@ bmlp_status bmlp_rms_alg1(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt, 
  * layout. A source is in its own output row only if it lies on a cycle.
  * R is n x n in format fmt. *iters_out receives the deepest frontier level.
  * Variants: BMLP_SMP_PACKED, BMLP_SMP_TC, BMLP_AUTO. BMLP_SMP_PACKED expands
- * up to 63 rows one per thread-block cluster straight from R; larger batches
- * one row per warp, or, over a relation whose rows widen fast (n >= 4096), 16
- * to 64 rows at a time with bit-sliced frontiers.
+ * up to 63 rows one per thread-block cluster straight from R (for n > 8192,
+ * rows that turn out too deep or too wide for that go on as those of larger
+ * batches do); larger batches one row per warp, or, over a relation whose rows
+ * widen fast (n >= 4096), 16 to 64 rows at a time with bit-sliced frontiers.
  */
 bmlp_status bmlp_smp(bmlp_ctx* ctx, const void* R, int64_t n, int32_t fmt,
                      const uint64_t* src_rows, int64_t nq, uint64_t* out_rows,

@@ -104,6 +104,8 @@ constexpr int WS_E8_IN0 = 31, WS_E8_IN1 = 32, WS_E8_OUT = 33;
 constexpr int WS_THIN_P = 35, WS_THIN_AUX = 36, WS_THIN_T = 37;
 // The second pair of bit rows, of calls that try a slice.
 constexpr int WS_THIN_P2 = 42;
+// Query rows between the form that reads R's rows and the one over word indexes.
+constexpr int WS_ROWS = 43;
 // The facts of an insertion (checked copy) and the chunk kernels' scratch.
 constexpr int WS_INS_FACTS = 38, WS_INS_SCRATCH = 39;
 // Facts from which an insertion runs in chunks of three launches instead of one launch per fact (n = 14,541: 19.5 us
@@ -1243,7 +1245,9 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
     if (ldw > smp_packed_max_words())
         return set_err(ctx, BMLP_ERR_UNSUPPORTED, "packed frontier path supports n <= %d", smp_packed_max_words() * 64);
     // a few query rows: expanded straight from R's rows, each row of a reached constant read once
-    if (const int ctas = square_first ? 0 : smp_rows_ctas(n, q)) {
+    RowState begun{nullptr, nullptr};  // rows that stopped there, to be finished over the word indexes
+    int row_levels = 0;
+    if (const RowQueryPlan plan = square_first ? RowQueryPlan{} : smp_rows_plan(n, q); plan.ctas > 0) {
         const int64_t wpr = words_of(n);
         const uint64_t* rows = static_cast<const uint64_t*>(R.dev);
         if (fmt == BMLP_FMT_U8) {
@@ -1252,20 +1256,30 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
             ST(to_packed(ctx, R, fmt, n, static_cast<uint64_t*>(p), wpr, s));
             rows = static_cast<const uint64_t*>(p);
         }
+        if (plan.may_stop) {
+            void* p = nullptr;
+            ST(ws_get(ctx, WS_ROWS, static_cast<size_t>(q * 3 * wpr * 8 + q * 4), &p));
+            begun.words = static_cast<uint64_t*>(p);
+            begun.levels = reinterpret_cast<int*>(begun.words + q * 3 * wpr);
+        }
         ProductTimer tm{ctx, o.profile != 0, s};
         ST(tm.begin());
         CK(launch_smp_rows(rows, wpr, n, src, ldw_src, q, out, ldw_out, o.reflexive, ctx->d_ctl + CTL_LEVELS,
-                           static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), ctas, s, deadline_of(ctx)),
+                           static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), plan, begun, ctx->d_ctl + CTL_STEP, s,
+                           deadline_of(ctx)),
            "query row kernel launch");
         ST(tm.end());
         ctx->stats.product_launches++;
         ctx->stats.launches++;
         ST(read_ctl(ctx, s, nullptr));
         ST(tm.collect());
-        *levels = ctx->h_ctl[CTL_LEVELS];
-        const int cap = o.max_iters > 0 ? o.max_iters : static_cast<int>(n + 1);
-        if (*levels > cap) return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "frontier did not empty within %d levels", cap);
-        return BMLP_OK;
+        row_levels = ctx->h_ctl[CTL_LEVELS];
+        if (ctx->h_ctl[CTL_STEP] == 0) {
+            *levels = row_levels;
+            const int cap = o.max_iters > 0 ? o.max_iters : static_cast<int>(n + 1);
+            if (*levels > cap) return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "frontier did not empty within %d levels", cap);
+            return BMLP_OK;
+        }
     }
     void* P = nullptr;
     WordIndex x;
@@ -1437,14 +1451,14 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
     if (src == nullptr) ST(identity_rows(ctx, n, ldw_src, s, &src));
     ST(tm.begin());
     CK(launch_smp_packed(x, xT, n, ldw, src, ldw_src, q, out, ldw_out, ctx->d_ctl + CTL_LEVELS, ctx->d_ctl + CTL_QCOUNT,
-                         o.reflexive, ctx->sm_count, s, deadline_of(ctx)),
+                         o.reflexive, ctx->sm_count, s, deadline_of(ctx), begun),
        "frontier kernel launch");
     ST(tm.end());
     ctx->stats.product_launches++;
     ctx->stats.launches++;
     ST(read_ctl(ctx, s, nullptr));
     ST(tm.collect());
-    *levels = ctx->h_ctl[CTL_LEVELS];
+    *levels = std::max(row_levels, ctx->h_ctl[CTL_LEVELS]);
     const int cap = o.max_iters > 0 ? o.max_iters : static_cast<int>(n + 1);
     if (*levels > cap) return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "frontier did not empty within %d levels", cap);
     return BMLP_OK;

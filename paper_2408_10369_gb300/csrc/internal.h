@@ -338,9 +338,15 @@ struct WordIndex {
     uint64_t* val;
 };
 cudaError_t launch_wcsr_build(const uint64_t* P, int64_t n, int64_t ldw, const WordIndex& x, cudaStream_t s);
+// Query rows that another form has begun (launch_smp_rows): of row r, words + 3 r ceil(n / 64) holds its frontier, the
+// constants it has reached and its source, ceil(n / 64) words each; levels[r] the levels done, or 0 when it is finished.
+struct RowState {
+    uint64_t* words;
+    int* levels;
+};
 cudaError_t launch_smp_packed(const WordIndex& x, const WordIndex& T, int64_t n, int64_t ldw, const uint64_t* src,
                               int64_t ldw_src, int64_t q, uint64_t* out, int64_t ldw_out, int* levels, int* qcounter,
-                              int reflexive, int sms, cudaStream_t s, Deadline dl);
+                              int reflexive, int sms, cudaStream_t s, Deadline dl, RowState from = RowState{nullptr, nullptr});
 // C = P | A B on packed rows through the word indexes of A and B (A = B = P: a squaring step); *changed (or null) is
 // raised when C != P
 cudaError_t launch_indexed_rows(const WordIndex& A, const WordIndex& B, const uint64_t* P, int64_t n, int64_t ldw,
@@ -369,13 +375,42 @@ cudaError_t launch_smp_tiles(const WordIndex& x, int64_t n, int64_t n1, int64_t 
                              bool derive, bool again, int* counts, unsigned long long* counter, int* levels, int max_levels,
                              int sms, cudaStream_t s, Deadline dl);
 // The expansion of a few query rows straight from R's packed rows (ld_r words, bits at columns >= n ignored), one cluster
-// of smp_rows_ctas() CTAs per row: 16, 8, 4 or 2, or 0 when q rows do not fit the GPU at once (or are more than
-// kRowsMaxQueries) or n is too large. Results and levels as launch_smp_tiles.
+// of plan.ctas CTAs per row: 16, 8, 4 or 2, or 0 when q rows do not fit the GPU at once (or are more than kRowsMaxQueries) or
+// n is too large. Results and levels as launch_smp_tiles, but for rows that stop (only with plan.may_stop and a `state`, and
+// *stopped is raised then): launch_smp_packed finishes those from the state.
 constexpr int64_t kRowsMaxQueries = 63;
-int smp_rows_ctas(int64_t n, int64_t q);
+struct RowQueryPlan {
+    int ctas;
+    bool may_stop;
+    int most;         // constants that a row reaches before it stops because reading their rows costs too much
+    int first_level;  // levels after which it may stop because more of them would
+    // what a level and a constant's row cost more than over word indexes, and what a row that stops has to gain (seconds)
+    float level_gain, row_gain, need;
+#ifdef __CUDACC__
+    // Whether a row that has reached `visited` of n constants after lv levels, `found` of them in the last one, has too many
+    // levels before it. Two kinds are told from the rows that end soon or fill up (visited ~ levels^alpha so far): a front that
+    // goes on widening like a grid's (alpha about 2), and after 96 levels a thin one that does not widen, a path, which is
+    // taken to go on for up to twice as long again. Either is taken to reach all constants, whose rows are cheap here.
+    __device__ __forceinline__ bool too_deep(int64_t n, int lv, int found, int visited) const {
+        if (lv < first_level || found == 0) return false;
+        const float l = static_cast<float>(lv), v = static_cast<float>(visited), left = static_cast<float>(n) / v;
+        const float alpha = fmaxf(1.0f, static_cast<float>(found) * l / v);
+        float more;
+        if (alpha >= 1.5f) {
+            if (alpha > 4.5f || 2 * found < lv) return false;
+            more = l * (exp2f(log2f(left) / alpha) - 1.0f);
+        } else {
+            if (lv < 96 || found > 8) return false;
+            more = l * fminf(2.0f, left - 1.0f);
+        }
+        return more * level_gain + (static_cast<float>(n) - v) * row_gain >= need;
+    }
+#endif
+};
+RowQueryPlan smp_rows_plan(int64_t n, int64_t q);
 cudaError_t launch_smp_rows(const uint64_t* R, int64_t ld_r, int64_t n, const uint64_t* src, int64_t ld_src, int64_t q,
-                            uint64_t* out, int64_t ld_out, int reflexive, int* levels, int max_levels, int ctas,
-                            cudaStream_t s, Deadline dl);
+                            uint64_t* out, int64_t ld_out, int reflexive, int* levels, int max_levels, const RowQueryPlan& plan,
+                            RowState state, int* stopped, cudaStream_t s, Deadline dl);
 // ---- a squaring restricted to the rows and columns that still hold zeros (thin.cu)
 // P, PT: bit rows (n_pad rows of ldw = n_pad / 64 words) of a matrix S with R <= S <= R' = R + R R and of S^T; Src, SrcT:
 // those of R and R^T (the same arrays when S = R). All are written by the squaring kernel's epilogue.

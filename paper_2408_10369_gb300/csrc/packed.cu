@@ -27,6 +27,7 @@
 //  * smp_sliced   Algorithm 2 for 64 sources at once, bit-sliced, for relations
 //                 too large for the tile form of frontier.cu.
 //  * insert_fact  one new fact into a transitive closure (rank-1 update).
+#include <algorithm>
 #include <atomic>
 
 #include "internal.h"
@@ -646,14 +647,17 @@ __device__ __forceinline__ void push_balanced(uint64_t d, int w, int lane, const
 
 // Algorithm 2 for one query row: the frontier expansion from the source row srcw(0 .. ) (words, bits >= n
 // ignored), visited set and result in V (ldw_out words), D / N / FL / GM the warp's shared-memory arrays
-// (sized for at least ldw words). Returns the levels run (the deepest BFS level + 1). Called by a whole warp.
+// (sized for at least ldw words). With `from` it goes on where the query-row kernel stopped after `lv` levels: from holds the
+// frontier and the visited set (ceil(n / 64) words each). Returns the levels run (the deepest BFS level + 1). Called by a
+// whole warp.
 template <class SrcWord>
 __device__ __forceinline__ int smp_expand_row(SrcWord srcw, uint64_t* __restrict__ V, int64_t ldw_out, int reflexive,
                                               const int64_t* __restrict__ wptr, const int32_t* __restrict__ widx,
                                               const uint64_t* __restrict__ wval, int64_t n, int64_t ldw,
                                               int max_levels, const Deadline& dl, const int64_t* __restrict__ wptrT,
                                               const int32_t* __restrict__ widxT, const uint64_t* __restrict__ wvalT,
-                                              uint64_t* D, uint64_t* N, uint16_t* FL, uint8_t* GM, int lane) {
+                                              uint64_t* D, uint64_t* N, uint16_t* FL, uint8_t* GM, int lane,
+                                              const uint64_t* __restrict__ from = nullptr, int lv = 0) {
     const unsigned lt = (1u << lane) - 1u;  // lanes below this one
     const int64_t wpr = (n + 63) / 64;
     // words of N form at most 64 groups of 2^gshift words; a push records the groups it wrote
@@ -664,12 +668,14 @@ __device__ __forceinline__ int smp_expand_row(SrcWord srcw, uint64_t* __restrict
     const float w_out = wptrT != nullptr ? static_cast<float>(wptr[2 * n]) / static_cast<float>(n) : 0.f;
     const float w_in = wptrT != nullptr ? static_cast<float>(wptrT[2 * n]) / static_cast<float>(n) : 0.f;
     // D = sources; FL = their nonzero words (ballot compaction); V = 0
-    int fcount = 0;
+    int fcount = 0, visited = 0;
     for (int64_t w0 = 0; w0 < ldw; w0 += 32) {
         const int64_t w = w0 + lane;
-        uint64_t s = 0;
+        uint64_t s = 0, v = 0;
         if (w < wpr) {
-            s = srcw(w);
+            s = from != nullptr ? from[w] : srcw(w);
+            if (from != nullptr) v = from[wpr + w];
+            visited += __popcll(v);
             const int64_t valid = n - w * 64;
             if (valid < 64) s &= (1ull << valid) - 1ull;
         }
@@ -677,15 +683,14 @@ __device__ __forceinline__ int smp_expand_row(SrcWord srcw, uint64_t* __restrict
             D[w] = s;
             N[w] = 0;
         }
-        if (w < ldw_out) V[w] = 0;
+        if (w < ldw_out) V[w] = v;
         const unsigned m = __ballot_sync(FULL, s != 0ull);
         if (s) FL[fcount + __popc(m & lt)] = static_cast<uint16_t>(w);
         fcount += __popc(m);
     }
     __syncwarp();
-    int lv = 0;
     bool pull = false;
-    int64_t nu = n;  // unvisited constants
+    int64_t nu = n - static_cast<int64_t>(__reduce_add_sync(FULL, static_cast<unsigned>(visited)));  // unvisited constants
     while (true) {
         if (dl.budget_ns && __shfl_sync(FULL, lane == 0 ? static_cast<int>(dl.past()) : 0, 0)) break;
         uint64_t gm = all_groups;  // groups of N that may be nonzero after this expansion
@@ -814,7 +819,7 @@ __global__ void __launch_bounds__(256, 4) smp_packed_kernel(const int64_t* __res
                                                          unsigned long long* qcounter, int reflexive, int max_levels,
                                                          Deadline dl, const int64_t* __restrict__ wptrT,
                                                          const int32_t* __restrict__ widxT,
-                                                         const uint64_t* __restrict__ wvalT) {
+                                                         const uint64_t* __restrict__ wvalT, RowState from) {
     extern __shared__ uint64_t sm[];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -829,8 +834,17 @@ __global__ void __launch_bounds__(256, 4) smp_packed_kernel(const int64_t* __res
         if (qi >= static_cast<unsigned long long>(q)) break;
         const uint64_t* srow = src + static_cast<int64_t>(qi) * ldw_src;
         uint64_t* V = out + static_cast<int64_t>(qi) * ldw_out;
-        const int lv = smp_expand_row([srow](int64_t w) { return srow[w]; }, V, ldw_out, reflexive, wptr, widx, wval,
-                                      n, ldw, max_levels, dl, wptrT, widxT, wvalT, D, N, FL, GM, lane);
+        const uint64_t* at = nullptr;
+        int lv = 0;
+        if (from.words != nullptr) {
+            lv = from.levels[qi];
+            if (lv == 0) continue;  // finished
+            const int64_t wpr = (n + 63) / 64;
+            at = from.words + static_cast<int64_t>(qi) * 3 * wpr;
+            srow = at + 2 * wpr;
+        }
+        lv = smp_expand_row([srow](int64_t w) { return srow[w]; }, V, ldw_out, reflexive, wptr, widx, wval, n, ldw,
+                            max_levels, dl, wptrT, widxT, wvalT, D, N, FL, GM, lane, at, lv);
         if (lane == 0) atomicMax(levels_max, lv);
         __syncwarp();
     }
@@ -1424,15 +1438,25 @@ __global__ void __launch_bounds__(kSlicedThreads) smp_sliced_kernel(const int64_
 // r ORs the rows of the frontier constants k = r mod C, four in flight per warp, into its own partial N; after a cluster
 // barrier it gathers its share of the words from every CTA's N, removes the visited constants and stores the new words
 // into every CTA's D; a second barrier ends the level. A query reads the row of each constant it reaches once, so it is
-// bound by the two barriers and the row latency per level (about 3 us) or, from some tens of thousands of constants on,
-// by the rows' bytes; no word index, no transpose and no column is needed. One warp per query over the word indexes of R
+// bound by the two barriers and the row latency per level (2.7 us at n = 5,000, 7 to 10 at 65,536) or, from some tens of
+// thousands of constants on, by the rows' bytes; no word index, no transpose and no column is needed. One warp per query over the word indexes of R
 // and R^T, which a call has to build first, took 302 us for a call with one query on n = 5,000 constants with 50 facts
-// each, 48 us now; n = 65,536 power law 6.1 ms, 0.55 ms now, and 16 queries 5.2 and 1.29 ms; a grid of n = 20,000 (117
-// levels) 1.63 and 0.57 ms, 16 queries 1.56 and 0.78 ms. For larger batches the indexes are shared and the forms that
-// use them stay.
+// each, 48 us now; n = 65,536 power law 6.1 ms, 0.55 ms now, and 16 queries 5.2 and 1.29 ms. For larger batches the indexes
+// are shared and the forms that use them stay.
+// Two kinds of rows would be slower here than over the indexes, and are not known from the start:
+// * A narrow frontier on its way through many levels (a path: one constant a level). Up to kNarrowN constants one warp
+//   then goes on alone, the words of a row in its lanes, without barriers (0.75 us a level). A path from its beginning, by
+//   levels of the cluster, over the indexes and so: n = 500: 1,336, 740 and 418 us; 5,000: 13.6, 6.8 and 3.8 ms.
+// * Beyond that size, deep or wide rows on large relations, whose levels or bytes cost more than building the indexes and
+//   going on there: the cluster writes down its frontier and visited set and stops (RowQueryPlan says when), and the call
+//   goes on from them over the indexes.
 constexpr int kRowsThreads = 512;
 constexpr int kRowsWarps = kRowsThreads / 32;
 constexpr int kRowsMaxCtas = 16;
+constexpr int kNarrowWords = 4;                          // words of a row in a lane of the warp that goes on alone
+constexpr int64_t kNarrowN = 32 * 64 * kNarrowWords;
+constexpr int kNarrowFrom = 8, kNarrowUntil = 16;       // constants of a frontier that it takes over, and gives back,
+constexpr int kNarrowAfter = 6;                          // and levels before it (most rows of dense relations end earlier)
 
 struct RowQueryArgs {
     const uint64_t* R;  // packed rows (bits at columns >= n ignored)
@@ -1445,12 +1469,97 @@ struct RowQueryArgs {
     int* levels_max;
     int max_levels;
     int reflexive;
+    RowQueryPlan plan;
+    RowState state;  // where a row that stops leaves its frontier, visited set and source (words null: none stops)
+    int* stopped;    // raised when one does
     Deadline dl;
 };
 
-__global__ void __launch_bounds__(kRowsThreads, 1) smp_rows_kernel(const RowQueryArgs a) {
+// Levels of a narrow frontier by one warp: until it is empty, has more than kNarrowUntil constants, or the levels or the time
+// are used up. The frontier and the visited constants are in its registers, lane l words l, l + 32, ... of a row; they come
+// from this CTA's frontier d_s and from every CTA's share of the visited ones, v_s (addresses in shared memory), and go back to
+// all of them. Returns the constants of the last frontier; *levels counts on, *stop: out of time. (Not inlined:
+// within the kernel's body it makes calls of few levels slower, 52 us instead of 46.)
+__device__ __noinline__ int narrow_levels(const uint64_t* __restrict__ R, int64_t ld_r, int n, int wpr, int share, int ctas,
+                                          uint32_t d_s, uint32_t v_s, int max_levels, Deadline dl, int* levels, int* stop) {
+    const int lane = threadIdx.x & 31;
+    uint64_t D[kNarrowWords], V[kNarrowWords], valid[kNarrowWords];
+#pragma unroll
+    for (int v = 0; v < kNarrowWords; ++v) {
+        const int w = 32 * v + lane, left = n - 64 * w;  // what lies beyond column n of a row is not a fact
+        D[v] = w < wpr ? ld_dsmem_u64(mapa_shared(d_s + 8u * w, 0)) : 0ull;
+        V[v] = w < wpr ? ld_dsmem_u64(mapa_shared(v_s + 8u * (w % share), w / share)) : 0ull;
+        valid[v] = left >= 64 ? ~0ull : left > 0 ? (1ull << left) - 1ull : 0ull;
+    }
+    int found = 0, lv = *levels;
+    do {
+        uint64_t acc[kNarrowWords];
+#pragma unroll
+        for (int v = 0; v < kNarrowWords; ++v) acc[v] = 0ull;
+#pragma unroll
+        for (int u = 0; u < kNarrowWords; ++u) {
+            unsigned m = __ballot_sync(FULL, D[u] != 0ull);
+            uint64_t bits = 0ull;
+            int kb = 0;
+            while (m != 0u || bits != 0ull) {
+                const uint64_t* row[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    row[q] = nullptr;
+                    if (bits == 0ull && m != 0u) {
+                        const int sl = __ffs(static_cast<int>(m)) - 1;
+                        m &= m - 1u;
+                        bits = __shfl_sync(FULL, D[u], sl);
+                        kb = (32 * u + sl) * 64;
+                    }
+                    if (bits != 0ull) {
+                        row[q] = R + static_cast<int64_t>(kb + __ffsll(static_cast<long long>(bits)) - 1) * ld_r + lane;
+                        bits &= bits - 1ull;
+                    }
+                }
+                uint64_t x[4][kNarrowWords];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int v = 0; v < kNarrowWords; ++v)
+                        x[q][v] = row[q] != nullptr && 32 * v + lane < wpr ? __ldg(row[q] + 32 * v) : 0ull;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int v = 0; v < kNarrowWords; ++v) acc[v] |= x[q][v];
+            }
+        }
+        unsigned c = 0;
+#pragma unroll
+        for (int v = 0; v < kNarrowWords; ++v) {
+            D[v] = acc[v] & valid[v] & ~V[v];
+            V[v] |= D[v];
+            c += static_cast<unsigned>(__popcll(D[v]));
+        }
+        found = static_cast<int>(__reduce_add_sync(FULL, c));
+        ++lv;
+        if ((lv & 15) == 0 && dl.budget_ns) *stop = __shfl_sync(FULL, lane == 0 ? static_cast<int>(dl.past()) : 0, 0);
+    } while (found > 0 && found <= kNarrowUntil && lv <= max_levels && *stop == 0);
+#pragma unroll
+    for (int v = 0; v < kNarrowWords; ++v) {
+        const int w = 32 * v + lane;
+        if (w < wpr) {
+            st_dsmem_u64(mapa_shared(v_s + 8u * (w % share), w / share), V[v]);
+            for (int c = 0; c < ctas; ++c) st_dsmem_u64(mapa_shared(d_s + 8u * w, c), D[v]);
+        }
+    }
+    *levels = lv;
+    return found;
+}
+
+// kNarrow: narrow frontiers go on in one warp (n <= kNarrowN); else rows may stop. (Two kernels: with both in one, unused, the
+// wide levels were 4 to 5 % slower.)
+template <bool kNarrow>
+__global__ void __launch_bounds__(kRowsThreads) smp_rows_kernel(const RowQueryArgs a) {
     extern __shared__ uint64_t rq_sm[];
-    __shared__ int s_flag[2][kRowsMaxCtas];  // by level parity, written by each CTA: 1 it found new constants, 2 stop
+    __shared__ int s_flag[2][kRowsMaxCtas];  // by level parity, by each CTA: 4 x the new constants it found, + 1: out of time, + 2: stop
+    __shared__ int s_found[2];               // by level parity: this CTA's new constants
+    __shared__ int s_narrow[3];              // after narrow levels: levels, constants of the frontier, out of time
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = static_cast<int>(cluster_ctarank()), ctas = static_cast<int>(cluster_nctarank());
     const int wpr = static_cast<int>((a.n + 63) >> 6);
@@ -1471,87 +1580,141 @@ __global__ void __launch_bounds__(kRowsThreads, 1) smp_rows_kernel(const RowQuer
         N[0][w] = N[1][w] = 0ull;
     }
     for (int w = tid; w < own; w += kRowsThreads) V[w] = 0ull;
+    if (tid < 2) s_found[tid] = 0;
     uint64_t mine = 0ull;  // this CTA's constants of a word: bits rank, rank + ctas, ... (ctas divides 64)
     for (int b = rank; b < 64; b += ctas) mine |= 1ull << b;
     cluster_sync();
-    int lv = 0;
+    int lv = 0, visited = 0, total = 0;  // constants reached, and those of the last level, of the whole relation
+    bool stopped = false;
+    int p = 0;
     while (true) {
-        const int p = lv & 1;
-        uint64_t* Np = N[p];
-        for (int c0 = 0; c0 < wpr; c0 += 256) {  // 256 words of the rows at a time: 8 per lane
-            uint64_t acc[8];
+        bool narrow = false;
+        for (;; p ^= 1) {
+            uint64_t* Np = N[p];
+            for (int c0 = 0; c0 < wpr; c0 += 256) {  // 256 words of the rows at a time: 8 per lane
+                uint64_t acc[8];
 #pragma unroll
-            for (int v = 0; v < 8; ++v) acc[v] = 0ull;
-            bool any = false;
-            for (int w0 = warp; w0 < wpr; w0 += kRowsThreads) {  // lane l: word w0 + kRowsWarps l
-                const int w = w0 + kRowsWarps * lane;
-                const uint64_t d = w < wpr ? D[w] & mine : 0ull;
-                unsigned m = __ballot_sync(FULL, d != 0ull);
-                any |= m != 0u;
-                uint64_t bits = 0ull;
-                int kb = 0;
-                while (m != 0u || bits != 0ull) {
-                    const uint64_t* row[4];
+                for (int v = 0; v < 8; ++v) acc[v] = 0ull;
+                bool any = false;
+                for (int w0 = warp; w0 < wpr; w0 += kRowsThreads) {  // lane l: word w0 + kRowsWarps l
+                    const int w = w0 + kRowsWarps * lane;
+                    const uint64_t d = w < wpr ? D[w] & mine : 0ull;
+                    unsigned m = __ballot_sync(FULL, d != 0ull);
+                    any |= m != 0u;
+                    uint64_t bits = 0ull;
+                    int kb = 0;
+                    while (m != 0u || bits != 0ull) {
+                        const uint64_t* row[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        row[q] = nullptr;
-                        if (bits == 0ull && m != 0u) {
-                            const int sl = __ffs(m) - 1;
-                            m &= m - 1u;
-                            bits = __shfl_sync(FULL, d, sl);
-                            kb = (w0 + kRowsWarps * sl) * 64;
+                        for (int q = 0; q < 4; ++q) {
+                            row[q] = nullptr;
+                            if (bits == 0ull && m != 0u) {
+                                const int sl = __ffs(m) - 1;
+                                m &= m - 1u;
+                                bits = __shfl_sync(FULL, d, sl);
+                                kb = (w0 + kRowsWarps * sl) * 64;
+                            }
+                            if (bits != 0ull) {
+                                row[q] = a.R + (kb + __ffsll(static_cast<long long>(bits)) - 1) * a.ld_r + c0 + lane;
+                                bits &= bits - 1ull;
+                            }
                         }
-                        if (bits != 0ull) {
-                            row[q] = a.R + (kb + __ffsll(static_cast<long long>(bits)) - 1) * a.ld_r + c0 + lane;
-                            bits &= bits - 1ull;
-                        }
+                        uint64_t x[4][8];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int v = 0; v < 8; ++v)
+                                x[q][v] = row[q] != nullptr && c0 + 32 * v + lane < wpr ? __ldg(row[q] + 32 * v) : 0ull;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int v = 0; v < 8; ++v) acc[v] |= x[q][v];
                     }
-                    uint64_t x[4][8];
+                }
+                if (any) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-#pragma unroll
-                        for (int v = 0; v < 8; ++v)
-                            x[q][v] = row[q] != nullptr && c0 + 32 * v + lane < wpr ? __ldg(row[q] + 32 * v) : 0ull;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-#pragma unroll
-                        for (int v = 0; v < 8; ++v) acc[v] |= x[q][v];
+                    for (int v = 0; v < 8; ++v)
+                        if (acc[v] != 0ull)  // zero beyond wpr
+                            atomicOr(reinterpret_cast<unsigned long long*>(&Np[c0 + 32 * v + lane]),
+                                     static_cast<unsigned long long>(acc[v]));
                 }
             }
-            if (any) {
+            cluster_sync();  // every CTA's N is complete, and nobody reads D any more
+            unsigned found = 0;
+            const uint32_t n_s = smem_u32(Np + base), d_s = smem_u32(D + base);
+            for (int i = tid; i < own; i += kRowsThreads) {
+                uint64_t x = 0ull;
 #pragma unroll
-                for (int v = 0; v < 8; ++v)
-                    if (acc[v] != 0ull)  // zero beyond wpr
-                        atomicOr(reinterpret_cast<unsigned long long*>(&Np[c0 + 32 * v + lane]),
-                                 static_cast<unsigned long long>(acc[v]));
+                for (int c = 0; c < kRowsMaxCtas; ++c)
+                    if (c < ctas) x |= ld_dsmem_u64(mapa_shared(n_s + 8u * i, c));
+                x &= valid(base + i) & ~V[i];
+                V[i] |= x;
+                found += static_cast<unsigned>(__popcll(x));
+                for (int c = 0; c < ctas; ++c) st_dsmem_u64(mapa_shared(d_s + 8u * i, c), x);
+            }
+            // the other N was last read before the previous barrier; the next level fills it
+            for (int w = tid; w < wpr; w += kRowsThreads) N[p ^ 1][w] = 0ull;
+            found = __reduce_add_sync(FULL, found);
+            if (lane == 0 && found != 0u) atomicAdd(&s_found[p], static_cast<int>(found));
+            __syncthreads();
+            if (tid < ctas) {
+                int stop = rank == 0 && a.dl.budget_ns && a.dl.past() ? 1 : 0;
+                // every 16 levels, by the counts after the level before this one: too deep, or another row has stopped (the
+                // indexes are built then, and would wait for this one)
+                if (!kNarrow && rank == 0 && a.state.words != nullptr && lv > 0 && (lv & 15) == 0 &&
+                    (*static_cast<volatile int*>(a.stopped) != 0 || a.plan.too_deep(a.n, lv, total, visited)))
+                    stop |= 2;
+                st_dsmem_s32(mapa_shared(smem_u32(&s_flag[p][rank]), tid), 4 * s_found[p] + stop);
+            }
+            if (tid == 0) s_found[p ^ 1] = 0;
+            cluster_sync();  // the new D and the flags are in place
+            const unsigned flags = lane < ctas ? static_cast<unsigned>(s_flag[p][lane]) : 0u;
+            const unsigned stop = __reduce_or_sync(FULL, flags & 3u);
+            total = static_cast<int>(__reduce_add_sync(FULL, flags >> 2));
+            visited += total;
+            ++lv;
+            if (total == 0 || (stop & 1u) != 0u || lv > a.max_levels) break;  // the same in every CTA: no barrier is left open
+            if (kNarrow && lv >= kNarrowAfter && total <= kNarrowFrom) {
+                narrow = true;
+                break;
+            }
+            if (!kNarrow && a.state.words != nullptr && (stop != 0u || visited > a.plan.most)) {
+                stopped = true;
+                break;
             }
         }
-        cluster_sync();  // every CTA's N is complete, and nobody reads D any more
-        bool grew = false;
-        const uint32_t n_s = smem_u32(Np + base), d_s = smem_u32(D + base);
-        for (int i = tid; i < own; i += kRowsThreads) {
-            uint64_t x = 0ull;
-#pragma unroll
-            for (int c = 0; c < kRowsMaxCtas; ++c)
-                if (c < ctas) x |= ld_dsmem_u64(mapa_shared(n_s + 8u * i, c));
-            x &= valid(base + i) & ~V[i];
-            V[i] |= x;
-            grew |= x != 0ull;
-            for (int c = 0; c < ctas; ++c) st_dsmem_u64(mapa_shared(d_s + 8u * i, c), x);
+        if (!kNarrow || !narrow) break;
+        // one warp goes on; the others wait at the barrier (each level of its loop ends)
+        if (rank == 0 && warp == 0) {
+            int levels = lv, out_of_time = 0;
+            const int last = narrow_levels(a.R, a.ld_r, static_cast<int>(a.n), wpr, share, ctas, smem_u32(D), smem_u32(V),
+                                           a.max_levels, a.dl, &levels, &out_of_time);
+            if (lane < ctas) {
+                st_dsmem_s32(mapa_shared(smem_u32(&s_narrow[0]), lane), levels);
+                st_dsmem_s32(mapa_shared(smem_u32(&s_narrow[1]), lane), last);
+                st_dsmem_s32(mapa_shared(smem_u32(&s_narrow[2]), lane), out_of_time);
+            }
+            __syncwarp();
         }
-        // the other N was last read before the previous barrier; the next level fills it
-        for (int w = tid; w < wpr; w += kRowsThreads) N[p ^ 1][w] = 0ull;
-        const int any = __syncthreads_or(grew);
-        if (tid < ctas) {
-            const int stop = rank == 0 && a.dl.budget_ns && a.dl.past() ? 2 : 0;
-            st_dsmem_s32(mapa_shared(smem_u32(&s_flag[p][rank]), tid), (any ? 1 : 0) | stop);
-        }
-        cluster_sync();  // the new D and the flags are in place
-        int f = 0;
-        for (int c = 0; c < ctas; ++c) f |= s_flag[p][c];
-        ++lv;
-        if ((f & 1) == 0 || (f & 2) != 0 || lv > a.max_levels) break;  // the same in every CTA: no barrier is left open
+        cluster_sync();
+        lv = s_narrow[0];
+        if (s_narrow[1] == 0 || s_narrow[2] != 0 || lv > a.max_levels) break;
+        p ^= 1;  // (N of the last level is cleared by the next one)
     }
+    if (!kNarrow && stopped) {
+        uint64_t* at = a.state.words + static_cast<int64_t>(cluster_id_x()) * 3 * wpr;
+        for (int i = tid; i < own; i += kRowsThreads) {
+            at[base + i] = D[base + i];
+            at[wpr + base + i] = V[i];
+            at[2 * wpr + base + i] = src[base + i] & valid(base + i);
+        }
+        if (rank == 0 && tid == 0) {
+            a.state.levels[cluster_id_x()] = lv;
+            atomicOr(a.stopped, 1);
+        }
+        return;
+    }
+    if (!kNarrow && a.state.words != nullptr && rank == 0 && tid == 0) a.state.levels[cluster_id_x()] = 0;
     if (rank == 0 && tid == 0) atomicMax(a.levels_max, lv);
     for (int i = tid; i < own; i += kRowsThreads)
         out[base + i] = V[i] | (a.reflexive ? src[base + i] & valid(base + i) : 0ull);
@@ -1689,13 +1852,16 @@ cudaLaunchConfig_t smp_rows_config(int64_t n, int64_t q, int ctas, cudaStream_t 
 // Shared memory of a CTA in steps of kRowsSmemStep, of which it has at most kRowsSmemSteps.
 constexpr size_t kRowsSmemStep = 16384, kRowsSmemSteps = 13;
 
-cudaError_t smp_rows_attributes() {
-    const cudaError_t e = allow_smem(smp_rows_kernel, kRowsSmemStep * kRowsSmemSteps);
-    return e != cudaSuccess ? e : cudaFuncSetAttribute(smp_rows_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+using RowsKernel = void (*)(RowQueryArgs);
+RowsKernel rows_kernel(int64_t n) { return n <= kNarrowN ? smp_rows_kernel<true> : smp_rows_kernel<false>; }
+
+cudaError_t smp_rows_attributes(RowsKernel kernel) {
+    const cudaError_t e = allow_smem(kernel, kRowsSmemStep * kRowsSmemSteps);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 }  // namespace
 
-int smp_rows_ctas(int64_t n, int64_t q) {
+static int rows_ctas(int64_t n, int64_t q) {
     // resident clusters by (device, cluster size, steps of shared memory), asked once each since the query costs more than
     // the launch (0: not asked; else the count + 1); written by any thread, always with the same value
     static std::atomic<unsigned char> known[16][4][kRowsSmemSteps + 1] = {};
@@ -1716,8 +1882,8 @@ int smp_rows_ctas(int64_t n, int64_t q) {
             cudaLaunchConfig_t cfg = smp_rows_config(n, 1, ctas, nullptr, &at);
             cfg.dynamicSmemBytes = step * kRowsSmemStep;
             clusters = 0;
-            if (smp_rows_attributes() != cudaSuccess ||
-                cudaOccupancyMaxActiveClusters(&clusters, smp_rows_kernel, &cfg) != cudaSuccess) {
+            if (smp_rows_attributes(rows_kernel(n)) != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&clusters, rows_kernel(n), &cfg) != cudaSuccess) {
                 cudaGetLastError();
                 continue;  // asked again by the next call
             }
@@ -1729,15 +1895,45 @@ int smp_rows_ctas(int64_t n, int64_t q) {
     return 0;
 }
 
+// When a row stops, from query rows of uniform random, power-law, grid and path relations of 500 to 262,144 constants. Here a
+// level takes 2.3 us + 0.1 ns n (half as much again with several clusters) + 3e-16 s n^2, and all rows' bytes come at 9.2 TB/s
+// or 98 GB/s a CTA; over the indexes it is 60 us + 1.3e-13 s n^2 to build them, 1.35 us a level and 40 ns a reached constant.
+// A row stops when going on is predicted to cost more by twice the build, and not before it has cost 15 % of what it would have
+// cost there: narrow rows on large relations end within a few levels, where the build alone is 0.6 ms at n = 65,536
+// and 9 ms at 262,144. Calls that never stop, that stop, and over the indexes from the start:
+//     63 rows, uniform random, n = 131,072, 3 facts a row    16.1     8.9     8.0 ms
+//     63 rows, uniform random, n = 262,144, 2 facts a row    57.8    21.9    18.9 ms
+//     63 rows, grid, n = 65,536                              10.0     6.0     4.8 ms
+//     1 row, path, n = 65,536                                 502      92      91 ms
+// and where the prediction fails: 63 rows, uniform random, n = 65,536, 1.2 facts a row 1.9, 2.6 and 2.1 ms; 1 row of a
+// grid, n = 131,072, 8.8, 10.3 and 9.5 ms.
+RowQueryPlan smp_rows_plan(int64_t n, int64_t q) {
+    RowQueryPlan p{};
+    p.ctas = rows_ctas(n, q);
+    p.may_stop = p.ctas > 0 && n > kNarrowN;
+    if (!p.may_stop) return p;
+    const double nn = static_cast<double>(n);
+    const double build = 60e-6 + 1.3e-13 * nn * nn, index_level = 1.35e-6, index_row = 40e-9;
+    const double level = 2.3e-6 + 0.1e-9 * nn * (q > 1 ? 1.5 : 1.0) + 3e-16 * nn * nn;
+    const double ctas = static_cast<double>(q) * p.ctas, row = nn / 8.0 * static_cast<double>(q) / std::min(9.2e12, 98e9 * ctas);
+    const double least = 0.15 * (build + nn * index_row);
+    p.level_gain = static_cast<float>(level - index_level);
+    p.row_gain = static_cast<float>(row - index_row);
+    p.need = static_cast<float>(2.0 * build);
+    p.first_level = std::max(32, static_cast<int>(least / level));
+    p.most = nn * (row - index_row) >= 2.0 * build ? static_cast<int>(least / row) : 0x7FFFFFFF;
+    return p;
+}
+
 cudaError_t launch_smp_rows(const uint64_t* R, int64_t ld_r, int64_t n, const uint64_t* src, int64_t ld_src, int64_t q,
-                            uint64_t* out, int64_t ld_out, int reflexive, int* levels, int max_levels, int ctas,
-                            cudaStream_t s, Deadline dl) {
+                            uint64_t* out, int64_t ld_out, int reflexive, int* levels, int max_levels, const RowQueryPlan& plan,
+                            RowState state, int* stopped, cudaStream_t s, Deadline dl) {
     cudaLaunchAttribute at;
-    const cudaLaunchConfig_t cfg = smp_rows_config(n, q, ctas, s, &at);
-    const cudaError_t e = smp_rows_attributes();
+    const cudaLaunchConfig_t cfg = smp_rows_config(n, q, plan.ctas, s, &at);
+    const cudaError_t e = smp_rows_attributes(rows_kernel(n));
     if (e != cudaSuccess) return e;
-    const RowQueryArgs a{R, ld_r, n, src, ld_src, out, ld_out, levels, max_levels, reflexive, dl};
-    return cudaLaunchKernelEx(&cfg, smp_rows_kernel, a);
+    const RowQueryArgs a{R, ld_r, n, src, ld_src, out, ld_out, levels, max_levels, reflexive, plan, state, stopped, dl};
+    return cudaLaunchKernelEx(&cfg, rows_kernel(n), a);
 }
 
 cudaError_t launch_square_growth(const WordIndex& x, int64_t n, int64_t ldw, unsigned long long* out, int sms, cudaStream_t s,
@@ -1765,7 +1961,7 @@ cudaError_t launch_indexed_cost(const WordIndex& A, const WordIndex& B, int64_t 
 
 cudaError_t launch_smp_packed(const WordIndex& x, const WordIndex& T, int64_t n, int64_t ldw, const uint64_t* src,
                               int64_t ldw_src, int64_t q, uint64_t* out, int64_t ldw_out, int* levels, int* qcounter,
-                              int reflexive, int sms, cudaStream_t s, Deadline dl) {
+                              int reflexive, int sms, cudaStream_t s, Deadline dl, RowState from) {
     // blocks of 1-8 warps, chosen so that as many warps as possible fit an SM's shared memory
     const int64_t per_warp = smp_warp_bytes(ldw);
     if (per_warp > static_cast<int64_t>(kMostWarpSmem)) return cudaErrorInvalidValue;
@@ -1782,7 +1978,7 @@ cudaError_t launch_smp_packed(const WordIndex& x, const WordIndex& T, int64_t n,
     const int max_levels = static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF);
     smp_packed_kernel<<<static_cast<int>(blocks), warps * 32, smem, s>>>(
         x.ptr, x.idx, x.val, n, ldw, src, ldw_src, q, out, ldw_out, levels,
-        reinterpret_cast<unsigned long long*>(qcounter), reflexive, max_levels, dl, T.ptr, T.idx, T.val);
+        reinterpret_cast<unsigned long long*>(qcounter), reflexive, max_levels, dl, T.ptr, T.idx, T.val, from);
     return cudaGetLastError();
 }
 
