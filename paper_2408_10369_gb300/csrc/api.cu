@@ -859,7 +859,7 @@ bmlp_status index_buffers(bmlp_ctx* ctx, int64_t n, int64_t ldw, int slot_ptr, i
 
 // Packed squaring fixpoint on P[0] (n rows x ldw words). *res = R1+. While fewer than half of R's words are
 // nonzero a squaring runs through R's word index (indexed_rows_kernel: only the nonzero words of the named rows are
-// ORed in, and the step streams R in and R' out), after that as the whole-row product (product_packed_kernel); a
+// ORed in, and the step streams R in and R' out), after that as the whole-row product (launch_product_packed); a
 // squaring that widens the rows past half their words hands the next ones to the whole-row product. *res_index (when
 // asked for) is the word index of the result when the last squaring was a word-indexed one, else its ptr is null.
 bmlp_status rms_packed_loop(bmlp_ctx* ctx, int64_t n, int64_t ldw, uint64_t* P[2], int max_iters,
@@ -1383,11 +1383,9 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         ctx->stats.product_launches++;
         ctx->stats.launches += 7;
         ctx->stats.sliced_closures++;
-        CK(cudaMemcpyAsync(ctx->h_ctl + CTL_HOST_I64, smp_tile_top_degree(prep, n), sizeof(int), cudaMemcpyDeviceToHost, s),
-           "read largest in-degree");
         ST(read_ctl(ctx, s, nullptr));
         ST(tm.collect());
-        const int top_degree = ctx->h_ctl[CTL_HOST_I64];
+        const int top_degree = ctx->h_ctl[CTL_PSTAT + 3];
         if (derive && ctx->h_ctl[CTL_PSTAT + 2] > ctx->h_ctl[CTL_LEVELS]) {
             // derived rows whose level count is not certain could be the deepest ones
             CK(tiles(true), "tile frontier kernel launch");

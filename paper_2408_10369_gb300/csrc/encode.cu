@@ -695,7 +695,7 @@ void launch_bytes_to_packed(const uint8_t* R, int64_t ld, int64_t rows, int64_t 
 }
 
 // Runs of the byte <-> bit converters: whole rows while a row has at most kUnitCols bytes, small enough that the runs
-// give each SM two blocks, but at least 2 KB.
+// give each of 152 SMs two blocks (a bound of their size only: any number of SMs takes them in turn), but at least 2 KB.
 static int64_t byte_units(int64_t n, int* rows_per, int* segs) {
     if (n > kUnitCols) {
         *rows_per = 1;

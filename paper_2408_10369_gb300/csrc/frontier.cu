@@ -43,7 +43,7 @@ constexpr int kUnclear = 1 << 30;        // in info: the row's deepest constants
 struct Lists {
     // `prep`, filled before the sizes are known on the host
     int32_t* deg;       // in-degree of each constant
-    int32_t* meta;      // [0] heavy constants, [1] the largest in-degree
+    int32_t* meta;      // [0] heavy constants
     int32_t* root;      // of each constant: the constant whose row its own follows from (itself: its row is expanded)
     int32_t* hops;      // steps to it; -1: the row is empty
     int32_t* rows;      // the rows to expand
@@ -140,7 +140,7 @@ __device__ __forceinline__ int only_fact(const WordIndex& x, int c, bool* empty)
     return j != c ? j : -1;
 }
 
-// counts[0] = constants that something reaches, counts[1] = rows to expand; the largest in-degree; and with `derive` which
+// counts[0] = constants that something reaches, counts[1] = rows to expand, counts[3] = the largest in-degree; and with `derive` which
 // rows those are: a row with one fact, c -> d, is d's row and d, so only the rows at the ends of such chains are expanded,
 // if they have facts at all. (A chain of more than kMaxHops, or a cycle, is expanded from its beginning.)
 __global__ void __launch_bounds__(kPrepThreads) lists_rows_kernel(const WordIndex x, int n, Lists l, int derive, int* counts) {
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kPrepThreads) lists_rows_kernel(const WordInde
     if (threadIdx.x == 0) {
         if (s_reached) atomicAdd(counts, s_reached);
         s_base = s_expand ? atomicAdd(counts + 1, s_expand) : 0;
-        if (s_top) atomicMax(&l.meta[1], s_top);
+        if (s_top) atomicMax(counts + 3, s_top);
     }
     __syncthreads();
     if (mine >= 0) l.rows[s_base + mine] = c;
@@ -764,8 +764,6 @@ int smp_tile_width(int64_t n1, int64_t rows, int sms) {
 
 size_t smp_tile_prep_bytes(int64_t n) { return static_cast<size_t>(5 * align64(n) + 64) * 4; }
 
-const int* smp_tile_top_degree(void* prep, int64_t n) { return lists_of(prep, nullptr, n).meta + 1; }
-
 size_t smp_tile_bytes(int64_t n, int64_t n1, int64_t ones, int width, int sms) {
     // words of the work area, lists (each tile's longest list, rounded up to a step), V and Dn of every CTA
     const int64_t ints = 4 * align64(n) + align64(n + n / 32 + 2) + kBins;
@@ -777,7 +775,7 @@ size_t smp_tile_bytes(int64_t n, int64_t n1, int64_t ones, int width, int sms) {
 cudaError_t launch_smp_tile_prep(const WordIndex& x, int64_t n, void* prep, int* counts, bool derive, int sms, cudaStream_t s) {
     const Lists l = lists_of(prep, nullptr, n);
     cudaError_t e = cudaMemsetAsync(l.deg, 0, static_cast<size_t>(align64(n) + 64) * 4, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, 3 * sizeof(int), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, 4 * sizeof(int), s);
     if (e != cudaSuccess) return e;
     const int rows_grid = static_cast<int>((n + 7) / 8 < sms * 8 ? (n + 7) / 8 : sms * 8);
     const int each = static_cast<int>((n + kPrepThreads - 1) / kPrepThreads);

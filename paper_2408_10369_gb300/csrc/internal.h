@@ -358,18 +358,17 @@ cudaError_t launch_smp_sliced(const WordIndex& T, int64_t n, uint64_t* scratch, 
                               int* levels, int max_levels, int sms, cudaStream_t s, Deadline dl);
 // The same expansion with the whole frontier of a batch in one SM's shared memory (frontier.cu; n <= 65,536): the rows
 // of src (ld_src words each), or of every constant when src is null, into out (ld_out words each), OR-ed with the source
-// row when reflexive. x: the word index of R, ones: its ones. In two parts, between which the host reads three counts:
+// row when reflexive. x: the word index of R, ones: its ones. In two parts, between which the host reads the counts:
 // launch_smp_tile_prep (prep: smp_tile_prep_bytes) counts the constants that something reaches (counts[0] = n1) and the
 // rows to expand (counts[1]; with `derive` those that do not follow from another row, else n). launch_smp_tiles expands
 // `rows` rows (q, or counts[1]), smp_tile_width(n1, rows) of them in a batch (0: n1 is too large; scratch:
 // smp_tile_bytes), and forms the derived ones. *counter = 0 and *levels = 0 beforehand; *levels receives the largest level
 // count. If counts[2] is then larger than *levels, a second call with `again` (same arguments) makes *levels exact.
-// *smp_tile_top_degree: the largest in-degree.
+// counts[3] is the largest in-degree.
 size_t smp_tile_prep_bytes(int64_t n);
 cudaError_t launch_smp_tile_prep(const WordIndex& x, int64_t n, void* prep, int* counts, bool derive, int sms, cudaStream_t s);
 int smp_tile_width(int64_t n1, int64_t rows, int sms);
 size_t smp_tile_bytes(int64_t n, int64_t n1, int64_t ones, int width, int sms);
-const int* smp_tile_top_degree(void* prep, int64_t n);
 cudaError_t launch_smp_tiles(const WordIndex& x, int64_t n, int64_t n1, int64_t ones, const uint64_t* src, int64_t ld_src,
                              int64_t rows, uint64_t* out, int64_t ld_out, int reflexive, int width, void* prep, void* scratch,
                              bool derive, bool again, int* counts, unsigned long long* counter, int* levels, int max_levels,

@@ -43,7 +43,7 @@ struct SmallArgs {
 };
 
 // All CTAs of the grid have arrived `round` times (they are resident at once: a cooperative launch). False if that takes
-// longer than the bound, or another CTA gave up.
+// longer than the bound; each CTA waits for its own (one that gave up never arrives, so the others' run out soon after).
 __device__ __forceinline__ bool grid_arrive_wait(const SmallArgs& a, unsigned round, int* s_ok) {
     __syncthreads();
     if (threadIdx.x == 0) {
