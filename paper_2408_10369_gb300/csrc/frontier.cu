@@ -810,7 +810,8 @@ cudaError_t launch_smp_tiles(const WordIndex& x, int64_t n, int64_t n1, int64_t 
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int64_t batches = (rows + width - 1) / width;
+    // the rows expanded after all are as many as the device finds, up to all of them
+    const int64_t batches = ((again ? n : rows) + width - 1) / width;
     const int grid = static_cast<int>(batches < sms ? batches : sms);
     TileArgs a{};
     a.l = l;
