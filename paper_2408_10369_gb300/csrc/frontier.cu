@@ -19,7 +19,9 @@
 // come last in the new numbers and have no place in D, V and the lists, and their facts are visited directly when they are
 // sources. And in a closure a row with one fact, c -> d, is d's row and d: only the rows at the ends of such chains are
 // expanded (batches from a list of rows), the others are copied afterwards. Their depths follow from the expanded row's,
-// except where the deepest constants of that row all lie on chains to it (lists_rows_kernel, derived_rows_kernel).
+// except where the deepest constants of that row all lie on chains to it and the other row's chain has more than one step
+// (lists_rows_kernel, derived_rows_kernel): such rows are expanded after all if they could be the deepest. Rows one step from
+// a hub that only they lead to, n = 30,000: 795 us, 1,573 with those rows expanded too; n = 4,200: 223 and 280 us.
 // Measured: closure of a power-law relation, n = 20,011 (32 levels; 64 % of the rows have one fact and 22 % of the
 // constants are not reached), the whole call: 6,590 us with clusters, 1,690 with every row expanded, 680 now; 4,096 query
 // rows on n = 65,536 (30 levels) 4,290, 1,740 (16 rows a batch) and 1,375 us (32 rows, one round of the SMs).
@@ -37,7 +39,8 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kPrepThreads = 256;
 constexpr int kMaxHops = 32;             // longest chain of one-fact rows that a row is derived over
 constexpr int kEmptyRoot = 1 << 30;      // in hops: the row at the end is empty
-constexpr int kUnclear = 1 << 30;        // in info: the row's deepest constants all have this row as their root
+constexpr int kUnclear = 1 << 30;        // in info: the row's deepest constants all have this row as their root,
+constexpr int kRootOnly = 1 << 29;       // and the only one is the row's own
 
 // Layout of the work areas: int32 words, then the 16-bit neighbour numbers.
 struct Lists {
@@ -47,7 +50,7 @@ struct Lists {
     int32_t* root;      // of each constant: the constant whose row its own follows from (itself: its row is expanded)
     int32_t* hops;      // steps to it; -1: the row is empty
     int32_t* rows;      // the rows to expand
-    int32_t* info;      // of each expanded row: its depth, and kUnclear
+    int32_t* info;      // of each expanded row: its depth, and kUnclear, kRootOnly
     // `scratch`
     int32_t* red;       // in-degree over constants that are reached themselves; counted down to 0 by the fill
     int32_t* rank;      // new number of each constant
@@ -521,7 +524,7 @@ __global__ void __launch_bounds__(kThreads, 1) smp_tile_kernel(const TileArgs a)
     using Word = typename S::Word;
     extern __shared__ __align__(16) unsigned char ti_sm[];
     __shared__ long long s_batch;
-    __shared__ unsigned long long s_active, s_pushed, s_clear;
+    __shared__ unsigned long long s_active, s_pushed, s_clear, s_more;
     __shared__ int s_stop, s_row[64];
     constexpr int VEC = 16 / static_cast<int>(sizeof(T));  // words of a 16-byte copy
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -597,7 +600,7 @@ __global__ void __launch_bounds__(kThreads, 1) smp_tile_kernel(const TileArgs a)
         int lv = 0;
         while (true) {
             if (tid == 0) {
-                s_active = s_clear = 0ull;
+                s_active = s_clear = s_more = 0ull;
                 s_stop = a.dl.budget_ns && a.dl.past() ? 1 : 0;
             }
             __syncthreads();  // D, V, the tiles' starts and the flags are in place
@@ -612,8 +615,9 @@ __global__ void __launch_bounds__(kThreads, 1) smp_tile_kernel(const TileArgs a)
             act = static_cast<T>(lv == 0 ? s_active | s_pushed : s_active);
             const T ended = static_cast<T>(before & ~act);
             if (a.info != nullptr && ended) {
-                // rows whose deepest constants are those of D (found one level ago): whether one of them has another root
-                T other = 0;
+                // rows whose deepest constants are those of D (found one level ago): whether one of them has another root, and
+                // whether one of this root is another constant than it
+                T other = 0, more = 0;
                 if (lv > 0)
                     for (int k = tid; k < n1; k += kThreads) {
                         unsigned long long w = static_cast<unsigned long long>(D[k] & ended);
@@ -621,16 +625,23 @@ __global__ void __launch_bounds__(kThreads, 1) smp_tile_kernel(const TileArgs a)
                             const int root = a.l.rroot[k];
                             for (unsigned long long x = w; x; x &= x - 1ull) {
                                 const int j = __ffsll(static_cast<long long>(x)) - 1;
-                                if (s_row[j] == root) w &= ~(1ull << j);
+                                if (s_row[j] == root) {
+                                    w &= ~(1ull << j);
+                                    if (a.l.rank[root] != k) more |= static_cast<T>(T(1) << j);
+                                }
                             }
                             other |= static_cast<T>(w);
                         }
                     }
                 other = or_warp(other);
+                more = or_warp(more);
                 if (lane == 0 && other) atomicOr(&s_clear, static_cast<unsigned long long>(other));
+                if (lane == 0 && more) atomicOr(&s_more, static_cast<unsigned long long>(more));
                 __syncthreads();
                 if (tid < cnt && ((static_cast<unsigned long long>(ended) >> tid) & 1ull))
-                    a.info[s_row[tid]] = lv > 0 && !((s_clear >> tid) & 1ull) ? lv | kUnclear : lv;
+                    a.info[s_row[tid]] = lv > 0 && !((s_clear >> tid) & 1ull)
+                                             ? lv | kUnclear | ((s_more >> tid) & 1ull ? 0 : kRootOnly)
+                                             : lv;
             }
             ++lv;
             if (act == 0 || lv > a.max_levels) break;
@@ -681,6 +692,14 @@ __global__ void __launch_bounds__(kThreads, 1) smp_tile_kernel(const TileArgs a)
     }
 }
 
+// Level count of a row of `hops` steps to an expanded row of info d, if it is certain, else an upper bound. The chain reaches
+// each of its constants within its steps, the expanded row's others come behind it. One step reaches the root alone: where the
+// root is the only constant of the deepest level, the level before it counts (it holds others), else that level does.
+__device__ __forceinline__ int derived_levels(int hops, int d, bool* certain) {
+    *certain = (d & kUnclear) == 0 || hops == 1;
+    return hops + (d & ~(kUnclear | kRootOnly)) + 1 - ((d & kRootOnly) != 0 ? 1 : 0);
+}
+
 // Rows that follow from an expanded row or from none: that row and the constants of the chain to it, a warp per row.
 // *levels: the largest level count of those whose depth is certain; counts[2] that of the others if it were what their
 // chain adds to the expanded row's (it is less when the deepest constants of that row all lie on their chain).
@@ -704,9 +723,10 @@ __global__ void __launch_bounds__(kPrepThreads) derived_rows_kernel(const WordIn
         }
         __syncwarp();
         if (mine >= 0) atomicOr(reinterpret_cast<unsigned long long*>(row) + (mine >> 6), 1ull << (mine & 63));
-        const int d = empty ? 0 : l.info[root], lv = hops + (d & ~kUnclear) + 1;
-        if (d & kUnclear) unclear = max(unclear, lv);
-        else top = max(top, lv);
+        bool certain = true;
+        const int lv = derived_levels(hops, empty ? 0 : l.info[root], &certain);
+        if (certain) top = max(top, lv);
+        else unclear = max(unclear, lv);
     }
     if (lane == 0) {
         if (top > 0) atomicMax(levels, top);
@@ -718,8 +738,8 @@ __global__ void __launch_bounds__(kPrepThreads) derived_rows_kernel(const WordIn
 __global__ void __launch_bounds__(kPrepThreads) unclear_rows_kernel(int n, Lists l, const int* levels, int* counts) {
     const int i = blockIdx.x * kPrepThreads + threadIdx.x;
     if (i >= n || l.root[i] == i || (l.hops[i] & kEmptyRoot)) return;
-    const int d = l.info[l.root[i]];
-    if ((d & kUnclear) && l.hops[i] + (d & ~kUnclear) + 1 > *levels) l.rows[atomicAdd(counts + 1, 1)] = i;
+    bool certain = true;
+    if (derived_levels(l.hops[i], l.info[l.root[i]], &certain) > *levels && !certain) l.rows[atomicAdd(counts + 1, 1)] = i;
 }
 
 // Shared memory of a CTA with `kept` of V, Dn in it.
