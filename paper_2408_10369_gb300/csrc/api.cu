@@ -108,9 +108,11 @@ constexpr int WS_THIN_P2 = 42;
 constexpr int WS_ROWS = 43;
 // The facts of an insertion (checked copy) and the chunk kernels' scratch.
 constexpr int WS_INS_FACTS = 38, WS_INS_SCRATCH = 39;
-// Facts from which an insertion runs in chunks of three launches instead of one launch per fact (n = 14,541: 19.5 us
-// for one fact and 23.1 for two by single launches, 25.6 us for three to eight as a chunk).
-constexpr int64_t kInsertChunkMin = 3;
+// Facts from which an insertion runs in chunks of three launches instead of one launch per fact. The whole call: three facts
+// by single launches and as a chunk, which is ordered with the insertion before it, bit rows, n = 300 to 3,000: 37 to 41 us
+// and 41 to 46, 8,192: 43 and 43, 14,541: 50 and 49, 20,000: 57 and 52 (bytes: 47 to 57, 50 to 58; 83, 83; 211, 206; 411,
+// 403). Four facts, n = 300 to 8,192: 42 to 46 and 44 to 48; 20,000: 65 and 55. Two, 20,000: 49 by single launches.
+constexpr int64_t insert_chunk_min(int64_t n) { return n <= 8192 ? 4 : 3; }
 constexpr int64_t kSquareMinN = 4096;
 // Bits per nonzero word of R from which a whole-row bit-row squaring uses the Four Russians tables instead of
 // gathering the named rows (measured at n = 8,192 and 16,384: equal times at 9.5 and 11.5 bits).
@@ -1808,8 +1810,8 @@ static bmlp_status core_insert(bmlp_ctx* ctx, void* closure, int64_t n, int32_t 
     // a capture records launches only: the facts travel as their arguments, since the copy of a chunk's would be replayed
     // from host memory that is gone by then, and its workspaces belong to whichever call comes next
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (m >= kInsertChunkMin && cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
-    bool chunks = m >= kInsertChunkMin && capture == cudaStreamCaptureStatusNone;
+    if (m >= insert_chunk_min(n) && cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+    bool chunks = m >= insert_chunk_min(n) && capture == cudaStreamCaptureStatusNone;
     void *dp = nullptr, *scratch = nullptr;
     if (chunks) {
         bmlp_status got = ws_get(ctx, WS_INS_FACTS, hp.size() * sizeof(int32_t), &dp);
