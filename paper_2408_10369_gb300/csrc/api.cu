@@ -1246,6 +1246,8 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
     const int64_t ldw = round_up(words_of(n), 2);
     if (ldw > smp_packed_max_words())
         return set_err(ctx, BMLP_ERR_UNSUPPORTED, "packed frontier path supports n <= %d", smp_packed_max_words() * 64);
+    // query rows: R is only read, so packed rows of the working width without padding bits are used where they are
+    const bool rows_in_place = !square_first && fmt == BMLP_FMT_PACKED64 && words_of(n) == ldw && n % 64 == 0;
     // a few query rows: expanded straight from R's rows, each row of a reached constant read once
     RowState begun{nullptr, nullptr};  // rows that stopped there, to be finished over the word indexes
     int row_levels = 0;
@@ -1254,29 +1256,51 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
         const uint64_t* rows = static_cast<const uint64_t*>(R.dev);
         if (fmt == BMLP_FMT_U8) {
             void* p = nullptr;
-            ST(ws_get(ctx, WS_M0, static_cast<size_t>(n * wpr * 8), &p));
+            ST(ws_get(ctx, WS_M0, static_cast<size_t>(n * (plan.may_stop ? ldw : wpr) * 8), &p));
             ST(to_packed(ctx, R, fmt, n, static_cast<uint64_t*>(p), wpr, s));
             rows = static_cast<const uint64_t*>(p);
         }
         if (plan.may_stop) {
             void* p = nullptr;
-            ST(ws_get(ctx, WS_ROWS, static_cast<size_t>(q * 3 * wpr * 8 + q * 4), &p));
-            begun.words = static_cast<uint64_t*>(p);
-            begun.levels = reinterpret_cast<int*>(begun.words + q * 3 * wpr);
+            const bmlp_status got = ws_get(ctx, WS_ROWS, static_cast<size_t>(q * 3 * wpr * 8 + q * 4), &p);
+            if (got != BMLP_OK && got != BMLP_ERR_OOM) return got;
+            if (got == BMLP_OK) {  // else no row stops
+                begun.words = static_cast<uint64_t*>(p);
+                begun.levels = reinterpret_cast<int*>(begun.words + q * 3 * wpr);
+            }
         }
-        ProductTimer tm{ctx, o.profile != 0, s};
-        ST(tm.begin());
-        CK(launch_smp_rows(rows, wpr, n, src, ldw_src, q, out, ldw_out, o.reflexive, ctx->d_ctl + CTL_LEVELS,
-                           static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), plan, begun, ctx->d_ctl + CTL_STEP, s,
-                           deadline_of(ctx)),
-           "query row kernel launch");
-        ST(tm.end());
-        ctx->stats.product_launches++;
-        ctx->stats.launches++;
-        ST(read_ctl(ctx, s, nullptr));
-        ST(tm.collect());
+        const auto expand_rows = [&](const uint64_t* from, int64_t ld_from, RowState state) -> bmlp_status {
+            ProductTimer tm{ctx, o.profile != 0, s};
+            ST(tm.begin());
+            CK(launch_smp_rows(rows, wpr, n, from, ld_from, q, out, ldw_out, o.reflexive, ctx->d_ctl + CTL_LEVELS,
+                               static_cast<int>(n + 1 < 0x7FFFFFFF ? n + 1 : 0x7FFFFFFF), plan, state, ctx->d_ctl + CTL_STEP,
+                               s, deadline_of(ctx)),
+               "query row kernel launch");
+            ST(tm.end());
+            ctx->stats.product_launches++;
+            ctx->stats.launches++;
+            ST(read_ctl(ctx, s, nullptr));
+            return tm.collect();
+        };
+        ST(expand_rows(src, ldw_src, begun));
         row_levels = ctx->h_ctl[CTL_LEVELS];
-        if (ctx->h_ctl[CTL_STEP] == 0) {
+        bool done = ctx->h_ctl[CTL_STEP] == 0;
+        if (!done) {
+            // the workspaces of the rest of this call; no room for them: the stopped rows from their sources to their ends
+            WordIndex xi;
+            void* p = nullptr;
+            bmlp_status got = index_buffers(ctx, n, ldw, WS_WPTR, WS_WIDX, WS_WVAL, &xi);
+            if (got == BMLP_OK) got = index_buffers(ctx, n, ldw, WS_WPTRT, WS_WIDXT, WS_WVALT, &xi);
+            if (got == BMLP_OK) got = ws_get(ctx, WS_PT, static_cast<size_t>(n * ldw * 8), &p);
+            if (got == BMLP_OK && !rows_in_place) got = ws_get(ctx, WS_M0, static_cast<size_t>(n * ldw * 8), &p);
+            if (got != BMLP_OK && got != BMLP_ERR_OOM) return got;
+            if (got == BMLP_ERR_OOM) {
+                ST(expand_rows(begun.words + 2 * wpr, 3 * wpr, RowState{nullptr, begun.levels}));
+                row_levels = ctx->h_ctl[CTL_LEVELS];
+                done = true;
+            }
+        }
+        if (done) {
             *levels = row_levels;
             const int cap = o.max_iters > 0 ? o.max_iters : static_cast<int>(n + 1);
             if (*levels > cap) return set_err(ctx, BMLP_ERR_NOT_CONVERGED, "frontier did not empty within %d levels", cap);
@@ -1286,9 +1310,7 @@ bmlp_status smp_packed_run(bmlp_ctx* ctx, const Operand& R, int32_t fmt, int64_t
     void* P = nullptr;
     WordIndex x;
     ST(index_buffers(ctx, n, ldw, WS_WPTR, WS_WIDX, WS_WVAL, &x));
-    if (!square_first && fmt == BMLP_FMT_PACKED64 && words_of(n) == ldw && n % 64 == 0) {
-        // query rows: R is only read, so packed rows of the working width without padding bits are used where
-        // they are
+    if (rows_in_place) {
         P = const_cast<void*>(R.dev);
     } else {
         ST(ws_get(ctx, WS_M0, static_cast<size_t>(n * ldw * 8), &P));

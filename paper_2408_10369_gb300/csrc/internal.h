@@ -376,7 +376,8 @@ cudaError_t launch_smp_tiles(const WordIndex& x, int64_t n, int64_t n1, int64_t 
 // The expansion of a few query rows straight from R's packed rows (ld_r words, bits at columns >= n ignored), one cluster
 // of plan.ctas CTAs per row: 16, 8, 4 or 2, or 0 when q rows do not fit the GPU at once (or are more than kRowsMaxQueries) or
 // n is too large. Results and levels as launch_smp_tiles, but for rows that stop (only with plan.may_stop and a `state`, and
-// *stopped is raised then): launch_smp_packed finishes those from the state.
+// *stopped is raised then): launch_smp_packed finishes those from the state, or a second launch from their sources in it
+// (src = words + 2 ceil(n / 64), ld_src = 3 ceil(n / 64), state {null, levels}), which leaves the others' results as they are.
 constexpr int64_t kRowsMaxQueries = 63;
 struct RowQueryPlan {
     int ctas;

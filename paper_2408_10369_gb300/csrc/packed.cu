@@ -1449,7 +1449,7 @@ __global__ void __launch_bounds__(kSlicedThreads) smp_sliced_kernel(const int64_
 //   levels of the cluster, over the indexes and so: n = 500: 1,336, 740 and 418 us; 5,000: 13.6, 6.8 and 3.8 ms.
 // * Beyond that size, deep or wide rows on large relations, whose levels or bytes cost more than building the indexes and
 //   going on there: the cluster writes down its frontier and visited set and stops (RowQueryPlan says when), and the call
-//   goes on from them over the indexes.
+//   goes on from them over the indexes (where these have no room on the device, from the sources again, without stopping).
 constexpr int kRowsThreads = 512;
 constexpr int kRowsWarps = kRowsThreads / 32;
 constexpr int kRowsMaxCtas = 16;
@@ -1470,7 +1470,8 @@ struct RowQueryArgs {
     int max_levels;
     int reflexive;
     RowQueryPlan plan;
-    RowState state;  // where a row that stops leaves its frontier, visited set and source (words null: none stops)
+    RowState state;  // where a row that stops leaves its frontier, visited set and source (words null: none stops, and with
+                     // levels only the rows that stopped before are expanded)
     int* stopped;    // raised when one does
     Deadline dl;
 };
@@ -1571,6 +1572,8 @@ __global__ void __launch_bounds__(kRowsThreads) smp_rows_kernel(const RowQueryAr
     uint64_t* V = rq_sm + 3 * wpr;  // visited, own words
     const uint64_t* src = a.src + static_cast<int64_t>(cluster_id_x()) * a.ld_src;
     uint64_t* out = a.out + static_cast<int64_t>(cluster_id_x()) * a.ld_out;
+    // finished by an earlier launch: the whole cluster leaves
+    if (!kNarrow && a.state.words == nullptr && a.state.levels != nullptr && a.state.levels[cluster_id_x()] == 0) return;
     const auto valid = [&](int w) {
         const int64_t v = a.n - 64ll * w;
         return v < 64 ? (1ull << v) - 1ull : ~0ull;
