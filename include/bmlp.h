@@ -39,10 +39,10 @@
  * has been decided (see bmlp_options.loop); host outputs are complete on
  * return. A context has one workspace for all of its calls: before a call on
  * another stream of the same context, the caller waits for the earlier ones or
- * orders the streams with an event. Insertions of three or more facts into
- * packed device closures order themselves with one another; insertions of
- * fewer facts into these, and unions and negations whose operands are separate
- * device memory, use no workspace.
+ * orders the streams with an event. Insertions into packed device closures
+ * need neither: those of many facts order themselves with one another, those
+ * of a few (up to two, or three for n <= 8192) use no workspace. Nor do unions
+ * and negations whose operands are separate device memory.
  *
  * Errors: every entry point returns a bmlp_status; nothing is thrown across
  * the ABI. bmlp_last_error() gives a message for the last failure on a
