@@ -2115,7 +2115,9 @@ static bmlp_status core_compose(bmlp_ctx* ctx, const void* R1, const void* R2, i
         if (st != BMLP_OK) return st;
         ST(to_packed(ctx, a, fmt, n, A1, ldw, s));
         bool indexed = false;
-        if (xc.ptr != nullptr && kSparseStepS < table_product_s(n)) {  // else not even an empty index product could win
+        // (up to some 4,300 constants not even an empty index product could win: with an empty R2 and n = 400, 1,500,
+        // 3,000 and 4,200 a call takes 106, 129, 145 and 169 us without the choice, 124, 145, 169 and 195 with it)
+        if (xc.ptr != nullptr && kSparseStepS < table_product_s(n)) {
             // a sparse closure: R1 + R2+ R1 through the word indexes of R2+ and R1, unless that is predicted to cost more
             // than the whole-row product, whose tables cost as much for few ones as for many
             WordIndex xr;
